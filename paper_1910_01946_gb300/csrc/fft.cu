@@ -1,4 +1,4 @@
-// Hand-written batched 3-D real FFT of tensor-component fields (FP64, and
+// Hand-written batched 3-D real FFT of tensor-component fields (FP64 data, and
 // FP32 for the mixed-precision conjugate gradients), with the frequency-space operators of the method fused between the
 // forward and inverse transforms along z:
 //   - the Galerkin projection with mixed control (Sec. 2.2, Eqs. weakarbi,
@@ -7,266 +7,474 @@
 //     with the same rotated-scheme derivative.
 //
 // Layout.  Real fields: [c][z][y][x] (x fastest).  Half spectrum:
-// [c][z][y][kx], kx = 0..n0/2.  Passes (each a kernel, each transform staged
-// in shared memory and done by a mixed-radix 8/4/2/3 Stockham autosort):
+// [c][z][y][kx], kx = 0..n0/2.  Passes (each a kernel):
 //   X  (R2C): two real rows y, y+1 packed as one complex row, one length-n0
 //             FFT, then the two half spectra are separated;
-//   Y  (C2C): tiles of consecutive kx columns, length-n1 FFTs;
-//   Z  (C2C + operator + C2C): the three fields of one tensor row i for a tile
-//             of (kx, ky) pencils (both operators act row by row), forward
-//             z FFT, operator, inverse z FFT;
+//   Y  (C2C): consecutive columns (z, kx), length-n1 FFTs;
+//   Z  (C2C + operator + C2C): pencils of consecutive (ky, kx), forward z
+//             FFT, operator, inverse z FFT;
 //   Y^-1, X^-1 (C2R).  The 1/nvox scaling is folded into the operator.
+//
+// A transform is held by T = n / R0 threads (R0: its first, largest radix), one
+// butterfly of R0 points per thread and pass.  The first butterfly takes its
+// points from global memory straight into registers, the last one of a Y or Z
+// transform stores to global memory, and only the passes between exchange
+// through shared memory (double-buffered: one barrier per pass).
+//
+// Arithmetic.  FP32 fields are transformed in FP32.  FP64 fields are
+// transformed in 64-bit fixed point (fix64.cuh): the FP64 pipe of this GPU
+// does 2 lanes per clock and SM and held every FP64 pass of a 64^3 grid to
+// 24-50 us, where the bytes need about 2.  A block takes the
+// largest magnitude of each transform's values, converts them to integers on that
+// scale with 57 or more bits (so that no sum of the transform can overflow),
+// and converts back on the way out.  Twiddles are Q62; a twiddled pass leaves the
+// values a factor 4 down (the high words of the products, no shift), which is about what its
+// sums grow by.  The rounding errors of a pass are 0.3 units of 2^-57 ...
+// 2^-53 of the transform's largest value, below the 2^-53 of each
+// intermediate value that every FP64 operation of a butterfly would leave.
+#include <cmath>
+#include <type_traits>
+
 #include "common.cuh"
+#include "fix64.cuh"
 #include "rve_internal.h"
 
 namespace {
 
-// complex value and storage pair type of a real type R (double or float)
-template <typename R> struct CX { R x, y; };
-template <typename R> struct V2T;
-template <> struct V2T<double> { typedef double2 t; };
-template <> struct V2T<float> { typedef float2 t; };
-template <typename R> using V2 = typename V2T<R>::t;
+using fix64::i64;
 
-template <typename R> __device__ __forceinline__ CX<R> mk(R a, R b) { CX<R> c; c.x = a; c.y = b; return c; }
-template <typename R> __device__ __forceinline__ CX<R> add(CX<R> a, CX<R> b) { return mk<R>(a.x + b.x, a.y + b.y); }
-template <typename R> __device__ __forceinline__ CX<R> sub(CX<R> a, CX<R> b) { return mk<R>(a.x - b.x, a.y - b.y); }
-template <typename R> __device__ __forceinline__ CX<R> scl(CX<R> a, R s) { return mk<R>(a.x * s, a.y * s); }
-template <typename R> __device__ __forceinline__ V2<R> st2(R a, R b) { V2<R> v; v.x = a; v.y = b; return v; }
+// storage pair, arithmetic type and twiddle type of a field type R
+template <typename R> struct FT;
+template <> struct FT<double> { typedef double2 pair; typedef i64 w; typedef int4 tw; };
+template <> struct FT<float> { typedef float2 pair; typedef float w; typedef float2 tw; };
+template <typename R> using V2 = typename FT<R>::pair;
+template <typename W> struct CX { W x, y; };
+template <typename R> using C = CX<typename FT<R>::w>;
+template <typename R> using TW = typename FT<R>::tw;
 
+template <typename W> __device__ __forceinline__ CX<W> mk(W a, W b) { CX<W> c; c.x = a; c.y = b; return c; }
+template <typename W> __device__ __forceinline__ CX<W> add(CX<W> a, CX<W> b) { return mk<W>(a.x + b.x, a.y + b.y); }
+template <typename W> __device__ __forceinline__ CX<W> sub(CX<W> a, CX<W> b) { return mk<W>(a.x - b.x, a.y - b.y); }
+template <int SIGN, typename W>
+__device__ __forceinline__ CX<W> mul_i(CX<W> a) { return SIGN > 0 ? mk<W>(-a.y, a.x) : mk<W>(a.y, -a.x); }
+__device__ __forceinline__ double2 st2(double a, double b) { return make_double2(a, b); }
+__device__ __forceinline__ float2 st2(float a, float b) { return make_float2(a, b); }
+
+// x / sqrt 2, x sqrt(3) / 2, x / 2
+__device__ __forceinline__ float by_r2(float x) { return 0.70710678f * x; }
+__device__ __forceinline__ float by_s3(float x) { return 0.86602540f * x; }
+__device__ __forceinline__ float by_half(float x) { return 0.5f * x; }
+constexpr i64 Q62_R2 = 3260954456333195553LL, Q62_S3 = 3993837246235628775LL;   // round(2^62 /sqrt 2), round(2^62 sqrt 3 /2)
+__host__ __device__ constexpr int q62_lo(i64 v) { return (int)(uint32_t)(uint64_t)v; }
+__host__ __device__ constexpr int q62_hi(i64 v) { return (int)((v - (i64)q62_lo(v)) >> 32); }
+__device__ __forceinline__ i64 by_r2(i64 x) { return fix64::mulq(x, q62_hi(Q62_R2), q62_lo(Q62_R2)); }
+__device__ __forceinline__ i64 by_s3(i64 x) { return fix64::mulq(x, q62_hi(Q62_S3), q62_lo(Q62_S3)); }
+__device__ __forceinline__ i64 by_half(i64 x) { return x >> 1; }
+
+// a * w (SIGN < 0) or a * conj(w) with w from the forward table
+template <int SIGN>
+__device__ __forceinline__ CX<float> twiddle(CX<float> a, const float2* tw, int idx) {
+  const float2 w = __ldg(tw + idx);
+  if (SIGN < 0) return mk<float>(fmaf(a.x, w.x, -a.y * w.y), fmaf(a.x, w.y, a.y * w.x));
+  return mk<float>(fmaf(a.x, w.x, a.y * w.y), fmaf(a.y, w.x, -a.x * w.y));
+}
+template <int SIGN>
+__device__ __forceinline__ CX<i64> twiddle(CX<i64> a, const int4* tw, int idx) {
+  const int4 w = __ldg(tw + idx);              // cosine (high, low), sine of the forward factor
+  const fix64::Sp x = fix64::split(a.x), y = fix64::split(a.y);
+  // (the result is a factor 4 down)
+  if (SIGN < 0) return mk<i64>(fix64::mulq2(x, w.x, w.y, y, -w.z, -w.w), fix64::mulq2(x, w.z, w.w, y, w.x, w.y));
+  return mk<i64>(fix64::mulq2(x, w.x, w.y, y, w.z, w.w), fix64::mulq2(y, w.x, w.y, x, -w.z, -w.w));
+}
+
+// ---- DFTs of RAD points in registers, natural order in and out ----
+template <int SIGN, typename W>
+__device__ __forceinline__ void dft3(CX<W>& a0, CX<W>& a1, CX<W>& a2) {
+  const CX<W> t = add(a1, a2), d = mul_i<SIGN, W>(sub(a1, a2));
+  const CX<W> u = mk<W>(by_s3(d.x), by_s3(d.y));
+  const CX<W> m = mk<W>(a0.x - by_half(t.x), a0.y - by_half(t.y));
+  a0 = add(a0, t);
+  a1 = add(m, u);
+  a2 = sub(m, u);
+}
+template <int SIGN, typename W>
+__device__ __forceinline__ void dft4(CX<W>& a0, CX<W>& a1, CX<W>& a2, CX<W>& a3) {
+  const CX<W> t0 = add(a0, a2), t1 = sub(a0, a2), t2 = add(a1, a3), t3 = mul_i<SIGN, W>(sub(a1, a3));
+  a0 = add(t0, t2);
+  a1 = add(t1, t3);
+  a2 = sub(t0, t2);
+  a3 = sub(t1, t3);
+}
+template <int SIGN, int RAD, typename W>
+__device__ __forceinline__ void dft(CX<W>* a) {
+  if (RAD == 2) {
+    const CX<W> t = a[0];
+    a[0] = add(t, a[1]);
+    a[1] = sub(t, a[1]);
+  } else if (RAD == 3) {
+    dft3<SIGN, W>(a[0], a[1], a[2]);
+  } else if (RAD == 4) {
+    dft4<SIGN, W>(a[0], a[1], a[2], a[3]);
+  } else if (RAD == 6) {
+    // Good-Thomas 2 x 3: input 3 i + 2 l, output 3 k1 + 4 k2 (mod 6), no factors between
+    CX<W> b0 = a[0], b1 = a[2], b2 = a[4], c0 = a[3], c1 = a[5], c2 = a[1];
+    dft3<SIGN, W>(b0, b1, b2);
+    dft3<SIGN, W>(c0, c1, c2);
+    a[0] = add(b0, c0); a[3] = sub(b0, c0);
+    a[4] = add(b1, c1); a[1] = sub(b1, c1);
+    a[2] = add(b2, c2); a[5] = sub(b2, c2);
+  } else {
+    // radix 8: a radix-2 step (a_m +/- a_{m+4}), the factors W8^m on the
+    // differences, then two radix-4 DFTs (even and odd outputs)
+    CX<W> b[4], c[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) { b[m] = add(a[m], a[m + 4]); c[m] = sub(a[m], a[m + 4]); }
+    const CX<W> c1 = c[1], c3 = c[3];
+    if (SIGN < 0) {
+      c[1] = mk<W>(by_r2(c1.x + c1.y), by_r2(c1.y - c1.x));
+      c[3] = mk<W>(by_r2(c3.y - c3.x), -by_r2(c3.x + c3.y));
+    } else {
+      c[1] = mk<W>(by_r2(c1.x - c1.y), by_r2(c1.x + c1.y));
+      c[3] = mk<W>(-by_r2(c3.x + c3.y), by_r2(c3.x - c3.y));
+    }
+    c[2] = mul_i<SIGN, W>(c[2]);
+    dft4<SIGN, W>(b[0], b[1], b[2], b[3]);
+    dft4<SIGN, W>(c[0], c[1], c[2], c[3]);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) { a[2 * m] = b[m]; a[2 * m + 1] = c[m]; }
+  }
+}
+
+constexpr int RMAX = 8;                 // largest radix
+
+// plan of one axis as the kernels take it
 struct PlanDev {
-  int n, npass;
-  int radix[RVE_MAX_RADIX_PASSES];
+  int n, npass, r0, T;                  // length, passes, first radix, threads per transform (n / r0)
+  int bits;                             // B: bits of a converted input (fixed point)
+  int down;                             // bits a fixed-point transform's values have moved down at its end
+  unsigned tdiv;                        // ceil(2^20 / T)
+  int radix[RVE_MAX_RADIX_PASSES], ns[RVE_MAX_RADIX_PASSES], step[RVE_MAX_RADIX_PASSES];
+  unsigned nsdiv[RVE_MAX_RADIX_PASSES]; // ceil(2^20 / ns)
 };
 
+// j / d for 0 <= j < 512 and 1 <= d <= 512 with m = ceil(2^20 / d): the
+// error j (m d - 2^20) / (2^20 d) stays below 1 / d
+__device__ __forceinline__ int fdiv(int j, unsigned m) { return (int)(((unsigned)j * m) >> 20); }
+unsigned div_magic(int d) { return ((1u << 20) + (unsigned)d - 1u) / (unsigned)d; }
+
 PlanDev to_dev(const FFTPlan& p) {
-  PlanDev d;
+  PlanDev d{};
   d.n = p.n;
   d.npass = p.npass;
-  for (int i = 0; i < RVE_MAX_RADIX_PASSES; ++i) d.radix[i] = p.radix[i];
+  d.T = p.npass > 0 ? p.n / p.radix[0] : 1;
+  d.r0 = p.npass > 0 ? p.radix[0] : 1;
+  d.tdiv = div_magic(d.T);
+  // A component below 2^B has |z| < 2^(B + 1/2) and a pass of radix r grows it
+  // by at most r; a twiddled pass (all but the first) takes values below
+  // 2^62 and moves them 2 bits down; the results stay below 2^61.5, so that
+  // the sums of the X passes' split fit
+  double grown = 0.5, bits = 61.0;
+  for (int i = 0; i < p.npass; ++i) {
+    if (i) {
+      bits = std::fmin(bits, 62.0 - grown);
+      grown -= 2.0;
+    }
+    grown += std::log2((double)p.radix[i]);
+  }
+  bits = std::fmin(bits, 61.5 - grown);
+  d.bits = (int)std::floor(bits + 1e-9);
+  d.down = p.npass > 1 ? 2 * (p.npass - 1) : 0;
+  int ns = 1;
+  for (int i = 0; i < p.npass; ++i) {
+    d.radix[i] = p.radix[i];
+    d.ns[i] = ns;
+    d.nsdiv[i] = div_magic(ns);
+    d.step[i] = p.n / (ns * p.radix[i]);
+    ns *= p.radix[i];
+  }
   return d;
 }
 
-// a * w or a * conj(w) (w from the forward table) with the sign fixed at
-// compile time, so the negation folds into the FMA operands; float
-// transforms read the float table
-template <int SIGN, typename R>
-__device__ __forceinline__ CX<R> twiddle(CX<R> a, const V2<R>* tw, int idx) {
-  const V2<R> w = __ldg(tw + idx);
-  if (SIGN < 0) return mk<R>(fma(a.x, w.x, -a.y * w.y), fma(a.x, w.y, a.y * w.x));
-  return mk<R>(fma(a.x, w.x, a.y * w.y), fma(a.y, w.x, -a.x * w.y));
+// the untwiddled point of a twiddled pass, on the scale of the others
+__device__ __forceinline__ CX<float> untwiddled(CX<float> a) { return a; }
+__device__ __forceinline__ CX<i64> untwiddled(CX<i64> a) { return mk<i64>((a.x + 2) >> 2, (a.y + 2) >> 2); }
+
+// Pass p of radix RAD of one transform: points ld(pos), results st(pos, value)
+template <int SIGN, typename R, int RAD, class Ld, class St>
+__device__ __forceinline__ void pass_r(const PlanDev& pl, int p, int tj, const TW<R>* __restrict__ tw, Ld ld, St st) {
+  const int nb = pl.n / RAD, ns = pl.ns[p];
+  for (int j = tj; j < nb; j += pl.T) {
+    C<R> a[RAD];
+#pragma unroll
+    for (int m = 0; m < RAD; ++m) a[m] = ld(j + m * nb);
+    const int q = fdiv(j, pl.nsdiv[p]), k = j - q * ns;
+    a[0] = untwiddled(a[0]);
+#pragma unroll
+    for (int m = 1; m < RAD; ++m) a[m] = twiddle<SIGN>(a[m], tw, m * k * pl.step[p]);
+    dft<SIGN, RAD>(a);
+    const int d = q * ns * RAD + k;
+#pragma unroll
+    for (int m = 0; m < RAD; ++m) st(d + m * ns, a[m]);
+  }
 }
 
-template <int SIGN, typename R>
-__device__ __forceinline__ CX<R> mul_i(CX<R> a) { return SIGN > 0 ? mk<R>(-a.y, a.x) : mk<R>(a.y, -a.x); }
-
-// One Stockham pass of radix R over `howmany` contiguous transforms of length
-// N from src to dst (both shared memory).
-template <int SIGN, typename RT>
-__device__ void stockham_pass(const CX<RT>* __restrict__ src, CX<RT>* __restrict__ dst, int N, int howmany,
-                              int R, int Ns, const V2<RT>* tw) {
-  typedef CX<RT> cplx;
-  const int nb = N / R;
-  const int total = nb * howmany;
-  const int twstep = N / (Ns * R);
-  for (int b = threadIdx.x; b < total; b += blockDim.x) {
-    const int tr = b / nb;
-    const int j = b - tr * nb;
-    const int k = j % Ns;
-    const cplx* X = src + tr * N;
-    cplx* Y = dst + tr * N;
-    const int d = (j / Ns) * Ns * R + k;
-    if (R == 8) {
-      // radix 8 as a radix-2 step (a_m +/- a_{m+4}), the factors W8^m on the
-      // differences, then two radix-4 DFTs (even and odd outputs)
-      cplx a[8];
+// The transform whose first butterfly's points (tj + m T) are in a[]: the
+// first pass writes b0, the others alternate b1, b0, ...; the caller
+// synchronises before it reads the result (in natural order) from the buffer
+// returned, the same for every thread.  idx maps a position of this thread's
+// transform to its shared-memory element.  All threads of the block call it
+// (barriers); `on`: this thread holds a transform.
+//
+// The results are converted and stored by a rolled loop of the caller and not
+// by the butterflies: inlined into every radix, the conversions made the code
+// a warp runs once so long that fetching it was the largest stall (6-8
+// cycles per instruction issued; y pass at 64^3 12 us instead of 8).
+template <int SIGN, typename R, class Idx>
+__device__ __forceinline__ C<R>* transform(C<R>* a, C<R>* b0, C<R>* b1, const PlanDev& pl, int tj, bool on, Idx idx,
+                                           const TW<R>* __restrict__ tw) {
+  if (on) {
+    auto first = [&](auto rad) {
+      constexpr int RAD = decltype(rad)::value;
+      dft<SIGN, RAD>(a);
 #pragma unroll
-      for (int m = 0; m < 8; ++m) a[m] = X[j + m * nb];
-      if (k) {
-#pragma unroll
-        for (int m = 1; m < 8; ++m) a[m] = twiddle<SIGN, RT>(a[m], tw, m * k * twstep);
-      }
-      const RT r2 = (RT)0.70710678118654752440;    // 1/sqrt(2)
-      cplx b[4], c[4];
-#pragma unroll
-      for (int m = 0; m < 4; ++m) { b[m] = add(a[m], a[m + 4]); c[m] = sub(a[m], a[m + 4]); }
-      // c1 *= W8^(sign), c2 *= -/+ i, c3 *= W8^(3 sign)
-      {
-        const cplx c1 = c[1], c3 = c[3];
-        if (SIGN < 0) {
-          c[1] = mk<RT>(r2 * (c1.x + c1.y), r2 * (c1.y - c1.x));
-          c[3] = mk<RT>(r2 * (c3.y - c3.x), -r2 * (c3.x + c3.y));
-        } else {
-          c[1] = mk<RT>(r2 * (c1.x - c1.y), r2 * (c1.x + c1.y));
-          c[3] = mk<RT>(-r2 * (c3.x + c3.y), r2 * (c3.x - c3.y));
-        }
-        c[2] = mul_i<SIGN, RT>(c[2]);
-      }
-      const cplx t0 = add(b[0], b[2]), t1 = sub(b[0], b[2]), t2 = add(b[1], b[3]), t3 = mul_i<SIGN, RT>(sub(b[1], b[3]));
-      const cplx u0 = add(c[0], c[2]), u1 = sub(c[0], c[2]), u2 = add(c[1], c[3]), u3 = mul_i<SIGN, RT>(sub(c[1], c[3]));
-      Y[d] = add(t0, t2);
-      Y[d + 4 * Ns] = sub(t0, t2);
-      Y[d + 2 * Ns] = add(t1, t3);
-      Y[d + 6 * Ns] = sub(t1, t3);
-      Y[d + Ns] = add(u0, u2);
-      Y[d + 5 * Ns] = sub(u0, u2);
-      Y[d + 3 * Ns] = add(u1, u3);
-      Y[d + 7 * Ns] = sub(u1, u3);
-    } else if (R == 4) {
-      cplx a0 = X[j], a1 = X[j + nb], a2 = X[j + 2 * nb], a3 = X[j + 3 * nb];
-      if (k) {
-        a1 = twiddle<SIGN, RT>(a1, tw, k * twstep);
-        a2 = twiddle<SIGN, RT>(a2, tw, 2 * k * twstep);
-        a3 = twiddle<SIGN, RT>(a3, tw, 3 * k * twstep);
-      }
-      cplx t0 = add(a0, a2), t1 = sub(a0, a2), t2 = add(a1, a3), t3 = mul_i<SIGN, RT>(sub(a1, a3));
-      Y[d] = add(t0, t2);
-      Y[d + Ns] = add(t1, t3);
-      Y[d + 2 * Ns] = sub(t0, t2);
-      Y[d + 3 * Ns] = sub(t1, t3);
-    } else if (R == 2) {
-      cplx a0 = X[j], a1 = X[j + nb];
-      if (k) a1 = twiddle<SIGN, RT>(a1, tw, k * twstep);
-      Y[d] = add(a0, a1);
-      Y[d + Ns] = sub(a0, a1);
-    } else {  // R == 3
-      cplx a0 = X[j], a1 = X[j + nb], a2 = X[j + 2 * nb];
-      if (k) {
-        a1 = twiddle<SIGN, RT>(a1, tw, k * twstep);
-        a2 = twiddle<SIGN, RT>(a2, tw, 2 * k * twstep);
-      }
-      const RT s3 = (RT)0.86602540378443864676;  // sqrt(3)/2
-      cplx t = add(a1, a2);
-      cplx u = scl(mul_i<SIGN, RT>(sub(a1, a2)), s3);
-      cplx m = mk<RT>(fma((RT)-0.5, t.x, a0.x), fma((RT)-0.5, t.y, a0.y));
-      Y[d] = add(a0, t);
-      Y[d + Ns] = add(m, u);
-      Y[d + 2 * Ns] = sub(m, u);
+      for (int m = 0; m < RAD; ++m) b0[idx(tj * RAD + m)] = a[m];
+    };
+    switch (pl.radix[0]) {
+      case 8: first(std::integral_constant<int, 8>()); break;
+      case 6: first(std::integral_constant<int, 6>()); break;
+      case 4: first(std::integral_constant<int, 4>()); break;
+      case 3: first(std::integral_constant<int, 3>()); break;
+      case 2: first(std::integral_constant<int, 2>()); break;
+      default: b0[idx(0)] = a[0]; break;
     }
   }
+  for (int p = 1; p < pl.npass; ++p) {
+    __syncthreads();
+    if (on) {
+      C<R>* src = (p & 1) ? b0 : b1;
+      C<R>* dst = (p & 1) ? b1 : b0;
+      auto ld = [&](int pos) { return src[idx(pos)]; };
+      auto st = [&](int pos, C<R> v) { dst[idx(pos)] = v; };
+      switch (pl.radix[p]) {
+        case 8: pass_r<SIGN, R, 8>(pl, p, tj, tw, ld, st); break;
+        case 6: pass_r<SIGN, R, 6>(pl, p, tj, tw, ld, st); break;
+        case 4: pass_r<SIGN, R, 4>(pl, p, tj, tw, ld, st); break;
+        case 3: pass_r<SIGN, R, 3>(pl, p, tj, tw, ld, st); break;
+        default: pass_r<SIGN, R, 2>(pl, p, tj, tw, ld, st); break;
+      }
+    }
+  }
+  return (pl.npass > 1 && !(pl.npass & 1)) ? b1 : b0;
 }
 
-// Full transform of `howmany` contiguous length-N sequences; the caller has
-// synchronised after filling `a`.  Returns the buffer that holds the result.
-template <int SIGN, typename RT>
-__device__ CX<RT>* block_fft(CX<RT>* a, CX<RT>* b, const PlanDev& pl, int howmany, const V2<RT>* tw) {
-  int Ns = 1;
-  for (int p = 0; p < pl.npass; ++p) {
-    const int R = pl.radix[p];
-    stockham_pass<SIGN, RT>(a, b, pl.n, howmany, R, Ns, tw);
+// ---- conversions: doubles on the block's common scale, floats as they are ----
+__device__ __forceinline__ unsigned mag_of(double2 v) { return max(fix64::mag(v.x), fix64::mag(v.y)); }
+__device__ __forceinline__ unsigned mag_of(float2) { return 0u; }
+__device__ __forceinline__ unsigned mag_of(double v) { return fix64::mag(v); }
+__device__ __forceinline__ unsigned mag_of(float) { return 0u; }
+__device__ __forceinline__ i64 to_work(double x, int s0) { return fix64::to_fix(x, s0); }
+__device__ __forceinline__ float to_work(float x, int) { return x; }
+template <typename R> __device__ __forceinline__ R from_work(typename FT<R>::w v, int eb);
+template <> __device__ __forceinline__ double from_work<double>(i64 v, int eb) { return fix64::from_fix(v, eb); }
+template <> __device__ __forceinline__ float from_work<float>(float v, int) { return v; }
+
+// Exponent of the largest magnitude of a transform's points (FP64; all
+// threads call it).  Each transform has its own: the spectra of neighbouring
+// columns differ by orders of magnitude (the divergence has almost nothing
+// near the Nyquist frequencies, where the inverse Laplacian is largest), and a
+// column on a larger scale than its own would lose what FP64 keeps.
+// Columns (Y, Z): the transform of column c is held by the threads c, c + cpb, ...
+// (cpb a power of two <= 32): shuffles within the warps, one word per warp and
+// column across them.
+constexpr int MAX_WARPS = 8;
+template <typename R>
+__device__ __forceinline__ int column_exp(unsigned key, int cpb, unsigned* red) {
+  if (sizeof(R) == 4) return 0;
+  for (int o = cpb; o < 32; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
+  const int nw = blockDim.x >> 5;
+  if (nw > 1) {
+    const int lane = threadIdx.x & 31, c = lane & (cpb - 1);
+    if (lane < cpb) red[(threadIdx.x >> 5) * 32 + lane] = key;
     __syncthreads();
-    CX<RT>* t = a; a = b; b = t;
-    Ns *= R;
+    for (int w = 0; w < nw; ++w) key = max(key, red[w * 32 + c]);
   }
-  return a;
+  return fix64::tile_exp(key);
 }
+// Rows (X): T consecutive threads.  T a power of two up to 32: shuffles only;
+// other lengths share the block's largest magnitude (rows next to each other
+// in real space, or of one kx range).
+template <typename R>
+__device__ __forceinline__ int row_exp(unsigned key, int T, unsigned* red) {
+  if (sizeof(R) == 4) return 0;
+  if (T <= 32 && (T & (T - 1)) == 0) {
+    for (int o = 1; o < T; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
+    return fix64::tile_exp(key);
+  }
+  key = __reduce_max_sync(0xffffffffu, key);
+  const int nw = blockDim.x >> 5;
+  if (nw > 1) {
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = key;
+    __syncthreads();
+    for (int w = 0; w < nw; ++w) key = max(key, red[w]);
+  }
+  return fix64::tile_exp(key);
+}
+
+extern __shared__ __align__(16) unsigned char fft_smem[];
+
+// element of position p of row `row` in the X passes (one pad element every
+// eight: the strided writes of a radix-8 pass spread over the banks)
+__device__ __forceinline__ int row_elem(int row, int n, int p) { return row * (n + (n >> 3) + 1) + p + (p >> 3); }
 
 // ---------------------------------------------------------------- pass X (R2C)
-// in: real fields (type R); spec: half spectrum (pairs of R)
+// in: real fields (type R); spec: half spectrum (pairs of R).  rows: number of
+// row pairs over all fields; rpb of them per block, T threads each.
 template <typename R>
-__global__ void __launch_bounds__(256) k_fft_x_r2c(const R* __restrict__ in, V2<R>* __restrict__ spec,
-                                                   int n0, int n1, int n2, int nkx, int rpb, PlanDev pl,
-                                                   const V2<R>* __restrict__ tw, const double* __restrict__ done) {
-  typedef CX<R> cplx;
-  if (done && *done != 0.0) return;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  cplx* a = reinterpret_cast<cplx*>(smraw);
-  cplx* b = a + rpb * n0;
-  const int f = blockIdx.z, z = blockIdx.y, j0 = blockIdx.x * rpb;
-  const size_t nvox = (size_t)n0 * n1 * n2;
-  const R* src = in + f * nvox + (size_t)z * n1 * n0;
-  for (int e = threadIdx.x; e < rpb * n0; e += blockDim.x) {
-    const int jj = e / n0, x = e - jj * n0;
-    const int y0 = 2 * (j0 + jj);
-    a[e] = mk<R>(src[(size_t)y0 * n0 + x], src[(size_t)(y0 + 1) * n0 + x]);
+__global__ void __launch_bounds__(256) k_fft_x_r2c(const R* __restrict__ in, V2<R>* __restrict__ spec, int rows,
+                                                   int nkx, int rpb, PlanDev pl, const TW<R>* __restrict__ tw,
+                                                   const double* __restrict__ done) {
+  __shared__ unsigned red[MAX_WARPS];
+  __shared__ int ebs[256];               // output scale of each row pair
+  const int n0 = pl.n;
+  C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
+  C<R>* b1 = b0 + rpb * (n0 + (n0 >> 3) + 1);
+  const int row = fdiv(threadIdx.x, pl.tdiv), tj = threadIdx.x - row * pl.T;
+  const long g0 = (long)blockIdx.x * rpb, g = g0 + row;
+  const bool on = row < rpb && g < rows;
+  const R* src = in + (size_t)(on ? g : 0) * 2 * n0;
+  R u[RMAX], v[RMAX];
+  unsigned key = 0u;
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m) {
+    u[m] = v[m] = (R)0;
+    if (on && m < pl.r0) {
+      u[m] = src[tj + m * pl.T];
+      v[m] = src[n0 + tj + m * pl.T];
+      key = max(key, max(mag_of(u[m]), mag_of(v[m])));
+    }
   }
+  if (done && *done != 0.0) return;
+  const int e = row_exp<R>(key, pl.T, red), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
+  C<R> a[RMAX];
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[m], s0), to_work(v[m], s0));
+  const C<R>* res = transform<-1, R>(a, b0, b1, pl, tj, on, [&](int p) { return row_elem(row, n0, p); }, tw);
+  if (tj == 0 && row < rpb) ebs[row] = eb;
   __syncthreads();
-  cplx* res = block_fft<-1, R>(a, b, pl, rpb, tw);
-  V2<R>* dst = spec + ((size_t)f * n2 + z) * n1 * nkx;
   // the two half spectra are Z(k) +/- conj(Z(n0 - k)) without the factor 1/2
   // of the split: every operator applied between the z passes carries it in
   // its 1/nvox (SPEC_SCALE), exactly, as a power of two
-  for (int e = threadIdx.x; e < rpb * nkx; e += blockDim.x) {
-    const int jj = e / nkx, k = e - jj * nkx;
-    const cplx zk = res[jj * n0 + k];
-    const cplx zc = res[jj * n0 + (k == 0 ? 0 : n0 - k)];
-    const cplx zm = mk<R>(zc.x, -zc.y);
-    const cplx s = add(zk, zm), d = sub(zk, zm);
-    const int y0 = 2 * (j0 + jj);
-    dst[(size_t)y0 * nkx + k] = st2<R>(s.x, s.y);
-    dst[(size_t)(y0 + 1) * nkx + k] = st2<R>(d.y, -d.x);
+  const int live = (int)min((long)rpb, rows - g0);
+#pragma unroll 1
+  for (int q = threadIdx.x; q < live * nkx; q += blockDim.x) {
+    const int jj = q / nkx, k = q - jj * nkx;
+    const C<R> zk = res[row_elem(jj, n0, k)];
+    const C<R> zc = res[row_elem(jj, n0, k == 0 ? 0 : n0 - k)];
+    const int ej = ebs[jj];
+    V2<R>* dst = spec + (size_t)(g0 + jj) * 2 * nkx + k;
+    dst[0] = st2(from_work<R>(zk.x + zc.x, ej), from_work<R>(zk.y - zc.y, ej));
+    dst[nkx] = st2(from_work<R>(zk.y + zc.y, ej), from_work<R>(zc.x - zk.x, ej));
   }
 }
 
 // ---------------------------------------------------------------- pass X^-1 (C2R)
 template <typename R>
-__global__ void __launch_bounds__(256) k_fft_x_c2r(const V2<R>* __restrict__ spec, R* __restrict__ out,
-                                                   int n0, int n1, int n2, int nkx, int rpb, PlanDev pl,
-                                                   const V2<R>* __restrict__ tw, const double* __restrict__ done) {
-  typedef CX<R> cplx;
-  if (done && *done != 0.0) return;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  cplx* a = reinterpret_cast<cplx*>(smraw);
-  cplx* b = a + rpb * n0;
-  const int f = blockIdx.z, z = blockIdx.y, j0 = blockIdx.x * rpb;
-  const size_t nvox = (size_t)n0 * n1 * n2;
-  const V2<R>* src = spec + ((size_t)f * n2 + z) * n1 * nkx;
-  for (int e = threadIdx.x; e < rpb * n0; e += blockDim.x) {
-    const int jj = e / n0, k = e - jj * n0;
-    const int y0 = 2 * (j0 + jj);
-    cplx A, B;
-    if (k < nkx) {
-      V2<R> u = src[(size_t)y0 * nkx + k], v = src[(size_t)(y0 + 1) * nkx + k];
-      A = mk<R>(u.x, u.y); B = mk<R>(v.x, v.y);
-    } else {
-      V2<R> u = src[(size_t)y0 * nkx + (n0 - k)], v = src[(size_t)(y0 + 1) * nkx + (n0 - k)];
-      A = mk<R>(u.x, -u.y); B = mk<R>(v.x, -v.y);
+__global__ void __launch_bounds__(256) k_fft_x_c2r(const V2<R>* __restrict__ spec, R* __restrict__ out, int rows,
+                                                   int nkx, int rpb, PlanDev pl, const TW<R>* __restrict__ tw,
+                                                   const double* __restrict__ done) {
+  __shared__ unsigned red[MAX_WARPS];
+  const int n0 = pl.n;
+  C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
+  C<R>* b1 = b0 + rpb * (n0 + (n0 >> 3) + 1);
+  const int row = fdiv(threadIdx.x, pl.tdiv), tj = threadIdx.x - row * pl.T;
+  const long g = (long)blockIdx.x * rpb + row;
+  const bool on = row < rpb && g < rows;
+  const V2<R>* src = spec + (size_t)(on ? g : 0) * 2 * nkx;
+  // the row pair's spectra A, B at k = tj + m T <= n0 / 2 (at most RMAX / 2
+  // + 1 of them) give Z(k) = A + i B and Z(n0 - k) = conj(A) + i conj(B)
+  constexpr int HM = RMAX / 2 + 1;
+  V2<R> A[HM], B[HM];
+  unsigned key = 0u;
+#pragma unroll
+  for (int m = 0; m < HM; ++m) {
+    A[m] = B[m] = st2((R)0, (R)0);
+    if (on && tj + m * pl.T < nkx) {
+      A[m] = src[tj + m * pl.T];
+      B[m] = src[nkx + tj + m * pl.T];
+      key = max(key, max(mag_of(A[m]), mag_of(B[m])));
     }
-    a[e] = mk<R>(A.x - B.y, A.y + B.x);  // A + i B
+  }
+  if (done && *done != 0.0) return;
+  // (the sums A + i B double the components: one bit less)
+  const int e = row_exp<R>(key, pl.T, red), bits = pl.bits - 1;
+  const int s0 = e + 63 - bits, eb = fix64::out_base(e, bits, pl.down);
+  if (on) {
+#pragma unroll
+    for (int m = 0; m < HM; ++m) {
+      const int k = tj + m * pl.T;
+      if (k < nkx) {
+        const C<R> z = mk(to_work(A[m].x, s0), to_work(A[m].y, s0)), w = mk(to_work(B[m].x, s0), to_work(B[m].y, s0));
+        b1[row_elem(row, n0, k)] = mk(z.x - w.y, z.y + w.x);
+        if (k > 0 && 2 * k < n0) b1[row_elem(row, n0, n0 - k)] = mk(z.x + w.y, w.x - z.y);
+      }
+    }
   }
   __syncthreads();
-  cplx* res = block_fft<+1, R>(a, b, pl, rpb, tw);
-  R* dst = out + f * nvox + (size_t)z * n1 * n0;
-  for (int e = threadIdx.x; e < rpb * n0; e += blockDim.x) {
-    const int jj = e / n0, x = e - jj * n0;
-    const int y0 = 2 * (j0 + jj);
-    dst[(size_t)y0 * n0 + x] = res[e].x;
-    dst[(size_t)(y0 + 1) * n0 + x] = res[e].y;
+  C<R> a[RMAX];
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m)
+    if (on && m < pl.r0) a[m] = b1[row_elem(row, n0, tj + m * pl.T)];
+  R* dst = out + (size_t)g * 2 * n0;
+  const C<R>* res = transform<+1, R>(a, b0, b1, pl, tj, on, [&](int p) { return row_elem(row, n0, p); }, tw);
+  __syncthreads();
+  if (!on) return;
+#pragma unroll 1
+  for (int p = tj; p < n0; p += pl.T) {
+    const C<R> z = res[row_elem(row, n0, p)];
+    dst[p] = from_work<R>(z.x, eb);
+    dst[n0 + p] = from_work<R>(z.y, eb);
   }
 }
 
 // ---------------------------------------------------------------- pass Y (C2C)
+// ncol columns (field, z, kx), cpb consecutive ones per block, kx fastest
 template <int SIGN, typename R>
-__global__ void __launch_bounds__(256) k_fft_y(V2<R>* __restrict__ spec, int n1, int n2, int nkx, int tx,
-                                               PlanDev pl, const V2<R>* __restrict__ tw,
-                                               const double* __restrict__ done) {
-  typedef CX<R> cplx;
-  if (done && *done != 0.0) return;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  cplx* a = reinterpret_cast<cplx*>(smraw);
-  cplx* b = a + tx * n1;
-  const int f = blockIdx.z, z = blockIdx.y, kx0 = blockIdx.x * tx;
-  V2<R>* base = spec + ((size_t)f * n2 + z) * n1 * nkx;
-  for (int e = threadIdx.x; e < tx * n1; e += blockDim.x) {
-    const int y = e / tx, t = e - y * tx;
-    const int kx = kx0 + t;
-    V2<R> v = kx < nkx ? base[(size_t)y * nkx + kx] : st2<R>((R)0, (R)0);
-    a[t * n1 + y] = mk<R>(v.x, v.y);
-  }
-  __syncthreads();
-  cplx* res = block_fft<SIGN, R>(a, b, pl, tx, tw);
-  for (int e = threadIdx.x; e < tx * n1; e += blockDim.x) {
-    const int y = e / tx, t = e - y * tx;
-    const int kx = kx0 + t;
-    if (kx < nkx) {
-      cplx v = res[t * n1 + y];
-      base[(size_t)y * nkx + kx] = st2<R>(v.x, v.y);
+__global__ void __launch_bounds__(256) k_fft_y(V2<R>* __restrict__ spec, int ncol, int nkx, int cpb, PlanDev pl,
+                                               const TW<R>* __restrict__ tw, const double* __restrict__ done) {
+  __shared__ unsigned red[MAX_WARPS * 32];
+  C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
+  C<R>* b1 = b0 + cpb * pl.n;
+  const int tj = threadIdx.x / cpb, c = threadIdx.x - tj * cpb;     // cpb: a power of two
+  const long col = (long)blockIdx.x * cpb + c;
+  const bool on = tj < pl.T && col < ncol;
+  const int plane = on ? (int)(col / nkx) : 0, kx = on ? (int)(col - (long)plane * nkx) : 0;
+  V2<R>* base = spec + (size_t)plane * pl.n * nkx + kx;
+  V2<R> u[RMAX];
+  unsigned key = 0u;
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m) {
+    u[m] = st2((R)0, (R)0);
+    if (on && m < pl.r0) {
+      u[m] = base[(size_t)(tj + m * pl.T) * nkx];
+      key = max(key, mag_of(u[m]));
     }
+  }
+  if (done && *done != 0.0) return;
+  const int e = column_exp<R>(key, cpb, red), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
+  C<R> a[RMAX];
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[m].x, s0), to_work(u[m].y, s0));
+  const C<R>* res = transform<SIGN, R>(a, b0, b1, pl, tj, on, [&](int p) { return p * cpb + c; }, tw);
+  __syncthreads();
+  if (!on) return;
+#pragma unroll 1
+  for (int p = tj; p < pl.n; p += pl.T) {
+    const C<R> z = res[p * cpb + c];
+    base[(size_t)p * nkx] = st2(from_work<R>(z.x, eb), from_work<R>(z.y, eb));
   }
 }
 
 struct OpTables {
-  const double* lapw;   // OP_LAPINV weight per spectrum point, SPEC_SCALE included (FP64 path)
   const double* s20; const double* s21; const double* s22;
   const double* c20; const double* c21; const double* c22;
   const double* tan0; const double* tan1; const double* tan2;
@@ -290,13 +498,10 @@ __device__ __forceinline__ double lapinv_weight(const OpTables& T, double inv_nv
 
 // Operator at one frequency on the three fields of a tensor row (in double).
 __device__ __forceinline__ void apply_op(const OpTables& T, const SpecParams& sp, int i, int kx, int ky, int kz,
-                                         size_t kidx, cplx& X0, cplx& X1, cplx& X2) {
+                                         cplx& X0, cplx& X1, cplx& X2) {
   cplx Y0, Y1, Y2;
   const double sc = SPEC_SCALE * sp.inv_nvox;
-  if (sp.op == OP_LAPINV) {
-    const double w = T.lapw ? __ldg(T.lapw + kidx) : lapinv_weight(T, sp.inv_nvox, kx, ky, kz);
-    Y0 = cscale(X0, w); Y1 = cscale(X1, w); Y2 = cscale(X2, w);
-  } else if (sp.op == OP_PROJECT) {
+  if (sp.op == OP_PROJECT) {
     if (kx == 0 && ky == 0 && kz == 0) {
       if (sp.mean_out) {
         sp.mean_out[3 * i + 0] = X0.x * sc;
@@ -346,129 +551,180 @@ __device__ __forceinline__ void apply_op(const OpTables& T, const SpecParams& sp
   X0 = Y0; X1 = Y1; X2 = Y2;
 }
 
-// inverse-Laplacian weight in float for the float path (SPEC_SCALE included
-// through the caller's scale)
-__device__ __forceinline__ float lapinv_weight_f(const OpTables& T, float scale, int kx, int ky, int kz) {
-  const float sx = (float)T.s20[kx], sy = (float)T.s21[ky], sz = (float)T.s22[kz];
-  const float cx = (float)T.c20[kx], cy = (float)T.c21[ky], cz = (float)T.c22[kz];
-  const float lap = fmaf(sx, cy * cz, fmaf(cx, sy * cz, cx * cy * sz));
-  return lap > 0.0f ? scale / (64.0f * lap) : 0.0f;
-}
-
 // the OP_LAPINV weight of every spectrum point (layout of one field's half
-// spectrum, [kz][ky][kx]), built once per handle
-__global__ void k_lapinv_table(double* __restrict__ w, OpTables T, int nkx, int n1, int n2, double inv_nvox) {
+// spectrum, [kz][ky][kx]), built once per handle; w32: its rounding to float
+// for the FP32 transforms (nullable)
+__global__ void k_lapinv_table(double* __restrict__ w, float* __restrict__ w32, OpTables T, int nkx, int n1, int n2,
+                               double inv_nvox) {
   const size_t n = (size_t)nkx * n1 * n2;
   for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
     const int kx = (int)(e % nkx), ky = (int)((e / nkx) % n1), kz = (int)(e / ((size_t)nkx * n1));
-    w[e] = lapinv_weight(T, inv_nvox, kx, ky, kz);
+    const double v = lapinv_weight(T, inv_nvox, kx, ky, kz);
+    w[e] = v;
+    if (w32) w32[e] = (float)v;
   }
 }
 
 // ---------------------------------------------------------------- pass Z + operator
+// np pencils (ky, kx) of every field, cpb consecutive ones per block; the
+// inverse Laplacian treats each field by itself (blockIdx.y: the field)
 template <typename R>
-__global__ void __launch_bounds__(256) k_fft_z_op(V2<R>* __restrict__ spec, int n1, int n2, int nkx, int tx,
-                                                  PlanDev pl, const V2<R>* __restrict__ tw, OpTables T,
-                                                  SpecParams sp, const double* __restrict__ done) {
-  typedef CX<R> cx;
-  if (done && *done != 0.0) return;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int cnt = 3 * tx * n2;
-  cx* a = reinterpret_cast<cx*>(smraw);
-  cx* b = a + cnt;
-  const int i = blockIdx.z, ky = blockIdx.y, kx0 = blockIdx.x * tx;
-  const size_t zstride = (size_t)n1 * nkx;
-  for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-    const int c = e / (tx * n2);
-    const int rem = e - c * tx * n2;
-    const int z = rem / tx, t = rem - z * tx;
-    const int kx = kx0 + t;
-    const size_t f = 3 * i + c;
-    V2<R> v = kx < nkx ? spec[(f * n2 + z) * zstride + (size_t)ky * nkx + kx] : st2<R>((R)0, (R)0);
-    a[(c * tx + t) * n2 + z] = mk<R>(v.x, v.y);
-  }
-  __syncthreads();
-  cx* res = block_fft<-1, R>(a, b, pl, 3 * tx, tw);
-  cx* oth = (res == a) ? b : a;
-  const float inv_nvox_f = (float)(SPEC_SCALE * sp.inv_nvox);
-  for (int e = threadIdx.x; e < tx * n2; e += blockDim.x) {
-    const int t = e / n2, z = e - t * n2;
-    const int kx = kx0 + t;
-    cx Y0 = res[(0 * tx + t) * n2 + z], Y1 = res[(1 * tx + t) * n2 + z], Y2 = res[(2 * tx + t) * n2 + z];
-    if (kx >= nkx) {
-      Y0 = Y1 = Y2 = mk<R>((R)0, (R)0);
-    } else if (sizeof(R) == 4) {
-      // float path: the inverse Laplacian is the only operator it carries
-      const R w = (R)lapinv_weight_f(T, inv_nvox_f, kx, ky, z);
-      Y0 = scl(Y0, w); Y1 = scl(Y1, w); Y2 = scl(Y2, w);
-    } else {
-      cplx X0 = cmk((double)Y0.x, (double)Y0.y), X1 = cmk((double)Y1.x, (double)Y1.y),
-           X2 = cmk((double)Y2.x, (double)Y2.y);
-      apply_op(T, sp, i, kx, ky, z, ((size_t)z * gridDim.y + ky) * nkx + kx, X0, X1, X2);
-      Y0 = mk<R>((R)X0.x, (R)X0.y); Y1 = mk<R>((R)X1.x, (R)X1.y); Y2 = mk<R>((R)X2.x, (R)X2.y);
+__global__ void __launch_bounds__(256) k_fft_z_lap(V2<R>* __restrict__ spec, int np, int cpb, PlanDev pl,
+                                                   const TW<R>* __restrict__ tw, const R* __restrict__ weight,
+                                                   const double* __restrict__ done) {
+  __shared__ unsigned red[2][MAX_WARPS * 32];
+  C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
+  C<R>* b1 = b0 + cpb * pl.n;
+  const int tj = threadIdx.x / cpb, c = threadIdx.x - tj * cpb;
+  const int pc = blockIdx.x * cpb + c;
+  const bool on = tj < pl.T && pc < np;
+  V2<R>* base = spec + (size_t)blockIdx.y * pl.n * np + (on ? pc : 0);
+  V2<R> u[RMAX];
+  unsigned key = 0u;
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m) {
+    u[m] = st2((R)0, (R)0);
+    if (on && m < pl.r0) {
+      u[m] = base[(size_t)(tj + m * pl.T) * np];
+      key = max(key, mag_of(u[m]));
     }
-    oth[(0 * tx + t) * n2 + z] = Y0;
-    oth[(1 * tx + t) * n2 + z] = Y1;
-    oth[(2 * tx + t) * n2 + z] = Y2;
   }
+  if (done && *done != 0.0) return;
+  int e = column_exp<R>(key, cpb, red[0]), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
+  C<R> a[RMAX];
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[m].x, s0), to_work(u[m].y, s0));
+  auto idx = [&](int p) { return p * cpb + c; };
+  C<R>* res = transform<-1, R>(a, b0, b1, pl, tj, on, idx, tw);
   __syncthreads();
-  cx* res2 = block_fft<+1, R>(oth, res, pl, 3 * tx, tw);
-  for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-    const int c = e / (tx * n2);
-    const int rem = e - c * tx * n2;
-    const int z = rem / tx, t = rem - z * tx;
-    const int kx = kx0 + t;
-    if (kx < nkx) {
-      const size_t f = 3 * i + c;
-      cx v = res2[(c * tx + t) * n2 + z];
-      spec[(f * n2 + z) * zstride + (size_t)ky * nkx + kx] = st2<R>(v.x, v.y);
+  key = 0u;
+  // weighted in R and kept in place (a thread reads only the points it writes here)
+  V2<R>* wres = reinterpret_cast<V2<R>*>(res);
+  if (on) {
+#pragma unroll 1
+    for (int p = tj; p < pl.n; p += pl.T) {
+      const C<R> z = res[idx(p)];
+      const R w = __ldg(weight + (size_t)p * np + pc);
+      const V2<R> v = st2(from_work<R>(z.x, eb) * w, from_work<R>(z.y, eb) * w);
+      wres[idx(p)] = v;
+      key = max(key, mag_of(v));
+    }
+  }
+  e = column_exp<R>(key, cpb, red[1]);
+  s0 = e + 63 - pl.bits;
+  eb = fix64::out_base(e, pl.bits, pl.down);
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m)
+    if (on && m < pl.r0) {
+      const V2<R> v = wres[idx(tj + m * pl.T)];
+      a[m] = mk(to_work(v.x, s0), to_work(v.y, s0));
+    }
+  // the inverse starts in the other buffer: this one may still be read
+  res = transform<+1, R>(a, res == b0 ? b1 : b0, res, pl, tj, on, idx, tw);
+  __syncthreads();
+  if (!on) return;
+#pragma unroll 1
+  for (int p = tj; p < pl.n; p += pl.T) {
+    const C<R> z = res[idx(p)];
+    base[(size_t)p * np] = st2(from_work<R>(z.x, eb), from_work<R>(z.y, eb));
+  }
+}
+
+// The operators that couple the three fields of a tensor row (projection and
+// curls; blockIdx.y: the row): each thread carries its points of all three
+// through the forward transforms, applies the operator in FP64 and goes back.
+__global__ void __launch_bounds__(128) k_fft_z_op(double2* __restrict__ spec, int np, int nkx, int cpb, PlanDev pl,
+                                                  const int4* __restrict__ tw, OpTables T, SpecParams sp) {
+  typedef double R;
+  __shared__ unsigned red[4][MAX_WARPS * 32];
+  C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
+  C<R>* b1 = b0 + cpb * pl.n;
+  const int tj = threadIdx.x / cpb, c = threadIdx.x - tj * cpb;
+  const int pc = blockIdx.x * cpb + c, row = blockIdx.y;
+  const bool on = tj < pl.T && pc < np;
+  const size_t fstride = (size_t)pl.n * np;
+  double2* base = spec + (size_t)row * 3 * fstride + (on ? pc : 0);
+  auto idx = [&](int p) { return p * cpb + c; };
+  double2 u[3][RMAX];
+#pragma unroll
+  for (int f = 0; f < 3; ++f)
+#pragma unroll
+    for (int m = 0; m < RMAX; ++m) {
+      u[f][m] = st2(0.0, 0.0);
+      if (on && m < pl.r0) u[f][m] = base[f * fstride + (size_t)(tj + m * pl.T) * np];
+    }
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    unsigned key = 0u;
+#pragma unroll
+    for (int m = 0; m < RMAX; ++m) key = max(key, mag_of(u[f][m]));
+    if (f) __syncthreads();                       // the previous field's results are read
+    const int e = column_exp<R>(key, cpb, red[f]), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
+    C<R> a[RMAX];
+#pragma unroll
+    for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[f][m].x, s0), to_work(u[f][m].y, s0));
+    const C<R>* res = transform<-1, R>(a, b0, b1, pl, tj, on, idx, tw);
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < RMAX; ++m)
+      if (on && m < pl.r0) {
+        const C<R> z = res[idx(tj + m * pl.T)];
+        u[f][m] = st2(from_work<R>(z.x, eb), from_work<R>(z.y, eb));
+      }
+  }
+  unsigned key = 0u;
+  if (on) {
+    const int ky = pc / nkx, kx = pc - ky * nkx;
+#pragma unroll
+    for (int m = 0; m < RMAX; ++m)
+      if (m < pl.r0) {
+        cplx X0 = cmk(u[0][m].x, u[0][m].y), X1 = cmk(u[1][m].x, u[1][m].y), X2 = cmk(u[2][m].x, u[2][m].y);
+        apply_op(T, sp, row, kx, ky, tj + m * pl.T, X0, X1, X2);
+        u[0][m] = st2(X0.x, X0.y); u[1][m] = st2(X1.x, X1.y); u[2][m] = st2(X2.x, X2.y);
+        key = max(key, max(mag_of(u[0][m]), max(mag_of(u[1][m]), mag_of(u[2][m]))));
+      }
+  }
+  const int e = column_exp<R>(key, cpb, red[3]), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
+#pragma unroll
+  for (int f = 0; f < 3; ++f) {
+    __syncthreads();                              // the previous results are read
+    C<R> a[RMAX];
+#pragma unroll
+    for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[f][m].x, s0), to_work(u[f][m].y, s0));
+    const C<R>* res = transform<+1, R>(a, b0, b1, pl, tj, on, idx, tw);
+    __syncthreads();
+    if (on) {
+#pragma unroll 1
+      for (int p = tj; p < pl.n; p += pl.T) {
+        const C<R> z = res[idx(p)];
+        base[f * fstride + (size_t)p * np] = st2(from_work<R>(z.x, eb), from_work<R>(z.y, eb));
+      }
     }
   }
 }
 
-// Tile sizes: as large as shared memory allows (up to 1024 complex per
-// transform batch, 512 in the z pass that holds three fields), shrunk while
-// the grid would fill less than four blocks per SM, down to 256 elements.
-
-int rows_per_block(int n0, int n1, int n2, int nf, int fill) {
-  int r = 1024 / n0;
+// Transforms per block.  Small blocks keep the barriers cheap and the common
+// scale local; the tile starts at 1024 values (a block's shared memory is two
+// tiles) and halves while the grid has fewer blocks than `fill` or the block
+// more than 256 threads, down to one warp.
+int rows_per_block(const PlanDev& pl, long rows, int fill) {
+  int r = 1024 / pl.n;
   if (r < 1) r = 1;
-  if (r > n1 / 2) r = n1 / 2;
-  while (r > 1 && (n1 / 2) % r) --r;
-  while (r > 1 && (long)(n1 / 2 / r) * n2 * nf < fill && r * n0 > 256) {
-    int q = r / 2;
-    while (q > 1 && (n1 / 2) % q) --q;
-    r = q;
-  }
+  while (r > 1 && (r * pl.T > 256 || (r * pl.T > 32 && (rows + r - 1) / r < fill))) r /= 2;
   return r;
 }
-int tile_y(int n1, int n2, int nkx, int nf, int fill) {
-  int t = 1024 / n1;
-  if (t > 16) t = 16;
-  if (t < 1) t = 1;
-  while (t > 1 && (long)((nkx + t - 1) / t) * n2 * nf < fill && t * n1 > 256) t /= 2;
-  return t;
+// columns per block of the y and z passes: a power of two, at least 8 where
+// the shared memory allows it (128 bytes of consecutive FP64 columns)
+int cols_per_block(const PlanDev& pl, long cols, int fill, int max_threads) {
+  int c = 1;
+  while (2 * c * pl.n <= 1024 && 2 * c * pl.T <= max_threads && c < 32) c *= 2;
+  while (c > 8 && c * pl.T > 32 && (cols + c - 1) / c < fill) c /= 2;
+  return c;
 }
-int tile_z(int n1, int n2, int nkx, int nf, int fill) {
-  int t = 512 / n2;
-  if (t > 16) t = 16;
-  if (t < 1) t = 1;
-  while (t > 1 && (long)((nkx + t - 1) / t) * n1 * (nf / 3) < fill && 3 * t * n2 > 256) t /= 2;
-  return t;
-}
-// threads for a block holding `elems` complex values: one per `per` values
-// (the x and y passes: one butterfly of the plan's largest radix, its first
-// pass, per thread; the z pass, whose tiles are narrow and few per SM, keeps
-// one thread per four values for the warps that hide its latency)
-int threads_for(int elems, int per) {
-  int t = (elems / per + 31) / 32 * 32;
-  return t < 64 ? 64 : (t > 256 ? 256 : t);
-}
-int first_radix(const FFTPlan& pl) { return pl.npass > 0 ? pl.radix[0] : 4; }
+int round32(int t) { return (t + 31) / 32 * 32; }
 
 OpTables op_tables(const rve_s* h) {
   OpTables T;
-  T.lapw = h->lapw;
   T.tan0 = h->ax[0].tanh_; T.tan1 = h->ax[1].tanh_; T.tan2 = h->ax[2].tanh_;
   T.nyq0 = h->ax[0].nyq; T.nyq1 = h->ax[1].nyq; T.nyq2 = h->ax[2].nyq;
   T.ph0 = h->ax[0].ph; T.ph1 = h->ax[1].ph; T.ph2 = h->ax[2].ph;
@@ -478,65 +734,74 @@ OpTables op_tables(const rve_s* h) {
   return T;
 }
 
-template <typename R> const V2<R>* twt(const rve_s* h, int a);
-template <> const double2* twt<double>(const rve_s* h, int a) { return h->ax[a].tw; }
+template <typename R> const TW<R>* twt(const rve_s* h, int a);
+template <> const int4* twt<double>(const rve_s* h, int a) { return h->ax[a].twq; }
 template <> const float2* twt<float>(const rve_s* h, int a) { return h->ax[a].tw32; }
 template <typename R> V2<R>* spect(const rve_s* h);
 template <> double2* spect<double>(const rve_s* h) { return h->spec; }
 template <> float2* spect<float>(const rve_s* h) { return h->spec32; }
+template <typename R> const R* lap_weight(const rve_s* h);
+template <> const double* lap_weight<double>(const rve_s* h) { return h->lapw; }
+template <> const float* lap_weight<float>(const rve_s* h) { return h->lapw32; }
+
+template <typename R>
+size_t row_smem(int rpb, int n) { return 2 * (size_t)rpb * (n + (n >> 3) + 1) * sizeof(C<R>); }
+
+template <int SIGN, typename R>
+void launch_y(const rve_s* h, cudaStream_t s, const double* done, int nf, int cat) {
+  const PlanDev pl = to_dev(h->plan[1]);
+  const long cols = (long)nf * h->n2 * h->nkx;
+  const int c = cols_per_block(pl, cols, h->fft_fill_y, 256);
+  ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : cat, s);
+  k_fft_y<SIGN, R><<<(unsigned)((cols + c - 1) / c), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
+      spect<R>(h), (int)cols, h->nkx, c, pl, twt<R>(h, 1), done);
+}
 
 template <typename R>
 cudaError_t fwd(const rve_s* h, const R* in, cudaStream_t s, const double* done, int nf) {
-  const int rpb = rows_per_block(h->n0, h->n1, h->n2, nf, h->fft_fill);
-  dim3 gx(h->n1 / 2 / rpb, h->n2, nf);
-  size_t shx = 2 * (size_t)rpb * h->n0 * sizeof(CX<R>);
+  const PlanDev pl = to_dev(h->plan[0]);
+  const long rows = (long)nf * h->n2 * (h->n1 / 2);
+  const int rpb = rows_per_block(pl, rows, h->fft_fill);
   {
     ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : RVE_K_FFT_X_R2C, s);
-    k_fft_x_r2c<R><<<gx, threads_for(rpb * h->n0, first_radix(h->plan[0])), shx, s>>>(in, spect<R>(h), h->n0, h->n1, h->n2, h->nkx, rpb,
-                                                             to_dev(h->plan[0]), twt<R>(h, 0), done);
+    k_fft_x_r2c<R><<<(unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb, pl.n), s>>>(
+        in, spect<R>(h), (int)rows, h->nkx, rpb, pl, twt<R>(h, 0), done);
   }
-  const int ty = tile_y(h->n1, h->n2, h->nkx, nf, h->fft_fill_y);
-  dim3 gy((h->nkx + ty - 1) / ty, h->n2, nf);
-  size_t shy = 2 * (size_t)ty * h->n1 * sizeof(CX<R>);
-  {
-    ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : RVE_K_FFT_Y, s);
-    k_fft_y<-1, R><<<gy, threads_for(ty * h->n1, first_radix(h->plan[1])), shy, s>>>(spect<R>(h), h->n1, h->n2, h->nkx, ty,
-                                                            to_dev(h->plan[1]), twt<R>(h, 1), done);
-  }
+  launch_y<-1, R>(h, s, done, nf, RVE_K_FFT_Y);
   return cudaGetLastError();
 }
 
 template <typename R>
-cudaError_t zop(const rve_s* h, const SpecParams& sp, cudaStream_t s, const double* done, int nf) {
-  const int tz = tile_z(h->n1, h->n2, h->nkx, nf, h->fft_fill_z);
-  dim3 g((h->nkx + tz - 1) / tz, h->n1, nf / 3);
-  size_t sh = 2 * 3 * (size_t)tz * h->n2 * sizeof(CX<R>);
-  const int zthreads = threads_for(3 * tz * h->n2, 4);
-  {
-    ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : RVE_K_FFT_Z_OP, s);
-    k_fft_z_op<R><<<g, zthreads, sh, s>>>(spect<R>(h), h->n1, h->n2, h->nkx, tz, to_dev(h->plan[2]), twt<R>(h, 2),
-                                          op_tables(h), sp, done);
-  }
+cudaError_t lap(const rve_s* h, cudaStream_t s, const double* done) {
+  const PlanDev pl = to_dev(h->plan[2]);
+  const int np = h->n1 * h->nkx;
+  const int c = cols_per_block(pl, 3L * np, h->fft_fill_z, 256);
+  ProfScope ps_(h, RVE_K_FFT_Z_OP, s);
+  k_fft_z_lap<R><<<dim3((np + c - 1) / c, 3), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
+      spect<R>(h), np, c, pl, twt<R>(h, 2), lap_weight<R>(h), done);
+  return cudaGetLastError();
+}
+
+cudaError_t zop(const rve_s* h, const SpecParams& sp, cudaStream_t s) {
+  const PlanDev pl = to_dev(h->plan[2]);
+  const int np = h->n1 * h->nkx;
+  const int c = cols_per_block(pl, 3L * np, h->fft_fill_z, 128);
+  ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : RVE_K_FFT_Z_OP, s);
+  k_fft_z_op<<<dim3((np + c - 1) / c, 3), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<double>), s>>>(
+      h->spec, np, h->nkx, c, pl, h->ax[2].twq, op_tables(h), sp);
   return cudaGetLastError();
 }
 
 template <typename R>
 cudaError_t inv(const rve_s* h, R* out, cudaStream_t s, const double* done, int nf) {
-  const int ty = tile_y(h->n1, h->n2, h->nkx, nf, h->fft_fill_y);
-  dim3 gy((h->nkx + ty - 1) / ty, h->n2, nf);
-  size_t shy = 2 * (size_t)ty * h->n1 * sizeof(CX<R>);
-  {
-    ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : RVE_K_FFT_Y_INV, s);
-    k_fft_y<+1, R><<<gy, threads_for(ty * h->n1, first_radix(h->plan[1])), shy, s>>>(spect<R>(h), h->n1, h->n2, h->nkx, ty,
-                                                            to_dev(h->plan[1]), twt<R>(h, 1), done);
-  }
-  const int rpb = rows_per_block(h->n0, h->n1, h->n2, nf, h->fft_fill);
-  dim3 gx(h->n1 / 2 / rpb, h->n2, nf);
-  size_t shx = 2 * (size_t)rpb * h->n0 * sizeof(CX<R>);
+  launch_y<+1, R>(h, s, done, nf, RVE_K_FFT_Y_INV);
+  const PlanDev pl = to_dev(h->plan[0]);
+  const long rows = (long)nf * h->n2 * (h->n1 / 2);
+  const int rpb = rows_per_block(pl, rows, h->fft_fill);
   {
     ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : RVE_K_FFT_X_C2R, s);
-    k_fft_x_c2r<R><<<gx, threads_for(rpb * h->n0, first_radix(h->plan[0])), shx, s>>>(spect<R>(h), out, h->n0, h->n1, h->n2, h->nkx, rpb,
-                                                             to_dev(h->plan[0]), twt<R>(h, 0), done);
+    k_fft_x_c2r<R><<<(unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb, pl.n), s>>>(
+        spect<R>(h), out, (int)rows, h->nkx, rpb, pl, twt<R>(h, 0), done);
   }
   return cudaGetLastError();
 }
@@ -545,35 +810,41 @@ cudaError_t inv(const rve_s* h, R* out, cudaStream_t s, const double* done, int 
 
 cudaError_t launch_lapinv_table(const rve_s* h, cudaStream_t s) {
   if (!h->lapw) return cudaSuccess;
-  k_lapinv_table<<<RVE_RED_BLOCKS, 256, 0, s>>>(h->lapw, op_tables(h), h->nkx, h->n1, h->n2, 1.0 / (double)h->nvox);
+  k_lapinv_table<<<RVE_RED_BLOCKS, 256, 0, s>>>(h->lapw, h->lapw32, op_tables(h), h->nkx, h->n1, h->n2,
+                                                1.0 / (double)h->nvox);
   return cudaGetLastError();
 }
 
-void make_plan(int n, FFTPlan* p, int max_radix) {
+// Radices of a length 2^a 3^b, the largest first (a transform has n / radix[0]
+// threads): 8s, then 6s while both factors are left, then 4, 3s or 2.
+void make_plan(int n, FFTPlan* p) {
   p->n = n;
   p->npass = 0;
-  int m = n;
-  while (max_radix >= 8 && m % 8 == 0) { p->radix[p->npass++] = 8; m /= 8; }
-  while (m % 4 == 0) { p->radix[p->npass++] = 4; m /= 4; }
-  if (m % 2 == 0) { p->radix[p->npass++] = 2; m /= 2; }
-  while (m % 3 == 0) { p->radix[p->npass++] = 3; m /= 3; }
-  if (m != 1) p->npass = -1;  // unsupported length
+  int a = 0, b = 0, m = n;
+  while (m % 2 == 0) { ++a; m /= 2; }
+  while (m % 3 == 0) { ++b; m /= 3; }
+  if (m != 1) { p->npass = -1; return; }     // unsupported length
+  while (a >= 3) { p->radix[p->npass++] = 8; a -= 3; }
+  while (a >= 1 && b >= 1) { p->radix[p->npass++] = 6; --a; --b; }
+  if (a == 2) p->radix[p->npass++] = 4;
+  // 3s before a last 2: the first radix stays the largest
+  while (b > 0) { p->radix[p->npass++] = 3; --b; }
+  if (a == 1) p->radix[p->npass++] = 2;
 }
 
 cudaError_t launch_fft_forward(const rve_s* h, const double* in, cudaStream_t s, const double* done, int nf) {
   return fwd<double>(h, in, s, done, nf);
 }
-cudaError_t launch_fft_op(const rve_s* h, const SpecParams& sp, cudaStream_t s, const double* done, int nf) {
-  return zop<double>(h, sp, s, done, nf);
-}
+cudaError_t launch_fft_lapinv(const rve_s* h, cudaStream_t s, const double* done) { return lap<double>(h, s, done); }
+cudaError_t launch_fft_op(const rve_s* h, const SpecParams& sp, cudaStream_t s) { return zop(h, sp, s); }
 cudaError_t launch_fft_inverse(const rve_s* h, double* out, cudaStream_t s, const double* done, int nf) {
   return inv<double>(h, out, s, done, nf);
 }
 cudaError_t launch_fft_forward32(const rve_s* h, const float* in, cudaStream_t s, const double* done) {
   return fwd<float>(h, in, s, done, 3);
 }
-cudaError_t launch_fft_lapinv32(const rve_s* h, const SpecParams& sp, cudaStream_t s, const double* done) {
-  return zop<float>(h, sp, s, done, 3);
+cudaError_t launch_fft_lapinv32(const rve_s* h, cudaStream_t s, const double* done) {
+  return lap<float>(h, s, done);
 }
 cudaError_t launch_fft_inverse32(const rve_s* h, float* out, cudaStream_t s, const double* done) {
   return inv<float>(h, out, s, done, 3);

@@ -1,0 +1,106 @@
+// 64-bit fixed-point arithmetic for the FP64 transforms and stencils.
+//
+// One FP64 instruction of a warp occupies an SM of this GPU for 16 or more
+// cycles (2 lanes per clock; measured 1.7 additions and 2.0 FMAs), a 64-bit
+// integer addition (two 32-bit ones) or a 32 x 32 + 64-bit multiply-add half
+// a cycle (64 lanes per clock).  Sums of doubles of one tile are therefore
+// formed as integers on a common power-of-two scale taken from the tile's
+// largest magnitude: a value keeps every bit above 2^-B of that magnitude
+// (B >= 52, more than the 2^-53 relative rounding of each FP64 operation it
+// replaces leaves in a sum of the tile's values), and integer additions are
+// exact.
+//
+// A tile that holds an infinity or a NaN gives NaN throughout; a tile whose
+// values lie below 2^-767 is taken as zero (a sum of it is below 2^-767
+// times the sum's terms, an absolute error no FP64 caller here can see).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace fix64 {
+
+typedef long long i64;
+
+constexpr int EXP_MIN = 256;          // smallest common exponent field used
+constexpr int EXP_SLOW = 2000;        // output exponent bases above this take the checked path
+
+// magnitude key of a double: its high word without the sign (the exponent
+// field on top), to be maximised over a tile
+__device__ __forceinline__ unsigned mag(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
+
+// exponent field of a tile's largest magnitude key (0x7ff: infinity or NaN)
+__device__ __forceinline__ int tile_exp(unsigned key) {
+  const int e = (int)(key >> 20);
+  return e < EXP_MIN ? EXP_MIN : e;
+}
+
+// x as an integer on the scale of exponent field e: |result| < 2^B for every
+// |x| of that exponent or a smaller one (truncated toward zero); s0 = e + 63 - B
+__device__ __forceinline__ i64 to_fix(double x, int s0) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  // the significand with its leading bit at 2^62, moved down by d: below 2^(63 - d)
+  const unsigned mh = (((unsigned)hi & 0xfffffu) | 0x100000u) << 10 | ((unsigned)lo >> 22);
+  const unsigned ml = (unsigned)lo << 10;
+  const unsigned d = min((unsigned)(s0 - ((hi >> 20) & 0x7ff)), 63u);
+  const uint64_t m = (((uint64_t)mh << 32) | ml) >> d;
+  const i64 s = (i64)(hi >> 31);
+  return ((i64)m ^ s) - s;
+}
+
+static __device__ __noinline__ double from_fix_checked(i64 v, int eb) {
+  if (eb >= (1 << 20)) return __hiloint2double(0x7ff80000, 0);      // from a tile with an infinity or NaN
+  return scalbn((double)v, eb - 1086);                              // may overflow to infinity
+}
+
+// v on the scale given by eb (the exponent field of 2^63 on that scale) as
+// a double, rounded to nearest (ties away from zero)
+__device__ __forceinline__ double from_fix(i64 v, int eb) {
+  if (eb > EXP_SLOW) return from_fix_checked(v, eb);
+  const i64 s = v >> 63;
+  const uint64_t a = (uint64_t)((v ^ s) - s);
+  const int lz = __clzll((i64)a);
+  const uint64_t n = a << (lz & 63);
+  const uint64_t t = (n >> 11) + ((n >> 10) & 1u);                   // implicit bit at 2^52
+  int hi = (int)(t >> 32) + ((eb - 1 - lz) << 20);
+  hi = a ? (hi | ((int)s & (int)0x80000000)) : 0;
+  return __hiloint2double(hi, (int)t);
+}
+// exponent base of from_fix for integers on the scale to_fix(., e + 63 - B) gave, times 2^sh
+__device__ __forceinline__ int out_base(int e, int B, int sh = 0) {
+  return e == 0x7ff ? (1 << 20) : e + 64 - B + sh;
+}
+
+// ---- multiplication by Q62 factors (|w| <= 1) ----
+// w = wh 2^32 + wl with wl in (-2^31, 2^31): signed 32 x 32 products only
+struct Sp { int h, l; };
+__device__ __forceinline__ Sp split(i64 a) {
+  Sp s;
+  s.l = (int)a;
+  s.h = (int)(a >> 32) - (s.l >> 31);
+  return s;
+}
+__device__ __forceinline__ i64 wide(int a, int b) { return (i64)a * (i64)b; }
+// a w for a real factor, rounded (the product of the low words is dropped)
+__device__ __forceinline__ i64 mulq(i64 a, int wh, int wl) {
+  const Sp s = split(a);
+  const i64 mid = wide(s.h, wl) + wide(s.l, wh) + (1LL << 29);
+  return (wide(s.h, wh) << 2) + (mid >> 30);
+}
+// (x u + y v) / 4, rounded, for |x|, |y| < 2^62 and u^2 + v^2 = 1: the high
+// words of the products as they are, no shift
+__device__ __forceinline__ i64 mulq2(Sp x, int uh, int ul, Sp y, int vh, int vl) {
+  const i64 mid = wide(x.h, ul) + wide(x.l, uh) + wide(y.h, vl) + wide(y.l, vh) + (1LL << 31);
+  return wide(x.h, uh) + wide(y.h, vh) + (mid >> 32);
+}
+
+// a Q62 factor in the split form (F: long double on the host, double on the device)
+template <typename F>
+__host__ __device__ inline void split_q62(F w, int* h, int* l) {
+  int64_t v = (int64_t)(w * (F)4611686018427387904.0 + (w < 0 ? (F)-0.5 : (F)0.5));
+  if ((int32_t)(uint32_t)(uint64_t)v == INT32_MIN) v += 1;   // wl in (-2^31, 2^31): its negation stays in range
+  const int64_t lo = (int32_t)(uint32_t)(uint64_t)v;
+  *l = (int)lo;
+  *h = (int)((v - lo) >> 32);
+}
+
+}  // namespace fix64

@@ -9,13 +9,14 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "fix64.cuh"
 #include "rve_internal.h"
 
 namespace {
 
 constexpr size_t SPEC_MAX_BYTES = RVE_NOALLOC_SPEC_BYTES;
 constexpr int AXIS_MAX = 512;
-constexpr size_t AXIS_BYTES = AXIS_MAX * (sizeof(double2) + sizeof(double2) + sizeof(double) + sizeof(int8_t));
+constexpr size_t AXIS_BYTES = AXIS_MAX * (sizeof(int4) + sizeof(double2) + sizeof(double) + sizeof(int8_t));
 constexpr size_t AXIS_PITCH = (AXIS_BYTES + 255) & ~(size_t)255;
 constexpr size_t TABLE_BYTES = 3 * AXIS_PITCH;
 
@@ -34,7 +35,7 @@ std::mutex g_mutex;
 DeviceSlot g_slot[MAX_DEVICES];
 
 // Frequency tables of one axis of length n in the layout the FFT kernels read
-// (twiddles e^{-2 pi i t / n}; phases e^{i xi_t}, exactly -1 at Nyquist;
+// (twiddles e^{-2 pi i t / n} in Q62; phases e^{i xi_t}, exactly -1 at Nyquist;
 // tan(pi k / n) for the signed index k, 0 at Nyquist; Nyquist flags), built
 // on the device, so no call copies anything from the host.  sincospi gives
 // the quarter-turn values exactly.
@@ -42,8 +43,8 @@ __global__ void k_axis_tables(unsigned char* tab, int n0, int n1, int n2) {
   const int a = blockIdx.y;
   const int n = a == 0 ? n0 : (a == 1 ? n1 : n2);
   unsigned char* ax = tab + a * AXIS_PITCH;
-  double2* tw = reinterpret_cast<double2*>(ax);
-  double2* ph = tw + AXIS_MAX;
+  int4* tw = reinterpret_cast<int4*>(ax);
+  double2* ph = reinterpret_cast<double2*>(tw + AXIS_MAX);
   double* tn = reinterpret_cast<double*>(ph + AXIS_MAX);
   int8_t* nq = reinterpret_cast<int8_t*>(tn + AXIS_MAX);
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
@@ -51,7 +52,8 @@ __global__ void k_axis_tables(unsigned char* tab, int n0, int n1, int n2) {
     const int ks = (2 * t <= n) ? t : t - n;
     double s, c;
     sincospi(2.0 * (double)t / (double)n, &s, &c);
-    tw[t] = nyq ? make_double2(-1.0, 0.0) : make_double2(c, -s);
+    fix64::split_q62(c, &tw[t].x, &tw[t].y);
+    fix64::split_q62(-s, &tw[t].z, &tw[t].w);
     ph[t] = nyq ? make_double2(-1.0, 0.0) : make_double2(c, s);
     double sh, ch;
     sincospi((double)ks / (double)n, &sh, &ch);
@@ -82,7 +84,7 @@ extern "C" rve_status rve_project_noalloc(int n0, int n1, int n2, double L, cons
   h.stream = (cudaStream_t)cuda_stream;
   make_plan(n0, &h.plan[0]);
   make_plan(n1, &h.plan[1]);
-  make_plan(n2, &h.plan[2], 4);
+  make_plan(n2, &h.plan[2]);
 
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return RVE_ECUDA;
@@ -106,10 +108,9 @@ extern "C" rve_status rve_project_noalloc(int n0, int n1, int n2, double L, cons
   h.spec = reinterpret_cast<double2*>(base);
   for (int a = 0; a < 3; ++a) {
     unsigned char* ax = base + SPEC_MAX_BYTES + a * AXIS_PITCH;
-    const double2* tw = reinterpret_cast<const double2*>(ax);
-    h.ax[a].tw = tw;
-    h.ax[a].ph = tw + AXIS_MAX;
-    h.ax[a].tanh_ = reinterpret_cast<const double*>(tw + 2 * AXIS_MAX);
+    h.ax[a].twq = reinterpret_cast<const int4*>(ax);
+    h.ax[a].ph = reinterpret_cast<const double2*>(h.ax[a].twq + AXIS_MAX);
+    h.ax[a].tanh_ = reinterpret_cast<const double*>(h.ax[a].ph + AXIS_MAX);
     h.ax[a].nyq = reinterpret_cast<const int8_t*>(h.ax[a].tanh_ + AXIS_MAX);
   }
 

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fix64.cuh"
 #include "rve_internal.h"
 
 namespace {
@@ -68,7 +69,7 @@ void carve(rve_s* h, Carver& c) {
   h->screw_of = c.take<int32_t>(12);
   const int ns[3] = {h->n0, h->n1, h->n2};
   for (int a = 0; a < 3; ++a) {
-    h->ax[a].tw = c.take<double2>(ns[a]);
+    h->ax[a].twq = c.take<int4>(ns[a]);
     h->ax[a].tanh_ = c.take<double>(ns[a]);
     h->ax[a].nyq = c.take<int8_t>(ns[a]);
     h->ax[a].ph = c.take<double2>(ns[a]);
@@ -107,6 +108,7 @@ void carve(rve_s* h, Carver& c) {
   h->lapw = c.take<double>(h->nspec);
   if (h->opt.precision == 1) {
     for (int a = 0; a < 3; ++a) h->ax[a].tw32 = c.take<float2>(ns[a]);
+    h->lapw32 = c.take<float>(h->nspec);
     h->spec32 = c.take<float2>(3 * h->nspec);
     h->x32 = c.take<float>(9 * nv);
     h->r32 = c.take<float>(9 * nv);
@@ -116,6 +118,7 @@ void carve(rve_s* h, Carver& c) {
   } else {
     for (int a = 0; a < 3; ++a) h->ax[a].tw32 = nullptr;
     h->spec32 = nullptr;
+    h->lapw32 = nullptr;
     h->x32 = h->r32 = h->p32 = h->t32 = h->du32 = nullptr;
   }
   h->partial = c.take<double>(9 * 4096 + 27 * (size_t)RVE_RED_BLOCKS);
@@ -237,6 +240,27 @@ rve_status read_scalars(rve_s* h) {
 }
 
 
+// e^{-2 pi i t / n} in Q62 for t = 0 .. n - 1.  The angle is reduced to an
+// eighth turn in integers, so the quadruple-precision functions (slow on some
+// hosts) run for n / 8 angles where 4 divides n, and the symmetric values agree
+// to the last bit.
+void q62_twiddles(int n, std::vector<int4>& w) {
+  w.resize(n);
+  std::vector<long double> cs(n / 2 + 1, 2.0L), sn(n / 2 + 1);
+  for (int t = 0; t < n; ++t) {
+    const int quarter = 4 * t / n, a = 4 * t - quarter * n, b = 2 * a <= n ? a : n - a;   // a / n of a quarter turn
+    if (cs[b] == 2.0L) {
+      const long double x = 1.57079632679489661923132169163975144L * b / n;
+      cs[b] = std::cos(x);
+      sn[b] = std::sin(x);
+    }
+    const long double c = a == b ? cs[b] : sn[b], s = a == b ? sn[b] : cs[b];
+    const long double co[4] = {c, -s, -c, s}, si[4] = {s, c, -s, -c};
+    fix64::split_q62(co[quarter], &w[t].x, &w[t].y);
+    fix64::split_q62(-si[quarter], &w[t].z, &w[t].w);
+  }
+}
+
 SpecParams project_params(const rve_s* h, const uint8_t* mask, const double* shift, double* mean_out) {
   SpecParams sp;
   sp.op = OP_PROJECT;
@@ -275,11 +299,9 @@ rve_status run_project_stencil(rve_s* h, const double* X, double* Y, const uint8
                                bool all_means = false) {
   double* d = h->q;
   double* u = h->q + 3 * h->nvox;
-  SpecParams sp = project_params(h, mask, nullptr, nullptr);
-  sp.op = OP_LAPINV;
   RVE_CUDA(h, launch_div(h, X, d, 0, all_means ? 0x1FFu : kept_means(mask), h->stream));
   RVE_CUDA(h, launch_fft_forward(h, d, h->stream, nullptr, 3));
-  RVE_CUDA(h, launch_fft_op(h, sp, h->stream, nullptr, 3));
+  RVE_CUDA(h, launch_fft_lapinv(h, h->stream, nullptr));
   RVE_CUDA(h, launch_fft_inverse(h, u, h->stream, nullptr, 3));
   RVE_CUDA(h, launch_grad(h, u, Y, mask, shift, h->stream));
   return RVE_OK;
@@ -388,8 +410,6 @@ rve_status cg_chunk(rve_s* h, const uint8_t* mask, Issue issue) {
 
 rve_status cg_solve(rve_s* h, const uint8_t* mask, double eta, int* iters, bool* ok) {
   RVE_CUDA(h, launch_cg_init(h, eta, h->stream));
-  SpecParams sp = project_params(h, mask, nullptr, nullptr);
-  sp.op = OP_LAPINV;
   const double* done = h->dscal + DS_DONE;
   double* d = h->q;
   double* u = h->q + 3 * h->nvox;
@@ -403,7 +423,7 @@ rve_status cg_solve(rve_s* h, const uint8_t* mask, double eta, int* iters, bool*
         RVE_CUDA(h, launch_tangent_apply(h, h->stream));
         RVE_CUDA(h, launch_div(h, h->t, d, 1, kept_means(mask), h->stream));
         RVE_CUDA(h, launch_fft_forward(h, d, h->stream, done, 3));
-        RVE_CUDA(h, launch_fft_op(h, sp, h->stream, done, 3));
+        RVE_CUDA(h, launch_fft_lapinv(h, h->stream, done));
         RVE_CUDA(h, launch_fft_inverse(h, u, h->stream, done, 3));
         RVE_CUDA(h, launch_grad_cg(h, u, mask, h->stream));
       }
@@ -425,8 +445,6 @@ rve_status cg_solve(rve_s* h, const uint8_t* mask, double eta, int* iters, bool*
 rve_status cg_solve32(rve_s* h, const uint8_t* mask, double eta, int* iters, bool* ok) {
   eta = std::fmax(eta, 1e-5);
   RVE_CUDA(h, launch_cg_init32(h, eta, h->stream));
-  SpecParams sp = project_params(h, mask, nullptr, nullptr);
-  sp.op = OP_LAPINV;
   const double* done = h->dscal + DS_DONE;
   float* d = h->du32;
   float* u = h->du32 + 3 * h->nvox;
@@ -439,7 +457,7 @@ rve_status cg_solve32(rve_s* h, const uint8_t* mask, double eta, int* iters, boo
         RVE_CUDA(h, launch_tangent_apply32(h, h->stream));
         RVE_CUDA(h, launch_div32(h, h->t32, d, kept_means(mask), h->stream));
         RVE_CUDA(h, launch_fft_forward32(h, d, h->stream, done));
-        RVE_CUDA(h, launch_fft_lapinv32(h, sp, h->stream, done));
+        RVE_CUDA(h, launch_fft_lapinv32(h, h->stream, done));
         RVE_CUDA(h, launch_fft_inverse32(h, u, h->stream, done));
         RVE_CUDA(h, launch_grad_cg32(h, u, mask, h->stream));
       }
@@ -616,8 +634,6 @@ rve_status autotune(rve_s* h) {
   // FFT tile fill targets of the x, y and z passes, one at a time with the
   // others held (forward, Laplace solve, inverse of three fields)
   for (int* target : {&h->fft_fill, &h->fft_fill_y, &h->fft_fill_z}) {
-    SpecParams sp = project_params(h, mask, nullptr, nullptr);
-    sp.op = OP_LAPINV;
     const int cand[4] = {2 * sms, 4 * sms, 8 * sms, 16 * sms};
     float best = 1e30f;
     int pick = *target;
@@ -627,11 +643,11 @@ rve_status autotune(rve_s* h) {
       RVE_TRY(timed([&]() -> cudaError_t {
         if (f32) {
           if (cudaError_t e = launch_fft_forward32(h, h->du32, st, nullptr)) return e;
-          if (cudaError_t e = launch_fft_lapinv32(h, sp, st, nullptr)) return e;
+          if (cudaError_t e = launch_fft_lapinv32(h, st, nullptr)) return e;
           return launch_fft_inverse32(h, h->du32 + 3 * h->nvox, st, nullptr);
         }
         if (cudaError_t e = launch_fft_forward(h, h->q, st, nullptr, 3)) return e;
-        if (cudaError_t e = launch_fft_op(h, sp, st, nullptr, 3)) return e;
+        if (cudaError_t e = launch_fft_lapinv(h, st, nullptr)) return e;
         return launch_fft_inverse(h, h->q + 3 * h->nvox, st, nullptr, 3);
       }, &ms));
       if (ms < best) { best = ms; pick = c; }
@@ -822,7 +838,7 @@ rve_status rve_create(const int32_t* grain_id, int n0, int n1, int n2, const dou
   for (int c = 0; c < 9; ++c) { h->dFbar_prev[c] = 0.0; h->Pmacro[c] = 0.0; h->Smacro[c] = 0.0; }
   make_plan(n0, &h->plan[0]);
   make_plan(n1, &h->plan[1]);
-  make_plan(n2, &h->plan[2], 4);
+  make_plan(n2, &h->plan[2]);
   Consts& c = h->cst;
   c.C11 = mat->C11; c.C12 = mat->C12; c.C44 = mat->C44; c.mu = h->mu; c.b = mat->b;
   c.tau0 = mat->tau0; c.alpha = mat->alpha; c.gdot0 = mat->gdot0; c.n = mat->n; c.K = mat->K; c.yc = mat->yc;
@@ -852,17 +868,18 @@ rve_status rve_create(const int32_t* grain_id, int n0, int n1, int n2, const dou
   for (int g = 0; g < n_grains; ++g) quat_to_R(quat + 4 * g, &R[9 * g]);
   build_tables(*mat, q, Ap, screw);
   const int ns[3] = {n0, n1, n2};
-  std::vector<double2> tw[3], ph[3];
+  std::vector<int4> twq[3];
+  std::vector<double2> ph[3];
   std::vector<double> tn[3], s2[3], c2[3], xi[3];
   std::vector<int8_t> nq[3];
   const double PI = 3.14159265358979323846;
   for (int a = 0; a < 3; ++a) {
     const int n = ns[a];
-    tw[a].resize(n); ph[a].resize(n); tn[a].resize(n); nq[a].resize(n); s2[a].resize(n); c2[a].resize(n);
+    q62_twiddles(n, twq[a]);
+    ph[a].resize(n); tn[a].resize(n); nq[a].resize(n); s2[a].resize(n); c2[a].resize(n);
     xi[a].resize(n);
     for (int t = 0; t < n; ++t) {
       const double ang = 2.0 * PI * (double)t / n;
-      tw[a][t] = make_double2(std::cos(ang), -std::sin(ang));
       const bool nyq = (2 * t == n);
       const int ks = (2 * t <= n) ? t : t - n;
       nq[a][t] = nyq ? 1 : 0;
@@ -875,11 +892,9 @@ rve_status rve_create(const int32_t* grain_id, int n0, int n1, int n2, const dou
     }
     // exact values at the quarter points
     for (int t = 0; t < n; ++t) {
-      if (4 * t == n) { tw[a][t] = make_double2(0.0, -1.0); ph[a][t] = make_double2(0.0, 1.0); }
-      if (4 * t == 3 * n) { tw[a][t] = make_double2(0.0, 1.0); ph[a][t] = make_double2(0.0, -1.0); }
-      if (2 * t == n) tw[a][t] = make_double2(-1.0, 0.0);
+      if (4 * t == n) ph[a][t] = make_double2(0.0, 1.0);
+      if (4 * t == 3 * n) ph[a][t] = make_double2(0.0, -1.0);
     }
-    tw[a][0] = make_double2(1.0, 0.0);
     ph[a][0] = make_double2(1.0, 0.0);
   }
   cudaStream_t s = h->stream;
@@ -889,7 +904,7 @@ rve_status rve_create(const int32_t* grain_id, int n0, int n1, int n2, const dou
                bad(cudaMemcpyAsync(h->Apinv, Ap.data(), 162 * sizeof(double), cudaMemcpyHostToDevice, s)) ||
                bad(cudaMemcpyAsync(h->screw_of, screw.data(), 12 * sizeof(int32_t), cudaMemcpyHostToDevice, s));
   for (int a = 0; a < 3 && !fail_; ++a) {
-    fail_ = bad(cudaMemcpyAsync((void*)h->ax[a].tw, tw[a].data(), ns[a] * sizeof(double2), cudaMemcpyHostToDevice, s)) ||
+    fail_ = bad(cudaMemcpyAsync((void*)h->ax[a].twq, twq[a].data(), ns[a] * sizeof(int4), cudaMemcpyHostToDevice, s)) ||
             bad(cudaMemcpyAsync((void*)h->ax[a].tanh_, tn[a].data(), ns[a] * sizeof(double), cudaMemcpyHostToDevice, s)) ||
             bad(cudaMemcpyAsync((void*)h->ax[a].nyq, nq[a].data(), ns[a] * sizeof(int8_t), cudaMemcpyHostToDevice, s)) ||
             bad(cudaMemcpyAsync((void*)h->ax[a].ph, ph[a].data(), ns[a] * sizeof(double2), cudaMemcpyHostToDevice, s)) ||
@@ -898,7 +913,7 @@ rve_status rve_create(const int32_t* grain_id, int n0, int n1, int n2, const dou
             bad(cudaMemcpyAsync((void*)h->ax[a].xi, xi[a].data(), ns[a] * sizeof(double), cudaMemcpyHostToDevice, s));
     if (!fail_ && h->opt.precision == 1) {
       std::vector<float2> t32(ns[a]);
-      for (int t = 0; t < ns[a]; ++t) t32[t] = make_float2((float)tw[a][t].x, (float)tw[a][t].y);
+      for (int t = 0; t < ns[a]; ++t) t32[t] = make_float2((float)std::cos(2.0 * PI * t / ns[a]), (float)-std::sin(2.0 * PI * t / ns[a]));
       fail_ = bad(cudaMemcpyAsync((void*)h->ax[a].tw32, t32.data(), ns[a] * sizeof(float2), cudaMemcpyHostToDevice, s)) ||
               bad(cudaStreamSynchronize(s));
     }
@@ -1414,17 +1429,16 @@ rve_status rve_time_fft(rve_t* h, int nf, int fp32, int reps, double* ms) {
     return RVE_EINVAL;
   const uint8_t mask[9] = {1, 0, 0, 1, 0, 0, 1, 1, 0};
   SpecParams sp = project_params(h, mask, nullptr, nullptr);
-  sp.op = nf == 3 ? OP_LAPINV : OP_PROJECT;
   cudaStream_t s = h->stream;
   auto pair = [&]() -> cudaError_t {
     cudaError_t e;
     if (fp32) {
       if ((e = launch_fft_forward32(h, h->t32, s, nullptr)) != cudaSuccess) return e;
-      if ((e = launch_fft_lapinv32(h, sp, s, nullptr)) != cudaSuccess) return e;
+      if ((e = launch_fft_lapinv32(h, s, nullptr)) != cudaSuccess) return e;
       return launch_fft_inverse32(h, h->x32, s, nullptr);
     }
     if ((e = launch_fft_forward(h, h->R, s, nullptr, nf)) != cudaSuccess) return e;
-    if ((e = launch_fft_op(h, sp, s, nullptr, nf)) != cudaSuccess) return e;
+    if ((e = nf == 3 ? launch_fft_lapinv(h, s, nullptr) : launch_fft_op(h, sp, s)) != cudaSuccess) return e;
     return launch_fft_inverse(h, h->t, s, nullptr, nf);
   };
   cudaEvent_t e0 = nullptr, e1 = nullptr;

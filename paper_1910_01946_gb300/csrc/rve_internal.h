@@ -23,11 +23,13 @@ struct FFTPlan {
 // Operator applied in frequency space between the forward and inverse z passes.
 //   OP_PROJECT: 9 fields, (G X)_ij = n_j sum_l X_il n_l with the zero-mode mixed control
 //   OP_CURL:    9 fields, G_ij = -eps_jkl D_k X_il
-//   OP_LAPINV:  3 fields, each multiplied by 1 / (64 nvox sum_m s2_m prod_{j!=m} c2_j),
-//               the inverse of D^H D for the unscaled rotated-scheme stencils (0 where it vanishes)
 //   OP_CURL_STD: 9 fields, G_ij = -eps_jkl D_k X_il with the standard (continuous)
 //               spectral derivative D_k = i xi_k / h (Nyquist: 0), for comparison
-enum SpecOp { OP_PROJECT = 0, OP_CURL = 1, OP_LAPINV = 2, OP_CURL_STD = 3 };
+// (The inverse Laplacian of the stencil-factored projection, three fields each
+// multiplied by 1 / (64 nvox sum_m s2_m prod_{j!=m} c2_j), the inverse of D^H D
+// for the unscaled rotated-scheme stencils and 0 where it vanishes, is a pass of
+// its own: launch_fft_lapinv.)
+enum SpecOp { OP_PROJECT = 0, OP_CURL = 1, OP_CURL_STD = 2 };
 
 struct SpecParams {
   int op;
@@ -40,13 +42,13 @@ struct SpecParams {
 
 // Device tables per axis (in the workspace).
 struct AxisTables {
-  const double2* tw;    // e^{-2 pi i t / n}, t = 0..n-1
+  const int4* twq;      // e^{-2 pi i t / n}, t = 0..n-1, in Q62: cosine (high, low), sine (high, low) as fix64.cuh splits them
   const double* tanh_;  // tan(pi k' / n) for the frequency index k (signed k'), Nyquist: 0
   const int8_t* nyq;    // 1 at the Nyquist index of an even n
   const double2* ph;    // e^{i xi_k}, exactly -1 at Nyquist
   const double* s2;     // sin^2(xi_k / 2)
   const double* c2;     // cos^2(xi_k / 2)
-  const float2* tw32;   // the twiddles rounded to float (mixed precision)
+  const float2* tw32;   // the twiddles in float (mixed precision)
   const double* xi;     // xi_k = 2 pi k' / n (signed k'), 0 at Nyquist: the standard frequency
 };
 
@@ -153,6 +155,7 @@ struct rve_s {
   double *bv, *bs;      // BiCGStab vectors v and s
   double2* spec;        // 9 * nspec
   double* lapw;         // nspec: inverse-Laplacian weight of the projection's Laplace solve
+  float* lapw32;        // the same in float (mixed precision)
   // mixed precision (precision == 1): FP32 conjugate-gradient state
   float2* spec32;       // 3 * nspec
   float *x32, *r32, *p32, *t32, *du32;   // 9, 9, 9, 9, 6 components
@@ -192,18 +195,18 @@ enum { DS_RR = 0, DS_PKP = 1, DS_ALPHA = 2, DS_BETA = 3, DS_NORM = 4, DS_STOP = 
 // nf: number of fields transformed (9, or 3 for OP_LAPINV)
 cudaError_t launch_fft_forward(const rve_s* h, const double* in, cudaStream_t s, const double* done = nullptr,
                                int nf = 9);
-cudaError_t launch_fft_op(const rve_s* h, const SpecParams& sp, cudaStream_t s, const double* done = nullptr,
-                          int nf = 9);
+// the operator between the z passes: the inverse Laplacian on three fields, or
+// one of the nine-field operators of SpecParams
+cudaError_t launch_fft_lapinv(const rve_s* h, cudaStream_t s, const double* done);
+cudaError_t launch_fft_op(const rve_s* h, const SpecParams& sp, cudaStream_t s);
 cudaError_t launch_fft_inverse(const rve_s* h, double* out, cudaStream_t s, const double* done = nullptr,
                                int nf = 9);
-// radix passes 8 (up to max_radix), 4, 2, 3.  The x and y passes take radix 8
-// (two shared-memory round trips for 64 points instead of three); the z pass,
-// whose narrow tiles leave few threads per block, is faster with radix 4
-void make_plan(int n, FFTPlan* p, int max_radix = 8);
-// fills h->lapw (once, at create)
+// radix passes 8, 6, 4, 3, 2, the largest first
+void make_plan(int n, FFTPlan* p);
+// fills h->lapw and h->lapw32 (once, at create)
 cudaError_t launch_lapinv_table(const rve_s* h, cudaStream_t s);
 cudaError_t launch_fft_forward32(const rve_s* h, const float* in, cudaStream_t s, const double* done);
-cudaError_t launch_fft_lapinv32(const rve_s* h, const SpecParams& sp, cudaStream_t s, const double* done);
+cudaError_t launch_fft_lapinv32(const rve_s* h, cudaStream_t s, const double* done);
 cudaError_t launch_fft_inverse32(const rve_s* h, float* out, cudaStream_t s, const double* done);
 
 // ---- stencil.cu: G* = D (D^H D)^-1 D^H with real-space rotated-scheme stencils ----

@@ -1,0 +1,119 @@
+"""The hand-written transforms behind the two projections, at axis lengths that
+exercise every radix (8, 6, 4, 3, 2), plans of one to five passes and
+transforms wider than a warp, against numpy's FP64 FFT; and the edges of the
+fixed-point arithmetic inside the FP64 transforms (scales, zeros, NaN)."""
+import numpy as np
+import pytest
+
+import rvegen
+from oracle import spectral as sp
+
+pytestmark = pytest.mark.gpu
+
+MASK = rvegen.UNIAXIAL_X_MASK
+LENGTHS = (2, 4, 6, 12, 16, 18, 24, 32, 36, 54, 64, 96, 108, 128, 162, 192, 256, 324, 432, 486, 512)
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1910_01946_gb300 import _build
+    _build.build()
+    import paper_1910_01946_gb300 as p
+    p.load_library()
+    return p
+
+
+def device_field(X):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(np.moveaxis(X.reshape(X.shape[:3] + (9,)), -1, 0).reshape(9, -1))).cuda()
+
+
+def handle(pkg, shape):
+    n2, n1, n0 = shape
+    return pkg.RVE(np.zeros(shape, dtype=np.int32), np.array([[1.0, 0, 0, 0]]), rvegen.material("Cu"), 1e-5)
+
+
+def noalloc(pkg, shape, Xd):
+    import torch
+    n2, n1, n0 = shape
+    Y = torch.empty_like(Xd)
+    assert pkg.rve_project_noalloc(n0, n1, n2, 1e-5, MASK, Xd.data_ptr(), Y.data_ptr(), 0) == pkg.RVE_OK
+    torch.cuda.synchronize()
+    return Y
+
+
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_every_axis_length_matches_numpy(pkg, axis):
+    """Tolerances: a transform's rounding errors stay within a few 2^-53 of its
+    largest value, and the Fourier-space projection (noalloc) has norm one:
+    1e-14.  The stencil-factored projection divides by the symbol of the
+    derivative, as small as about pi / n near the Nyquist frequencies, so
+    errors of 2^-52 grow by up to n: 4e-15 n."""
+    lengths = LENGTHS + ((1, 3, 9, 27, 81, 243) if axis == 2 else ())
+    for n in lengths:
+        size = [4, 6, 3]
+        size[axis] = n
+        shape = (size[2], size[1], size[0])
+        X = np.random.default_rng(100 * axis + n).standard_normal(shape + (3, 3))
+        ref = device_field(sp.project(X, MASK, 1e-5 / size[0])).cpu()
+        scale = float(ref.abs().max())
+        Xd = device_field(X)
+        r = handle(pkg, shape)
+        Y = r.project(MASK, Xd).cpu()
+        r.close()
+        assert float((Y - ref).abs().max()) < 4e-15 * max(size) * scale, (axis, n, "handle")
+        assert float((noalloc(pkg, shape, Xd).cpu() - ref).abs().max()) < 1e-14 * scale, (axis, n, "noalloc")
+
+
+@pytest.mark.parametrize("shape", [(6, 12, 16), (9, 18, 64)])
+def test_fixed_point_scales(pkg, shape):
+    """Powers of two pass through the projection exactly; near the ends of the
+    FP64 range (where the conversion takes its checked path) the result is the
+    scaled one to round-off; a zero field gives zero."""
+    import torch
+    Xd = device_field(np.random.default_rng(7).standard_normal(shape + (3, 3)))
+    r = handle(pkg, shape)
+    for run in (lambda x: r.project(MASK, x).clone(), lambda x: noalloc(pkg, shape, x)):
+        Y = run(Xd)
+        for k in (-600, -40, 300, 900):
+            assert torch.equal(run(Xd * 2.0 ** k), Y * 2.0 ** k), k
+        big = run(Xd * 2.0 ** 1000) * 2.0 ** -1000
+        assert float((big - Y).abs().max()) < 1e-13 * float(Y.abs().max())
+        assert float(run(torch.zeros_like(Xd)).abs().max()) == 0.0
+    r.close()
+
+
+def test_columns_of_very_different_size_keep_their_digits(pkg):
+    """A field whose rows differ by 2^-30 along y and z: the small tensor row's
+    projection is as accurate as when it stands alone (each transform has its
+    own scale)."""
+    import torch
+    shape = (8, 12, 32)
+    X = np.random.default_rng(11).standard_normal(shape + (3, 3))
+    X[..., 1, :] *= 2.0 ** -30
+    X[..., 2, :] *= 2.0 ** 30
+    ref = device_field(sp.project(X, MASK, 1e-5 / 32)).cpu()
+    Xd = device_field(X)
+    r = handle(pkg, shape)
+    for Y in (r.project(MASK, Xd).cpu(), noalloc(pkg, shape, Xd).cpu()):
+        for i in range(3):
+            rows = slice(3 * i, 3 * i + 3)
+            assert float((Y[rows] - ref[rows]).abs().max()) < 2e-13 * float(ref[rows].abs().max())
+    r.close()
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf"), -float("inf")])
+def test_non_finite_values_reach_every_value_of_their_rows(pkg, bad):
+    import torch
+    shape = (6, 12, 16)
+    Xd = device_field(np.random.default_rng(13).standard_normal(shape + (3, 3)))
+    Xd[4, 77] = bad                                     # component 11: tensor row 1
+    r = handle(pkg, shape)
+    for Y in (r.project(MASK, Xd), noalloc(pkg, shape, Xd)):
+        # (the mean and the constant modes of the other rows do not see it)
+        assert not torch.isfinite(Y[3:6]).any()
+        assert torch.isfinite(Y[:3]).all() and torch.isfinite(Y[6:]).all()
+    r.close()
