@@ -107,8 +107,9 @@ typedef struct {
                             The choice follows measured times, so two tuned handles may differ in
                             reduction order: equal results to round-off, not bit for bit. */
   int32_t stencils;      /* divergence and gradient stencils of the projection: 0 row strips (one
-                            warp per x line, separable, no halo) where n0 is 32, 64, 96 or 128, else
-                            tiles; 1 tiles always.  Equal results to round-off. */
+                            warp per x line, separable, no halo; FP64 fields in 64-bit fixed point)
+                            where n0 is at most 128 (FP32: 32 or 64), else tiles; 1 tiles always.
+                            Equal results to round-off. */
   int32_t continuation;  /* 0..6: when Newton-Raphson fails on an increment (RVE_ENOCONV_NEWTON,
                             _CG or _LOCAL), solve the same increment again from its start with the
                             macroscopic load in 2^k equal stages, k = 1 .. continuation, each stage

@@ -57,8 +57,6 @@ template <typename W> __device__ __forceinline__ CX<W> add(CX<W> a, CX<W> b) { r
 template <typename W> __device__ __forceinline__ CX<W> sub(CX<W> a, CX<W> b) { return mk<W>(a.x - b.x, a.y - b.y); }
 template <int SIGN, typename W>
 __device__ __forceinline__ CX<W> mul_i(CX<W> a) { return SIGN > 0 ? mk<W>(-a.y, a.x) : mk<W>(a.y, -a.x); }
-__device__ __forceinline__ double2 st2(double a, double b) { return make_double2(a, b); }
-__device__ __forceinline__ float2 st2(float a, float b) { return make_float2(a, b); }
 
 // x / sqrt 2, x sqrt(3) / 2, x / 2
 __device__ __forceinline__ float by_r2(float x) { return 0.70710678f * x; }
@@ -219,25 +217,29 @@ __device__ __forceinline__ void pass_r(const PlanDev& pl, int p, int tj, const T
 }
 
 // The transform whose first butterfly's points (tj + m T) are in a[]: the
-// first pass writes b0, the others alternate b1, b0, ...; the caller
-// synchronises before it reads the result (in natural order) from the buffer
-// returned, the same for every thread.  idx maps a position of this thread's
-// transform to its shared-memory element.  All threads of the block call it
-// (barriers); `on`: this thread holds a transform.
+// first pass writes b0, the others alternate b1, b0, ..., the last one hands
+// its results to st(pos, value); with `shared`, st is not used and the last pass
+// goes to a buffer as well, which last_buffer() names.  idx maps a position of
+// this thread's transform to its shared-memory element.  All threads of the
+// block call it (barriers); `on`: this thread holds a transform.
 //
-// The results are converted and stored by a rolled loop of the caller and not
-// by the butterflies: inlined into every radix, the conversions made the code
-// a warp runs once so long that fetching it was the largest stall (6-8
-// cycles per instruction issued; y pass at 64^3 12 us instead of 8).
-template <int SIGN, typename R, class Idx>
-__device__ __forceinline__ C<R>* transform(C<R>* a, C<R>* b0, C<R>* b1, const PlanDev& pl, int tj, bool on, Idx idx,
-                                           const TW<R>* __restrict__ tw) {
+// st only stores: conversions belong into a rolled loop over a shared result.
+// Inlined into every radix they made the code a warp runs once so long that
+// fetching it was the largest stall (6-8 cycles per instruction issued).
+template <int SIGN, typename R, class Idx, class St>
+__device__ __forceinline__ void transform(C<R>* a, C<R>* b0, C<R>* b1, const PlanDev& pl, int tj, bool on, Idx idx,
+                                          const TW<R>* __restrict__ tw, bool shared, St st) {
+  const int last = shared ? -1 : pl.npass - 1;        // the pass that goes to st
   if (on) {
+    auto put = [&](int pos, C<R> v) {
+      if (last >= 0 && last == 0) st(pos, v);
+      else b0[idx(pos)] = v;
+    };
     auto first = [&](auto rad) {
       constexpr int RAD = decltype(rad)::value;
       dft<SIGN, RAD>(a);
 #pragma unroll
-      for (int m = 0; m < RAD; ++m) b0[idx(tj * RAD + m)] = a[m];
+      for (int m = 0; m < RAD; ++m) put(tj * RAD + m, a[m]);
     };
     switch (pl.radix[0]) {
       case 8: first(std::integral_constant<int, 8>()); break;
@@ -245,7 +247,10 @@ __device__ __forceinline__ C<R>* transform(C<R>* a, C<R>* b0, C<R>* b1, const Pl
       case 4: first(std::integral_constant<int, 4>()); break;
       case 3: first(std::integral_constant<int, 3>()); break;
       case 2: first(std::integral_constant<int, 2>()); break;
-      default: b0[idx(0)] = a[0]; break;
+      default:                                        // length 1
+        if (shared) b0[idx(0)] = a[0];
+        else st(0, a[0]);
+        break;
     }
   }
   for (int p = 1; p < pl.npass; ++p) {
@@ -254,32 +259,28 @@ __device__ __forceinline__ C<R>* transform(C<R>* a, C<R>* b0, C<R>* b1, const Pl
       C<R>* src = (p & 1) ? b0 : b1;
       C<R>* dst = (p & 1) ? b1 : b0;
       auto ld = [&](int pos) { return src[idx(pos)]; };
-      auto st = [&](int pos, C<R> v) { dst[idx(pos)] = v; };
+      auto put = [&](int pos, C<R> v) {
+        if (p == last) st(pos, v);
+        else dst[idx(pos)] = v;
+      };
       switch (pl.radix[p]) {
-        case 8: pass_r<SIGN, R, 8>(pl, p, tj, tw, ld, st); break;
-        case 6: pass_r<SIGN, R, 6>(pl, p, tj, tw, ld, st); break;
-        case 4: pass_r<SIGN, R, 4>(pl, p, tj, tw, ld, st); break;
-        case 3: pass_r<SIGN, R, 3>(pl, p, tj, tw, ld, st); break;
-        default: pass_r<SIGN, R, 2>(pl, p, tj, tw, ld, st); break;
+        case 8: pass_r<SIGN, R, 8>(pl, p, tj, tw, ld, put); break;
+        case 6: pass_r<SIGN, R, 6>(pl, p, tj, tw, ld, put); break;
+        case 4: pass_r<SIGN, R, 4>(pl, p, tj, tw, ld, put); break;
+        case 3: pass_r<SIGN, R, 3>(pl, p, tj, tw, ld, put); break;
+        default: pass_r<SIGN, R, 2>(pl, p, tj, tw, ld, put); break;
       }
     }
   }
+}
+template <typename W>
+__device__ __forceinline__ CX<W>* last_buffer(const PlanDev& pl, CX<W>* b0, CX<W>* b1) {
   return (pl.npass > 1 && !(pl.npass & 1)) ? b1 : b0;
 }
+struct NoStore { template <typename Z> __device__ void operator()(int, Z) const {} };
 
-// ---- conversions: doubles on the block's common scale, floats as they are ----
-__device__ __forceinline__ unsigned mag_of(double2 v) { return max(fix64::mag(v.x), fix64::mag(v.y)); }
-__device__ __forceinline__ unsigned mag_of(float2) { return 0u; }
-__device__ __forceinline__ unsigned mag_of(double v) { return fix64::mag(v); }
-__device__ __forceinline__ unsigned mag_of(float) { return 0u; }
-__device__ __forceinline__ i64 to_work(double x, int s0) { return fix64::to_fix(x, s0); }
-__device__ __forceinline__ float to_work(float x, int) { return x; }
-template <typename R> __device__ __forceinline__ R from_work(typename FT<R>::w v, int eb);
-template <> __device__ __forceinline__ double from_work<double>(i64 v, int eb) { return fix64::from_fix(v, eb); }
-template <> __device__ __forceinline__ float from_work<float>(float v, int) { return v; }
-
-// Exponent of the largest magnitude of a transform's points (FP64; all
-// threads call it).  Each transform has its own: the spectra of neighbouring
+// ---- the common scale of a transform's points (FP64; all threads call it) ----
+// Each transform has its own: the spectra of neighbouring
 // columns differ by orders of magnitude (the divergence has almost nothing
 // near the Nyquist frequencies, where the inverse Laplacian is largest), and a
 // column on a larger scale than its own would lose what FP64 keeps.
@@ -288,7 +289,7 @@ template <> __device__ __forceinline__ float from_work<float>(float v, int) { re
 // column across them.
 constexpr int MAX_WARPS = 8;
 template <typename R>
-__device__ __forceinline__ int column_exp(unsigned key, int cpb, unsigned* red) {
+__device__ __forceinline__ int column_max(int key, int cpb, int* red) {
   if (sizeof(R) == 4) return 0;
   for (int o = cpb; o < 32; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
   const int nw = blockDim.x >> 5;
@@ -298,17 +299,17 @@ __device__ __forceinline__ int column_exp(unsigned key, int cpb, unsigned* red) 
     __syncthreads();
     for (int w = 0; w < nw; ++w) key = max(key, red[w * 32 + c]);
   }
-  return fix64::tile_exp(key);
+  return key;
 }
 // Rows (X): T consecutive threads.  T a power of two up to 32: shuffles only;
-// other lengths share the block's largest magnitude (rows next to each other
+// other lengths share the block's largest key (rows next to each other
 // in real space, or of one kx range).
 template <typename R>
-__device__ __forceinline__ int row_exp(unsigned key, int T, unsigned* red) {
+__device__ __forceinline__ int row_max(int key, int T, int* red) {
   if (sizeof(R) == 4) return 0;
   if (T <= 32 && (T & (T - 1)) == 0) {
     for (int o = 1; o < T; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
-    return fix64::tile_exp(key);
+    return key;
   }
   key = __reduce_max_sync(0xffffffffu, key);
   const int nw = blockDim.x >> 5;
@@ -317,23 +318,74 @@ __device__ __forceinline__ int row_exp(unsigned key, int T, unsigned* red) {
     __syncthreads();
     for (int w = 0; w < nw; ++w) key = max(key, red[w]);
   }
-  return fix64::tile_exp(key);
+  return key;
 }
 
+// Points as they lie in memory, their key and their conversion to a transform's
+// scale.  Three storages:
+//   Plain<float>:  floats, no scale;
+//   Plain<double>: doubles, scaled by the exponent of the largest (to_fix);
+//   Fixed:         64-bit integers with a scale of their own per row or column
+//                  (the ex arrays), as the three-field transforms of the
+//                  projection keep them between their passes: no conversion, only shifts.
+__device__ __forceinline__ double2 st2(double a, double b) { return make_double2(a, b); }
+__device__ __forceinline__ float2 st2(float a, float b) { return make_float2(a, b); }
+template <typename R> struct Plain {
+  typedef V2<R> pair;
+  typedef R real;
+  static constexpr bool FIX = false;
+  static constexpr bool direct = sizeof(R) == 4;      // the last pass stores its results itself
+  __device__ static int key(pair v, int) { return max(key(v.x, 0), key(v.y, 0)); }
+  __device__ static int key(double v, int) { return (int)fix64::mag(v); }
+  __device__ static int key(float, int) { return 0; }
+  // the scale as an output exponent base (see fix64::from_fix)
+  __device__ static int scale(int key, int B) { return sizeof(R) == 4 ? 0 : fix64::out_base(fix64::tile_exp((unsigned)key), B); }
+  __device__ static i64 work(double x, int, int E, int B) {
+    // (NaN tiles: any shift; their results are marked by E)
+    return fix64::to_fix(x, E >= fix64::EXP_BAD ? 0x7ff : E - 1);
+  }
+  __device__ static float work(float x, int, int, int) { return x; }
+  // a result on the scale eb
+  __device__ static pair store(C<R> z, int eb) {
+    if constexpr (sizeof(R) == 4) return st2(z.x, z.y);
+    else return st2(fix64::from_fix(z.x, eb), fix64::from_fix(z.y, eb));
+  }
+};
+struct Fixed {
+  typedef longlong2 pair;
+  typedef i64 real;
+  static constexpr bool FIX = true;
+  static constexpr bool direct = true;
+  __device__ static int key(pair v, int ex) { return fix64::fit_key(fix64::abs_hi(v.x) | fix64::abs_hi(v.y), ex); }
+  __device__ static int key(i64 v, int ex) { return fix64::fit_key(fix64::abs_hi(v), ex); }
+  __device__ static int scale(int key, int B) { return fix64::key_scale(key, B); }
+  __device__ static i64 work(i64 v, int ex, int E, int) { return fix64::rescale(v, ex, E); }
+  __device__ static pair store(CX<i64> z, int) { return make_longlong2(z.x, z.y); }
+};
+template <class S> __device__ __forceinline__ typename S::pair zero_pair() {
+  typename S::pair z;
+  z.x = z.y = (typename S::real)0;
+  return z;
+}
 extern __shared__ __align__(16) unsigned char fft_smem[];
 
 // element of position p of row `row` in the X passes (one pad element every
 // eight: the strided writes of a radix-8 pass spread over the banks)
 __device__ __forceinline__ int row_elem(int row, int n, int p) { return row * (n + (n >> 3) + 1) + p + (p >> 3); }
 
+// Scales of the three-field transforms, one int each: of the divergence's rows
+// (tensor row, z, y), of the row pairs of both X passes (field, z, y / 2), and of the columns
+// (field, z, kx) after the Y passes and (field, ky, kx) after the Z pass.  Unused by the other storages.
+
 // ---------------------------------------------------------------- pass X (R2C)
-// in: real fields (type R); spec: half spectrum (pairs of R).  rows: number of
-// row pairs over all fields; rpb of them per block, T threads each.
-template <typename R>
-__global__ void __launch_bounds__(256) k_fft_x_r2c(const R* __restrict__ in, V2<R>* __restrict__ spec, int rows,
-                                                   int nkx, int rpb, PlanDev pl, const TW<R>* __restrict__ tw,
-                                                   const double* __restrict__ done) {
-  __shared__ unsigned red[MAX_WARPS];
+// in: real fields; spec: half spectrum.  rows: number of row pairs over all
+// fields; rpb of them per block, T threads each.
+template <typename R, class In, class Out>
+__global__ void __launch_bounds__(256) k_fft_x_r2c(const typename In::real* __restrict__ in, const int* __restrict__ exin,
+                                                   typename Out::pair* __restrict__ spec, int* __restrict__ exout,
+                                                   int rows, int nkx, int rpb, PlanDev pl,
+                                                   const TW<R>* __restrict__ tw, const double* __restrict__ done) {
+  __shared__ int red[MAX_WARPS];
   __shared__ int ebs[256];               // output scale of each row pair
   const int n0 = pl.n;
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
@@ -341,25 +393,32 @@ __global__ void __launch_bounds__(256) k_fft_x_r2c(const R* __restrict__ in, V2<
   const int row = fdiv(threadIdx.x, pl.tdiv), tj = threadIdx.x - row * pl.T;
   const long g0 = (long)blockIdx.x * rpb, g = g0 + row;
   const bool on = row < rpb && g < rows;
-  const R* src = in + (size_t)(on ? g : 0) * 2 * n0;
-  R u[RMAX], v[RMAX];
-  unsigned key = 0u;
+  const typename In::real* src = in + (size_t)(on ? g : 0) * 2 * n0;
+  const int eu = In::FIX && on ? exin[2 * g] : 0, ev = In::FIX && on ? exin[2 * g + 1] : 0;
+  typename In::real u[RMAX], v[RMAX];
 #pragma unroll
   for (int m = 0; m < RMAX; ++m) {
-    u[m] = v[m] = (R)0;
+    u[m] = v[m] = 0;
     if (on && m < pl.r0) {
       u[m] = src[tj + m * pl.T];
       v[m] = src[n0 + tj + m * pl.T];
-      key = max(key, max(mag_of(u[m]), mag_of(v[m])));
     }
   }
   if (done && *done != 0.0) return;
-  const int e = row_exp<R>(key, pl.T, red), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
+  int key = In::FIX ? 2 * fix64::EXP_ZERO : 0;
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m)
+    if (on && m < pl.r0) key = max(key, max(In::key(u[m], eu), In::key(v[m], ev)));
+  const int E = In::scale(row_max<R>(key, pl.T, red), pl.bits), eb = E + pl.down;
   C<R> a[RMAX];
 #pragma unroll
-  for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[m], s0), to_work(v[m], s0));
-  const C<R>* res = transform<-1, R>(a, b0, b1, pl, tj, on, [&](int p) { return row_elem(row, n0, p); }, tw);
-  if (tj == 0 && row < rpb) ebs[row] = eb;
+  for (int m = 0; m < RMAX; ++m) a[m] = mk(In::work(u[m], eu, E, pl.bits), In::work(v[m], ev, E, pl.bits));
+  transform<-1, R>(a, b0, b1, pl, tj, on, [&](int p) { return row_elem(row, n0, p); }, tw, true, NoStore());
+  const C<R>* res = last_buffer(pl, b0, b1);
+  if (tj == 0 && on) {
+    ebs[row] = eb;
+    if (Out::FIX) exout[g] = eb;
+  }
   __syncthreads();
   // the two half spectra are Z(k) +/- conj(Z(n0 - k)) without the factor 1/2
   // of the split: every operator applied between the z passes carries it in
@@ -371,49 +430,58 @@ __global__ void __launch_bounds__(256) k_fft_x_r2c(const R* __restrict__ in, V2<
     const C<R> zk = res[row_elem(jj, n0, k)];
     const C<R> zc = res[row_elem(jj, n0, k == 0 ? 0 : n0 - k)];
     const int ej = ebs[jj];
-    V2<R>* dst = spec + (size_t)(g0 + jj) * 2 * nkx + k;
-    dst[0] = st2(from_work<R>(zk.x + zc.x, ej), from_work<R>(zk.y - zc.y, ej));
-    dst[nkx] = st2(from_work<R>(zk.y + zc.y, ej), from_work<R>(zc.x - zk.x, ej));
+    typename Out::pair* dst = spec + (size_t)(g0 + jj) * 2 * nkx + k;
+    dst[0] = Out::store(mk(zk.x + zc.x, zk.y - zc.y), ej);
+    dst[nkx] = Out::store(mk(zk.y + zc.y, zc.x - zk.x), ej);
   }
 }
 
 // ---------------------------------------------------------------- pass X^-1 (C2R)
-template <typename R>
-__global__ void __launch_bounds__(256) k_fft_x_c2r(const V2<R>* __restrict__ spec, R* __restrict__ out, int rows,
-                                                   int nkx, int rpb, PlanDev pl, const TW<R>* __restrict__ tw,
-                                                   const double* __restrict__ done) {
-  __shared__ unsigned red[MAX_WARPS];
+// S: storage of the spectrum (In) and of the real fields (Out)
+template <typename R, class In, class Out>
+__global__ void __launch_bounds__(256) k_fft_x_c2r(const typename In::pair* __restrict__ spec, const int* __restrict__ exin,
+                                                   typename Out::real* __restrict__ out, int* __restrict__ exout,
+                                                   int rows, int rows_per_plane, int nkx, int rpb, PlanDev pl,
+                                                   const TW<R>* __restrict__ tw, const double* __restrict__ done) {
+  __shared__ int red[MAX_WARPS];
   const int n0 = pl.n;
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
   C<R>* b1 = b0 + rpb * (n0 + (n0 >> 3) + 1);
   const int row = fdiv(threadIdx.x, pl.tdiv), tj = threadIdx.x - row * pl.T;
   const long g = (long)blockIdx.x * rpb + row;
   const bool on = row < rpb && g < rows;
-  const V2<R>* src = spec + (size_t)(on ? g : 0) * 2 * nkx;
+  const typename In::pair* src = spec + (size_t)(on ? g : 0) * 2 * nkx;
+  const int* exs = In::FIX ? exin + (size_t)(on ? g / rows_per_plane : 0) * nkx : nullptr;
   // the row pair's spectra A, B at k = tj + m T <= n0 / 2 (at most RMAX / 2
   // + 1 of them) give Z(k) = A + i B and Z(n0 - k) = conj(A) + i conj(B)
   constexpr int HM = RMAX / 2 + 1;
-  V2<R> A[HM], B[HM];
-  unsigned key = 0u;
+  typename In::pair A[HM], B[HM];
+  int ex[HM];
+  const int bits = pl.bits - 1;          // (the sums A + i B double the components: one bit less)
 #pragma unroll
   for (int m = 0; m < HM; ++m) {
-    A[m] = B[m] = st2((R)0, (R)0);
+    A[m] = B[m] = zero_pair<In>();
+    ex[m] = 0;
     if (on && tj + m * pl.T < nkx) {
       A[m] = src[tj + m * pl.T];
       B[m] = src[nkx + tj + m * pl.T];
-      key = max(key, max(mag_of(A[m]), mag_of(B[m])));
+      if (In::FIX) ex[m] = exs[tj + m * pl.T];
     }
   }
   if (done && *done != 0.0) return;
-  // (the sums A + i B double the components: one bit less)
-  const int e = row_exp<R>(key, pl.T, red), bits = pl.bits - 1;
-  const int s0 = e + 63 - bits, eb = fix64::out_base(e, bits, pl.down);
+  int key = In::FIX ? 2 * fix64::EXP_ZERO : 0;
+#pragma unroll
+  for (int m = 0; m < HM; ++m)
+    if (on && tj + m * pl.T < nkx) key = max(key, max(In::key(A[m], ex[m]), In::key(B[m], ex[m])));
+  const int E = In::scale(row_max<R>(key, pl.T, red), bits), eb = E + pl.down;
   if (on) {
+    if (Out::FIX && tj == 0) exout[g] = eb;
 #pragma unroll
     for (int m = 0; m < HM; ++m) {
       const int k = tj + m * pl.T;
       if (k < nkx) {
-        const C<R> z = mk(to_work(A[m].x, s0), to_work(A[m].y, s0)), w = mk(to_work(B[m].x, s0), to_work(B[m].y, s0));
+        const C<R> z = mk(In::work(A[m].x, ex[m], E, bits), In::work(A[m].y, ex[m], E, bits));
+        const C<R> w = mk(In::work(B[m].x, ex[m], E, bits), In::work(B[m].y, ex[m], E, bits));
         b1[row_elem(row, n0, k)] = mk(z.x - w.y, z.y + w.x);
         if (k > 0 && 2 * k < n0) b1[row_elem(row, n0, n0 - k)] = mk(z.x + w.y, w.x - z.y);
       }
@@ -424,53 +492,76 @@ __global__ void __launch_bounds__(256) k_fft_x_c2r(const V2<R>* __restrict__ spe
 #pragma unroll
   for (int m = 0; m < RMAX; ++m)
     if (on && m < pl.r0) a[m] = b1[row_elem(row, n0, tj + m * pl.T)];
-  R* dst = out + (size_t)g * 2 * n0;
-  const C<R>* res = transform<+1, R>(a, b0, b1, pl, tj, on, [&](int p) { return row_elem(row, n0, p); }, tw);
-  __syncthreads();
-  if (!on) return;
+  typename Out::real* dst = out + (size_t)(on ? g : 0) * 2 * n0;
+  transform<+1, R>(a, b0, b1, pl, tj, on, [&](int p) { return row_elem(row, n0, p); }, tw, !Out::direct,
+                   [&](int p, C<R> z) {
+                     if constexpr (Out::direct) {
+                       dst[p] = (typename Out::real)z.x;
+                       dst[n0 + p] = (typename Out::real)z.y;
+                     }
+                   });
+  if constexpr (!Out::direct) {
+    __syncthreads();
+    if (!on) return;
+    const C<R>* res = last_buffer(pl, b0, b1);
 #pragma unroll 1
-  for (int p = tj; p < n0; p += pl.T) {
-    const C<R> z = res[row_elem(row, n0, p)];
-    dst[p] = from_work<R>(z.x, eb);
-    dst[n0 + p] = from_work<R>(z.y, eb);
+    for (int p = tj; p < n0; p += pl.T) {
+      const typename Out::pair v = Out::store(res[row_elem(row, n0, p)], eb);
+      dst[p] = v.x;
+      dst[n0 + p] = v.y;
+    }
   }
 }
 
 // ---------------------------------------------------------------- pass Y (C2C)
-// ncol columns (field, z, kx), cpb consecutive ones per block, kx fastest
-template <int SIGN, typename R>
-__global__ void __launch_bounds__(256) k_fft_y(V2<R>* __restrict__ spec, int ncol, int nkx, int cpb, PlanDev pl,
+// ncol columns (field, z, kx), cpb consecutive ones per block, kx fastest.
+// Scales of stored integers, in: forward, of the row pairs (plane, y / 2); inverse,
+// of the columns (field, y, kx) of the Z pass.  Out: of the columns (plane, kx).
+template <int SIGN, typename R, class S>
+__global__ void __launch_bounds__(256) k_fft_y(typename S::pair* __restrict__ spec, const int* __restrict__ exin,
+                                               int* __restrict__ exout, int ncol, int n2, int nkx, int cpb, PlanDev pl,
                                                const TW<R>* __restrict__ tw, const double* __restrict__ done) {
-  __shared__ unsigned red[MAX_WARPS * 32];
+  __shared__ int red[MAX_WARPS * 32];
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
   C<R>* b1 = b0 + cpb * pl.n;
   const int tj = threadIdx.x / cpb, c = threadIdx.x - tj * cpb;     // cpb: a power of two
   const long col = (long)blockIdx.x * cpb + c;
   const bool on = tj < pl.T && col < ncol;
   const int plane = on ? (int)(col / nkx) : 0, kx = on ? (int)(col - (long)plane * nkx) : 0;
-  V2<R>* base = spec + (size_t)plane * pl.n * nkx + kx;
-  V2<R> u[RMAX];
-  unsigned key = 0u;
+  typename S::pair* base = spec + (size_t)plane * pl.n * nkx + kx;
+  const int* exs = nullptr;
+  if (S::FIX) exs = SIGN < 0 ? exin + (size_t)plane * (pl.n / 2) : exin + (size_t)(plane / n2) * pl.n * nkx + kx;
+  typename S::pair u[RMAX];
+  int ex[RMAX];
 #pragma unroll
   for (int m = 0; m < RMAX; ++m) {
-    u[m] = st2((R)0, (R)0);
+    u[m] = zero_pair<S>();
+    ex[m] = 0;
     if (on && m < pl.r0) {
-      u[m] = base[(size_t)(tj + m * pl.T) * nkx];
-      key = max(key, mag_of(u[m]));
+      const int y = tj + m * pl.T;
+      u[m] = base[(size_t)y * nkx];
+      if (S::FIX) ex[m] = SIGN < 0 ? exs[y >> 1] : exs[(size_t)y * nkx];
     }
   }
   if (done && *done != 0.0) return;
-  const int e = column_exp<R>(key, cpb, red), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
+  int key = S::FIX ? 2 * fix64::EXP_ZERO : 0;
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m)
+    if (on && m < pl.r0) key = max(key, S::key(u[m], ex[m]));
+  const int E = S::scale(column_max<R>(key, cpb, red), pl.bits), eb = E + pl.down;
   C<R> a[RMAX];
 #pragma unroll
-  for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[m].x, s0), to_work(u[m].y, s0));
-  const C<R>* res = transform<SIGN, R>(a, b0, b1, pl, tj, on, [&](int p) { return p * cpb + c; }, tw);
-  __syncthreads();
-  if (!on) return;
+  for (int m = 0; m < RMAX; ++m) a[m] = mk(S::work(u[m].x, ex[m], E, pl.bits), S::work(u[m].y, ex[m], E, pl.bits));
+  if (S::FIX && on && tj == 0) exout[col] = eb;
+  transform<SIGN, R>(a, b0, b1, pl, tj, on, [&](int p) { return p * cpb + c; }, tw, !S::direct, [&](int p, C<R> z) {
+    if constexpr (S::direct) base[(size_t)p * nkx] = S::store(z, 0);
+  });
+  if constexpr (!S::direct) {
+    __syncthreads();
+    if (!on) return;
+    const C<R>* res = last_buffer(pl, b0, b1);
 #pragma unroll 1
-  for (int p = tj; p < pl.n; p += pl.T) {
-    const C<R> z = res[p * cpb + c];
-    base[(size_t)p * nkx] = st2(from_work<R>(z.x, eb), from_work<R>(z.y, eb));
+    for (int p = tj; p < pl.n; p += pl.T) base[(size_t)p * nkx] = S::store(res[p * cpb + c], eb);
   }
 }
 
@@ -568,66 +659,79 @@ __global__ void k_lapinv_table(double* __restrict__ w, float* __restrict__ w32, 
 // ---------------------------------------------------------------- pass Z + operator
 // np pencils (ky, kx) of every field, cpb consecutive ones per block; the
 // inverse Laplacian treats each field by itself (blockIdx.y: the field)
-template <typename R>
-__global__ void __launch_bounds__(256) k_fft_z_lap(V2<R>* __restrict__ spec, int np, int cpb, PlanDev pl,
+__device__ __forceinline__ CX<float> weighted(CX<float> z, float w, int, int&) {
+  return mk<float>(z.x * w, z.y * w);
+}
+// the weight's significand as a Q62 factor, its exponent into the scale
+__device__ __forceinline__ CX<i64> weighted(CX<i64> z, double w, int eb, int& ex) {
+  const int hi = __double2hiint(w), lo = __double2loint(w);
+  const fix64::Sp m = fix64::split(((i64)((((hi & 0xfffff) | 0x100000) << 9) | (int)((unsigned)lo >> 23)) << 32) |
+                                   (i64)((unsigned)lo << 9));
+  ex = hi ? eb + (hi >> 20) - 1022 : fix64::EXP_ZERO;
+  return hi ? mk<i64>(fix64::mulq(z.x, m.h, m.l), fix64::mulq(z.y, m.h, m.l)) : mk<i64>(0, 0);
+}
+
+template <typename R, class S>
+__global__ void __launch_bounds__(256) k_fft_z_lap(typename S::pair* __restrict__ spec, const int* __restrict__ exin,
+                                                   int* __restrict__ exout, int np, int nkx, int cpb, PlanDev pl,
                                                    const TW<R>* __restrict__ tw, const R* __restrict__ weight,
                                                    const double* __restrict__ done) {
-  __shared__ unsigned red[2][MAX_WARPS * 32];
+  __shared__ int red[2][MAX_WARPS * 32];
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
   C<R>* b1 = b0 + cpb * pl.n;
   const int tj = threadIdx.x / cpb, c = threadIdx.x - tj * cpb;
   const int pc = blockIdx.x * cpb + c;
   const bool on = tj < pl.T && pc < np;
-  V2<R>* base = spec + (size_t)blockIdx.y * pl.n * np + (on ? pc : 0);
-  V2<R> u[RMAX];
-  unsigned key = 0u;
+  typename S::pair* base = spec + (size_t)blockIdx.y * pl.n * np + (on ? pc : 0);
+  const int* exs = S::FIX ? exin + (size_t)blockIdx.y * pl.n * nkx + (on ? pc % nkx : 0) : nullptr;
+  typename S::pair u[RMAX];
+  R w[RMAX];
+  int ex[RMAX];
 #pragma unroll
   for (int m = 0; m < RMAX; ++m) {
-    u[m] = st2((R)0, (R)0);
+    u[m] = zero_pair<S>();
+    w[m] = (R)0;
+    ex[m] = 0;
     if (on && m < pl.r0) {
-      u[m] = base[(size_t)(tj + m * pl.T) * np];
-      key = max(key, mag_of(u[m]));
+      const int z = tj + m * pl.T;
+      u[m] = base[(size_t)z * np];
+      if (S::FIX) ex[m] = exs[(size_t)z * nkx];
+      w[m] = __ldg(weight + (size_t)z * np + pc);
     }
   }
   if (done && *done != 0.0) return;
-  int e = column_exp<R>(key, cpb, red[0]), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
-  C<R> a[RMAX];
-#pragma unroll
-  for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[m].x, s0), to_work(u[m].y, s0));
-  auto idx = [&](int p) { return p * cpb + c; };
-  C<R>* res = transform<-1, R>(a, b0, b1, pl, tj, on, idx, tw);
-  __syncthreads();
-  key = 0u;
-  // weighted in R and kept in place (a thread reads only the points it writes here)
-  V2<R>* wres = reinterpret_cast<V2<R>*>(res);
-  if (on) {
-#pragma unroll 1
-    for (int p = tj; p < pl.n; p += pl.T) {
-      const C<R> z = res[idx(p)];
-      const R w = __ldg(weight + (size_t)p * np + pc);
-      const V2<R> v = st2(from_work<R>(z.x, eb) * w, from_work<R>(z.y, eb) * w);
-      wres[idx(p)] = v;
-      key = max(key, mag_of(v));
-    }
-  }
-  e = column_exp<R>(key, cpb, red[1]);
-  s0 = e + 63 - pl.bits;
-  eb = fix64::out_base(e, pl.bits, pl.down);
+  int key = S::FIX ? 2 * fix64::EXP_ZERO : 0;
 #pragma unroll
   for (int m = 0; m < RMAX; ++m)
-    if (on && m < pl.r0) {
-      const V2<R> v = wres[idx(tj + m * pl.T)];
-      a[m] = mk(to_work(v.x, s0), to_work(v.y, s0));
-    }
-  // the inverse starts in the other buffer: this one may still be read
-  res = transform<+1, R>(a, res == b0 ? b1 : b0, res, pl, tj, on, idx, tw);
+    if (on && m < pl.r0) key = max(key, S::key(u[m], ex[m]));
+  int E = S::scale(column_max<R>(key, cpb, red[0]), pl.bits), eb = E + pl.down;
+  C<R> a[RMAX];
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m) a[m] = mk(S::work(u[m].x, ex[m], E, pl.bits), S::work(u[m].y, ex[m], E, pl.bits));
+  auto idx = [&](int p) { return p * cpb + c; };
+  transform<-1, R>(a, b0, b1, pl, tj, on, idx, tw, true, NoStore());
+  C<R>* res = last_buffer(pl, b0, b1);
   __syncthreads();
-  if (!on) return;
-#pragma unroll 1
-  for (int p = tj; p < pl.n; p += pl.T) {
-    const C<R> z = res[idx(p)];
-    base[(size_t)p * np] = st2(from_work<R>(z.x, eb), from_work<R>(z.y, eb));
+  key = S::FIX ? 2 * fix64::EXP_ZERO : 0;
+#pragma unroll
+  for (int m = 0; m < RMAX; ++m) {
+    a[m] = mk((typename FT<R>::w)0, (typename FT<R>::w)0);
+    if (on && m < pl.r0) {
+      a[m] = weighted(res[idx(tj + m * pl.T)], w[m], eb, ex[m]);
+      if constexpr (S::FIX) key = max(key, S::key(make_longlong2(a[m].x, a[m].y), ex[m]));
+    }
   }
+  E = S::scale(column_max<R>(key, cpb, red[1]), pl.bits);
+  eb = E + pl.down;
+  if constexpr (S::FIX) {
+#pragma unroll
+    for (int m = 0; m < RMAX; ++m) a[m] = mk(S::work(a[m].x, ex[m], E, pl.bits), S::work(a[m].y, ex[m], E, pl.bits));
+    if (on && tj == 0) exout[(size_t)blockIdx.y * np + pc] = eb;
+  }
+  // the inverse starts in the other buffer: this one may still be read
+  transform<+1, R>(a, res == b0 ? b1 : b0, res, pl, tj, on, idx, tw, false, [&](int p, C<R> z) {
+    base[(size_t)p * np] = S::store(z, 0);
+  });
 }
 
 // The operators that couple the three fields of a tensor row (projection and
@@ -636,7 +740,8 @@ __global__ void __launch_bounds__(256) k_fft_z_lap(V2<R>* __restrict__ spec, int
 __global__ void __launch_bounds__(128) k_fft_z_op(double2* __restrict__ spec, int np, int nkx, int cpb, PlanDev pl,
                                                   const int4* __restrict__ tw, OpTables T, SpecParams sp) {
   typedef double R;
-  __shared__ unsigned red[4][MAX_WARPS * 32];
+  __shared__ int red[4][MAX_WARPS * 32];
+  typedef Plain<double> S;
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
   C<R>* b1 = b0 + cpb * pl.n;
   const int tj = threadIdx.x / cpb, c = threadIdx.x - tj * cpb;
@@ -655,24 +760,25 @@ __global__ void __launch_bounds__(128) k_fft_z_op(double2* __restrict__ spec, in
     }
 #pragma unroll
   for (int f = 0; f < 3; ++f) {
-    unsigned key = 0u;
+    int key = 0;
 #pragma unroll
-    for (int m = 0; m < RMAX; ++m) key = max(key, mag_of(u[f][m]));
+    for (int m = 0; m < RMAX; ++m) key = max(key, S::key(u[f][m], 0));
     if (f) __syncthreads();                       // the previous field's results are read
-    const int e = column_exp<R>(key, cpb, red[f]), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
+    const int E = S::scale(column_max<R>(key, cpb, red[f]), pl.bits), eb = E + pl.down;
     C<R> a[RMAX];
 #pragma unroll
-    for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[f][m].x, s0), to_work(u[f][m].y, s0));
-    const C<R>* res = transform<-1, R>(a, b0, b1, pl, tj, on, idx, tw);
+    for (int m = 0; m < RMAX; ++m) a[m] = mk(S::work(u[f][m].x, 0, E, pl.bits), S::work(u[f][m].y, 0, E, pl.bits));
+    transform<-1, R>(a, b0, b1, pl, tj, on, idx, tw, true, NoStore());
+    const C<R>* res = last_buffer(pl, b0, b1);
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < RMAX; ++m)
       if (on && m < pl.r0) {
         const C<R> z = res[idx(tj + m * pl.T)];
-        u[f][m] = st2(from_work<R>(z.x, eb), from_work<R>(z.y, eb));
+        u[f][m] = S::store(z, eb);
       }
   }
-  unsigned key = 0u;
+  int key = 0;
   if (on) {
     const int ky = pc / nkx, kx = pc - ky * nkx;
 #pragma unroll
@@ -681,24 +787,22 @@ __global__ void __launch_bounds__(128) k_fft_z_op(double2* __restrict__ spec, in
         cplx X0 = cmk(u[0][m].x, u[0][m].y), X1 = cmk(u[1][m].x, u[1][m].y), X2 = cmk(u[2][m].x, u[2][m].y);
         apply_op(T, sp, row, kx, ky, tj + m * pl.T, X0, X1, X2);
         u[0][m] = st2(X0.x, X0.y); u[1][m] = st2(X1.x, X1.y); u[2][m] = st2(X2.x, X2.y);
-        key = max(key, max(mag_of(u[0][m]), max(mag_of(u[1][m]), mag_of(u[2][m]))));
+        key = max(key, max(S::key(u[0][m], 0), max(S::key(u[1][m], 0), S::key(u[2][m], 0))));
       }
   }
-  const int e = column_exp<R>(key, cpb, red[3]), s0 = e + 63 - pl.bits, eb = fix64::out_base(e, pl.bits, pl.down);
+  const int E = S::scale(column_max<R>(key, cpb, red[3]), pl.bits), eb = E + pl.down;
 #pragma unroll
   for (int f = 0; f < 3; ++f) {
     __syncthreads();                              // the previous results are read
     C<R> a[RMAX];
 #pragma unroll
-    for (int m = 0; m < RMAX; ++m) a[m] = mk(to_work(u[f][m].x, s0), to_work(u[f][m].y, s0));
-    const C<R>* res = transform<+1, R>(a, b0, b1, pl, tj, on, idx, tw);
+    for (int m = 0; m < RMAX; ++m) a[m] = mk(S::work(u[f][m].x, 0, E, pl.bits), S::work(u[f][m].y, 0, E, pl.bits));
+    transform<+1, R>(a, b0, b1, pl, tj, on, idx, tw, true, NoStore());
+    const C<R>* res = last_buffer(pl, b0, b1);
     __syncthreads();
     if (on) {
 #pragma unroll 1
-      for (int p = tj; p < pl.n; p += pl.T) {
-        const C<R> z = res[idx(p)];
-        base[f * fstride + (size_t)p * np] = st2(from_work<R>(z.x, eb), from_work<R>(z.y, eb));
-      }
+      for (int p = tj; p < pl.n; p += pl.T) base[f * fstride + (size_t)p * np] = S::store(res[idx(p)], eb);
     }
   }
 }
@@ -737,73 +841,66 @@ OpTables op_tables(const rve_s* h) {
 template <typename R> const TW<R>* twt(const rve_s* h, int a);
 template <> const int4* twt<double>(const rve_s* h, int a) { return h->ax[a].twq; }
 template <> const float2* twt<float>(const rve_s* h, int a) { return h->ax[a].tw32; }
-template <typename R> V2<R>* spect(const rve_s* h);
-template <> double2* spect<double>(const rve_s* h) { return h->spec; }
-template <> float2* spect<float>(const rve_s* h) { return h->spec32; }
 template <typename R> const R* lap_weight(const rve_s* h);
 template <> const double* lap_weight<double>(const rve_s* h) { return h->lapw; }
 template <> const float* lap_weight<float>(const rve_s* h) { return h->lapw32; }
+template <class S> typename S::pair* spect(const rve_s* h);
+template <> double2* spect<Plain<double>>(const rve_s* h) { return h->spec; }
+template <> longlong2* spect<Fixed>(const rve_s* h) { return reinterpret_cast<longlong2*>(h->spec); }
+template <> float2* spect<Plain<float>>(const rve_s* h) { return h->spec32; }
 
 template <typename R>
 size_t row_smem(int rpb, int n) { return 2 * (size_t)rpb * (n + (n >> 3) + 1) * sizeof(C<R>); }
 
-template <int SIGN, typename R>
-void launch_y(const rve_s* h, cudaStream_t s, const double* done, int nf, int cat) {
-  const PlanDev pl = to_dev(h->plan[1]);
-  const long cols = (long)nf * h->n2 * h->nkx;
-  const int c = cols_per_block(pl, cols, h->fft_fill_y, 256);
-  ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : cat, s);
-  k_fft_y<SIGN, R><<<(unsigned)((cols + c - 1) / c), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
-      spect<R>(h), (int)cols, h->nkx, c, pl, twt<R>(h, 1), done);
-}
+int fft_category(const rve_s* h, int cat) { return h->fft_cat >= 0 ? h->fft_cat : cat; }
 
-template <typename R>
-cudaError_t fwd(const rve_s* h, const R* in, cudaStream_t s, const double* done, int nf) {
+template <typename R, class In, class S>
+void launch_r2c(const rve_s* h, const typename In::real* in, cudaStream_t s, const double* done, int nf) {
   const PlanDev pl = to_dev(h->plan[0]);
   const long rows = (long)nf * h->n2 * (h->n1 / 2);
   const int rpb = rows_per_block(pl, rows, h->fft_fill);
-  {
-    ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : RVE_K_FFT_X_R2C, s);
-    k_fft_x_r2c<R><<<(unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb, pl.n), s>>>(
-        in, spect<R>(h), (int)rows, h->nkx, rpb, pl, twt<R>(h, 0), done);
-  }
-  launch_y<-1, R>(h, s, done, nf, RVE_K_FFT_Y);
-  return cudaGetLastError();
+  ProfScope ps_(h, fft_category(h, RVE_K_FFT_X_R2C), s);
+  k_fft_x_r2c<R, In, S><<<(unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb, pl.n), s>>>(
+      in, h->ex.div, spect<S>(h), h->ex.x, (int)rows, h->nkx, rpb, pl, twt<R>(h, 0), done);
 }
 
-template <typename R>
-cudaError_t lap(const rve_s* h, cudaStream_t s, const double* done) {
+template <int SIGN, typename R, class S>
+void launch_y(const rve_s* h, cudaStream_t s, const double* done, int nf) {
+  const PlanDev pl = to_dev(h->plan[1]);
+  const long cols = (long)nf * h->n2 * h->nkx;
+  const int c = cols_per_block(pl, cols, h->fft_fill_y, 256);
+  ProfScope ps_(h, fft_category(h, SIGN < 0 ? RVE_K_FFT_Y : RVE_K_FFT_Y_INV), s);
+  k_fft_y<SIGN, R, S><<<(unsigned)((cols + c - 1) / c), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
+      spect<S>(h), SIGN < 0 ? h->ex.x : h->ex.z, h->ex.y, (int)cols, h->n2, h->nkx, c, pl, twt<R>(h, 1), done);
+}
+
+template <typename R, class S>
+void launch_lap(const rve_s* h, cudaStream_t s, const double* done) {
   const PlanDev pl = to_dev(h->plan[2]);
   const int np = h->n1 * h->nkx;
   const int c = cols_per_block(pl, 3L * np, h->fft_fill_z, 256);
   ProfScope ps_(h, RVE_K_FFT_Z_OP, s);
-  k_fft_z_lap<R><<<dim3((np + c - 1) / c, 3), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
-      spect<R>(h), np, c, pl, twt<R>(h, 2), lap_weight<R>(h), done);
-  return cudaGetLastError();
+  k_fft_z_lap<R, S><<<dim3((np + c - 1) / c, 3), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
+      spect<S>(h), h->ex.y, h->ex.z, np, h->nkx, c, pl, twt<R>(h, 2), lap_weight<R>(h), done);
 }
 
-cudaError_t zop(const rve_s* h, const SpecParams& sp, cudaStream_t s) {
+void zop(const rve_s* h, const SpecParams& sp, cudaStream_t s) {
   const PlanDev pl = to_dev(h->plan[2]);
   const int np = h->n1 * h->nkx;
   const int c = cols_per_block(pl, 3L * np, h->fft_fill_z, 128);
-  ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : RVE_K_FFT_Z_OP, s);
+  ProfScope ps_(h, fft_category(h, RVE_K_FFT_Z_OP), s);
   k_fft_z_op<<<dim3((np + c - 1) / c, 3), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<double>), s>>>(
       h->spec, np, h->nkx, c, pl, h->ax[2].twq, op_tables(h), sp);
-  return cudaGetLastError();
 }
 
-template <typename R>
-cudaError_t inv(const rve_s* h, R* out, cudaStream_t s, const double* done, int nf) {
-  launch_y<+1, R>(h, s, done, nf, RVE_K_FFT_Y_INV);
+template <typename R, class S, class Out>
+void launch_c2r(const rve_s* h, typename Out::real* out, cudaStream_t s, const double* done, int nf) {
   const PlanDev pl = to_dev(h->plan[0]);
   const long rows = (long)nf * h->n2 * (h->n1 / 2);
   const int rpb = rows_per_block(pl, rows, h->fft_fill);
-  {
-    ProfScope ps_(h, h->fft_cat >= 0 ? h->fft_cat : RVE_K_FFT_X_C2R, s);
-    k_fft_x_c2r<R><<<(unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb, pl.n), s>>>(
-        spect<R>(h), out, (int)rows, h->nkx, rpb, pl, twt<R>(h, 0), done);
-  }
-  return cudaGetLastError();
+  ProfScope ps_(h, fft_category(h, RVE_K_FFT_X_C2R), s);
+  k_fft_x_c2r<R, S, Out><<<(unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb, pl.n), s>>>(
+      spect<S>(h), h->ex.y, out, h->ex.u, (int)rows, h->n1 / 2, h->nkx, rpb, pl, twt<R>(h, 0), done);
 }
 
 }  // namespace
@@ -816,7 +913,9 @@ cudaError_t launch_lapinv_table(const rve_s* h, cudaStream_t s) {
 }
 
 // Radices of a length 2^a 3^b, the largest first (a transform has n / radix[0]
-// threads): 8s, then 6s while both factors are left, then 4, 3s or 2.
+// threads): 8s, and what is left of the 2s as a 6 (with a 3), as 4 4 instead of 8 2
+// (four radix-2 butterflies per thread would follow one of radix 8), or as a 4;
+// then 3s.
 void make_plan(int n, FFTPlan* p) {
   p->n = n;
   p->npass = 0;
@@ -824,28 +923,47 @@ void make_plan(int n, FFTPlan* p) {
   while (m % 2 == 0) { ++a; m /= 2; }
   while (m % 3 == 0) { ++b; m /= 3; }
   if (m != 1) { p->npass = -1; return; }     // unsupported length
-  while (a >= 3) { p->radix[p->npass++] = 8; a -= 3; }
-  while (a >= 1 && b >= 1) { p->radix[p->npass++] = 6; --a; --b; }
-  if (a == 2) p->radix[p->npass++] = 4;
-  // 3s before a last 2: the first radix stays the largest
-  while (b > 0) { p->radix[p->npass++] = 3; --b; }
-  if (a == 1) p->radix[p->npass++] = 2;
+  auto add = [&](int r) { p->radix[p->npass++] = r; };
+  const bool fours = a % 3 == 1 && a > 1 && b == 0;
+  for (int q = a / 3 - (fours ? 1 : 0); q > 0; --q) add(8);
+  if (fours) { add(4); add(4); }
+  else if (a % 3 == 1 && b > 0) { add(6); --b; }
+  else if (a % 3 == 1) add(2);
+  else if (a % 3 == 2 && b > 1) { add(6); add(6); b -= 2; }
+  else if (a % 3 == 2) add(4);
+  for (; b > 0; --b) add(3);
 }
 
-cudaError_t launch_fft_forward(const rve_s* h, const double* in, cudaStream_t s, const double* done, int nf) {
-  return fwd<double>(h, in, s, done, nf);
+// nine fields (double spectra) around the operators that couple a tensor row
+cudaError_t launch_fft9(const rve_s* h, const double* in, double* out, const SpecParams& sp, cudaStream_t s) {
+  typedef Plain<double> S;
+  launch_r2c<double, S, S>(h, in, s, nullptr, 9);
+  launch_y<-1, double, S>(h, s, nullptr, 9);
+  zop(h, sp, s);
+  launch_y<+1, double, S>(h, s, nullptr, 9);
+  launch_c2r<double, S, S>(h, out, s, nullptr, 9);
+  return cudaGetLastError();
 }
-cudaError_t launch_fft_lapinv(const rve_s* h, cudaStream_t s, const double* done) { return lap<double>(h, s, done); }
-cudaError_t launch_fft_op(const rve_s* h, const SpecParams& sp, cudaStream_t s) { return zop(h, sp, s); }
-cudaError_t launch_fft_inverse(const rve_s* h, double* out, cudaStream_t s, const double* done, int nf) {
-  return inv<double>(h, out, s, done, nf);
+// three fields around the inverse Laplacian.  FP64: the divergence comes and the
+// solution goes as integers with a scale per row (h->ex), or as doubles where the
+// stencils of this grid work on doubles
+cudaError_t launch_laplace_solve(const rve_s* h, const double* d, double* u, bool fixed, cudaStream_t s,
+                                 const double* done) {
+  if (fixed) launch_r2c<double, Fixed, Fixed>(h, reinterpret_cast<const i64*>(d), s, done, 3);
+  else launch_r2c<double, Plain<double>, Fixed>(h, d, s, done, 3);
+  launch_y<-1, double, Fixed>(h, s, done, 3);
+  launch_lap<double, Fixed>(h, s, done);
+  launch_y<+1, double, Fixed>(h, s, done, 3);
+  if (fixed) launch_c2r<double, Fixed, Fixed>(h, reinterpret_cast<i64*>(u), s, done, 3);
+  else launch_c2r<double, Fixed, Plain<double>>(h, u, s, done, 3);
+  return cudaGetLastError();
 }
-cudaError_t launch_fft_forward32(const rve_s* h, const float* in, cudaStream_t s, const double* done) {
-  return fwd<float>(h, in, s, done, 3);
-}
-cudaError_t launch_fft_lapinv32(const rve_s* h, cudaStream_t s, const double* done) {
-  return lap<float>(h, s, done);
-}
-cudaError_t launch_fft_inverse32(const rve_s* h, float* out, cudaStream_t s, const double* done) {
-  return inv<float>(h, out, s, done, 3);
+cudaError_t launch_laplace_solve32(const rve_s* h, const float* d, float* u, cudaStream_t s, const double* done) {
+  typedef Plain<float> S;
+  launch_r2c<float, S, S>(h, d, s, done, 3);
+  launch_y<-1, float, S>(h, s, done, 3);
+  launch_lap<float, S>(h, s, done);
+  launch_y<+1, float, S>(h, s, done, 3);
+  launch_c2r<float, S, S>(h, u, s, done, 3);
+  return cudaGetLastError();
 }

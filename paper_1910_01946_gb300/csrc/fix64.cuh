@@ -23,6 +23,8 @@ typedef long long i64;
 
 constexpr int EXP_MIN = 256;          // smallest common exponent field used
 constexpr int EXP_SLOW = 2000;        // output exponent bases above this take the checked path
+constexpr int EXP_BAD = 1 << 20;      // scale of values that an infinity or a NaN went into
+constexpr int EXP_ZERO = -(1 << 20);  // scale of exact zeros
 
 // magnitude key of a double: its high word without the sign (the exponent
 // field on top), to be maximised over a tile
@@ -48,7 +50,7 @@ __device__ __forceinline__ i64 to_fix(double x, int s0) {
 }
 
 static __device__ __noinline__ double from_fix_checked(i64 v, int eb) {
-  if (eb >= (1 << 20)) return __hiloint2double(0x7ff80000, 0);      // from a tile with an infinity or NaN
+  if (eb >= EXP_BAD / 2) return __hiloint2double(0x7ff80000, 0);    // an infinity or NaN went in
   return scalbn((double)v, eb - 1086);                              // may overflow to infinity
 }
 
@@ -67,7 +69,22 @@ __device__ __forceinline__ double from_fix(i64 v, int eb) {
 }
 // exponent base of from_fix for integers on the scale to_fix(., e + 63 - B) gave, times 2^sh
 __device__ __forceinline__ int out_base(int e, int B, int sh = 0) {
-  return e == 0x7ff ? (1 << 20) : e + 64 - B + sh;
+  return e == 0x7ff ? EXP_BAD : e + 64 - B + sh;
+}
+
+// ---- integers already on a scale eb (v 2^(eb - 1086), |v| < 2^63) ----
+// |v| < 2^(33 + top_bit(high(v)))
+__device__ __forceinline__ int abs_hi(i64 v) { const int h = (int)(v >> 32); return h ^ (h >> 31); }
+__device__ __forceinline__ int top_bit(int h) { return 31 - __clz(h); }
+// Key of values on the scale ex whose magnitudes' high words or to h: maximised
+// over the values that are to share a scale, key_scale() of it is the scale on which
+// all of them just fit B bits.
+__device__ __forceinline__ int fit_key(int h, int ex) { return ex + top_bit(h); }
+__device__ __forceinline__ int key_scale(int key, int B) { return key + 33 - B; }
+// v from the scale ex to the scale E (up only as far as the key allowed)
+__device__ __forceinline__ i64 rescale(i64 v, int ex, int E) {
+  const int d = E - ex;
+  return (v << min(max(-d, 0), 63)) >> min(max(d, 0), 63);
 }
 
 // ---- multiplication by Q62 factors (|w| <= 1) ----

@@ -123,8 +123,6 @@ extern "C" rve_status rve_project_noalloc(int n0, int n1, int n2, double L, cons
   sp.inv_nvox = 1.0 / (double)h.nvox;
   sp.inv4h = 0.25 / h.h;
   sp.mean_out = nullptr;
-  if (launch_fft_forward(&h, d_X, h.stream) != cudaSuccess) return RVE_ECUDA;
-  if (launch_fft_op(&h, sp, h.stream) != cudaSuccess) return RVE_ECUDA;
-  if (launch_fft_inverse(&h, d_Y, h.stream) != cudaSuccess) return RVE_ECUDA;
+  if (launch_fft9(&h, d_X, d_Y, sp, h.stream) != cudaSuccess) return RVE_ECUDA;
   return RVE_OK;
 }

@@ -106,6 +106,11 @@ void carve(rve_s* h, Carver& c) {
   h->bs = c.take<double>(9 * nv);
   h->spec = c.take<double2>(9 * h->nspec);
   h->lapw = c.take<double>(h->nspec);
+  h->ex.div = c.take<int>(3 * (size_t)h->n1 * h->n2);
+  h->ex.x = c.take<int>(3 * (size_t)(h->n1 / 2) * h->n2);
+  h->ex.y = c.take<int>(3 * (size_t)h->nkx * h->n2);
+  h->ex.z = c.take<int>(3 * (size_t)h->nkx * h->n1);
+  h->ex.u = c.take<int>(3 * (size_t)(h->n1 / 2) * h->n2);
   if (h->opt.precision == 1) {
     for (int a = 0; a < 3; ++a) h->ax[a].tw32 = c.take<float2>(ns[a]);
     h->lapw32 = c.take<float>(h->nspec);
@@ -274,13 +279,6 @@ SpecParams project_params(const rve_s* h, const uint8_t* mask, const double* shi
   return sp;
 }
 
-rve_status run_project(rve_s* h, const double* in, double* out, const SpecParams& sp) {
-  RVE_CUDA(h, launch_fft_forward(h, in, h->stream));
-  RVE_CUDA(h, launch_fft_op(h, sp, h->stream));
-  RVE_CUDA(h, launch_fft_inverse(h, out, h->stream));
-  return RVE_OK;
-}
-
 // Y = G*(X) (minus the prescribed mean `shift` on the kept components) as
 // divergence stencil, scalar Laplace solve by FFT, gradient stencil; leaves
 // mean(X) in DS_XMEAN and sum Y^2 in DS_NORM.  Scratch: the first six
@@ -300,9 +298,7 @@ rve_status run_project_stencil(rve_s* h, const double* X, double* Y, const uint8
   double* d = h->q;
   double* u = h->q + 3 * h->nvox;
   RVE_CUDA(h, launch_div(h, X, d, 0, all_means ? 0x1FFu : kept_means(mask), h->stream));
-  RVE_CUDA(h, launch_fft_forward(h, d, h->stream, nullptr, 3));
-  RVE_CUDA(h, launch_fft_lapinv(h, h->stream, nullptr));
-  RVE_CUDA(h, launch_fft_inverse(h, u, h->stream, nullptr, 3));
+  RVE_CUDA(h, launch_laplace_solve(h, d, u, stencils_fixed(h), h->stream, nullptr));
   RVE_CUDA(h, launch_grad(h, u, Y, mask, shift, h->stream));
   return RVE_OK;
 }
@@ -312,9 +308,10 @@ rve_status run_curl(rve_s* h, const double* in, double* out) {
   SpecParams sp = project_params(h, (const uint8_t*)"\0\0\0\0\0\0\0\0\0", nullptr, nullptr);
   sp.op = OP_CURL;
   h->fft_cat = RVE_K_FFT_CURL;
-  const rve_status st = run_project(h, in, out, sp);
+  const cudaError_t e = launch_fft9(h, in, out, sp, h->stream);
   h->fft_cat = -1;
-  return st;
+  RVE_CUDA(h, e);
+  return RVE_OK;
 }
 
 rve_status run_hardening(rve_s* h) {
@@ -422,9 +419,7 @@ rve_status cg_solve(rve_s* h, const uint8_t* mask, double eta, int* iters, bool*
         // t = K : p, then q = G*(t) as div -> Laplace solve -> grad fused with the update
         RVE_CUDA(h, launch_tangent_apply(h, h->stream));
         RVE_CUDA(h, launch_div(h, h->t, d, 1, kept_means(mask), h->stream));
-        RVE_CUDA(h, launch_fft_forward(h, d, h->stream, done, 3));
-        RVE_CUDA(h, launch_fft_lapinv(h, h->stream, done));
-        RVE_CUDA(h, launch_fft_inverse(h, u, h->stream, done, 3));
+        RVE_CUDA(h, launch_laplace_solve(h, d, u, stencils_fixed(h), h->stream, done));
         RVE_CUDA(h, launch_grad_cg(h, u, mask, h->stream));
       }
       return RVE_OK;
@@ -456,9 +451,7 @@ rve_status cg_solve32(rve_s* h, const uint8_t* mask, double eta, int* iters, boo
       for (int i = 0; i < chunk; ++i) {
         RVE_CUDA(h, launch_tangent_apply32(h, h->stream));
         RVE_CUDA(h, launch_div32(h, h->t32, d, kept_means(mask), h->stream));
-        RVE_CUDA(h, launch_fft_forward32(h, d, h->stream, done));
-        RVE_CUDA(h, launch_fft_lapinv32(h, h->stream, done));
-        RVE_CUDA(h, launch_fft_inverse32(h, u, h->stream, done));
+        RVE_CUDA(h, launch_laplace_solve32(h, d, u, h->stream, done));
         RVE_CUDA(h, launch_grad_cg32(h, u, mask, h->stream));
       }
       return RVE_OK;
@@ -632,7 +625,8 @@ rve_status autotune(rve_s* h) {
     h->div_blocks = pick;
   }
   // FFT tile fill targets of the x, y and z passes, one at a time with the
-  // others held (forward, Laplace solve, inverse of three fields)
+  // others held (forward, Laplace solve, inverse of three fields; FP64: of the
+  // divergence the loop above left)
   for (int* target : {&h->fft_fill, &h->fft_fill_y, &h->fft_fill_z}) {
     const int cand[4] = {2 * sms, 4 * sms, 8 * sms, 16 * sms};
     float best = 1e30f;
@@ -641,14 +635,8 @@ rve_status autotune(rve_s* h) {
       *target = c;
       float ms = 0.f;
       RVE_TRY(timed([&]() -> cudaError_t {
-        if (f32) {
-          if (cudaError_t e = launch_fft_forward32(h, h->du32, st, nullptr)) return e;
-          if (cudaError_t e = launch_fft_lapinv32(h, st, nullptr)) return e;
-          return launch_fft_inverse32(h, h->du32 + 3 * h->nvox, st, nullptr);
-        }
-        if (cudaError_t e = launch_fft_forward(h, h->q, st, nullptr, 3)) return e;
-        if (cudaError_t e = launch_fft_lapinv(h, st, nullptr)) return e;
-        return launch_fft_inverse(h, h->q + 3 * h->nvox, st, nullptr, 3);
+        if (f32) return launch_laplace_solve32(h, h->du32, h->du32 + 3 * h->nvox, st, nullptr);
+        return launch_laplace_solve(h, h->q, h->q + 3 * h->nvox, stencils_fixed(h), st, nullptr);
       }, &ms));
       if (ms < best) { best = ms; pick = c; }
     }
@@ -1289,9 +1277,9 @@ rve_status rve_eval_nye(rve_t* h, int scheme) {
     SpecParams sp = project_params(h, (const uint8_t*)"\0\0\0\0\0\0\0\0\0", nullptr, nullptr);
     sp.op = OP_CURL_STD;
     h->fft_cat = RVE_K_FFT_CURL;
-    const rve_status st = run_project(h, h->Fp, h->nye, sp);
+    const cudaError_t e = launch_fft9(h, h->Fp, h->nye, sp, h->stream);
     h->fft_cat = -1;
-    RVE_TRY(st);
+    RVE_CUDA(h, e);
   }
   RVE_CUDA(h, cudaStreamSynchronize(h->stream));
   return RVE_OK;
@@ -1430,16 +1418,12 @@ rve_status rve_time_fft(rve_t* h, int nf, int fp32, int reps, double* ms) {
   const uint8_t mask[9] = {1, 0, 0, 1, 0, 0, 1, 1, 0};
   SpecParams sp = project_params(h, mask, nullptr, nullptr);
   cudaStream_t s = h->stream;
+  if (nf == 3 && !fp32)          // a divergence in the form the transforms take
+    RVE_CUDA(h, launch_div(h, h->F, h->q, 0, 0u, s));
   auto pair = [&]() -> cudaError_t {
-    cudaError_t e;
-    if (fp32) {
-      if ((e = launch_fft_forward32(h, h->t32, s, nullptr)) != cudaSuccess) return e;
-      if ((e = launch_fft_lapinv32(h, s, nullptr)) != cudaSuccess) return e;
-      return launch_fft_inverse32(h, h->x32, s, nullptr);
-    }
-    if ((e = launch_fft_forward(h, h->R, s, nullptr, nf)) != cudaSuccess) return e;
-    if ((e = nf == 3 ? launch_fft_lapinv(h, s, nullptr) : launch_fft_op(h, sp, s)) != cudaSuccess) return e;
-    return launch_fft_inverse(h, h->t, s, nullptr, nf);
+    if (fp32) return launch_laplace_solve32(h, h->t32, h->x32, s, nullptr);
+    if (nf == 3) return launch_laplace_solve(h, h->q, h->q + 3 * h->nvox, stencils_fixed(h), s, nullptr);
+    return launch_fft9(h, h->R, h->t, sp, s);
   };
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   RVE_CUDA(h, cudaEventCreate(&e0));

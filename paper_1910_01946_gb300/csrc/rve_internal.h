@@ -138,7 +138,7 @@ struct rve_s {
   bool autotuned = false;
   bool tma_apply = false;   // FP32 tangent apply staged by bulk copies (rve_options.tma)
   int fft_cat = -1;         // >= 0: the FFT passes are counted in this category (the Nye curl)
-  bool row_stencils = true; // row-strip stencils where the grid suits them (n0 = 32, 64, 96, 128)
+  bool row_stencils = true; // row-strip stencils where the grid suits them (FP64: n0 <= 128; FP32: 32, 64)
   unsigned wait_polls = RVE_WAIT_POLLS_DEFAULT;   // its per-tile wait limit (rve_set_wait_limit)
   // forward-mode sensitivities (rve_sensitivity_enable): state tangents
   // dFp (9) and d rho_SSD (12) per parameter, double-buffered so that a
@@ -154,6 +154,14 @@ struct rve_s {
   double *R, *x, *r, *p, *t, *q;
   double *bv, *bs;      // BiCGStab vectors v and s
   double2* spec;        // 9 * nspec
+  // scales of the integers of the three-field FP64 transforms (v 2^(ex - 1086), see fix64.cuh)
+  struct {
+    int* div;           // divergence: per tensor row and x line (i, z, y)
+    int* x;             // spectra after the X pass: per field and line pair
+    int* y;             // after a Y pass: per column (field, z, kx)
+    int* z;             // after the Z pass: per column (field, ky, kx)
+    int* u;             // solution: per field and line pair
+  } ex;
   double* lapw;         // nspec: inverse-Laplacian weight of the projection's Laplace solve
   float* lapw32;        // the same in float (mixed precision)
   // mixed precision (precision == 1): FP32 conjugate-gradient state
@@ -190,27 +198,25 @@ enum { DS_RR = 0, DS_PKP = 1, DS_ALPHA = 2, DS_BETA = 3, DS_NORM = 4, DS_STOP = 
        DS_XMEAN = 48 };
 
 // ---- fft.cu ----
-// `done` (nullable, device): when *done != 0 every block returns at once (the
-// conjugate-gradient loop has converged on the device)
-// nf: number of fields transformed (9, or 3 for OP_LAPINV)
-cudaError_t launch_fft_forward(const rve_s* h, const double* in, cudaStream_t s, const double* done = nullptr,
-                               int nf = 9);
-// the operator between the z passes: the inverse Laplacian on three fields, or
-// one of the nine-field operators of SpecParams
-cudaError_t launch_fft_lapinv(const rve_s* h, cudaStream_t s, const double* done);
-cudaError_t launch_fft_op(const rve_s* h, const SpecParams& sp, cudaStream_t s);
-cudaError_t launch_fft_inverse(const rve_s* h, double* out, cudaStream_t s, const double* done = nullptr,
-                               int nf = 9);
+// nine fields through the operator sp of Fourier space (out may be in)
+cudaError_t launch_fft9(const rve_s* h, const double* in, double* out, const SpecParams& sp, cudaStream_t s);
+// three fields through the inverse Laplacian.  `done` (nullable, device): when
+// *done != 0 nothing is written (the conjugate-gradient loop has converged on
+// the device).  fixed: d and u are 64-bit integers with the scales h->ex.div and h->ex.u
+// (see stencils_fixed), else doubles
+cudaError_t launch_laplace_solve(const rve_s* h, const double* d, double* u, bool fixed, cudaStream_t s,
+                                 const double* done);
+cudaError_t launch_laplace_solve32(const rve_s* h, const float* d, float* u, cudaStream_t s, const double* done);
 // radix passes 8, 6, 4, 3, 2, the largest first
 void make_plan(int n, FFTPlan* p);
 // fills h->lapw and h->lapw32 (once, at create)
 cudaError_t launch_lapinv_table(const rve_s* h, cudaStream_t s);
-cudaError_t launch_fft_forward32(const rve_s* h, const float* in, cudaStream_t s, const double* done);
-cudaError_t launch_fft_lapinv32(const rve_s* h, cudaStream_t s, const double* done);
-cudaError_t launch_fft_inverse32(const rve_s* h, float* out, cudaStream_t s, const double* done);
 
 // ---- stencil.cu: G* = D (D^H D)^-1 D^H with real-space rotated-scheme stencils ----
-// number of tiles the stencils cover (their grids loop over them)
+// whether the FP64 stencils of this grid work in fixed point (row strips, n0 up
+// to 128), with the divergence and the solution as integers (launch_laplace_solve)
+bool stencils_fixed(const rve_s* h);
+// number of tiles the tiled stencils cover (their grids loop over them)
 int stencil_tiles(const rve_s* h);
 // mean_mask: bit c set = the mean of field c is reduced into ds[DS_XMEAN + c]
 // (others read 0)

@@ -86,6 +86,25 @@ def test_fixed_point_scales(pkg, shape):
     r.close()
 
 
+@pytest.mark.parametrize("n0", [4, 24, 48, 54, 64, 72, 108, 128])
+def test_projection_of_fields_on_an_odd_eight_byte_boundary(pkg, n0):
+    """The row strips load 16 bytes at a time where the caller's field allows
+    it; one that starts 8 bytes off gives the same bits, and so does a run of
+    many rows per warp (sums of the means are taken down in between)."""
+    import torch
+    shape = (40, 54, n0) if n0 < 8 else (3, 4, n0)
+    Xd = device_field(np.random.default_rng(n0).standard_normal(shape + (3, 3)) + 5.0)
+    shifted = torch.empty(Xd.numel() + 1, dtype=Xd.dtype, device=Xd.device)[1:].view_as(Xd)
+    shifted.copy_(Xd)
+    assert shifted.data_ptr() % 16 == 8
+    r = handle(pkg, shape)
+    out = torch.empty(Xd.numel() + 1, dtype=Xd.dtype, device=Xd.device)[1:].view_as(Xd)
+    Y = r.project(MASK, Xd)
+    assert torch.equal(r.project(MASK, shifted, out), Y)
+    assert float((Y[8].mean() - Xd[8].mean()).abs()) < 1e-14 * float(Xd.abs().max())
+    r.close()
+
+
 def test_columns_of_very_different_size_keep_their_digits(pkg):
     """A field whose rows differ by 2^-30 along y and z: the small tensor row's
     projection is as accurate as when it stands alone (each transform has its
