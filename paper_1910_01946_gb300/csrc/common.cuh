@@ -267,3 +267,66 @@ __device__ __forceinline__ bool last_block_sums(const double* partial, int nval,
   }
   return true;
 }
+
+// The same for one value per block: sum over the blocks into *out of thread 0.
+__device__ __forceinline__ bool last_block_sum1(const double* partial, unsigned int* ticket, double* sh, double* out) {
+  __shared__ bool last;
+  const int t = lin_tid(), nt = lin_nthreads(), n = (int)gridDim.x;
+  __threadfence();
+  __syncthreads();
+  if (t == 0) last = (atomicAdd(ticket, 1u) == gridDim.x - 1);
+  __syncthreads();
+  if (!last) return false;
+  double acc = 0.0;
+  for (int i = t; i < n; i += 4 * nt) {                // four loads in flight
+    double v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = i + q * nt < n ? __ldcg(partial + i + q * nt) : 0.0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc += v[q];
+  }
+  *out = blk_sum(acc, sh);
+  if (t == 0) *ticket = 0u;
+  return true;
+}
+
+// Sums that a later kernel needs and that no launch in between does: the block
+// sums a kernel has left in memory are added up by extra blocks (one per value) of a
+// kernel that follows (the forward Y pass of the Laplace solve), whose other
+// blocks have their own work meanwhile.  Before, the last block of the
+// divergence did it (ticket and fence, then nine sums on the FP64 pipe): 13 of the
+// kernel's 26 us at 64^3 were that one block.
+struct Fold {
+  const double* mean;      // block sums of the divergence's input fields, [9][mean_blocks]
+  int mean_blocks;         // 0: none
+  unsigned mean_mask;      // fields summed (others: 0)
+  double inv_nvox;
+  const double* pkp;       // block sums of p . K p
+  int pkp_blocks;          // 0: none
+  double* xmean;           // 9 means
+  double* rr_pkp_alpha;    // r . r (read), p . K p, alpha = r . r / p . K p
+};
+constexpr int FOLD_BLOCKS = 10;            // extra blocks, one per value
+// the sum of value c (0..8: field means, 9: p . K p) by one block; sh: a double per warp
+__device__ __forceinline__ void fold_block(const Fold& f, int c, double* sh) {
+  const bool dot = c == 9;
+  const int n = dot ? f.pkp_blocks : f.mean_blocks;
+  const double* src = dot ? f.pkp : f.mean + (size_t)c * n;
+  double acc = 0.0;
+  if (dot || ((f.mean_mask >> c) & 1u)) {
+    for (int i = threadIdx.x; i < n; i += 8 * blockDim.x) {
+      double v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = i + q * (int)blockDim.x < n ? src[i + q * blockDim.x] : 0.0;
+      acc += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    }
+    acc = blk_sum(acc, sh);
+  }
+  if (threadIdx.x) return;
+  if (!dot) {
+    f.xmean[c] = acc * f.inv_nvox;
+  } else if (n) {
+    f.rr_pkp_alpha[1] = acc;
+    f.rr_pkp_alpha[2] = f.rr_pkp_alpha[0] / acc;
+  }
+}

@@ -517,15 +517,23 @@ __global__ void __launch_bounds__(256) k_fft_x_c2r(const typename In::pair* __re
 // ncol columns (field, z, kx), cpb consecutive ones per block, kx fastest.
 // Scales of stored integers, in: forward, of the row pairs (plane, y / 2); inverse,
 // of the columns (field, y, kx) of the Z pass.  Out: of the columns (plane, kx).
+// With fold.mean_blocks the first FOLD_BLOCKS blocks add up the divergence's and the tangent apply's
+// block sums instead (see Fold).
 template <int SIGN, typename R, class S>
 __global__ void __launch_bounds__(256) k_fft_y(typename S::pair* __restrict__ spec, const int* __restrict__ exin,
                                                int* __restrict__ exout, int ncol, int n2, int nkx, int cpb, PlanDev pl,
-                                               const TW<R>* __restrict__ tw, const double* __restrict__ done) {
+                                               const TW<R>* __restrict__ tw, const double* __restrict__ done, Fold fold) {
+  if (SIGN < 0 && fold.mean_blocks && blockIdx.x < FOLD_BLOCKS) {
+    __shared__ double fsh[MAX_WARPS];
+    if (!(done && *done != 0.0)) fold_block(fold, blockIdx.x, fsh);
+    return;
+  }
+  const int block = (int)blockIdx.x - (SIGN < 0 && fold.mean_blocks ? FOLD_BLOCKS : 0);
   __shared__ int red[MAX_WARPS * 32];
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
   C<R>* b1 = b0 + cpb * pl.n;
   const int tj = threadIdx.x / cpb, c = threadIdx.x - tj * cpb;     // cpb: a power of two
-  const long col = (long)blockIdx.x * cpb + c;
+  const long col = (long)block * cpb + c;
   const bool on = tj < pl.T && col < ncol;
   const int plane = on ? (int)(col / nkx) : 0, kx = on ? (int)(col - (long)plane * nkx) : 0;
   typename S::pair* base = spec + (size_t)plane * pl.n * nkx + kx;
@@ -865,13 +873,14 @@ void launch_r2c(const rve_s* h, const typename In::real* in, cudaStream_t s, con
 }
 
 template <int SIGN, typename R, class S>
-void launch_y(const rve_s* h, cudaStream_t s, const double* done, int nf) {
+void launch_y(const rve_s* h, cudaStream_t s, const double* done, int nf, const Fold& fold = Fold{}) {
   const PlanDev pl = to_dev(h->plan[1]);
   const long cols = (long)nf * h->n2 * h->nkx;
   const int c = cols_per_block(pl, cols, h->fft_fill_y, 256);
   ProfScope ps_(h, fft_category(h, SIGN < 0 ? RVE_K_FFT_Y : RVE_K_FFT_Y_INV), s);
-  k_fft_y<SIGN, R, S><<<(unsigned)((cols + c - 1) / c), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
-      spect<S>(h), SIGN < 0 ? h->ex.x : h->ex.z, h->ex.y, (int)cols, h->n2, h->nkx, c, pl, twt<R>(h, 1), done);
+  const unsigned blocks = (unsigned)((cols + c - 1) / c) + (fold.mean_blocks ? (unsigned)FOLD_BLOCKS : 0u);
+  k_fft_y<SIGN, R, S><<<blocks, round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
+      spect<S>(h), SIGN < 0 ? h->ex.x : h->ex.z, h->ex.y, (int)cols, h->n2, h->nkx, c, pl, twt<R>(h, 1), done, fold);
 }
 
 template <typename R, class S>
@@ -934,6 +943,22 @@ void make_plan(int n, FFTPlan* p) {
   for (; b > 0; --b) add(3);
 }
 
+// the block sums waiting to be added up, taken by the caller's Y pass
+Fold take_fold(const rve_s* h) {
+  Fold f{};
+  f.mean = h->partial;
+  f.mean_blocks = h->fold.mean_blocks;
+  f.mean_mask = h->fold.mean_mask;
+  f.inv_nvox = 1.0 / (double)h->nvox;
+  f.pkp = h->partial_pkp();
+  f.pkp_blocks = h->fold.pkp_blocks;
+  f.xmean = h->dscal + DS_XMEAN;
+  f.rr_pkp_alpha = h->dscal + DS_RR;
+  static_assert(DS_PKP == DS_RR + 1 && DS_ALPHA == DS_RR + 2, "Fold writes these scalars in a row");
+  h->fold.mean_blocks = h->fold.pkp_blocks = 0;
+  return f;
+}
+
 // nine fields (double spectra) around the operators that couple a tensor row
 cudaError_t launch_fft9(const rve_s* h, const double* in, double* out, const SpecParams& sp, cudaStream_t s) {
   typedef Plain<double> S;
@@ -951,7 +976,7 @@ cudaError_t launch_laplace_solve(const rve_s* h, const double* d, double* u, boo
                                  const double* done) {
   if (fixed) launch_r2c<double, Fixed, Fixed>(h, reinterpret_cast<const i64*>(d), s, done, 3);
   else launch_r2c<double, Plain<double>, Fixed>(h, d, s, done, 3);
-  launch_y<-1, double, Fixed>(h, s, done, 3);
+  launch_y<-1, double, Fixed>(h, s, done, 3, take_fold(h));
   launch_lap<double, Fixed>(h, s, done);
   launch_y<+1, double, Fixed>(h, s, done, 3);
   if (fixed) launch_c2r<double, Fixed, Fixed>(h, reinterpret_cast<i64*>(u), s, done, 3);
@@ -961,7 +986,7 @@ cudaError_t launch_laplace_solve(const rve_s* h, const double* d, double* u, boo
 cudaError_t launch_laplace_solve32(const rve_s* h, const float* d, float* u, cudaStream_t s, const double* done) {
   typedef Plain<float> S;
   launch_r2c<float, S, S>(h, d, s, done, 3);
-  launch_y<-1, float, S>(h, s, done, 3);
+  launch_y<-1, float, S>(h, s, done, 3, take_fold(h));
   launch_lap<float, S>(h, s, done);
   launch_y<+1, float, S>(h, s, done, 3);
   launch_c2r<float, S, S>(h, u, s, done, 3);

@@ -167,7 +167,9 @@ struct rve_s {
   // mixed precision (precision == 1): FP32 conjugate-gradient state
   float2* spec32;       // 3 * nspec
   float *x32, *r32, *p32, *t32, *du32;   // 9, 9, 9, 9, 6 components
-  double* partial;      // 4 * RVE_RED_BLOCKS
+  double* partial;      // block sums (9 * 4096 of the divergence, then those of p . K p: partial_pkp())
+  double* partial_pkp() const { return partial + 9 * 4096; }
+  mutable struct { int mean_blocks = 0; unsigned mean_mask = 0; int pkp_blocks = 0; } fold;   // block sums to be added up (see Fold)
   double* dscal;        // device scalars (see DS_*)
   int32_t* dcount;      // device counters: [0] local max iters, [1] local failures, [4] last-block ticket,
                         // [6] next voxel chunk of the local update, [8..11] 64-bit work totals
@@ -250,9 +252,6 @@ cudaError_t launch_constitutive(const rve_s* h, double dt, double lambda, int ou
 
 // ---- vec.cu ----
 cudaError_t launch_tangent_apply(const rve_s* h, cudaStream_t s);
-cudaError_t launch_cg_update(const rve_s* h, cudaStream_t s);
-cudaError_t launch_norm2(const rve_s* h, const double* a, int ncomp, cudaStream_t s);
-cudaError_t launch_reduce_final(const rve_s* h, int mode, cudaStream_t s);
 cudaError_t launch_cg_init(const rve_s* h, double eta, cudaStream_t s);
 cudaError_t launch_tangent_apply32(const rve_s* h, cudaStream_t s);
 // one-time kernel attributes (shared-memory sizes); before any launch or capture
@@ -277,4 +276,3 @@ cudaError_t launch_macro(const rve_s* h, cudaStream_t s);
 cudaError_t launch_output_field(const rve_s* h, int which, const double* P, const double* S, double* dst,
                                cudaStream_t s);
 
-enum { RED_PKP_ALPHA = 0, RED_RR_BETA = 1, RED_NORM = 2, RED_RR_INIT = 3, RED_MACRO = 4 };

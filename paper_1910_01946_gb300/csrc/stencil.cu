@@ -50,13 +50,12 @@ struct Tiling {
 __device__ __forceinline__ int wrapi(int a, int n) { return a < 0 ? a + n : (a >= n ? a - n : a); }
 
 // d_i = sum_l D_l^T X_il (unscaled); partial sums of the 9 input fields for
-// their means.  V is the field type (double, or float for the mixed-precision
-// conjugate gradients); block and grid sums are accumulated in double.
+// their means, one per block and field in `partial`.  V is the field type (double, or float for the mixed-precision
+// conjugate gradients); block sums are accumulated in double.
 template <typename V>
 __global__ void __launch_bounds__(NT) k_div(Grid3 g, Tiling T, const V* __restrict__ X,
                                            V* __restrict__ d, double* __restrict__ ds,
-                                           double* __restrict__ partial, unsigned int* __restrict__ ticket,
-                                           int check_done, unsigned mean_mask) {
+                                           double* __restrict__ partial, int check_done, unsigned mean_mask) {
   __shared__ V S[9][SMAX];
   __shared__ double sh[320];
   if (check_done && ds[DS_DONE] != 0.0) return;
@@ -131,10 +130,6 @@ __global__ void __launch_bounds__(NT) k_div(Grid3 g, Tiling T, const V* __restri
   if (tx == 0 && ty == 0) {
 #pragma unroll
     for (int c = 0; c < 9; ++c) partial[(size_t)c * gridDim.x + blockIdx.x] = bs[c];
-  }
-  double tot[9];
-  if (last_block_sums(partial, 9, ticket, sh, tot, mean_mask) && tx == 0 && ty == 0) {
-    for (int c = 0; c < 9; ++c) ds[DS_XMEAN + c] = tot[c] / (double)g.nvox;
   }
 }
 
@@ -239,7 +234,7 @@ __global__ void __launch_bounds__(NT) k_grad_t(Grid3 g, Tiling T, const V* __res
   const double s = blk_sum_v<V>(acc, sh);
   if (tx == 0 && ty == 0) partial[blockIdx.x] = s;
   double tot;
-  if (last_block_sums(partial, 1, ticket, sh, &tot) && tx == 0 && ty == 0) {
+  if (last_block_sum1(partial, ticket, sh, &tot) && tx == 0 && ty == 0) {
     if (CG) {
       ds[DS_BETA] = tot / ds[DS_RR];
       ds[DS_RR] = tot;
@@ -322,8 +317,7 @@ __device__ __forceinline__ RowRange row_range(const Grid3& g, int planes, int wa
 template <typename V, int NPL>
 __global__ void __launch_bounds__(32 * RW) k_div_rows(Grid3 g, const V* __restrict__ X,
                                                      V* __restrict__ d, double* __restrict__ ds,
-                                                     double* __restrict__ partial, unsigned int* __restrict__ ticket,
-                                                     int check_done, unsigned mean_mask) {
+                                                     double* __restrict__ partial, int check_done, unsigned mean_mask) {
   __shared__ double sh[320];
   if (check_done && ds[DS_DONE] != 0.0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -408,7 +402,7 @@ __global__ void __launch_bounds__(32 * RW) k_div_rows(Grid3 g, const V* __restri
     }
   }
   // means: one transposed warp reduction of the (up to nine) selected fields,
-  // the block's warps combined in shared memory, then the grid's last block
+  // the block's warps combined in shared memory
   V m16[16];
 #pragma unroll
   for (int f = 0; f < 16; ++f) m16[f] = f < 9 ? mean[f] : (V)0;
@@ -420,10 +414,6 @@ __global__ void __launch_bounds__(32 * RW) k_div_rows(Grid3 g, const V* __restri
     double t = 0.0;
     for (int q = 0; q < RW; ++q) t += sh[q * 16 + threadIdx.x];
     partial[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = ((mean_mask >> threadIdx.x) & 1u) ? t : 0.0;
-  }
-  double tot[9];
-  if (last_block_sums(partial, 9, ticket, sh, tot, mean_mask) && threadIdx.x == 0) {
-    for (int c = 0; c < 9; ++c) ds[DS_XMEAN + c] = tot[c] / (double)g.nvox;
   }
 }
 
@@ -537,7 +527,7 @@ __global__ void __launch_bounds__(32 * RW, NPL <= 2 ? 4 : 1) k_grad_rows(Grid3 g
   const double s = blk_sum_v<V>(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
   double tot;
-  if (last_block_sums(partial, 1, ticket, sh, &tot) && threadIdx.x == 0) {
+  if (last_block_sum1(partial, ticket, sh, &tot) && threadIdx.x == 0) {
     ds[DS_BETA] = tot / ds[DS_RR];
     ds[DS_RR] = tot;
     ds[DS_ITERS] += 1.0;
@@ -589,17 +579,16 @@ __device__ __forceinline__ void store_row(i64* dst, const i64 (&v)[NPL]) {
 // d_i = sum_l D_l^T X_il (unscaled) on the scale ex[(i n2 + z) n1 + y].  With the z pairs A, B,
 // C of k_div_rows, YS_A = A(y) + A(y-1), YD_B = B(y-1) - B(y), YS_C = C(y) +
 // C(y-1) and Q = YD_B + YS_C: d_i(x) = (Q - YS_A)(x) + (Q + YS_A)(x - 1).
-// Sums of 24 values below 2^DIV_BITS.  Means of the fields as k_div.
+// Sums of 24 values below 2^DIV_BITS.  Sums of the fields as in k_div, exact within a warp.
 // lanes: n0 / NPL; vec: X is 16-byte aligned.
 constexpr int DIV_BITS = 57;
 template <int NPL>
 __global__ void __launch_bounds__(32 * RW) k_div_fix(Grid3 g, int lanes, const double* __restrict__ X, i64* __restrict__ d,
                                                     int* __restrict__ ex, double* __restrict__ ds,
-                                                    double* __restrict__ partial, unsigned int* __restrict__ ticket,
-                                                    int check_done, unsigned mean_mask, int vec) {
+                                                    double* __restrict__ partial, int check_done, unsigned mean_mask,
+                                                    int vec) {
   constexpr int B = DIV_BITS;
   constexpr int FLUSH = 32 / NPL;                       // rows after which a lane's sums of a field could overflow
-  __shared__ double sh[320];
   __shared__ double macc[RW][9];
   if (check_done && ds[DS_DONE] != 0.0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -707,10 +696,6 @@ __global__ void __launch_bounds__(32 * RW) k_div_fix(Grid3 g, int lanes, const d
     double t = 0.0;
     for (int q = 0; q < RW; ++q) t += macc[q][threadIdx.x];
     partial[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = t;
-  }
-  double tot[9];
-  if (last_block_sums(partial, 9, ticket, sh, tot, mean_mask) && threadIdx.x == 0) {
-    for (int c = 0; c < 9; ++c) ds[DS_XMEAN + c] = tot[c] / (double)g.nvox;
   }
 }
 
@@ -857,7 +842,7 @@ __global__ void __launch_bounds__(32 * RW) k_grad_fix(Grid3 g, int lanes, const 
   const double s = blk_sum_v<double>(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
   double tot;
-  if (last_block_sums(partial, 1, ticket, sh, &tot) && threadIdx.x == 0) {
+  if (last_block_sum1(partial, ticket, sh, &tot) && threadIdx.x == 0) {
     if (CG) {
       ds[DS_BETA] = tot / ds[DS_RR];
       ds[DS_RR] = tot;
@@ -890,6 +875,12 @@ int resident_blocks(K kernel) {
   return n;
 }
 
+// the block sums of the field means are added up by launch_laplace_solve (see Fold)
+void set_fold(const rve_s* h, int blocks, unsigned mean_mask) {
+  h->fold.mean_blocks = blocks;
+  h->fold.mean_mask = mean_mask;
+}
+
 unsigned int* ticket_of(const rve_s* h) { return (unsigned int*)(h->dcount + 4); }
 
 template <int NPL>
@@ -897,8 +888,9 @@ void div_fix_n(const rve_s* h, const double* X, i64* d, int check_done, unsigned
                const Grid3& g) {
   static const int bps = resident_blocks(k_div_fix<NPL>);
   const int nb = row_blocks(h, 3L * h->n1 * h->n2, bps, h->div_blocks);
-  k_div_fix<NPL><<<nb, 32 * RW, 0, s>>>(g, h->n0 / NPL, X, d, h->ex.div, h->dscal, h->partial, ticket_of(h), check_done,
+  k_div_fix<NPL><<<nb, 32 * RW, 0, s>>>(g, h->n0 / NPL, X, d, h->ex.div, h->dscal, h->partial, check_done,
                                         mean_mask, (reinterpret_cast<uintptr_t>(X) & 15) == 0);
+  set_fold(h, nb, mean_mask);
 }
 
 template <bool CG, int NPL>
@@ -923,7 +915,8 @@ template <int NPL>
 void div_rows_n(const rve_s* h, const float* X, float* d, unsigned mean_mask, cudaStream_t s, const Grid3& g) {
   static const int bps = resident_blocks(k_div_rows<float, NPL>);
   const int nb = row_blocks(h, (long)h->n1 * h->n2, bps, h->div_blocks);
-  k_div_rows<float, NPL><<<nb, 32 * RW, 0, s>>>(g, X, d, h->dscal, h->partial, ticket_of(h), 1, mean_mask);
+  k_div_rows<float, NPL><<<nb, 32 * RW, 0, s>>>(g, X, d, h->dscal, h->partial, 1, mean_mask);
+  set_fold(h, nb, mean_mask);
 }
 
 template <int NPL>
@@ -989,8 +982,9 @@ cudaError_t launch_div(const rve_s* h, const double* X, double* d, int check_don
   Tiling T = tiling_of(h);
   if ((T.tx + 1) * (T.ty + 1) > SMAX) return cudaErrorInvalidValue;   // n0 odd: not a valid grid
   if (T.nblocks > h->div_blocks) T.nblocks = h->div_blocks;
-  k_div<double><<<T.nblocks, dim3(T.tx, T.ty), 0, s>>>(grid_of(h), T, X, d, h->dscal, h->partial, ticket_of(h),
-                                                       check_done, mean_mask);
+  k_div<double><<<T.nblocks, dim3(T.tx, T.ty), 0, s>>>(grid_of(h), T, X, d, h->dscal, h->partial, check_done,
+                                                       mean_mask);
+  set_fold(h, T.nblocks, mean_mask);
   return cudaGetLastError();
 }
 
@@ -1033,8 +1027,8 @@ cudaError_t launch_div32(const rve_s* h, const float* X, float* d, unsigned mean
   Tiling T = tiling_of(h);
   if ((T.tx + 1) * (T.ty + 1) > SMAX) return cudaErrorInvalidValue;   // n0 odd: not a valid grid
   if (T.nblocks > h->div_blocks) T.nblocks = h->div_blocks;
-  k_div<float><<<T.nblocks, dim3(T.tx, T.ty), 0, s>>>(grid_of(h), T, X, d, h->dscal, h->partial, ticket_of(h), 1,
-                                                      mean_mask);
+  k_div<float><<<T.nblocks, dim3(T.tx, T.ty), 0, s>>>(grid_of(h), T, X, d, h->dscal, h->partial, 1, mean_mask);
+  set_fold(h, T.nblocks, mean_mask);
   return cudaGetLastError();
 }
 

@@ -46,13 +46,13 @@ __device__ __forceinline__ double last_block_sum(const double* partial, unsigned
   return s;
 }
 
-// p = r (first) or r + beta p; t = K : p; pKp = p . t; alpha = rr / pKp.
+// p = r (first) or r + beta p; t = K : p; block sums of p . t (added up, and
+// alpha = rr / p . t formed, by launch_laplace_solve: see Fold).
 // Returns at once when the CG loop has converged (done != 0).
 __global__ void __launch_bounds__(RVE_RED_THREADS, 3) k_tangent_apply(size_t nvox, const double* __restrict__ K,
                                                                       const double* __restrict__ r, double* __restrict__ p,
                                                                       double* __restrict__ t, double* __restrict__ ds,
-                                                                      double* __restrict__ partial,
-                                                                      unsigned int* __restrict__ ticket) {
+                                                                      double* __restrict__ partial) {
   __shared__ double sh[320];
   if (ds[DS_DONE] != 0.0) return;
   // the first iteration of a solve (the counter is reset by the CG init and
@@ -87,47 +87,14 @@ __global__ void __launch_bounds__(RVE_RED_THREADS, 3) k_tangent_apply(size_t nvo
   }
   const double s = block_sum(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
-  const double tot = last_block_sum(partial, ticket, sh);
-  if (threadIdx.x == 0 && !isnan(tot)) {
-    ds[DS_PKP] = tot;
-    ds[DS_ALPHA] = ds[DS_RR] / tot;
-  }
-}
-
-// x += alpha p; r -= alpha q; rr' = r . r; beta = rr' / rr; one more
-// iteration counted; done once rr' <= stop.
-__global__ void __launch_bounds__(RVE_RED_THREADS) k_cg_update(size_t n, double* __restrict__ x, double* __restrict__ r,
-                                                               const double* __restrict__ p, const double* __restrict__ q,
-                                                               double* __restrict__ ds, double* __restrict__ partial,
-                                                               unsigned int* __restrict__ ticket) {
-  __shared__ double sh[320];
-  if (ds[DS_DONE] != 0.0) return;
-  const double alpha = ds[DS_ALPHA];
-  double acc = 0.0;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    x[e] = fma(alpha, p[e], x[e]);
-    const double rv = fma(-alpha, q[e], r[e]);
-    r[e] = rv;
-    acc = fma(rv, rv, acc);
-  }
-  const double s = block_sum(acc, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = s;
-  const double tot = last_block_sum(partial, ticket, sh);
-  if (threadIdx.x == 0 && !isnan(tot)) {
-    ds[DS_BETA] = tot / ds[DS_RR];
-    ds[DS_RR] = tot;
-    ds[DS_ITERS] += 1.0;
-    if (!(tot > ds[DS_STOP])) ds[DS_DONE] = 1.0;   // also stops on NaN
-  }
 }
 
 // Mixed precision: the same CG step with FP32 tangent and vectors (warp sums
-// in FP32, block and grid sums in FP64).  p = r (first) or r + beta p; t = K : p; alpha = rr / p.t
+// in FP32, block and grid sums in FP64).  p = r (first) or r + beta p; t = K : p; block sums of p . t
 __global__ void __launch_bounds__(RVE_RED_THREADS, 2) k_tangent_apply32(size_t nvox, const float* __restrict__ K,
                                                                      const float* __restrict__ r, float* __restrict__ p,
                                                                      float* __restrict__ t, double* __restrict__ ds,
-                                                                     double* __restrict__ partial,
-                                                                     unsigned int* __restrict__ ticket) {
+                                                                     double* __restrict__ partial) {
   __shared__ double sh[320];
   if (ds[DS_DONE] != 0.0) return;
   const bool first = ds[DS_ITERS] == 0.0;
@@ -157,11 +124,6 @@ __global__ void __launch_bounds__(RVE_RED_THREADS, 2) k_tangent_apply32(size_t n
   }
   const double s = blk_sum_v<float>(acc, sh);   // warp stage in FP32
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
-  const double tot = last_block_sum(partial, ticket, sh);
-  if (threadIdx.x == 0 && !isnan(tot)) {
-    ds[DS_PKP] = tot;
-    ds[DS_ALPHA] = ds[DS_RR] / tot;
-  }
 }
 
 // ---- TMA-staged FP32 tangent apply ----
@@ -232,9 +194,7 @@ __device__ __forceinline__ void ta_issue(const float* __restrict__ K, const floa
 __global__ void __launch_bounds__(TA_TV, 1) k_tangent_apply32_tma(size_t nvox, const float* __restrict__ K,
                                                                  const float* __restrict__ r, float* __restrict__ p,
                                                                  float* __restrict__ t, double* __restrict__ ds,
-                                                                 double* __restrict__ partial,
-                                                                 unsigned int* __restrict__ ticket,
-                                                                 unsigned tile_wait_polls) {
+                                                                 double* __restrict__ partial, unsigned tile_wait_polls) {
   extern __shared__ __align__(128) unsigned char ta_smem[];
   float* stage[2] = {reinterpret_cast<float*>(ta_smem), reinterpret_cast<float*>(ta_smem) + TA_STAGE};
   uint64_t* bar = reinterpret_cast<uint64_t*>(ta_smem + 2 * (size_t)TA_STAGE_BYTES);
@@ -300,11 +260,6 @@ __global__ void __launch_bounds__(TA_TV, 1) k_tangent_apply32_tma(size_t nvox, c
   }
   const double s = blk_sum_v<float>(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
-  const double tot = last_block_sum(partial, ticket, sh);
-  if (threadIdx.x == 0 && !isnan(tot)) {
-    ds[DS_PKP] = tot;
-    ds[DS_ALPHA] = ds[DS_RR] / tot;
-  }
 }
 
 // x32 = 0; r32 = -R (rounded); rr; stop = eta^2 rr; iteration count 0
@@ -360,38 +315,15 @@ __global__ void __launch_bounds__(RVE_RED_THREADS) k_cg_init(size_t n, double* _
   }
 }
 
-__global__ void __launch_bounds__(RVE_RED_THREADS) k_norm2(size_t n, const double* __restrict__ a, double* __restrict__ partial) {
-  __shared__ double sh[320];
+// the 27 sums of k_macro
+__global__ void __launch_bounds__(256) k_macro_final(const double* __restrict__ partial, int nparts, double* __restrict__ ds) {
+  const int c = threadIdx.x >> 3, part = threadIdx.x & 7;       // eight threads per value
   double acc = 0.0;
-  for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
-    acc = fma(a[e], a[e], acc);
-  const double s = block_sum(acc, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = s;
-}
-
-__global__ void __launch_bounds__(1024) k_reduce_final(const double* __restrict__ partial, int nparts, int nval,
-                                                       int mode, double* __restrict__ ds) {
-  __shared__ double sh[320];
-  for (int c = 0; c < nval; ++c) {
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += partial[(size_t)c * nparts + i];
-    const double s = block_sum(acc, sh);
-    if (threadIdx.x == 0) {
-      if (mode == RED_PKP_ALPHA) {
-        ds[DS_PKP] = s;
-        ds[DS_ALPHA] = ds[DS_RR] / s;
-      } else if (mode == RED_RR_BETA) {
-        ds[DS_BETA] = s / ds[DS_RR];
-        ds[DS_RR] = s;
-      } else if (mode == RED_RR_INIT) {
-        ds[DS_RR] = s;
-      } else if (mode == RED_NORM) {
-        ds[DS_NORM] = s;
-      } else {  // RED_MACRO: 27 averages -> mean P, mean sigma, mean F
-        ds[DS_MEANP + c] = s;
-      }
-    }
-  }
+  if (c < 27)
+    for (int i = part; i < nparts; i += 8) acc += partial[(size_t)c * nparts + i];
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (c < 27 && part == 0) ds[DS_MEANP + c] = acc;               // mean P, sigma, F
 }
 
 __global__ void k_axpy(size_t n, double* __restrict__ y, const double* __restrict__ x, double a) {
@@ -546,16 +478,8 @@ cudaError_t launch_tangent_apply(const rve_s* h, cudaStream_t s) {
   {
     ProfScope ps_(h, RVE_K_TANGENT_APPLY, s);
     k_tangent_apply<<<blocks, RVE_RED_THREADS, 0, s>>>(h->nvox, h->K[h->cur], h->r, h->p, h->t, h->dscal,
-                                                       h->partial, (unsigned int*)(h->dcount + 4));
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_cg_update(const rve_s* h, cudaStream_t s) {
-  {
-    ProfScope ps_(h, RVE_K_CG_UPDATE, s);
-    k_cg_update<<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>(9 * h->nvox, h->x, h->r, h->p, h->q, h->dscal, h->partial,
-                                                           (unsigned int*)(h->dcount + 4));
+                                                       h->partial_pkp());
+    h->fold.pkp_blocks = blocks;
   }
   return cudaGetLastError();
 }
@@ -565,26 +489,6 @@ cudaError_t launch_cg_init(const rve_s* h, double eta, cudaStream_t s) {
     ProfScope ps_(h, RVE_K_OTHER, s);
     k_cg_init<<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>(9 * h->nvox, h->x, h->r, h->R, h->dscal, eta, h->partial,
                                                          (unsigned int*)(h->dcount + 4));
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_norm2(const rve_s* h, const double* a, int ncomp, cudaStream_t s) {
-  {
-    ProfScope ps_(h, RVE_K_REDUCE, s);
-    k_norm2<<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>((size_t)ncomp * h->nvox, a, h->partial);
-  }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return launch_reduce_final(h, RED_NORM, s);
-}
-
-cudaError_t launch_reduce_final(const rve_s* h, int mode, cudaStream_t s) {
-  const int nval = mode == RED_MACRO ? 27 : 1;
-  const int nparts = mode == RED_MACRO ? MACRO_BLOCKS : RVE_RED_BLOCKS;
-  {
-    ProfScope ps_(h, RVE_K_REDUCE, s);
-    k_reduce_final<<<1, 1024, 0, s>>>(h->partial, nparts, nval, mode, h->dscal);
   }
   return cudaGetLastError();
 }
@@ -633,9 +537,11 @@ cudaError_t launch_macro(const rve_s* h, cudaStream_t s) {
     ProfScope ps_(h, RVE_K_REDUCE, s);
     k_macro<<<MACRO_BLOCKS, RVE_RED_THREADS, 0, s>>>(h->nvox, h->P_c, h->F_c, h->partial);
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  return launch_reduce_final(h, RED_MACRO, s);
+  {
+    ProfScope ps_(h, RVE_K_REDUCE, s);
+    k_macro_final<<<1, 256, 0, s>>>(h->partial, MACRO_BLOCKS, h->dscal);
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t launch_output_field(const rve_s* h, int which, const double* P, const double* S, double* dst,
@@ -656,12 +562,12 @@ cudaError_t launch_tangent_apply32(const rve_s* h, cudaStream_t s) {
     ProfScope ps_(h, RVE_K_TANGENT_APPLY, s);
     if (h->tma_apply)   // persistent: one block per SM
       k_tangent_apply32_tma<<<h->num_sms, TA_TV, TA_SMEM, s>>>(h->nvox, reinterpret_cast<const float*>(h->K[h->cur]),
-                                                               h->r32, h->p32, h->t32, h->dscal, h->partial,
-                                                               (unsigned int*)(h->dcount + 4), h->wait_polls);
+                                                               h->r32, h->p32, h->t32, h->dscal, h->partial_pkp(),
+                                                               h->wait_polls);
     else
       k_tangent_apply32<<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>(h->nvox, reinterpret_cast<const float*>(h->K[h->cur]),
-                                                                   h->r32, h->p32, h->t32, h->dscal, h->partial,
-                                                                   (unsigned int*)(h->dcount + 4));
+                                                                   h->r32, h->p32, h->t32, h->dscal, h->partial_pkp());
+    h->fold.pkp_blocks = h->tma_apply ? h->num_sms : RVE_RED_BLOCKS;
   }
   return cudaGetLastError();
 }

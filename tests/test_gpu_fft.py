@@ -92,7 +92,7 @@ def test_projection_of_fields_on_an_odd_eight_byte_boundary(pkg, n0):
     it; one that starts 8 bytes off gives the same bits, and so does a run of
     many rows per warp (sums of the means are taken down in between)."""
     import torch
-    shape = (40, 54, n0) if n0 < 8 else (3, 4, n0)
+    shape = (36, 54, n0) if n0 < 8 else (3, 4, n0)
     Xd = device_field(np.random.default_rng(n0).standard_normal(shape + (3, 3)) + 5.0)
     shifted = torch.empty(Xd.numel() + 1, dtype=Xd.dtype, device=Xd.device)[1:].view_as(Xd)
     shifted.copy_(Xd)
