@@ -264,8 +264,8 @@ __global__ void __launch_bounds__(128) k_hardening(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
     const double* __restrict__ qhat, const double* __restrict__ Apinv, const int32_t* __restrict__ screw_of,
     const double* __restrict__ nye, const double* __restrict__ rho_ssd, const double* __restrict__ Fp,
-    double* __restrict__ rho18, double* __restrict__ rho_gnd, double* __restrict__ tauc, double* __restrict__ ell,
-    double* __restrict__ Fp0inv, Consts c) {
+    double* __restrict__ rho18, double* __restrict__ rho_gnd, double* __restrict__ tauc, double* __restrict__ tinv,
+    double* __restrict__ ell, double* __restrict__ Fp0inv, Consts c) {
   __shared__ double sq[144], sA[162];
   __shared__ int sscrew[12];
   for (int i = threadIdx.x; i < 144; i += blockDim.x) sq[i] = qhat[i];
@@ -305,7 +305,9 @@ __global__ void __launch_bounds__(128) k_hardening(
     double s = 0.0;
 #pragma unroll
     for (int b = 0; b < 12; ++b) s = fma(sq[12 * a + b], rho[b], s);
-    tauc[a * nvox + v] = fma(amb, sqrt(s), c.tau0);
+    const double t = fma(amb, sqrt(s), c.tau0);
+    tauc[a * nvox + v] = t;
+    tinv[a * nvox + v] = 1.0 / t;      // read by every evaluation of the increment
     ell[a * nvox + v] = c.K / sqrt(sum - rho[a]);
   }
   double Fpv[9], Fi[9];
@@ -329,7 +331,7 @@ struct VoxelIn {
 __device__ __forceinline__ void load_voxel(size_t nvox, size_t v, const int32_t* __restrict__ grain,
                                            const double* __restrict__ grainR, const double* __restrict__ Fin,
                                            const double* __restrict__ xdir, double lambda,
-                                           const double* __restrict__ Fp0inv, const double* __restrict__ tauc_g,
+                                           const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
                                            VoxelIn& in) {
   double Fs[9], T[9], FeTr[9];
   const int g = grain[v];
@@ -347,8 +349,571 @@ __device__ __forceinline__ void load_voxel(size_t nvox, size_t v, const int32_t*
   mat3_mul(in.Ft, in.Fpi0, FeTr);
   mat3_tmul(FeTr, FeTr, in.A);
 #pragma unroll
-  for (int a = 0; a < 12; ++a) in.tinv[a] = 1.0 / tauc_g[a * nvox + v];
+  for (int a = 0; a < 12; ++a) in.tinv[a] = tinv_g[a * nvox + v];
 }
+
+// ---- the local Newton iteration ----
+// Its FP64 work is the residual alone.  The Newton matrix and its solve run in
+// FP32, which is 60 times faster here: they only propose the step, and a step is taken
+// if the FP64 residual says so, until that is below the same tolerance.  (An FP32
+// direction errs by about 1e-5 of the step, so the last digits converge by that
+// factor per iteration instead of quadratically.)
+
+// magnitude of a double as an ordered integer (NaN above infinity)
+__device__ __forceinline__ unsigned long long mag_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
+}
+constexpr unsigned long long INF_BITS = 0x7ff0000000000000ull;
+
+// double to float and back by integer instructions (the conversions of the
+// FP64 pipe cost as much as an FMA there); truncated; below 2^-126: zero
+__device__ __forceinline__ float f32_of(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  const unsigned m = (__funnelshift_l((unsigned)lo, (unsigned)hi, 3) - (896u << 23)) & 0x7fffffffu;
+  const unsigned v = e <= 896 ? 0u : (e >= 1151 ? 0x7f7fffffu : m);
+  return __uint_as_float(v | ((unsigned)hi & 0x80000000u));
+}
+__device__ __forceinline__ double f64_of(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  const unsigned hi = (m >> 3) + (896u << 20);
+  return m < 0x00800000u ? 0.0 : __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+
+// sqrt 6 times the resolved shears of the twelve systems: every one is a
+// difference of two normal components and a sum or difference of two shears
+__device__ __forceinline__ void resolved12(const double* S, double* t) {
+  const double a = S[1] - S[2], b = S[2] - S[0], c = S[0] - S[1];
+  const double am = S[5] - S[4], ap = S[5] + S[4], bm = S[3] - S[5], bp = S[3] + S[5], cm = S[4] - S[3], cp = S[4] + S[3];
+  t[0] = a + am; t[1] = b + bm; t[2] = c + cm;
+  t[3] = a - am; t[4] = b + bp; t[5] = cp - c;
+  t[6] = ap - a; t[7] = bm - b; t[8] = c + cp;
+  t[9] = a + ap; t[10] = bp - b; t[11] = c - cm;
+}
+
+// sum_a g_a s'^a (x) m'^a (unnormalised): the three directions of each plane first
+__device__ __forceinline__ void schmid_sum(const double* g, double* M) {
+  const double v[4][3] = {{g[2] - g[1], g[0] - g[2], g[1] - g[0]},
+                          {g[4] + g[5], g[3] + g[5], g[4] - g[3]},
+                          {g[7] + g[8], g[6] + g[8], g[6] - g[7]},
+                          {g[10] + g[11], g[9] - g[11], g[9] + g[10]}};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const double t = v[0][i] + v[1][i], u = v[0][i] - v[1][i], s = v[2][i] + v[3][i], w = v[3][i] - v[2][i];
+    M[3 * i] = u + s;
+    M[3 * i + 1] = t + w;
+    M[3 * i + 2] = t - w;
+  }
+}
+
+// adjugate of M and its determinant
+__device__ __forceinline__ double adjugate(const double* M, double* B) {
+  B[0] = fma(M[4], M[8], -M[5] * M[7]);
+  B[1] = fma(M[2], M[7], -M[1] * M[8]);
+  B[2] = fma(M[1], M[5], -M[2] * M[4]);
+  B[3] = fma(M[5], M[6], -M[3] * M[8]);
+  B[4] = fma(M[0], M[8], -M[2] * M[6]);
+  B[5] = fma(M[2], M[3], -M[0] * M[5]);
+  B[6] = fma(M[3], M[7], -M[4] * M[6]);
+  B[7] = fma(M[1], M[6], -M[0] * M[7]);
+  B[8] = fma(M[0], M[4], -M[1] * M[3]);
+  return fma(M[0], B[0], fma(M[1], B[3], M[2] * B[6]));
+}
+
+// A^T A of a 3x3 matrix, Voigt order
+__device__ __forceinline__ void gram(const double* A, double* G) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const int i = V_I(k), j = V_J(k);
+    G[k] = fma(A[i], A[j], fma(A[3 + i], A[3 + j], A[6 + i] * A[6 + j]));
+  }
+}
+
+// The residual r(S) and what the Newton matrix and the stress need: the ratios
+// x = tau / tauc, M^-1 = adj * id, Ce (Voigt).  A (Voigt): trial elastic right
+// Cauchy-Green tensor; tq = 1 / (sqrt 6 tauc).  dg(a, value) receives the slips.
+// rn: max |r| as bits, INF_BITS when a slip exceeds its cap or the residual is not finite.
+struct Residual {
+  double x[12], adj[9], id, Ce[6], r[6];
+  unsigned long long rn;
+};
+template <class Slip>
+__device__ __forceinline__ void residual(const Consts& c, const double* S, const double* A, const double* tq, double dt,
+                                         Residual& e, Slip dg) {
+  double g[12];
+  resolved12(S, e.x);
+  const double rate = dt * c.gdot0;
+  unsigned long long most = 0ull;
+#pragma unroll
+  for (int a = 0; a < 12; ++a) {
+    e.x[a] *= tq[a];
+    g[a] = rate * pow_n(c, fabs(e.x[a]));
+    most = max(most, mag_bits(g[a]));
+    g[a] = copysign(g[a], e.x[a]);
+    dg(a, g[a]);
+  }
+  e.rn = INF_BITS;
+  if (most > mag_bits(c.dgam_max)) return;
+  double M[9], X[6];
+  schmid_sum(g, M);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) M[k] = k % 4 == 0 ? fma(INV_SQRT6, M[k], 1.0) : INV_SQRT6 * M[k];
+  e.id = 1.0 / adjugate(M, e.adj);
+  const double Af[9] = {A[0], A[5], A[4], A[5], A[1], A[3], A[4], A[3], A[2]};
+  double B[9];
+  mat3_mul(Af, e.adj, B);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const int i = V_I(k), j = V_J(k);
+    X[k] = fma(e.adj[i], B[j], fma(e.adj[3 + i], B[3 + j], e.adj[6 + i] * B[6 + j]));
+  }
+  // Ce = id^2 X, E = (Ce - I) / 2, r = S - C : E
+  const double id2 = e.id * e.id, h = 0.5 * id2, c44 = c.C44 * id2, cd = c.C11 - c.C12;
+  const double E0 = fma(h, X[0], -0.5), E1 = fma(h, X[1], -0.5), E2 = fma(h, X[2], -0.5);
+  const double q = c.C12 * (E0 + E1 + E2);
+  e.r[0] = fma(-cd, E0, S[0] - q);
+  e.r[1] = fma(-cd, E1, S[1] - q);
+  e.r[2] = fma(-cd, E2, S[2] - q);
+  unsigned long long rn = 0ull;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    if (k >= 3) e.r[k] = fma(-c44, X[k], S[k]);
+    e.Ce[k] = X[k];                                 // times id2: applied where it is used
+    rn = max(rn, mag_bits(e.r[k]));
+  }
+  e.rn = rn < INF_BITS ? rn : INF_BITS;
+}
+
+// |x|^(n - 1) in FP32
+__device__ __forceinline__ float pow_n1f(const Consts& c, float x) {
+  if (c.n_int == 20) {
+    const float x2 = x * x, x3 = x * x2, x4 = x2 * x2, x8 = x4 * x4;
+    return x3 * (x8 * x8);
+  }
+  if (!c.n_int) return powf(x, (float)(c.n - 1.0));
+  float r = 1.0f;
+  for (int n = c.n_int - 1; n; n >>= 1) {
+    if (n & 1) r *= x;
+    x *= x;
+  }
+  return r;
+}
+
+__device__ __forceinline__ float faccf(float acc, bool& first, int k, float x) {
+  if (k == 0) return acc;
+  const float v = k < 0 ? -x : x;
+  const float r = first ? v : acc + v;
+  first = false;
+  return r;
+}
+
+// d = -J^-1 r for any stiffness: J = I + C : H, H without the compliance
+// (rve_create sets s11 = s12 = s44 = 0 when C11 + 2 C12 <= 0, where the compliance form does not apply)
+static __device__ __noinline__ void newton_direction_general(const Consts& c, const float* H, const double* r, float* d) {
+  double J[36], b[6];
+  int piv[6];
+  for (int j = 0; j < 6; ++j) {
+    double col[6], cc[6];
+    for (int i = 0; i < 6; ++i) col[i] = H[6 * i + j];
+    cubic(c, col, cc);
+    for (int i = 0; i < 6; ++i) J[6 * i + j] = (i == j ? 1.0 : 0.0) + cc[i];
+  }
+  for (int i = 0; i < 6; ++i) b[i] = -r[i];
+  lu6(J, piv);
+  lu6_solve(J, piv, b);
+  for (int i = 0; i < 6; ++i) d[i] = (float)b[i];
+}
+
+// Newton direction d = -J^-1 r in FP32, from (C^-1 - N) d = -C^-1 r with N =
+// dE/dS = -sum_a gp^a sym(Ce S0^a Minv) (x) d tau^a / dS: C^-1 - N is close to
+// symmetric positive definite (compliance plus a sum of nearly symmetric
+// rank-one terms), so it is factorised without pivoting.
+__device__ __forceinline__ void newton_direction(const Consts& c, const Residual& e, const double* tq, double dt, float* d) {
+  float Ce[9], Mi[9], J[36];
+  const float id = f32_of(e.id), id2 = id * id;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Mi[k] = id * f32_of(e.adj[k]);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) Ce[3 * V_I(k) + V_J(k)] = Ce[3 * V_J(k) + V_I(k)] = id2 * f32_of(e.Ce[k]);
+  const float s11 = (float)c.s11, s12 = (float)c.s12, s44 = (float)c.s44;
+#pragma unroll
+  for (int i = 0; i < 6; ++i)
+#pragma unroll
+    for (int j = 0; j < 6; ++j) J[6 * i + j] = i == j ? (i < 3 ? s11 : s44) : (i < 3 && j < 3 ? s12 : 0.0f);
+  const float rate = (float)(dt * c.gdot0 * c.n * INV_SQRT6);
+#pragma unroll
+  for (int a = 0; a < 12; ++a) {
+    const float gp = rate * pow_n1f(c, fabsf(f32_of(e.x[a]))) * f32_of(tq[a]);
+    float u[3], w[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      bool fu = true, fw = true;
+      u[i] = w[i] = 0.0f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        u[i] = faccf(u[i], fu, fcc_s(a, k), Ce[3 * i + k]);
+        w[i] = faccf(w[i], fw, fcc_m(a, k), Mi[3 * k + i]);
+      }
+      u[i] *= gp;
+    }
+    const float T[6] = {u[0] * w[0], u[1] * w[1], u[2] * w[2], 0.5f * (u[1] * w[2] + u[2] * w[1]),
+                        0.5f * (u[0] * w[2] + u[2] * w[0]), 0.5f * (u[0] * w[1] + u[1] * w[0])};
+#pragma unroll
+    for (int i = 0; i < 6; ++i)
+#pragma unroll
+      for (int j = 0; j < 6; ++j)
+        if (tau_coef(a, j) != 0) J[6 * i + j] = tau_coef(a, j) > 0 ? J[6 * i + j] + T[i] : J[6 * i + j] - T[i];
+  }
+  if (!(c.s11 > 0.0)) {                          // no positive definite compliance: rows through the stiffness, pivoted
+    float Hc[36], dc[6];                         // (copies: the arrays of the other path stay in registers)
+    double rc[6];
+#pragma unroll
+    for (int k = 0; k < 36; ++k) Hc[k] = J[k];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) rc[k] = e.r[k];
+    newton_direction_general(c, Hc, rc, dc);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) d[k] = dc[k];
+    return;
+  }
+  const float r0 = f32_of(e.r[0]), r1 = f32_of(e.r[1]), r2 = f32_of(e.r[2]);
+  d[0] = -(s11 * r0 + s12 * (r1 + r2));
+  d[1] = -(s11 * r1 + s12 * (r0 + r2));
+  d[2] = -(s11 * r2 + s12 * (r0 + r1));
+#pragma unroll
+  for (int k = 3; k < 6; ++k) d[k] = -s44 * f32_of(e.r[k]);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const float inv = 1.0f / J[6 * k + k];
+    J[6 * k + k] = inv;
+#pragma unroll
+    for (int i = k + 1; i < 6; ++i) {
+      const float l = J[6 * i + k] * inv;
+#pragma unroll
+      for (int j = k + 1; j < 6; ++j) J[6 * i + j] = fmaf(-l, J[6 * k + j], J[6 * i + j]);
+      d[i] = fmaf(-l, d[k], d[i]);
+    }
+  }
+#pragma unroll
+  for (int i = 5; i >= 0; --i) {
+#pragma unroll
+    for (int j = i + 1; j < 6; ++j) d[i] = fmaf(-J[6 * i + j], d[j], d[i]);
+    d[i] *= J[6 * i + i];
+  }
+}
+
+// F (with the line-search step) times R, and F~ = R^T F R
+__device__ __forceinline__ void load_F(size_t nvox, size_t v, const double* __restrict__ R, const double* __restrict__ Fin,
+                                       const double* __restrict__ xdir, double lambda, double* FR, double* Ft) {
+  double Fs[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    double f = Fin[k * nvox + v];
+    if (lambda != 0.0) f = fma(lambda, xdir[k * nvox + v], f);
+    Fs[k] = f;
+  }
+  mat3_mul(Fs, R, FR);
+  if (Ft) mat3_tmul(R, FR, Ft);
+}
+
+// Local Newton on S at one voxel (data-dependent iteration counts): writes S,
+// dgam and P; returns the Newton iterations, residual evaluations and whether
+// it failed.  One residual call serves the warm start, the restart from the
+// elastic-free state, the trials and their halvings; the slips go to memory at every
+// evaluation, and F and R are read again for P, so that few registers live through the loop.
+__device__ __forceinline__ void local_voxel(size_t nvox, size_t v, const int32_t* __restrict__ grain,
+                                            const double* __restrict__ grainR, const double* __restrict__ Fin,
+                                            const double* __restrict__ xdir, double lambda,
+                                            const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
+                                            const double* __restrict__ Swarm, double* __restrict__ Sout,
+                                            double* __restrict__ dgout, double* __restrict__ Pout, double dt,
+                                            const Consts& c, int& iters, int& evals, int& failed) {
+  double A[6], tq[12], S[6], St[6];
+  const double* Rg = grainR + 9 * grain[v];
+  {
+    double R[9], FR[9], Ft[9], Fpi0[9], FeTr[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) { R[k] = __ldg(Rg + k); Fpi0[k] = Fp0inv[k * nvox + v]; }
+    load_F(nvox, v, R, Fin, xdir, lambda, FR, Ft);
+    mat3_mul(Ft, Fpi0, FeTr);
+    gram(FeTr, A);
+  }
+#pragma unroll
+  for (int a = 0; a < 12; ++a) tq[a] = INV_SQRT6 * tinv_g[a * nvox + v];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) St[k] = S[k] = Swarm[k * nvox + v];
+  const unsigned long long tol = mag_bits(c.local_tol_abs), floor_ = mag_bits(c.floor_abs);
+  Residual e;
+  unsigned long long rn = 0ull;                  // of S
+  float d[6];
+  double lam = 1.0;
+  int halved = 0;
+  bool first = true, restarted = false, conv = false, last = false;
+  for (;;) {
+    residual(c, St, A, tq, dt, e, [&](int a, double g) { dgout[a * nvox + v] = g; });
+    if (last) break;                             // e is that of S again
+    ++evals;
+    bool accept = e.rn < rn;
+    if (first) {
+      if (e.rn >= INF_BITS && !restarted) {      // warm start rejected: restart from the elastic-free state
+        restarted = true;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) St[k] = S[k] = 0.0;
+        continue;
+      }
+      first = false;
+      accept = true;
+    } else if (accept) {
+      ++iters;
+    }
+    if (accept) {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) S[k] = St[k];
+      rn = e.rn;
+      conv = rn <= tol;
+      if (conv || iters >= c.max_local) break;
+      newton_direction(c, e, tq, dt, d);
+      lam = 1.0;
+      halved = 0;
+    } else {
+      // no decrease: halve; at the round-off floor (or after all halvings) stop at S
+      lam *= 0.5;
+      ++halved;
+      if (halved > c.max_halvings || (rn <= floor_ && halved > 3)) {
+        ++iters;
+        conv = rn <= floor_;
+        last = true;
+        lam = 0.0;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) St[k] = fma(lam, f64_of(d[k]), S[k]);
+  }
+  failed = conv ? 0 : 1;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) Sout[k * nvox + v] = S[k];
+  // P = F~ Q rotated to the sample frame = (F R) Q R^T, Q = Fp^-1 S Fp^-T,
+  // Fp^-1 = Fp_prev^-1 M^-1 (Eq. Piola)
+  double R[9], FR[9], Fpi0[9], Fpinv[9], Sf[9], W[9], Q[9], T[9], P[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) { R[k] = __ldg(Rg + k); Fpi0[k] = Fp0inv[k * nvox + v]; }
+#pragma unroll
+  for (int k = 0; k < 9; ++k) e.adj[k] *= e.id;
+  mat3_mul(Fpi0, e.adj, Fpinv);
+  sym_full(S, Sf);
+  mat3_mult(Sf, Fpinv, W);
+  mat3_mul(Fpinv, W, Q);
+  load_F(nvox, v, R, Fin, xdir, lambda, FR, nullptr);
+  mat3_mul(FR, Q, T);
+  mat3_mult(T, R, P);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Pout[k * nvox + v] = P[k];
+}
+
+constexpr int LOCAL_THREADS = 128, LOCAL_BLOCKS = 3;
+
+// Local update over all voxels.  The number of local Newton iterations
+// differs from voxel to voxel (grains near their yield point need several),
+// so the kernel is persistent and balanced dynamically: each warp takes the
+// next chunk of 32 voxels from a device counter (counters[6], zeroed before
+// the launch) until none is left, and an SM whose voxels converge quickly
+// takes more chunks.  Each voxel's arithmetic is the same as with a fixed
+// assignment.
+__global__ void __launch_bounds__(LOCAL_THREADS, LOCAL_BLOCKS) k_local(
+    size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
+    const double* __restrict__ Fin, const double* __restrict__ xdir, double lambda,
+    const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g, const double* __restrict__ Swarm,
+    double* __restrict__ Sout, double* __restrict__ dgout, double* __restrict__ Pout,
+    int32_t* __restrict__ counters, double dt, Consts c) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const long nchunks = (long)((nvox + 31) / 32);
+  int mx = 0, nf = 0;
+  unsigned si = 0, se = 0;
+  for (;;) {
+    int chunk = 0;
+    if (lane == 0) chunk = atomicAdd(&counters[6], 1);
+    chunk = __shfl_sync(full, chunk, 0);
+    if (chunk >= nchunks) break;
+    const size_t v = (size_t)chunk * 32 + lane;
+    int iters = 0, failed = 0, evals = 0;
+    if (v < nvox)
+      local_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c,
+                  iters, evals, failed);
+    mx = max(mx, iters);
+    nf += failed;
+    si += (unsigned)iters;
+    se += (unsigned)evals;
+  }
+  // counters: warp-aggregated
+  mx = __reduce_max_sync(full, mx);
+  nf = __reduce_add_sync(full, nf);
+  si = __reduce_add_sync(full, si);
+  se = __reduce_add_sync(full, se);
+  if (lane == 0) {
+    if (mx) atomicMax(&counters[0], mx);
+    if (nf) atomicAdd(&counters[1], nf);
+    // 64-bit totals of local Newton iterations and residual evaluations (work accounting)
+    unsigned long long* tot = reinterpret_cast<unsigned long long*>(counters + 8);
+    atomicAdd(&tot[0], (unsigned long long)si);
+    atomicAdd(&tot[1], (unsigned long long)se);
+  }
+}
+
+// The consistent tangent at the converged S: the same work for every voxel
+// (no data-dependent iterations), so whole warps stay converged.
+//
+// With L_k = sum_a dgp^a (d tau^a / dS_k) s^a (x) m^a (so dM = sum_k L_k dS_k), the Newton matrix is
+// J = I + C : sym(Ce L_k Minv) column by column, and a strain increment dE gives
+// dS = J^-1 C : dE and
+//   F~ dQ = Fe B Fp^-T,  B = dS - dM V - (dM V)^T,  V = Minv S,
+// which is the change of P~ at fixed F~; B = T dS with one 6 x 6 matrix T.  A direction
+// dF = e_k e_l^T of the sample frame has dE = sym(U_k (x) W_l) with the rows of U = R Fe and W =
+// R Fp^-1, and
+//   dP_ij = delta_ik (W S W^T)_jl + (U B W^T)_ij,
+// so the six unit strains are carried to the sample frame once (H = U B W^T, 9 x 6 in shared
+// memory) and each of the nine directions costs H dE.
+//
+// Bound by the FP64 pipe: 2.6 thousand instructions per voxel, against 4.9
+// thousand with the Schmid sums, the products of dQ and the rotation formed per
+// strain and per direction: 2.39 -> 1.43 ms at 64^3.
+constexpr int TAN_THREADS = 64;
+
+__global__ void __launch_bounds__(TAN_THREADS) k_tangent(
+    size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
+    const double* __restrict__ Fin, const double* __restrict__ xdir, double lambda,
+    const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g, const double* __restrict__ Sin,
+    double* __restrict__ Kout, double dt, Consts c, int k32) {
+  __shared__ double Hs[54 * TAN_THREADS], Ts[36 * TAN_THREADS];   // [slot][thread]
+  double* H = Hs + threadIdx.x;
+  double* T = Ts + threadIdx.x;
+  const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= nvox) return;
+  double J[36];
+  int piv[6];
+  double U[9], W[9], Qs[9];
+  {
+    double R[9], FR[9], Fpi0[9], S[6], Mi[9], Ce[9], V[9], gp[12];
+    const double* Rg = grainR + 9 * grain[v];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) { R[k] = __ldg(Rg + k); Fpi0[k] = Fp0inv[k * nvox + v]; }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) S[k] = Sin[k * nvox + v];
+    {
+      double Ft[9], FeTr[9], A[6], tq[12];
+      load_F(nvox, v, R, Fin, xdir, lambda, FR, Ft);
+      mat3_mul(Ft, Fpi0, FeTr);
+      gram(FeTr, A);
+#pragma unroll
+      for (int a = 0; a < 12; ++a) tq[a] = INV_SQRT6 * tinv_g[a * nvox + v];
+      Residual e;
+      residual(c, S, A, tq, dt, e, [](int, double) {});
+      const double rate = dt * c.gdot0 * c.n * INV_SQRT6;
+#pragma unroll
+      for (int a = 0; a < 12; ++a) gp[a] = rate * pow_n1(c, fabs(e.x[a])) * tq[a];    // dgp / 6
+#pragma unroll
+      for (int k = 0; k < 9; ++k) Mi[k] = e.adj[k] * e.id;
+      const double id2 = e.id * e.id;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) Ce[3 * V_I(k) + V_J(k)] = Ce[3 * V_J(k) + V_I(k)] = id2 * e.Ce[k];
+    }
+    {
+      double Sf[9], Fpinv[9], Z[9];
+      sym_full(S, Sf);
+      mat3_mul(Mi, Sf, V);
+      mat3_mul(Fpi0, Mi, Fpinv);
+      mat3_mul(R, Fpinv, W);
+      mat3_mul(FR, Fpinv, U);
+      mat3_mul(W, Sf, Z);
+      mat3_mult(Z, W, Qs);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      double L[9], X[9], Z[9], col[6], cc[6];
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        double w4[4];
+#pragma unroll
+        for (int p = 0; p < 4; ++p) {
+          bool f = true;
+          w4[p] = 0.0;
+#pragma unroll
+          for (int a = 3 * p; a < 3 * p + 3; ++a) w4[p] = cacc(w4[p], f, fcc_s(a, i) * tau_coef(a, k), gp[a]);
+        }
+        const double t = w4[0] + w4[1], u = w4[0] - w4[1], s = w4[2] + w4[3], w = w4[3] - w4[2];
+        L[3 * i] = u + s;
+        L[3 * i + 1] = t + w;
+        L[3 * i + 2] = t - w;
+      }
+      mat3_mul(L, Mi, X);
+      mat3_mul(Ce, X, Z);
+      col[0] = Z[0]; col[1] = Z[4]; col[2] = Z[8];
+      col[3] = 0.5 * (Z[5] + Z[7]); col[4] = 0.5 * (Z[2] + Z[6]); col[5] = 0.5 * (Z[1] + Z[3]);
+      cubic(c, col, cc);
+#pragma unroll
+      for (int i = 0; i < 6; ++i) J[6 * i + k] = i == k ? 1.0 + cc[i] : cc[i];
+      mat3_mul(L, V, Z);
+      const double tk[6] = {-2.0 * Z[0], -2.0 * Z[4], -2.0 * Z[8], -(Z[5] + Z[7]), -(Z[2] + Z[6]), -(Z[1] + Z[3])};
+#pragma unroll
+      for (int i = 0; i < 6; ++i) T[(6 * k + i) * TAN_THREADS] = i == k ? 1.0 + tk[i] : tk[i];
+    }
+    lu6(J, piv);
+  }
+  // H for the six unit strain increments (tensor components E11, E22, E33, E23, E13, E12, as `cubic` takes them)
+#pragma unroll 1
+  for (int m = 0; m < 6; ++m) {
+    double dE[6], dS[6], B[6] = {0, 0, 0, 0, 0, 0}, Bf[9], Z[9], P[9];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) dE[k] = k == m ? 1.0 : 0.0;
+    cubic(c, dE, dS);
+    lu6_solve(J, piv, dS);
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+#pragma unroll
+      for (int i = 0; i < 6; ++i) B[i] = fma(T[(6 * k + i) * TAN_THREADS], dS[k], B[i]);
+    sym_full(B, Bf);
+    mat3_mul(U, Bf, Z);
+    mat3_mult(Z, W, P);
+#pragma unroll
+    for (int ij = 0; ij < 9; ++ij) H[(9 * m + ij) * TAN_THREADS] = P[ij];
+  }
+  // T is done with: its place takes U, W and W S W^T for the rolled loop over directions
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    T[k * TAN_THREADS] = U[k];
+    T[(9 + k) * TAN_THREADS] = W[k];
+    T[(18 + k) * TAN_THREADS] = Qs[k];
+  }
+#pragma unroll 1
+  for (int kl = 0; kl < 9; ++kl) {
+    const int kk = kl / 3, ll = kl % 3;
+    double u[3], w[3], q[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      u[i] = T[(3 * kk + i) * TAN_THREADS];
+      w[i] = T[(9 + 3 * ll + i) * TAN_THREADS];
+      q[i] = T[(18 + 3 * ll + i) * TAN_THREADS];
+    }
+    const double dE[6] = {u[0] * w[0], u[1] * w[1], u[2] * w[2], 0.5 * fma(u[1], w[2], u[2] * w[1]),
+                          0.5 * fma(u[0], w[2], u[2] * w[0]), 0.5 * fma(u[0], w[1], u[1] * w[0])};
+#pragma unroll
+    for (int ij = 0; ij < 9; ++ij) {
+      double t = ij / 3 == kk ? q[ij % 3] : 0.0;
+#pragma unroll
+      for (int m = 0; m < 6; ++m) t = fma(H[(9 * m + ij) * TAN_THREADS], dE[m], t);
+      if (k32)   // mixed precision: the tangent only drives the FP32 conjugate gradients
+        reinterpret_cast<float*>(Kout)[(size_t)(9 * ij + kl) * nvox + v] = (float)t;
+      else
+        Kout[(size_t)(9 * ij + kl) * nvox + v] = t;
+    }
+  }
+}
+
+// ---- the same with FP64 directions and the products formed one by one ----
+// For rve_eval_constitutive on a mixed-precision handle, whose tangent is
+// rounded to FP32 (see curl_fp64.cu): the exact Jacobian's Newton path and the order of the products stay as they
+// are, so that the rounded values are the same bits.  3.05 and 2.43 ms at 64^3 within an increment, against
+// 1.07 and 1.44 ms above.
 
 // P = Fe S Fp^-T = F~ (Fp^-1 S Fp^-T) in the crystal frame, rotated to the
 // sample frame, with Fp^-1 = Fp_prev^-1 M^-1 (Eq. Piola)
@@ -363,18 +928,16 @@ __device__ __forceinline__ void piola(const VoxelIn& in, const double* S, const 
   mat3_mul(in.R, U, P);
 }
 
-// Local Newton on S at one voxel (data-dependent iteration counts): writes S,
-// dgam and P; returns the Newton iterations, residual evaluations and whether
-// it failed.
-__device__ __forceinline__ void local_voxel(size_t nvox, size_t v, const int32_t* __restrict__ grain,
+// Local Newton on S at one voxel, with the exact Jacobian
+__device__ __forceinline__ void local_voxel_fp64(size_t nvox, size_t v, const int32_t* __restrict__ grain,
                                             const double* __restrict__ grainR, const double* __restrict__ Fin,
                                             const double* __restrict__ xdir, double lambda,
-                                            const double* __restrict__ Fp0inv, const double* __restrict__ tauc_g,
+                                            const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
                                             const double* __restrict__ Swarm, double* __restrict__ Sout,
                                             double* __restrict__ dgout, double* __restrict__ Pout, double dt,
                                             const Consts& c, int& iters, int& evals, int& failed) {
   VoxelIn in;
-  load_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tauc_g, in);
+  load_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, in);
   const double* A = in.A;
   const double* tinv = in.tinv;      // 1 / tauc
   double S[6];
@@ -436,17 +999,10 @@ __device__ __forceinline__ void local_voxel(size_t nvox, size_t v, const int32_t
   for (int k = 0; k < 9; ++k) Pout[k * nvox + v] = P[k];
 }
 
-// Local update over all voxels.  The number of local Newton iterations
-// differs from voxel to voxel (grains near their yield point need several),
-// so the kernel is persistent and balanced dynamically: each warp takes the
-// next chunk of 32 voxels from a device counter (counters[6], zeroed before
-// the launch) until none is left, and an SM whose voxels converge quickly
-// takes more chunks.  Each voxel's arithmetic is the same as with a fixed
-// assignment.
-__global__ void __launch_bounds__(128) k_local(
+__global__ void __launch_bounds__(128) k_local_fp64(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
     const double* __restrict__ Fin, const double* __restrict__ xdir, double lambda,
-    const double* __restrict__ Fp0inv, const double* __restrict__ tauc_g, const double* __restrict__ Swarm,
+    const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g, const double* __restrict__ Swarm,
     double* __restrict__ Sout, double* __restrict__ dgout, double* __restrict__ Pout,
     int32_t* __restrict__ counters, double dt, Consts c) {
   const unsigned full = 0xffffffffu;
@@ -462,7 +1018,7 @@ __global__ void __launch_bounds__(128) k_local(
     const size_t v = (size_t)chunk * 32 + lane;
     int iters = 0, failed = 0, evals = 0;
     if (v < nvox)
-      local_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tauc_g, Swarm, Sout, dgout, Pout, dt, c,
+      local_voxel_fp64(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c,
                   iters, evals, failed);
     mx = max(mx, iters);
     nf += failed;
@@ -484,31 +1040,22 @@ __global__ void __launch_bounds__(128) k_local(
   }
 }
 
-// The consistent tangent at the converged S: the same work for every voxel
-// (no data-dependent iterations), so whole warps stay converged.
-//
 // For a direction dF~ = a b^T of the crystal-frame deformation gradient,
 // dE = sym(u w^T) with u = Fe^T a, w = Fp^-T b, and
 //   dP~ = F~ dQ + a (Q b)^T,  dQ = Fp^-1 dS Fp^-T - (dFpi W + (dFpi W)^T),
 // where dS = J^-1 C : dE, dM = sum_a dgp^a tau^a(dS) s^a (x) m^a,
-// dFpi = Fp^-1 dM M^-1, W = S Fp^-T and Q = Fp^-1 S Fp^-T.  Everything but
-// a (Q b)^T is linear in the six components of dE, so F~ dQ is formed once
-// for each unit dE (the columns of H, 9 x 6, in shared memory) and each of
-// the nine directions costs H dE plus the rank-one term and the rotation:
-// six solves through the chain instead of nine.
-constexpr int TAN_THREADS = 64;
-
-__global__ void __launch_bounds__(TAN_THREADS) k_tangent(
+// dFpi = Fp^-1 dM M^-1, W = S Fp^-T and Q = Fp^-1 S Fp^-T.
+__global__ void __launch_bounds__(TAN_THREADS) k_tangent_fp64(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
     const double* __restrict__ Fin, const double* __restrict__ xdir, double lambda,
-    const double* __restrict__ Fp0inv, const double* __restrict__ tauc_g, const double* __restrict__ Sin,
+    const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g, const double* __restrict__ Sin,
     double* __restrict__ Kout, double dt, Consts c, int k32) {
   __shared__ double Hs[54 * TAN_THREADS];     // H[9 m + ij] of this thread at Hs[(9 m + ij) T + tid]
   double* H = Hs + threadIdx.x;
   const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (v < nvox) {
     VoxelIn in;
-    load_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tauc_g, in);
+    load_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, in);
     const double* R = in.R;
     const double* Ft = in.Ft;
     const double* Fpi0 = in.Fpi0;
@@ -692,7 +1239,7 @@ __global__ void __launch_bounds__(128) k_hard_jvp(
 // into mean_out[9].
 __global__ void __launch_bounds__(128) k_local_jvp(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
-    const double* __restrict__ Fin, const double* __restrict__ Fp0inv, const double* __restrict__ tauc_g,
+    const double* __restrict__ Fin, const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
     const double* __restrict__ Sin, const double* __restrict__ dFin, const double* __restrict__ dFp0_g,
     const double* __restrict__ dtauc_g, const double* __restrict__ ell_g, const double* __restrict__ dell_g,
     const double* __restrict__ rho_g, const double* __restrict__ drho_g, double* __restrict__ dP_out,
@@ -704,7 +1251,7 @@ __global__ void __launch_bounds__(128) k_local_jvp(
   for (int k = 0; k < 9; ++k) acc[k] = 0.0;
   for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvox; v += (size_t)gridDim.x * blockDim.x) {
     VoxelIn in;
-    load_voxel(nvox, v, grain, grainR, Fin, nullptr, 0.0, Fp0inv, tauc_g, in);
+    load_voxel(nvox, v, grain, grainR, Fin, nullptr, 0.0, Fp0inv, tinv_g, in);
     const double* R = in.R;
     double S[6];
 #pragma unroll
@@ -839,7 +1386,7 @@ cudaError_t launch_hardening(const rve_s* h, cudaStream_t s) {
   {
     ProfScope ps_(h, RVE_K_HARDENING, s);
     k_hardening<<<blocks, 128, 0, s>>>(h->nvox, h->grain, h->grainR, h->qhat, h->Apinv, h->screw_of, h->nye,
-                                     h->rho_ssd, h->Fp, h->rho18, h->rho_gnd, h->tauc, h->ell, h->Fp0inv, h->cst);
+                                     h->rho_ssd, h->Fp, h->rho18, h->rho_gnd, h->tauc, h->tinv, h->ell, h->Fp0inv, h->cst);
   }
   return cudaGetLastError();
 }
@@ -848,16 +1395,16 @@ cudaError_t launch_local(const rve_s* h, double dt, double lambda, int out_buf, 
   // persistent: as many blocks as are resident at once (no more than the chunks need)
   static const int per_sm = [] {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local, 128, 0) != cudaSuccess || n < 1) n = 1;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local, LOCAL_THREADS, 0) != cudaSuccess || n < 1) n = 1;
     return n;
   }();
-  const long need = (long)((h->nvox + 127) / 128);
+  const long need = (long)((h->nvox + LOCAL_THREADS - 1) / LOCAL_THREADS);
   const unsigned blocks = (unsigned)std::min<long>(need, (long)per_sm * h->num_sms);
   const double* warm = warm_buf < 0 ? h->S_c : h->S[warm_buf];
   if (cudaError_t e = cudaMemsetAsync(h->dcount + 6, 0, sizeof(int32_t), s)) return e;
   {
     ProfScope ps_(h, RVE_K_CONSTITUTIVE, s);
-    k_local<<<blocks, 128, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv, h->tauc, warm,
+    k_local<<<blocks, LOCAL_THREADS, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv, h->tinv, warm,
                                    h->S[out_buf], h->dgam[out_buf], h->P[out_buf], h->dcount, dt, h->cst);
   }
   return cudaGetLastError();
@@ -868,15 +1415,37 @@ cudaError_t launch_tangent(const rve_s* h, double dt, double lambda, int buf, cu
   {
     ProfScope ps_(h, RVE_K_TANGENT_BUILD, s);
     k_tangent<<<blocks, TAN_THREADS, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv,
-                                             h->tauc, h->S[buf], h->K[buf], dt, h->cst, h->opt.precision == 1);
+                                             h->tinv, h->S[buf], h->K[buf], dt, h->cst, h->opt.precision == 1);
   }
   return cudaGetLastError();
 }
 
 cudaError_t launch_constitutive(const rve_s* h, double dt, double lambda, int out_buf, int warm_buf,
                                 cudaStream_t s) {
-  if (cudaError_t e = launch_local(h, dt, lambda, out_buf, warm_buf, s)) return e;
-  return launch_tangent(h, dt, lambda, out_buf, s);
+  if (h->opt.precision == 0) {
+    if (cudaError_t e = launch_local(h, dt, lambda, out_buf, warm_buf, s)) return e;
+    return launch_tangent(h, dt, lambda, out_buf, s);
+  }
+  const double* warm = warm_buf < 0 ? h->S_c : h->S[warm_buf];
+  if (cudaError_t e = cudaMemsetAsync(h->dcount + 6, 0, sizeof(int32_t), s)) return e;
+  {
+    static const int per_sm = [] {
+      int n = 0;
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local_fp64, 128, 0) != cudaSuccess || n < 1) n = 1;
+      return n;
+    }();
+    const unsigned blocks = (unsigned)std::min<long>((long)((h->nvox + 127) / 128), (long)per_sm * h->num_sms);
+    ProfScope ps_(h, RVE_K_CONSTITUTIVE, s);
+    k_local_fp64<<<blocks, 128, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv, h->tinv, warm,
+                                        h->S[out_buf], h->dgam[out_buf], h->P[out_buf], h->dcount, dt, h->cst);
+  }
+  {
+    const unsigned blocks = (unsigned)((h->nvox + TAN_THREADS - 1) / TAN_THREADS);
+    ProfScope ps_(h, RVE_K_TANGENT_BUILD, s);
+    k_tangent_fp64<<<blocks, TAN_THREADS, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv, h->tinv,
+                                                  h->S[out_buf], h->K[out_buf], dt, h->cst, 1);
+  }
+  return cudaGetLastError();
 }
 
 constexpr int JVP_BLOCKS = 4 * 152;
@@ -897,7 +1466,7 @@ cudaError_t launch_local_jvp(const rve_s* h, double dt, int mode, const double* 
                              double* dFp_out, double* drho_out, double* mean_out, Theta dth, cudaStream_t s) {
   {
     ProfScope ps_(h, RVE_K_CONSTITUTIVE, s);
-    k_local_jvp<<<JVP_BLOCKS, 128, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->Fp0inv, h->tauc, h->S[h->cur], dF,
+    k_local_jvp<<<JVP_BLOCKS, 128, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->Fp0inv, h->tinv, h->S[h->cur], dF,
                                            dFp0, dtauc, h->ell, dell, h->rho_ssd, drho, dP, dFp_out, drho_out,
                                            h->partial, (unsigned int*)(h->dcount + 4), mean_out, dt, h->cst, dth,
                                            mode);

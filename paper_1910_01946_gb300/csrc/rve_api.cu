@@ -87,6 +87,7 @@ void carve(rve_s* h, Carver& c) {
   h->rho18 = c.take<double>(18 * nv);
   h->rho_gnd = c.take<double>(12 * nv);
   h->tauc = c.take<double>(12 * nv);
+  h->tinv = c.take<double>(12 * nv);
   h->ell = c.take<double>(12 * nv);
   h->Fp0inv = c.take<double>(9 * nv);
   h->F = c.take<double>(9 * nv);
@@ -113,6 +114,7 @@ void carve(rve_s* h, Carver& c) {
   h->ex.u = c.take<int>(3 * (size_t)(h->n1 / 2) * h->n2);
   if (h->opt.precision == 1) {
     for (int a = 0; a < 3; ++a) h->ax[a].tw32 = c.take<float2>(ns[a]);
+    for (int a = 0; a < 3; ++a) h->ax[a].tw64 = c.take<double2>(ns[a]);
     h->lapw32 = c.take<float>(h->nspec);
     h->spec32 = c.take<float2>(3 * h->nspec);
     h->x32 = c.take<float>(9 * nv);
@@ -121,7 +123,7 @@ void carve(rve_s* h, Carver& c) {
     h->t32 = c.take<float>(9 * nv);
     h->du32 = c.take<float>(6 * nv);
   } else {
-    for (int a = 0; a < 3; ++a) h->ax[a].tw32 = nullptr;
+    for (int a = 0; a < 3; ++a) { h->ax[a].tw32 = nullptr; h->ax[a].tw64 = nullptr; }
     h->spec32 = nullptr;
     h->lapw32 = nullptr;
     h->x32 = h->r32 = h->p32 = h->t32 = h->du32 = nullptr;
@@ -830,6 +832,11 @@ rve_status rve_create(const int32_t* grain_id, int n0, int n1, int n2, const dou
   Consts& c = h->cst;
   c.C11 = mat->C11; c.C12 = mat->C12; c.C44 = mat->C44; c.mu = h->mu; c.b = mat->b;
   c.tau0 = mat->tau0; c.alpha = mat->alpha; c.gdot0 = mat->gdot0; c.n = mat->n; c.K = mat->K; c.yc = mat->yc;
+  const double det = (mat->C11 - mat->C12) * (mat->C11 + 2.0 * mat->C12);
+  const bool compliant = det > 0;
+  c.s11 = compliant ? (mat->C11 + mat->C12) / det : 0.0;
+  c.s12 = compliant ? -mat->C12 / det : 0.0;
+  c.s44 = compliant ? 0.5 / mat->C44 : 0.0;
   c.n_int = (mat->n == std::floor(mat->n) && mat->n >= 1 && mat->n <= 64) ? (int)mat->n : 0;
   c.gnd_enabled = mat->gnd_enabled ? 1 : 0;
   c.local_tol_abs = opt->local_tol * h->mu;
@@ -901,8 +908,18 @@ rve_status rve_create(const int32_t* grain_id, int n0, int n1, int n2, const dou
             bad(cudaMemcpyAsync((void*)h->ax[a].xi, xi[a].data(), ns[a] * sizeof(double), cudaMemcpyHostToDevice, s));
     if (!fail_ && h->opt.precision == 1) {
       std::vector<float2> t32(ns[a]);
+      std::vector<double2> t64(ns[a]);
+      for (int t = 0; t < ns[a]; ++t) {
+        const double ang = 2.0 * PI * (double)t / ns[a];
+        t64[t] = make_double2(std::cos(ang), -std::sin(ang));
+        if (4 * t == ns[a]) t64[t] = make_double2(0.0, -1.0);
+        if (4 * t == 3 * ns[a]) t64[t] = make_double2(0.0, 1.0);
+        if (2 * t == ns[a]) t64[t] = make_double2(-1.0, 0.0);
+        if (t == 0) t64[t] = make_double2(1.0, 0.0);
+      }
       for (int t = 0; t < ns[a]; ++t) t32[t] = make_float2((float)std::cos(2.0 * PI * t / ns[a]), (float)-std::sin(2.0 * PI * t / ns[a]));
       fail_ = bad(cudaMemcpyAsync((void*)h->ax[a].tw32, t32.data(), ns[a] * sizeof(float2), cudaMemcpyHostToDevice, s)) ||
+              bad(cudaMemcpyAsync((void*)h->ax[a].tw64, t64.data(), ns[a] * sizeof(double2), cudaMemcpyHostToDevice, s)) ||
               bad(cudaStreamSynchronize(s));
     }
   }
@@ -1287,7 +1304,12 @@ rve_status rve_eval_nye(rve_t* h, int scheme) {
 
 rve_status rve_eval_constitutive(rve_t* h, double dt, int32_t* local_max_iters, int32_t* local_failures) {
   if (!h || !(dt > 0)) return RVE_EINVAL;
-  RVE_TRY(run_hardening(h));
+  if (h->opt.precision == 1) {                  // see curl_fp64.cu
+    RVE_CUDA(h, launch_curl_fp64(h, h->Fp, h->nye, h->stream));
+    RVE_CUDA(h, launch_hardening(h, h->stream));
+  } else {
+    RVE_TRY(run_hardening(h));
+  }
   RVE_CUDA(h, cudaMemcpyAsync(h->F, h->F_c, 9 * h->nvox * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
   RVE_CUDA(h, cudaMemsetAsync(h->dcount, 0, 2 * sizeof(int32_t), h->stream));
   RVE_CUDA(h, launch_constitutive(h, dt, 0.0, h->cur, -1, h->stream));

@@ -49,6 +49,7 @@ struct AxisTables {
   const double* s2;     // sin^2(xi_k / 2)
   const double* c2;     // cos^2(xi_k / 2)
   const float2* tw32;   // the twiddles in float (mixed precision)
+  const double2* tw64;  // and in double (mixed precision: launch_curl_fp64)
   const double* xi;     // xi_k = 2 pi k' / n (signed k'), 0 at Nyquist: the standard frequency
 };
 
@@ -60,6 +61,7 @@ struct Theta {
 
 struct Consts {        // material constants read by the hardening and constitutive kernels
   double C11, C12, C44, mu, b, tau0, alpha, gdot0, n, K, yc;
+  double s11, s12, s44; // cubic compliance: E = s11 S + s12 (the other two), shear E = s44 S
   int n_int;            // n if it is a positive integer <= 64, else 0 (use pow)
   int gnd_enabled;
   double local_tol_abs, floor_abs, dgam_max;
@@ -122,7 +124,7 @@ struct rve_s {
   double* Apinv;        // 162: A^+ (18 x 9, crystal frame, divided by b)
   int32_t* screw_of;    // 12
   double *F_c, *Fp, *S_c, *rho_ssd, *dF_last, *P_c;  // committed
-  double *nye, *rho18, *rho_gnd, *tauc, *ell, *Fp0inv;  // per increment
+  double *nye, *rho18, *rho_gnd, *tauc, *tinv, *ell, *Fp0inv;  // per increment (tinv = 1 / tauc)
   double* F;            // Newton iterate
   double *P[2], *K[2], *S[2], *dgam[2];             // evaluation double buffer
   int cur;
@@ -209,6 +211,9 @@ cudaError_t launch_fft9(const rve_s* h, const double* in, double* out, const Spe
 cudaError_t launch_laplace_solve(const rve_s* h, const double* d, double* u, bool fixed, cudaStream_t s,
                                  const double* done);
 cudaError_t launch_laplace_solve32(const rve_s* h, const float* d, float* u, cudaStream_t s, const double* done);
+// ---- curl_fp64.cu: the Nye curl in FP64 floating point (mixed-precision handles) ----
+cudaError_t launch_curl_fp64(const rve_s* h, const double* in, double* out, cudaStream_t s);
+
 // radix passes 8, 6, 4, 3, 2, the largest first
 void make_plan(int n, FFTPlan* p);
 // fills h->lapw and h->lapw32 (once, at create)
@@ -246,7 +251,7 @@ cudaError_t launch_hard_jvp(const rve_s* h, const double* dnye, const double* dr
 cudaError_t launch_local_jvp(const rve_s* h, double dt, int mode, const double* dF, const double* dFp0,
                              const double* dtauc, const double* dell, const double* drho, double* dP,
                              double* dFp_out, double* drho_out, double* mean_out, Theta dth, cudaStream_t s);
-// both
+// both, as rve_eval_constitutive runs them (mixed precision: FP64 directions, see constitutive.cu)
 cudaError_t launch_constitutive(const rve_s* h, double dt, double lambda, int out_buf, int warm_buf,
                                 cudaStream_t s);
 

@@ -1,0 +1,90 @@
+"""The local update (FP32 directions, FP64 residual) and the consistent tangent
+in the sample frame against the oracle, at the edges of their dispatch: voxel
+counts that fill no warp, one and two voxels past a block, flow-rule exponents
+with and without the integer fast path, a stiffness without a positive definite
+compliance; and the mixed-precision entry point (FP64 directions, FP32 tangent)
+against the FP64 one."""
+import numpy as np
+import pytest
+
+import rvegen
+from oracle import solver
+
+pytestmark = pytest.mark.gpu
+
+CASES = {
+    "one block": (dict(), (4, 4, 4)),
+    "two voxels": (dict(), (1, 2, 2)),
+    "past a block": (dict(), (9, 6, 12)),
+    "integer exponent": (dict(n=7.0), (3, 4, 6)),
+    "real exponent": (dict(n=12.5), (3, 4, 6)),
+    "linear flow": (dict(n=1.0), (2, 4, 4)),
+    "soft bulk": (dict(C11=100e3, C12=-55e3, C44=60e3, mu=45e3), (2, 4, 6)),
+}
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1910_01946_gb300 import _build
+    _build.build()
+    import paper_1910_01946_gb300 as p
+    p.load_library()
+    return p
+
+
+def relerr(a, b):
+    return float(np.abs(a - b).max() / max(np.abs(b).max(), 1e-300))
+
+
+def state(case, seed=23):
+    over, shape = CASES[case]
+    n2, n1, n0 = shape
+    gid, _ = rvegen.voronoi_grain_map(0, 3, seed, shape=(n0, n1, n2))
+    mat = rvegen.material("Cu", **over)
+    rng = np.random.default_rng(seed)
+    F = np.eye(3) + np.diag([2e-3, -6e-4, -6e-4]) + 5e-4 * rng.standard_normal(shape + (3, 3))
+    Fp = np.eye(3) + 5e-4 * rng.standard_normal(shape + (3, 3))
+    return gid, rvegen.random_quaternions(3, seed + 1), mat, F, Fp
+
+
+def evaluate(pkg, args, **options):
+    gid, quat, mat, F, Fp = args
+    g = pkg.RVE(gid, quat, mat, 2e-5, **options)
+    g.set_field("F", F.reshape(gid.shape + (9,)))
+    g.set_field("FP", Fp.reshape(gid.shape + (9,)))
+    _, failed = g.eval_constitutive(1.0)
+    assert failed == 0
+    out = {k: g.field(k).reshape(gid.size, -1) for k in ("P_EVAL", "S_EVAL", "DGAM", "TANGENT")}
+    g.close()
+    return out
+
+
+@pytest.mark.parametrize("case", sorted(CASES))
+def test_local_update_and_tangent_match_oracle(pkg, case):
+    args = state(case)
+    gid, quat, mat, F, Fp = args
+    out = evaluate(pkg, args)
+    o = solver.RVE(gid, quat, mat, 2e-5)
+    o.Fp = Fp.reshape(-1, 3, 3).copy()
+    tauc, _ = o.hardening()
+    P, K, S, M, dg, iters, failed = o.constitutive(F.reshape(-1, 3, 3), tauc, np.zeros_like(o.S), 1.0)
+    assert failed == 0
+    assert relerr(out["P_EVAL"], P.reshape(-1, 9)) < 1e-11
+    assert relerr(out["DGAM"], dg.reshape(-1, 12)) < 1e-9
+    assert relerr(out["TANGENT"], K.reshape(-1, 81)) < 1e-10
+
+
+@pytest.mark.parametrize("case", ["one block", "past a block", "real exponent"])
+def test_mixed_evaluation_is_the_fp64_one_with_a_rounded_tangent(pkg, case):
+    """FP32 rounding of the tangent: half a unit of the last place, 2^-24."""
+    args = state(case)
+    a, b = evaluate(pkg, args), evaluate(pkg, args, precision=1)
+    for k in ("P_EVAL", "S_EVAL"):
+        assert relerr(b[k], a[k]) < 1e-11
+    assert relerr(b["DGAM"], a["DGAM"]) < 1e-9
+    K = b["TANGENT"]
+    assert np.array_equal(K, K.astype(np.float32).astype(np.float64))
+    assert np.all(np.abs(K - a["TANGENT"]) <= 2.0 ** -24 * np.abs(a["TANGENT"]) + 1e-10 * np.abs(a["TANGENT"]).max())
