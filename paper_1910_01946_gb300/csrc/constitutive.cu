@@ -25,6 +25,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "fix64.cuh"
 #include "rve_internal.h"
 
 namespace {
@@ -779,11 +780,13 @@ __global__ void __launch_bounds__(LOCAL_THREADS, LOCAL_BLOCKS) k_local(
 // strain and per direction: 2.39 -> 1.43 ms at 64^3.
 constexpr int TAN_THREADS = 64;
 
+constexpr int TAN_BITS = 60;        // of an integer entry of K (high words below 2^28: see fixed_row in vec.cu)
+
 __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
     const double* __restrict__ Fin, const double* __restrict__ xdir, double lambda,
     const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g, const double* __restrict__ Sin,
-    double* __restrict__ Kout, double dt, Consts c, int k32) {
+    double* __restrict__ Kout, int* __restrict__ kex, double dt, Consts c, int k32) {
   __shared__ double Hs[54 * TAN_THREADS], Ts[36 * TAN_THREADS];   // [slot][thread]
   double* H = Hs + threadIdx.x;
   double* T = Ts + threadIdx.x;
@@ -859,6 +862,14 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
     }
     lu6(J, piv);
   }
+  // scale of the voxel's tangent: |K| <= |W S W^T| + 6 |H| |U| |W| in largest entries
+  unsigned mU = 0u, mW = 0u, mQ = 0u, mH = 0u;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    mU = max(mU, fix64::mag(U[k]));
+    mW = max(mW, fix64::mag(W[k]));
+    mQ = max(mQ, fix64::mag(Qs[k]));
+  }
   // H for the six unit strain increments (tensor components E11, E22, E33, E23, E13, E12, as `cubic` takes them)
 #pragma unroll 1
   for (int m = 0; m < 6; ++m) {
@@ -875,8 +886,15 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
     mat3_mul(U, Bf, Z);
     mat3_mult(Z, W, P);
 #pragma unroll
-    for (int ij = 0; ij < 9; ++ij) H[(9 * m + ij) * TAN_THREADS] = P[ij];
+    for (int ij = 0; ij < 9; ++ij) {
+      H[(9 * m + ij) * TAN_THREADS] = P[ij];
+      mH = max(mH, fix64::mag(P[ij]));
+    }
   }
+  const bool finite = max(max(mU, mW), max(mQ, mH)) < 0x7ff00000u;
+  const int ek = min(max(max((int)(mH >> 20) + (int)(mU >> 20) + (int)(mW >> 20) - 2046 + 5, (int)(mQ >> 20)) + 1,
+                         fix64::EXP_MIN), 0x7fe);
+  if (!k32) kex[v] = finite ? fix64::out_base(ek, TAN_BITS) : fix64::EXP_BAD;
   // T is done with: its place takes U, W and W S W^T for the rolled loop over directions
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -901,10 +919,13 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
       double t = ij / 3 == kk ? q[ij % 3] : 0.0;
 #pragma unroll
       for (int m = 0; m < 6; ++m) t = fma(H[(9 * m + ij) * TAN_THREADS], dE[m], t);
-      if (k32)   // mixed precision: the tangent only drives the FP32 conjugate gradients
-        reinterpret_cast<float*>(Kout)[(size_t)(9 * ij + kl) * nvox + v] = (float)t;
-      else
-        Kout[(size_t)(9 * ij + kl) * nvox + v] = t;
+      const size_t at = (size_t)(9 * ij + kl) * nvox + v;
+      if (k32) {   // mixed precision: the tangent only drives the FP32 conjugate gradients
+        reinterpret_cast<float*>(Kout)[at] = (float)t;
+      } else {     // integers for the FP64 apply: signed low word, high word
+        const fix64::Sp k = fix64::split(fix64::to_fix(t, ek + 63 - TAN_BITS));
+        reinterpret_cast<int2*>(Kout)[at] = make_int2(k.l, k.h);
+      }
     }
   }
 }
@@ -1415,7 +1436,8 @@ cudaError_t launch_tangent(const rve_s* h, double dt, double lambda, int buf, cu
   {
     ProfScope ps_(h, RVE_K_TANGENT_BUILD, s);
     k_tangent<<<blocks, TAN_THREADS, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv,
-                                             h->tinv, h->S[buf], h->K[buf], dt, h->cst, h->opt.precision == 1);
+                                             h->tinv, h->S[buf], h->K[buf], h->kex[buf], dt, h->cst,
+                                             h->opt.precision == 1);
   }
   return cudaGetLastError();
 }

@@ -94,6 +94,7 @@ void carve(rve_s* h, Carver& c) {
   for (int b = 0; b < 2; ++b) {
     h->P[b] = c.take<double>(9 * nv);
     h->K[b] = c.take<double>(81 * nv);
+    h->kex[b] = h->opt.precision == 0 ? c.take<int>(nv) : nullptr;
     h->S[b] = c.take<double>(6 * nv);
     h->dgam[b] = c.take<double>(12 * nv);
   }
@@ -1232,13 +1233,15 @@ rve_status rve_get_fields(rve_t* h, uint32_t which, void* dst, size_t bytes, int
     case RVE_FIELD_DGAM: src = h->dgam[h->cur]; break;
     case RVE_FIELD_TANGENT:
       RVE_TRY(build_stale_tangent(h));
-      if (h->opt.precision == 1) {   // stored as float: widen into the other evaluation buffer
-        double* tmp = h->K[1 - h->cur];
-        RVE_CUDA(h, launch_widen(h, reinterpret_cast<const float*>(h->K[h->cur]), tmp, 81 * h->nvox, h->stream));
-        src = tmp;
-      } else {
-        src = h->K[h->cur];
+      // stored as floats or as integers: as doubles into the caller's device memory, or by way of the
+      // other evaluation buffer
+      if (dst_is_device) {
+        RVE_CUDA(h, launch_tangent_values(h, static_cast<double*>(dst), h->stream));
+        RVE_CUDA(h, cudaStreamSynchronize(h->stream));
+        return RVE_OK;
       }
+      RVE_CUDA(h, launch_tangent_values(h, h->K[1 - h->cur], h->stream));
+      src = h->K[1 - h->cur];
       break;
     case RVE_FIELD_GRAIN: src = h->grain; break;
     case RVE_FIELD_P_EVAL: src = h->P[h->cur]; break;

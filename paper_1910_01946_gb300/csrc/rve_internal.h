@@ -126,7 +126,9 @@ struct rve_s {
   double *F_c, *Fp, *S_c, *rho_ssd, *dF_last, *P_c;  // committed
   double *nye, *rho18, *rho_gnd, *tauc, *tinv, *ell, *Fp0inv;  // per increment (tinv = 1 / tauc)
   double* F;            // Newton iterate
-  double *P[2], *K[2], *S[2], *dgam[2];             // evaluation double buffer
+  double *P[2], *K[2], *S[2], *dgam[2];             // evaluation double buffer (K: floats in mixed
+                                                    // precision, else integers on the scales kex, see k_tangent)
+  int* kex[2];
   int cur;
   bool K_stale = false;   // the converged evaluation's tangent is not built yet (built on request)
   CgGraph graphs[RVE_CG_GRAPHS];
@@ -264,6 +266,8 @@ cudaError_t vec_init();
 cudaError_t launch_cg_init32(const rve_s* h, double eta, cudaStream_t s);
 cudaError_t launch_widen_x(const rve_s* h, cudaStream_t s);
 cudaError_t launch_widen(const rve_s* h, const float* a, double* b, size_t n, cudaStream_t s);
+// the tangent K[cur] as doubles (81 * nvox)
+cudaError_t launch_tangent_values(const rve_s* h, double* dst, cudaStream_t s);
 // x_c -= mean(x_c) for the components whose bit is set (uses DS_XMEAN)
 cudaError_t launch_zero_means(const rve_s* h, double* x, unsigned bits, cudaStream_t s);
 cudaError_t launch_kmul(const rve_s* h, const double* in, double* out, cudaStream_t s);

@@ -7,6 +7,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "fix64.cuh"
 #include "rve_internal.h"
 
 namespace {
@@ -44,49 +45,6 @@ __device__ __forceinline__ double last_block_sum(const double* partial, unsigned
   const double s = block_sum(acc, sh);
   if (threadIdx.x == 0) *ticket = 0u;
   return s;
-}
-
-// p = r (first) or r + beta p; t = K : p; block sums of p . t (added up, and
-// alpha = rr / p . t formed, by launch_laplace_solve: see Fold).
-// Returns at once when the CG loop has converged (done != 0).
-__global__ void __launch_bounds__(RVE_RED_THREADS, 3) k_tangent_apply(size_t nvox, const double* __restrict__ K,
-                                                                      const double* __restrict__ r, double* __restrict__ p,
-                                                                      double* __restrict__ t, double* __restrict__ ds,
-                                                                      double* __restrict__ partial) {
-  __shared__ double sh[320];
-  if (ds[DS_DONE] != 0.0) return;
-  // the first iteration of a solve (the counter is reset by the CG init and
-  // bumped by each completed iteration): every launch of the loop has the
-  // same arguments, so chunks of iterations can be replayed as a CUDA graph
-  const bool first = ds[DS_ITERS] == 0.0;
-  const double beta = first ? 0.0 : ds[DS_BETA];
-  double acc = 0.0;
-  for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvox; v += (size_t)gridDim.x * blockDim.x) {
-    double pv[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const double rv = r[k * nvox + v];
-      pv[k] = first ? rv : fma(beta, p[k * nvox + v], rv);
-      p[k * nvox + v] = pv[k];
-    }
-    // three rows of K (27 streamed loads in flight) per stage
-#pragma unroll
-    for (int ib = 0; ib < 3; ++ib) {
-      double kk[27];
-#pragma unroll
-      for (int e = 0; e < 27; ++e) kk[e] = __ldcs(K + (size_t)(27 * ib + e) * nvox + v);
-#pragma unroll
-      for (int ii = 0; ii < 3; ++ii) {
-        double s = 0.0;
-#pragma unroll
-        for (int j = 0; j < 9; ++j) s = fma(kk[9 * ii + j], pv[j], s);
-        t[(3 * ib + ii) * nvox + v] = s;
-        acc = fma(pv[3 * ib + ii], s, acc);
-      }
-    }
-  }
-  const double s = block_sum(acc, sh);
-  if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
 // Mixed precision: the same CG step with FP32 tangent and vectors (warp sums
@@ -259,6 +217,94 @@ __global__ void __launch_bounds__(TA_TV, 1) k_tangent_apply32_tma(size_t nvox, c
     if (pending[1]) mbar_wait(&bar[1], phase[1]);
   }
   const double s = blk_sum_v<float>(acc, sh);
+  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+}
+
+// ---- FP64 tangent apply ----
+// The 81 FMAs of K : p per voxel take 41 us at 64^3 on the FP64 pipe (2 lanes per clock and SM), the
+// bytes (648 of K of 936 in all) 31, so the products are formed in fixed point on the integer pipes:
+// k_tangent stores K as integers on one scale per voxel (kex), each split into a high word and a
+// signed low word, p becomes integers on the scale of its largest component, and three 32 x 32
+// multiply-adds per entry sum the high and the mixed products exactly (the low words' product, below
+// 2^-58 of the row's largest, is dropped).  K keeps 54 or more bits of the voxel's
+// largest entry, p 56 of its largest component, against the 2^-53 of each FP64 FMA.  FP64 keeps p = r + beta p and p . t (18 FMAs).
+constexpr int TAF_P_BITS = 56, TAF_SHIFT = 7;
+
+// p of one voxel as split integers; returns their scale
+__device__ __forceinline__ int fixed_vector(const double* pv, fix64::Sp* pf) {
+  unsigned pm = 0u;
+#pragma unroll
+  for (int c = 0; c < 9; ++c) pm = max(pm, fix64::mag(pv[c]));
+  const int e = fix64::tile_exp(pm);
+#pragma unroll
+  for (int c = 0; c < 9; ++c) pf[c] = fix64::split(fix64::to_fix(pv[c], e + 63 - TAF_P_BITS));
+  return fix64::out_base(e, TAF_P_BITS);
+}
+// one row of K (entries `stride` apart, on the scale ek) times p (on the scale ep)
+__device__ __forceinline__ double fixed_row(const int2* K, size_t stride, const fix64::Sp* pf, int ek, int ep) {
+  using namespace fix64;
+  i64 hi = 0, mid = 0;
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    const int2 k = K[j * stride];                          // low (signed), high
+    hi += wide(k.y, pf[j].h);
+    mid += wide(k.y, pf[j].l) + wide(k.x, pf[j].h);
+  }
+  const int eb = max(ek, ep) >= EXP_BAD / 2 ? EXP_BAD : ek + ep - 1022 - TAF_SHIFT;
+  return eb < 70 ? 0.0 : from_fix((hi << TAF_SHIFT) + (mid >> (32 - TAF_SHIFT)), eb);
+}
+
+// p = r (first) or r + beta p; t = K : p; block sums of p . t (added up, and
+// alpha = rr / p . t formed, by launch_laplace_solve: see Fold).
+// Returns at once when the CG loop has converged (done != 0).
+//
+// 55.3 -> 46.0 us at 64^3 (4.9 TB/s).  Plain loads, three rows of K in flight per thread: staged through
+// shared memory (bulk copies, two or four threads per voxel) it took 53, with the next voxel's rows
+// prefetched 49, at four and three blocks per SM 47 and 50 us.
+constexpr int TAF_THREADS = 128, TAF_BLOCKS = 5;  // per SM: 102 registers, 27 rows of K in flight per thread
+__global__ void __launch_bounds__(TAF_THREADS, TAF_BLOCKS) k_tangent_apply(size_t nvox, const int2* __restrict__ K,
+                                                                           const int* __restrict__ kex,
+                                                                           const double* __restrict__ r, double* __restrict__ p,
+                                                                           double* __restrict__ t, double* __restrict__ ds,
+                                                                           double* __restrict__ partial) {
+  __shared__ double sh[32];
+  if (ds[DS_DONE] != 0.0) return;
+  // the first iteration of a solve (the counter is reset by the CG init and
+  // bumped by each completed iteration): every launch of the loop has the
+  // same arguments, so chunks of iterations can be replayed as a CUDA graph
+  const bool first = ds[DS_ITERS] == 0.0;
+  const double beta = first ? 0.0 : ds[DS_BETA];
+  double acc = 0.0;
+  for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvox; v += (size_t)gridDim.x * blockDim.x) {
+    int2 kk[27];
+#pragma unroll
+    for (int e = 0; e < 27; ++e) kk[e] = __ldcs(K + (size_t)e * nvox + v);
+    const int ek = __ldcs(kex + v);
+    double pv[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const double rv = r[k * nvox + v];
+      pv[k] = first ? rv : fma(beta, p[k * nvox + v], rv);
+      p[k * nvox + v] = pv[k];
+    }
+    fix64::Sp pf[9];
+    const int ep = fixed_vector(pv, pf);
+#pragma unroll
+    for (int ib = 0; ib < 3; ++ib) {
+#pragma unroll
+      for (int ii = 0; ii < 3; ++ii) {
+        const int i = 3 * ib + ii;
+        const double s = fixed_row(kk + 9 * ii, 1, pf, ek, ep);
+        t[i * nvox + v] = s;
+        acc = fma(pv[i], s, acc);
+        if (ib < 2) {
+#pragma unroll
+          for (int e = 0; e < 9; ++e) kk[9 * ii + e] = __ldcs(K + (size_t)(27 * (ib + 1) + 9 * ii + e) * nvox + v);
+        }
+      }
+    }
+  }
+  const double s = block_sum(acc, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
@@ -471,13 +517,11 @@ unsigned grid_for(size_t n, int threads) {
 }  // namespace
 
 cudaError_t launch_tangent_apply(const rve_s* h, cudaStream_t s) {
-  // one wave of resident blocks (three per SM): each thread covers more
-  // voxels, so the block reduction of p . t is spread over more of them, and
-  // no partial last wave trails
-  const int blocks = std::min(RVE_RED_BLOCKS, 3 * h->num_sms);
+  // one wave of resident blocks, no more than the voxels need
+  const int blocks = (int)std::min<size_t>((h->nvox + TAF_THREADS - 1) / TAF_THREADS, (size_t)TAF_BLOCKS * h->num_sms);
   {
     ProfScope ps_(h, RVE_K_TANGENT_APPLY, s);
-    k_tangent_apply<<<blocks, RVE_RED_THREADS, 0, s>>>(h->nvox, h->K[h->cur], h->r, h->p, h->t, h->dscal,
+    k_tangent_apply<<<blocks, TAF_THREADS, 0, s>>>(h->nvox, reinterpret_cast<const int2*>(h->K[h->cur]), h->kex[h->cur], h->r, h->p, h->t, h->dscal,
                                                        h->partial_pkp());
     h->fold.pkp_blocks = blocks;
   }
@@ -600,19 +644,41 @@ cudaError_t launch_widen(const rve_s* h, const float* a, double* b, size_t n, cu
 // ---- BiCGStab support (FP64): w = K : v; fused dot products; linear combinations
 namespace {
 
-template <typename KT>
-__global__ void __launch_bounds__(RVE_RED_THREADS, 2) k_kmul(size_t nvox, const KT* __restrict__ K,
+// FIXED: K as k_tangent stores it for the FP64 apply, else floats
+template <bool FIXED>
+__global__ void __launch_bounds__(RVE_RED_THREADS, 2) k_kmul(size_t nvox, const double* __restrict__ K, const int* __restrict__ kex,
                                                              const double* __restrict__ in, double* __restrict__ out) {
   for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvox; v += (size_t)gridDim.x * blockDim.x) {
     double pv[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) pv[k] = in[k * nvox + v];
+    if (FIXED) {
+      fix64::Sp pf[9];
+      const int ep = fixed_vector(pv, pf), ek = kex[v];
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      double s = 0.0;
+      for (int i = 0; i < 9; ++i)
+        out[i * nvox + v] = fixed_row(reinterpret_cast<const int2*>(K) + (size_t)9 * i * nvox + v, nvox, pf, ek, ep);
+    } else {
+      const float* Kf = reinterpret_cast<const float*>(K);
 #pragma unroll
-      for (int j = 0; j < 9; ++j) s = fma((double)__ldcs(K + (size_t)(9 * i + j) * nvox + v), pv[j], s);
-      out[i * nvox + v] = s;
+      for (int i = 0; i < 9; ++i) {
+        double s = 0.0;
+#pragma unroll
+        for (int j = 0; j < 9; ++j) s = fma((double)__ldcs(Kf + (size_t)(9 * i + j) * nvox + v), pv[j], s);
+        out[i * nvox + v] = s;
+      }
+    }
+  }
+}
+
+// the FP64 path's tangent as doubles
+__global__ void k_tangent_values(size_t nvox, const int2* __restrict__ K, const int* __restrict__ kex, double* __restrict__ out) {
+  for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvox; v += (size_t)gridDim.x * blockDim.x) {
+    const int ek = kex[v];
+#pragma unroll 9
+    for (int e = 0; e < 81; ++e) {
+      const int2 k = __ldcs(K + (size_t)e * nvox + v);
+      out[(size_t)e * nvox + v] = fix64::from_fix(((fix64::i64)k.y << 32) + k.x, ek);
     }
   }
 }
@@ -703,10 +769,19 @@ cudaError_t launch_kmul(const rve_s* h, const double* in, double* out, cudaStrea
   {
     ProfScope ps_(h, RVE_K_TANGENT_APPLY, s);
     if (h->opt.precision == 1)   // the tangent is stored as float in mixed precision
-      k_kmul<float><<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>(h->nvox, reinterpret_cast<const float*>(h->K[h->cur]),
-                                                               in, out);
+      k_kmul<false><<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>(h->nvox, h->K[h->cur], nullptr, in, out);
     else
-      k_kmul<double><<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>(h->nvox, h->K[h->cur], in, out);
+      k_kmul<true><<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>(h->nvox, h->K[h->cur], h->kex[h->cur], in, out);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_tangent_values(const rve_s* h, double* dst, cudaStream_t s) {
+  if (h->opt.precision == 1)   // stored as float
+    return launch_widen(h, reinterpret_cast<const float*>(h->K[h->cur]), dst, 81 * h->nvox, s);
+  {
+    ProfScope ps_(h, RVE_K_OTHER, s);
+    k_tangent_values<<<RVE_RED_BLOCKS, 128, 0, s>>>(h->nvox, reinterpret_cast<const int2*>(h->K[h->cur]), h->kex[h->cur], dst);
   }
   return cudaGetLastError();
 }
