@@ -385,6 +385,7 @@ __global__ void __launch_bounds__(256) k_fft_x_r2c(const typename In::real* __re
                                                    typename Out::pair* __restrict__ spec, int* __restrict__ exout,
                                                    int rows, int nkx, int rpb, PlanDev pl,
                                                    const TW<R>* __restrict__ tw, const double* __restrict__ done) {
+  chain_wait();
   __shared__ int red[MAX_WARPS];
   __shared__ int ebs[256];               // output scale of each row pair
   const int n0 = pl.n;
@@ -443,6 +444,7 @@ __global__ void __launch_bounds__(256) k_fft_x_c2r(const typename In::pair* __re
                                                    typename Out::real* __restrict__ out, int* __restrict__ exout,
                                                    int rows, int rows_per_plane, int nkx, int rpb, PlanDev pl,
                                                    const TW<R>* __restrict__ tw, const double* __restrict__ done) {
+  chain_wait();
   __shared__ int red[MAX_WARPS];
   const int n0 = pl.n;
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
@@ -523,6 +525,7 @@ template <int SIGN, typename R, class S>
 __global__ void __launch_bounds__(256) k_fft_y(typename S::pair* __restrict__ spec, const int* __restrict__ exin,
                                                int* __restrict__ exout, int ncol, int n2, int nkx, int cpb, PlanDev pl,
                                                const TW<R>* __restrict__ tw, const double* __restrict__ done, Fold fold) {
+  chain_wait();
   if (SIGN < 0 && fold.mean_blocks && blockIdx.x < FOLD_BLOCKS) {
     __shared__ double fsh[MAX_WARPS];
     if (!(done && *done != 0.0)) fold_block(fold, blockIdx.x, fsh);
@@ -684,6 +687,7 @@ __global__ void __launch_bounds__(256) k_fft_z_lap(typename S::pair* __restrict_
                                                    int* __restrict__ exout, int np, int nkx, int cpb, PlanDev pl,
                                                    const TW<R>* __restrict__ tw, const R* __restrict__ weight,
                                                    const double* __restrict__ done) {
+  chain_wait();
   __shared__ int red[2][MAX_WARPS * 32];
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
   C<R>* b1 = b0 + cpb * pl.n;
@@ -747,6 +751,7 @@ __global__ void __launch_bounds__(256) k_fft_z_lap(typename S::pair* __restrict_
 // through the forward transforms, applies the operator in FP64 and goes back.
 __global__ void __launch_bounds__(128) k_fft_z_op(double2* __restrict__ spec, int np, int nkx, int cpb, PlanDev pl,
                                                   const int4* __restrict__ tw, OpTables T, SpecParams sp) {
+  chain_wait();
   typedef double R;
   __shared__ int red[4][MAX_WARPS * 32];
   typedef Plain<double> S;
@@ -868,8 +873,8 @@ void launch_r2c(const rve_s* h, const typename In::real* in, cudaStream_t s, con
   const long rows = (long)nf * h->n2 * (h->n1 / 2);
   const int rpb = rows_per_block(pl, rows, h->fft_fill);
   ProfScope ps_(h, fft_category(h, RVE_K_FFT_X_R2C), s);
-  k_fft_x_r2c<R, In, S><<<(unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb, pl.n), s>>>(
-      in, h->ex.div, spect<S>(h), h->ex.x, (int)rows, h->nkx, rpb, pl, twt<R>(h, 0), done);
+  launch_chained(h, k_fft_x_r2c<R, In, S>, (unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb,
+                 pl.n), s, in, h->ex.div, spect<S>(h), h->ex.x, (int)rows, h->nkx, rpb, pl, twt<R>(h, 0), done);
 }
 
 template <int SIGN, typename R, class S>
@@ -879,8 +884,9 @@ void launch_y(const rve_s* h, cudaStream_t s, const double* done, int nf, const 
   const int c = cols_per_block(pl, cols, h->fft_fill_y, 256);
   ProfScope ps_(h, fft_category(h, SIGN < 0 ? RVE_K_FFT_Y : RVE_K_FFT_Y_INV), s);
   const unsigned blocks = (unsigned)((cols + c - 1) / c) + (fold.mean_blocks ? (unsigned)FOLD_BLOCKS : 0u);
-  k_fft_y<SIGN, R, S><<<blocks, round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
-      spect<S>(h), SIGN < 0 ? h->ex.x : h->ex.z, h->ex.y, (int)cols, h->n2, h->nkx, c, pl, twt<R>(h, 1), done, fold);
+  launch_chained(h, k_fft_y<SIGN, R, S>, blocks, round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s,
+                 spect<S>(h), SIGN < 0 ? h->ex.x : h->ex.z, h->ex.y, (int)cols, h->n2, h->nkx, c, pl, twt<R>(h, 1),
+                 done, fold);
 }
 
 template <typename R, class S>
@@ -889,8 +895,9 @@ void launch_lap(const rve_s* h, cudaStream_t s, const double* done) {
   const int np = h->n1 * h->nkx;
   const int c = cols_per_block(pl, 3L * np, h->fft_fill_z, 256);
   ProfScope ps_(h, RVE_K_FFT_Z_OP, s);
-  k_fft_z_lap<R, S><<<dim3((np + c - 1) / c, 3), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<R>), s>>>(
-      spect<S>(h), h->ex.y, h->ex.z, np, h->nkx, c, pl, twt<R>(h, 2), lap_weight<R>(h), done);
+  launch_chained(h, k_fft_z_lap<R, S>, dim3((np + c - 1) / c, 3), round32(c * pl.T), 2 * (size_t)c * pl.n *
+                 sizeof(C<R>), s, spect<S>(h), h->ex.y, h->ex.z, np, h->nkx, c, pl, twt<R>(h, 2), lap_weight<R>(h),
+                 done);
 }
 
 void zop(const rve_s* h, const SpecParams& sp, cudaStream_t s) {
@@ -898,8 +905,8 @@ void zop(const rve_s* h, const SpecParams& sp, cudaStream_t s) {
   const int np = h->n1 * h->nkx;
   const int c = cols_per_block(pl, 3L * np, h->fft_fill_z, 128);
   ProfScope ps_(h, fft_category(h, RVE_K_FFT_Z_OP), s);
-  k_fft_z_op<<<dim3((np + c - 1) / c, 3), round32(c * pl.T), 2 * (size_t)c * pl.n * sizeof(C<double>), s>>>(
-      h->spec, np, h->nkx, c, pl, h->ax[2].twq, op_tables(h), sp);
+  launch_chained(h, k_fft_z_op, dim3((np + c - 1) / c, 3), round32(c * pl.T), 2 * (size_t)c * pl.n *
+                 sizeof(C<double>), s, h->spec, np, h->nkx, c, pl, h->ax[2].twq, op_tables(h), sp);
 }
 
 template <typename R, class S, class Out>
@@ -908,8 +915,9 @@ void launch_c2r(const rve_s* h, typename Out::real* out, cudaStream_t s, const d
   const long rows = (long)nf * h->n2 * (h->n1 / 2);
   const int rpb = rows_per_block(pl, rows, h->fft_fill);
   ProfScope ps_(h, fft_category(h, RVE_K_FFT_X_C2R), s);
-  k_fft_x_c2r<R, S, Out><<<(unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb, pl.n), s>>>(
-      spect<S>(h), h->ex.y, out, h->ex.u, (int)rows, h->n1 / 2, h->nkx, rpb, pl, twt<R>(h, 0), done);
+  launch_chained(h, k_fft_x_c2r<R, S, Out>, (unsigned)((rows + rpb - 1) / rpb), round32(rpb * pl.T), row_smem<R>(rpb,
+                 pl.n), s, spect<S>(h), h->ex.y, out, h->ex.u, (int)rows, h->n1 / 2, h->nkx, rpb, pl, twt<R>(h, 0),
+                 done);
 }
 
 }  // namespace

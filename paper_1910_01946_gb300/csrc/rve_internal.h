@@ -196,6 +196,26 @@ struct ProfScope {
   ~ProfScope() { p.end(cat, s, a); }
 };
 
+// Launch as a programmatic dependent of the kernel before on the stream: the launch
+// overlaps that kernel's end (the kernel starts with chain_wait()).  The seven
+// launches of a projection are a few microseconds each on small grids: 62 -> 44 us at 16^3 and
+// 93 -> 79 us at 64^3 on a stream, and 14.6 -> 13.9 ms per 16^3 increment inside the CG graphs.
+// Not while every launch is timed: the events in between would order the launches anyway.
+template <class... P, class... A>
+void launch_chained(const rve_s* h, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = h->prof.on ? 0 : 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // device scalar slots
 enum { DS_RR = 0, DS_PKP = 1, DS_ALPHA = 2, DS_BETA = 3, DS_NORM = 4, DS_STOP = 5, DS_DONE = 6, DS_ITERS = 7,
        DS_MEANP = 8,

@@ -58,6 +58,7 @@ __global__ void __launch_bounds__(NT) k_div(Grid3 g, Tiling T, const V* __restri
                                            double* __restrict__ partial, int check_done, unsigned mean_mask) {
   __shared__ V S[9][SMAX];
   __shared__ double sh[320];
+  chain_wait();
   if (check_done && ds[DS_DONE] != 0.0) return;
   const int W = T.tx + 1;     // row pitch of the staged tile (with its halo)
   const int tx = threadIdx.x, ty = threadIdx.y;
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(NT) k_grad_t(Grid3 g, Tiling T, const V* __res
                                               unsigned int* __restrict__ ticket) {
   __shared__ V SP[3][SMAX], SM[3][SMAX];
   __shared__ double sh[320];
+  chain_wait();
   if (CG && ds[DS_DONE] != 0.0) return;
   const V alpha = CG ? (V)ds[DS_ALPHA] : (V)0;
   V off[9];
@@ -319,6 +321,7 @@ __global__ void __launch_bounds__(32 * RW) k_div_rows(Grid3 g, const V* __restri
                                                      V* __restrict__ d, double* __restrict__ ds,
                                                      double* __restrict__ partial, int check_done, unsigned mean_mask) {
   __shared__ double sh[320];
+  chain_wait();
   if (check_done && ds[DS_DONE] != 0.0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int left = (lane + 31) & 31;
@@ -429,6 +432,7 @@ __global__ void __launch_bounds__(32 * RW, NPL <= 2 ? 4 : 1) k_grad_rows(Grid3 g
                                                       double* __restrict__ ds, double* __restrict__ partial,
                                                       unsigned int* __restrict__ ticket) {
   __shared__ double sh[320];
+  chain_wait();
   if (ds[DS_DONE] != 0.0) return;
   const V alpha = (V)ds[DS_ALPHA];
   V off[9];
@@ -590,6 +594,7 @@ __global__ void __launch_bounds__(32 * RW) k_div_fix(Grid3 g, int lanes, const d
   constexpr int B = DIV_BITS;
   constexpr int FLUSH = 32 / NPL;                       // rows after which a lane's sums of a field could overflow
   __shared__ double macc[RW][9];
+  chain_wait();
   if (check_done && ds[DS_DONE] != 0.0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int left = lane == 0 ? lanes - 1 : lane - 1;
@@ -713,6 +718,7 @@ __global__ void __launch_bounds__(32 * RW) k_grad_fix(Grid3 g, int lanes, const 
                                                      double* __restrict__ partial, unsigned int* __restrict__ ticket) {
   constexpr int B = GRAD_BITS;
   __shared__ double sh[320];
+  chain_wait();
   if (CG && ds[DS_DONE] != 0.0) return;
   const double alpha = CG ? ds[DS_ALPHA] : 0.0;
   const int lane = threadIdx.x & 31;
@@ -888,8 +894,8 @@ void div_fix_n(const rve_s* h, const double* X, i64* d, int check_done, unsigned
                const Grid3& g) {
   static const int bps = resident_blocks(k_div_fix<NPL>);
   const int nb = row_blocks(h, 3L * h->n1 * h->n2, bps, h->div_blocks);
-  k_div_fix<NPL><<<nb, 32 * RW, 0, s>>>(g, h->n0 / NPL, X, d, h->ex.div, h->dscal, h->partial, check_done,
-                                        mean_mask, (reinterpret_cast<uintptr_t>(X) & 15) == 0);
+  launch_chained(h, k_div_fix<NPL>, nb, 32 * RW, 0, s, g, h->n0 / NPL, X, d, h->ex.div, h->dscal, h->partial,
+                 check_done, mean_mask, (reinterpret_cast<uintptr_t>(X) & 15) == 0);
   set_fold(h, nb, mean_mask);
 }
 
@@ -897,8 +903,8 @@ template <bool CG, int NPL>
 void grad_fix_n(const rve_s* h, const i64* u, const ZeroMode& zm, double* Y, cudaStream_t s, const Grid3& g) {
   static const int bps = resident_blocks(k_grad_fix<CG, NPL>);
   const int nb = row_blocks(h, 3L * h->n1 * h->n2, bps, 0);
-  k_grad_fix<CG, NPL><<<nb, 32 * RW, 0, s>>>(g, h->n0 / NPL, u, h->ex.u, zm, Y, h->x, h->r, h->p, h->dscal, h->partial,
-                                             ticket_of(h));
+  launch_chained(h, k_grad_fix<CG, NPL>, nb, 32 * RW, 0, s, g, h->n0 / NPL, u, h->ex.u, zm, Y, h->x, h->r, h->p,
+                 h->dscal, h->partial, ticket_of(h));
 }
 
 template <bool CG>
@@ -915,7 +921,7 @@ template <int NPL>
 void div_rows_n(const rve_s* h, const float* X, float* d, unsigned mean_mask, cudaStream_t s, const Grid3& g) {
   static const int bps = resident_blocks(k_div_rows<float, NPL>);
   const int nb = row_blocks(h, (long)h->n1 * h->n2, bps, h->div_blocks);
-  k_div_rows<float, NPL><<<nb, 32 * RW, 0, s>>>(g, X, d, h->dscal, h->partial, 1, mean_mask);
+  launch_chained(h, k_div_rows<float, NPL>, nb, 32 * RW, 0, s, g, X, d, h->dscal, h->partial, 1, mean_mask);
   set_fold(h, nb, mean_mask);
 }
 
@@ -923,7 +929,8 @@ template <int NPL>
 void grad_rows_n(const rve_s* h, const float* u, const ZeroMode& zm, cudaStream_t s, const Grid3& g) {
   static const int bps = resident_blocks(k_grad_rows<float, NPL>);
   const int nb = row_blocks(h, (long)h->n1 * h->n2, bps, 0);
-  k_grad_rows<float, NPL><<<nb, 32 * RW, 0, s>>>(g, u, zm, h->x32, h->r32, h->p32, h->dscal, h->partial, ticket_of(h));
+  launch_chained(h, k_grad_rows<float, NPL>, nb, 32 * RW, 0, s, g, u, zm, h->x32, h->r32, h->p32, h->dscal,
+                 h->partial, ticket_of(h));
 }
 
 // The FP32 row strips take n0 = 32 and 64.  Beyond: on the
@@ -982,8 +989,8 @@ cudaError_t launch_div(const rve_s* h, const double* X, double* d, int check_don
   Tiling T = tiling_of(h);
   if ((T.tx + 1) * (T.ty + 1) > SMAX) return cudaErrorInvalidValue;   // n0 odd: not a valid grid
   if (T.nblocks > h->div_blocks) T.nblocks = h->div_blocks;
-  k_div<double><<<T.nblocks, dim3(T.tx, T.ty), 0, s>>>(grid_of(h), T, X, d, h->dscal, h->partial, check_done,
-                                                       mean_mask);
+  launch_chained(h, k_div<double>, T.nblocks, dim3(T.tx, T.ty), 0, s, grid_of(h), T, X, d, h->dscal, h->partial,
+                 check_done, mean_mask);
   set_fold(h, T.nblocks, mean_mask);
   return cudaGetLastError();
 }
@@ -997,8 +1004,8 @@ cudaError_t launch_grad(const rve_s* h, const double* u, double* Y, const uint8_
   }
   const Tiling T = tiling_of(h);
   if ((T.tx + 1) * (T.ty + 1) > SMAX) return cudaErrorInvalidValue;   // n0 odd: not a valid grid
-  k_grad_t<false, double><<<T.nblocks, dim3(T.tx, T.ty), 0, s>>>(grid_of(h), T, u, zero_mode(mask, shift), Y, nullptr,
-                                                                 nullptr, nullptr, h->dscal, h->partial, ticket_of(h));
+  launch_chained(h, k_grad_t<false, double>, T.nblocks, dim3(T.tx, T.ty), 0, s, grid_of(h), T, u, zero_mode(mask,
+                 shift), Y, nullptr, nullptr, nullptr, h->dscal, h->partial, ticket_of(h));
   return cudaGetLastError();
 }
 
@@ -1010,8 +1017,8 @@ cudaError_t launch_grad_cg(const rve_s* h, const double* u, const uint8_t* mask,
   }
   const Tiling T = tiling_of(h);
   if ((T.tx + 1) * (T.ty + 1) > SMAX) return cudaErrorInvalidValue;   // n0 odd: not a valid grid
-  k_grad_t<true, double><<<T.nblocks, dim3(T.tx, T.ty), 0, s>>>(grid_of(h), T, u, zero_mode(mask, nullptr), nullptr,
-                                                                h->x, h->r, h->p, h->dscal, h->partial, ticket_of(h));
+  launch_chained(h, k_grad_t<true, double>, T.nblocks, dim3(T.tx, T.ty), 0, s, grid_of(h), T, u, zero_mode(mask,
+                 nullptr), nullptr, h->x, h->r, h->p, h->dscal, h->partial, ticket_of(h));
   return cudaGetLastError();
 }
 
@@ -1027,7 +1034,8 @@ cudaError_t launch_div32(const rve_s* h, const float* X, float* d, unsigned mean
   Tiling T = tiling_of(h);
   if ((T.tx + 1) * (T.ty + 1) > SMAX) return cudaErrorInvalidValue;   // n0 odd: not a valid grid
   if (T.nblocks > h->div_blocks) T.nblocks = h->div_blocks;
-  k_div<float><<<T.nblocks, dim3(T.tx, T.ty), 0, s>>>(grid_of(h), T, X, d, h->dscal, h->partial, 1, mean_mask);
+  launch_chained(h, k_div<float>, T.nblocks, dim3(T.tx, T.ty), 0, s, grid_of(h), T, X, d, h->dscal, h->partial, 1,
+                 mean_mask);
   set_fold(h, T.nblocks, mean_mask);
   return cudaGetLastError();
 }
@@ -1041,8 +1049,7 @@ cudaError_t launch_grad_cg32(const rve_s* h, const float* u, const uint8_t* mask
   }
   const Tiling T = tiling_of(h);
   if ((T.tx + 1) * (T.ty + 1) > SMAX) return cudaErrorInvalidValue;   // n0 odd: not a valid grid
-  k_grad_t<true, float><<<T.nblocks, dim3(T.tx, T.ty), 0, s>>>(grid_of(h), T, u, zero_mode(mask, nullptr), nullptr,
-                                                               h->x32, h->r32, h->p32, h->dscal, h->partial,
-                                                               ticket_of(h));
+  launch_chained(h, k_grad_t<true, float>, T.nblocks, dim3(T.tx, T.ty), 0, s, grid_of(h), T, u, zero_mode(mask,
+                 nullptr), nullptr, h->x32, h->r32, h->p32, h->dscal, h->partial, ticket_of(h));
   return cudaGetLastError();
 }

@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(RVE_RED_THREADS, 2) k_tangent_apply32(size_t n
                                                                      float* __restrict__ t, double* __restrict__ ds,
                                                                      double* __restrict__ partial) {
   __shared__ double sh[320];
+  chain_wait();
   if (ds[DS_DONE] != 0.0) return;
   const bool first = ds[DS_ITERS] == 0.0;
   const float beta = first ? 0.0f : (float)ds[DS_BETA];
@@ -157,6 +158,7 @@ __global__ void __launch_bounds__(TA_TV, 1) k_tangent_apply32_tma(size_t nvox, c
   float* stage[2] = {reinterpret_cast<float*>(ta_smem), reinterpret_cast<float*>(ta_smem) + TA_STAGE};
   uint64_t* bar = reinterpret_cast<uint64_t*>(ta_smem + 2 * (size_t)TA_STAGE_BYTES);
   __shared__ double sh[320];
+  chain_wait();
   if (ds[DS_DONE] != 0.0) return;
   const bool first = ds[DS_ITERS] == 0.0;
   const float beta = first ? 0.0f : (float)ds[DS_BETA];
@@ -268,6 +270,7 @@ __global__ void __launch_bounds__(TAF_THREADS, TAF_BLOCKS) k_tangent_apply(size_
                                                                            double* __restrict__ t, double* __restrict__ ds,
                                                                            double* __restrict__ partial) {
   __shared__ double sh[32];
+  chain_wait();
   if (ds[DS_DONE] != 0.0) return;
   // the first iteration of a solve (the counter is reset by the CG init and
   // bumped by each completed iteration): every launch of the loop has the
@@ -521,8 +524,8 @@ cudaError_t launch_tangent_apply(const rve_s* h, cudaStream_t s) {
   const int blocks = (int)std::min<size_t>((h->nvox + TAF_THREADS - 1) / TAF_THREADS, (size_t)TAF_BLOCKS * h->num_sms);
   {
     ProfScope ps_(h, RVE_K_TANGENT_APPLY, s);
-    k_tangent_apply<<<blocks, TAF_THREADS, 0, s>>>(h->nvox, reinterpret_cast<const int2*>(h->K[h->cur]), h->kex[h->cur], h->r, h->p, h->t, h->dscal,
-                                                       h->partial_pkp());
+    launch_chained(h, k_tangent_apply, blocks, TAF_THREADS, 0, s, h->nvox, reinterpret_cast<const
+                   int2*>(h->K[h->cur]), h->kex[h->cur], h->r, h->p, h->t, h->dscal, h->partial_pkp());
     h->fold.pkp_blocks = blocks;
   }
   return cudaGetLastError();
@@ -609,8 +612,8 @@ cudaError_t launch_tangent_apply32(const rve_s* h, cudaStream_t s) {
                                                                h->r32, h->p32, h->t32, h->dscal, h->partial_pkp(),
                                                                h->wait_polls);
     else
-      k_tangent_apply32<<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>(h->nvox, reinterpret_cast<const float*>(h->K[h->cur]),
-                                                                   h->r32, h->p32, h->t32, h->dscal, h->partial_pkp());
+      launch_chained(h, k_tangent_apply32, RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s, h->nvox, reinterpret_cast<const
+                     float*>(h->K[h->cur]), h->r32, h->p32, h->t32, h->dscal, h->partial_pkp());
     h->fold.pkp_blocks = h->tma_apply ? h->num_sms : RVE_RED_BLOCKS;
   }
   return cudaGetLastError();
