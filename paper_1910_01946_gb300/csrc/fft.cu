@@ -301,24 +301,22 @@ __device__ __forceinline__ int column_max(int key, int cpb, int* red) {
   }
   return key;
 }
-// Rows (X): T consecutive threads.  T a power of two up to 32: shuffles only;
-// other lengths share the block's largest key (rows next to each other
-// in real space, or of one kx range).
+// Rows (X): row pair `row` of the block is held by T consecutive threads.  T a power of two up
+// to 32: shuffles; other lengths by shared-memory atomics.  (Not the block's largest key: the
+// rows of a block can belong to two tensor rows of very different size.)
+constexpr int MAX_ROWS = 256;
 template <typename R>
-__device__ __forceinline__ int row_max(int key, int T, int* red) {
+__device__ __forceinline__ int row_max(int key, int T, int row, int tj, int* red) {
   if (sizeof(R) == 4) return 0;
   if (T <= 32 && (T & (T - 1)) == 0) {
     for (int o = 1; o < T; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
     return key;
   }
-  key = __reduce_max_sync(0xffffffffu, key);
-  const int nw = blockDim.x >> 5;
-  if (nw > 1) {
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = key;
-    __syncthreads();
-    for (int w = 0; w < nw; ++w) key = max(key, red[w]);
-  }
-  return key;
+  if (tj == 0) red[row] = key;
+  __syncthreads();
+  atomicMax(&red[row], key);
+  __syncthreads();
+  return red[row];
 }
 
 // Points as they lie in memory, their key and their conversion to a transform's
@@ -386,8 +384,8 @@ __global__ void __launch_bounds__(256) k_fft_x_r2c(const typename In::real* __re
                                                    int rows, int nkx, int rpb, PlanDev pl,
                                                    const TW<R>* __restrict__ tw, const double* __restrict__ done) {
   chain_wait();
-  __shared__ int red[MAX_WARPS];
-  __shared__ int ebs[256];               // output scale of each row pair
+  __shared__ int red[MAX_ROWS];
+  __shared__ int ebs[MAX_ROWS];             // output scale of each row pair
   const int n0 = pl.n;
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
   C<R>* b1 = b0 + rpb * (n0 + (n0 >> 3) + 1);
@@ -410,7 +408,7 @@ __global__ void __launch_bounds__(256) k_fft_x_r2c(const typename In::real* __re
 #pragma unroll
   for (int m = 0; m < RMAX; ++m)
     if (on && m < pl.r0) key = max(key, max(In::key(u[m], eu), In::key(v[m], ev)));
-  const int E = In::scale(row_max<R>(key, pl.T, red), pl.bits), eb = E + pl.down;
+  const int E = In::scale(row_max<R>(key, pl.T, row, tj, red), pl.bits), eb = E + pl.down;
   C<R> a[RMAX];
 #pragma unroll
   for (int m = 0; m < RMAX; ++m) a[m] = mk(In::work(u[m], eu, E, pl.bits), In::work(v[m], ev, E, pl.bits));
@@ -445,7 +443,7 @@ __global__ void __launch_bounds__(256) k_fft_x_c2r(const typename In::pair* __re
                                                    int rows, int rows_per_plane, int nkx, int rpb, PlanDev pl,
                                                    const TW<R>* __restrict__ tw, const double* __restrict__ done) {
   chain_wait();
-  __shared__ int red[MAX_WARPS];
+  __shared__ int red[MAX_ROWS];
   const int n0 = pl.n;
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
   C<R>* b1 = b0 + rpb * (n0 + (n0 >> 3) + 1);
@@ -475,7 +473,7 @@ __global__ void __launch_bounds__(256) k_fft_x_c2r(const typename In::pair* __re
 #pragma unroll
   for (int m = 0; m < HM; ++m)
     if (on && tj + m * pl.T < nkx) key = max(key, max(In::key(A[m], ex[m]), In::key(B[m], ex[m])));
-  const int E = In::scale(row_max<R>(key, pl.T, red), bits), eb = E + pl.down;
+  const int E = In::scale(row_max<R>(key, pl.T, row, tj, red), bits), eb = E + pl.down;
   if (on) {
     if (Out::FIX && tj == 0) exout[g] = eb;
 #pragma unroll

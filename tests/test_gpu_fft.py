@@ -136,3 +136,29 @@ def test_non_finite_values_reach_every_value_of_their_rows(pkg, bad):
         assert not torch.isfinite(Y[3:6]).any()
         assert torch.isfinite(Y[:3]).all() and torch.isfinite(Y[6:]).all()
     r.close()
+
+
+@pytest.mark.parametrize("shape", [(3, 54, 48), (1, 8, 512), (3, 12, 486)])
+def test_rows_that_share_a_block_with_another_tensor_row(pkg, shape):
+    """Transforms along x whose threads are no power of two up to 32 (6, 64 and
+    81 of them): the last rows of one tensor row lie in a block with the first of the
+    next, 2^60 as large or with a NaN in it, and keep their digits (4e-15 n, as
+    above) all the same."""
+    import torch
+    X = np.random.default_rng(17).standard_normal(shape + (3, 3))
+    X[..., 1, :] *= 2.0 ** -30
+    X[..., 2, :] *= 2.0 ** 30
+    ref = device_field(sp.project(X, MASK, 1e-5 / shape[2])).cpu()
+    Xd = device_field(X)
+    Xn = Xd.clone()
+    Xn[4, 5] = float("nan")
+    r = handle(pkg, shape)
+    for run in (lambda x: r.project(MASK, x).clone(), lambda x: noalloc(pkg, shape, x)):
+        Y = run(Xd)
+        for i in range(3):
+            rows = slice(3 * i, 3 * i + 3)
+            assert float((Y.cpu()[rows] - ref[rows]).abs().max()) < 4e-15 * max(shape) * float(ref[rows].abs().max()), i
+        Z = run(Xn)
+        assert not torch.isfinite(Z[3:6]).any()
+        assert torch.equal(Z[:3], Y[:3]) and torch.equal(Z[6:], Y[6:])
+    r.close()
