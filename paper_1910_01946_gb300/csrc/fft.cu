@@ -14,6 +14,8 @@
 //   Z  (C2C + operator + C2C): pencils of consecutive (ky, kx), forward z
 //             FFT, operator, inverse z FFT;
 //   Y^-1, X^-1 (C2R).  The 1/nvox scaling is folded into the operator.
+// Of small grids the X and Y passes of the three-field transforms run in one kernel each way
+// (k_fft_xy, k_fft_yx).
 //
 // A transform is held by T = n / R0 threads (R0: its first, largest radix), one
 // butterfly of R0 points per thread and pass.  The first butterfly takes its
@@ -32,6 +34,7 @@
 // sums grow by.  The rounding errors of a pass are 0.3 units of 2^-57 ...
 // 2^-53 of the transform's largest value, below the 2^-53 of each
 // intermediate value that every FP64 operation of a butterfly would leave.
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -160,6 +163,23 @@ struct PlanDev {
 __device__ __forceinline__ int fdiv(int j, unsigned m) { return (int)(((unsigned)j * m) >> 20); }
 unsigned div_magic(int d) { return ((1u << 20) + (unsigned)d - 1u) / (unsigned)d; }
 
+// n / d for 0 <= n < 2^31 and 1 <= d < 2^31 by one multiplication: with s = ceil(log2 d) and m = ceil(2^(31 + s) / d)
+// the error n (m d - 2^(31 + s)) / (2^(31 + s) d) stays below 1 / d.  (A division by a run-time
+// number is a call of 30 to 100 instructions at the start of every block.)
+struct Div {
+  unsigned m;
+  int s, d;
+  __device__ __forceinline__ int operator()(int n) const {
+    return s ? (int)(__umulhi((unsigned)n, m) >> (s - 1)) : n;
+  }
+};
+Div make_div(int d) {
+  Div r{0u, 0, d};
+  while ((1LL << r.s) < d) ++r.s;
+  r.m = (unsigned)(((1ULL << (31 + r.s)) + (unsigned)d - 1ULL) / (unsigned)d);
+  return r;
+}
+
 PlanDev to_dev(const FFTPlan& p) {
   PlanDev d{};
   d.n = p.n;
@@ -197,8 +217,9 @@ PlanDev to_dev(const FFTPlan& p) {
 __device__ __forceinline__ CX<float> untwiddled(CX<float> a) { return a; }
 __device__ __forceinline__ CX<i64> untwiddled(CX<i64> a) { return mk<i64>((a.x + 2) >> 2, (a.y + 2) >> 2); }
 
-// Pass p of radix RAD of one transform: points ld(pos), results st(pos, value)
-template <int SIGN, typename R, int RAD, class Ld, class St>
+// Pass p of radix RAD of one transform: points ld(pos), results st(pos, value); the FIRST
+// pass has no twiddles
+template <int SIGN, typename R, int RAD, bool FIRST = false, class Ld, class St>
 __device__ __forceinline__ void pass_r(const PlanDev& pl, int p, int tj, const TW<R>* __restrict__ tw, Ld ld, St st) {
   const int nb = pl.n / RAD, ns = pl.ns[p];
   for (int j = tj; j < nb; j += pl.T) {
@@ -206,9 +227,11 @@ __device__ __forceinline__ void pass_r(const PlanDev& pl, int p, int tj, const T
 #pragma unroll
     for (int m = 0; m < RAD; ++m) a[m] = ld(j + m * nb);
     const int q = fdiv(j, pl.nsdiv[p]), k = j - q * ns;
-    a[0] = untwiddled(a[0]);
+    if (!FIRST) {
+      a[0] = untwiddled(a[0]);
 #pragma unroll
-    for (int m = 1; m < RAD; ++m) a[m] = twiddle<SIGN>(a[m], tw, m * k * pl.step[p]);
+      for (int m = 1; m < RAD; ++m) a[m] = twiddle<SIGN>(a[m], tw, m * k * pl.step[p]);
+    }
     dft<SIGN, RAD>(a);
     const int d = q * ns * RAD + k;
 #pragma unroll
@@ -571,6 +594,269 @@ __global__ void __launch_bounds__(256) k_fft_y(typename S::pair* __restrict__ sp
     const C<R>* res = last_buffer(pl, b0, b1);
 #pragma unroll 1
     for (int p = tj; p < pl.n; p += pl.T) base[(size_t)p * nkx] = S::store(res[p * cpb + c], eb);
+  }
+}
+
+// ---------------------------------------------------------------- planes
+// The X and Y passes of one (field, z) plane in one kernel, the plane in shared
+// memory in between.  On small grids a Laplace solve is bound by its chain of
+// launches (about 2 us each, dependent launches included), not by their work: two of five
+// go (planes_fit has the line and both sides measured).  The transforms and scales are
+// those of the separate passes; a transform's threads find its largest value by
+// shared-memory atomics, since a plane's transforms need not fill whole warps.
+// Buffers: two of Plane::cap complex values; X transforms in row_elem's layout, Y transforms as [y][kx].
+
+// one pass of every transform: slot q is thread tj of transform t
+template <int SIGN, typename R, bool FIRST, class Slot, class Ld, class St>
+__device__ __forceinline__ void plane_pass(const PlanDev& pl, int p, int slots, const TW<R>* __restrict__ tw, Slot slot, Ld ld,
+                                           St st) {
+#pragma unroll 1
+  for (int q = threadIdx.x; q < slots; q += blockDim.x) {
+    int t, tj;
+    slot(q, t, tj);
+    auto l = [&](int pos) { return ld(t, pos); };
+    auto w = [&](int pos, C<R> v) { st(t, pos, v); };
+    switch (pl.radix[p]) {
+      case 8: pass_r<SIGN, R, 8, FIRST>(pl, p, tj, tw, l, w); break;
+      case 6: pass_r<SIGN, R, 6, FIRST>(pl, p, tj, tw, l, w); break;
+      case 4: pass_r<SIGN, R, 4, FIRST>(pl, p, tj, tw, l, w); break;
+      case 3: pass_r<SIGN, R, 3, FIRST>(pl, p, tj, tw, l, w); break;
+      default: pass_r<SIGN, R, 2, FIRST>(pl, p, tj, tw, l, w); break;
+    }
+  }
+}
+
+// sizes of one plane kernel, for its launch and its pointers
+struct Plane {
+  int n0, n1, nkx, rows, cap;            // rows: line pairs; cap: complex values per buffer
+  Div dkx, dTx;
+  PlanDev x, y;
+};
+template <typename R>
+size_t plane_bytes(const Plane& g, bool inverse) {
+  return 2 * (size_t)g.cap * sizeof(C<R>) +
+         (sizeof(R) == 8 ? (2 * (size_t)g.rows + 2 * (size_t)g.nkx + (inverse ? (size_t)g.n1 * g.nkx : 0)) * sizeof(int) : 0);
+}
+
+template <typename R, class S>
+__global__ void __launch_bounds__(512) k_fft_xy(const typename S::real* __restrict__ in, const int* __restrict__ exin,
+                                                typename S::pair* __restrict__ spec, int* __restrict__ exout, Plane g,
+                                                const TW<R>* __restrict__ twx, const TW<R>* __restrict__ twy,
+                                                const double* __restrict__ done, Fold fold) {
+  chain_wait();
+  if (done && *done != 0.0) return;
+  if (fold.mean_blocks && blockIdx.x < FOLD_BLOCKS) {
+    __shared__ double fsh[32];
+    fold_block(fold, blockIdx.x, fsh);
+    return;
+  }
+  const int plane = (int)blockIdx.x - (fold.mean_blocks ? FOLD_BLOCKS : 0);
+  C<R>* A = reinterpret_cast<C<R>*>(fft_smem);
+  C<R>* B = A + g.cap;
+  int* rowkey = reinterpret_cast<int*>(B + g.cap);   // largest key, then output scale, of each line pair
+  int* rowex = rowkey + g.rows;
+  int* colkey = rowex + g.rows;
+  const int n0 = g.n0, nkx = g.nkx;
+  if (S::FIX) {
+    for (int i = threadIdx.x; i < g.rows; i += blockDim.x) rowkey[i] = 2 * fix64::EXP_ZERO;
+    for (int i = threadIdx.x; i < nkx; i += blockDim.x) colkey[i] = 2 * fix64::EXP_ZERO;
+    __syncthreads();
+  }
+  auto xslot = [&](int q, int& t, int& tj) { t = g.dTx(q); tj = q - t * g.x.T; };
+  const typename S::real* src = in + (size_t)plane * g.n1 * n0;
+  const int* exr = exin + (size_t)plane * g.n1;
+#pragma unroll 1
+  for (int q = threadIdx.x; q < g.rows * g.x.T; q += blockDim.x) {
+    int row, tj;
+    xslot(q, row, tj);
+    typename S::real u[RMAX], v[RMAX];
+#pragma unroll
+    for (int m = 0; m < RMAX; ++m)
+      if (m < g.x.r0) {
+        u[m] = src[(size_t)2 * row * n0 + tj + m * g.x.T];
+        v[m] = src[(size_t)(2 * row + 1) * n0 + tj + m * g.x.T];
+      }
+    int hu = 0, hv = 0;
+#pragma unroll
+    for (int m = 0; m < RMAX; ++m)
+      if (m < g.x.r0) {
+        if constexpr (S::FIX) { hu |= fix64::abs_hi(u[m]); hv |= fix64::abs_hi(v[m]); }
+        B[row_elem(row, n0, tj + m * g.x.T)] = mk((typename FT<R>::w)u[m], (typename FT<R>::w)v[m]);
+      }
+    if constexpr (S::FIX)
+      atomicMax(&rowkey[row], max(fix64::fit_key(hu, exr[2 * row]), fix64::fit_key(hv, exr[2 * row + 1])));
+  }
+  __syncthreads();
+  C<R>* from = B;
+  C<R>* to = A;
+  plane_pass<-1, R, true>(g.x, 0, g.rows * g.x.T, twx, xslot,
+                          [&](int row, int pos) {
+                            C<R> z = from[row_elem(row, n0, pos)];
+                            if constexpr (S::FIX) {
+                              const int E = S::scale(rowkey[row], g.x.bits);
+                              z = mk(S::work(z.x, exr[2 * row], E, 0), S::work(z.y, exr[2 * row + 1], E, 0));
+                            }
+                            return z;
+                          },
+                          [&](int row, int pos, C<R> v) { to[row_elem(row, n0, pos)] = v; });
+  for (int p = 1; p < g.x.npass; ++p) {
+    __syncthreads();
+    C<R>* o = from; from = to; to = o;
+    plane_pass<-1, R, false>(g.x, p, g.rows * g.x.T, twx, xslot, [&](int row, int pos) { return from[row_elem(row, n0, pos)]; },
+                             [&](int row, int pos, C<R> v) { to[row_elem(row, n0, pos)] = v; });
+  }
+  if constexpr (S::FIX) {
+    for (int i = threadIdx.x; i < g.rows; i += blockDim.x) rowex[i] = S::scale(rowkey[i], g.x.bits) + g.x.down;
+  }
+  __syncthreads();
+  { C<R>* o = from; from = to; to = o; }
+  // the two half spectra of each pair (without the factor 1/2, as in k_fft_x_r2c)
+#pragma unroll 1
+  for (int q = threadIdx.x; q < g.rows * nkx; q += blockDim.x) {
+    const int row = g.dkx(q), k = q - row * nkx;
+    const C<R> zk = from[row_elem(row, n0, k)], zc = from[row_elem(row, n0, k == 0 ? 0 : n0 - k)];
+    const C<R> a = mk(zk.x + zc.x, zk.y - zc.y), b = mk(zk.y + zc.y, zc.x - zk.x);
+    to[2 * row * nkx + k] = a;
+    to[(2 * row + 1) * nkx + k] = b;
+    if constexpr (S::FIX)
+      atomicMax(&colkey[k], fix64::fit_key(fix64::abs_hi(a.x) | fix64::abs_hi(a.y) | fix64::abs_hi(b.x) | fix64::abs_hi(b.y),
+                                           rowex[row]));
+  }
+  __syncthreads();
+  typename S::pair* dst = spec + (size_t)plane * g.n1 * nkx;
+  auto yslot = [&](int q, int& t, int& tj) { tj = g.dkx(q); t = q - tj * nkx; };
+  if constexpr (S::FIX) {
+    for (int k = threadIdx.x; k < nkx; k += blockDim.x)
+      exout[(size_t)plane * nkx + k] = S::scale(colkey[k], g.y.bits) + g.y.down;
+  }
+  { C<R>* o = from; from = to; to = o; }
+  plane_pass<-1, R, true>(g.y, 0, nkx * g.y.T, twy, yslot,
+                          [&](int k, int pos) {
+                            C<R> z = from[pos * nkx + k];
+                            if constexpr (S::FIX) {
+                              const int E = S::scale(colkey[k], g.y.bits);
+                              z = mk(S::work(z.x, rowex[pos >> 1], E, 0), S::work(z.y, rowex[pos >> 1], E, 0));
+                            }
+                            return z;
+                          },
+                          [&](int k, int pos, C<R> v) {
+                            if (g.y.npass == 1) dst[pos * nkx + k] = S::store(v, 0);
+                            else to[pos * nkx + k] = v;
+                          });
+  for (int p = 1; p < g.y.npass; ++p) {
+    __syncthreads();
+    C<R>* o = from; from = to; to = o;
+    plane_pass<-1, R, false>(g.y, p, nkx * g.y.T, twy, yslot, [&](int k, int pos) { return from[pos * nkx + k]; },
+                             [&](int k, int pos, C<R> v) {
+                               if (p + 1 == g.y.npass) dst[pos * nkx + k] = S::store(v, 0);
+                               else to[pos * nkx + k] = v;
+                             });
+  }
+}
+
+template <typename R, class S>
+__global__ void __launch_bounds__(512) k_fft_yx(const typename S::pair* __restrict__ spec, const int* __restrict__ exin,
+                                                typename S::real* __restrict__ out, int* __restrict__ exout, int n2, Plane g,
+                                                const TW<R>* __restrict__ twx, const TW<R>* __restrict__ twy,
+                                                const double* __restrict__ done) {
+  chain_wait();
+  if (done && *done != 0.0) return;
+  const int plane = blockIdx.x, n0 = g.n0, nkx = g.nkx;
+  C<R>* A = reinterpret_cast<C<R>*>(fft_smem);
+  C<R>* B = A + g.cap;
+  int* rowkey = reinterpret_cast<int*>(B + g.cap);
+  int* colkey = rowkey + 2 * g.rows;
+  int* colex = colkey + nkx;             // scale of each column after its inverse
+  int* ex = colex + nkx;                 // scale of each value of the plane as it comes in
+  if (S::FIX) {
+    for (int i = threadIdx.x; i < g.rows; i += blockDim.x) rowkey[i] = 2 * fix64::EXP_ZERO;
+    for (int i = threadIdx.x; i < nkx; i += blockDim.x) colkey[i] = 2 * fix64::EXP_ZERO;
+    __syncthreads();
+  }
+  const typename S::pair* src = spec + (size_t)plane * g.n1 * nkx;
+  const int* exs = exin + (size_t)((unsigned)plane / (unsigned)n2) * g.n1 * nkx;
+#pragma unroll 4
+  for (int q = threadIdx.x; q < g.n1 * nkx; q += blockDim.x) {
+    const typename S::pair v = src[q];
+    B[q] = mk((typename FT<R>::w)v.x, (typename FT<R>::w)v.y);
+    if constexpr (S::FIX) {
+      const int e = exs[q];
+      ex[q] = e;
+      atomicMax(&colkey[q - g.dkx(q) * nkx], S::key(v, e));
+    }
+  }
+  __syncthreads();
+  auto yslot = [&](int q, int& t, int& tj) { tj = g.dkx(q); t = q - tj * nkx; };
+  C<R>* from = B;
+  C<R>* to = A;
+  plane_pass<+1, R, true>(g.y, 0, nkx * g.y.T, twy, yslot,
+                          [&](int k, int pos) {
+                            C<R> z = from[pos * nkx + k];
+                            if constexpr (S::FIX) {
+                              const int E = S::scale(colkey[k], g.y.bits);
+                              z = mk(S::work(z.x, ex[pos * nkx + k], E, 0), S::work(z.y, ex[pos * nkx + k], E, 0));
+                            }
+                            return z;
+                          },
+                          [&](int k, int pos, C<R> v) { to[pos * nkx + k] = v; });
+  for (int p = 1; p < g.y.npass; ++p) {
+    __syncthreads();
+    C<R>* o = from; from = to; to = o;
+    plane_pass<+1, R, false>(g.y, p, nkx * g.y.T, twy, yslot, [&](int k, int pos) { return from[pos * nkx + k]; },
+                             [&](int k, int pos, C<R> v) { to[pos * nkx + k] = v; });
+  }
+  if constexpr (S::FIX) {
+    for (int k = threadIdx.x; k < nkx; k += blockDim.x) colex[k] = S::scale(colkey[k], g.y.bits) + g.y.down;
+  }
+  __syncthreads();
+  { C<R>* o = from; from = to; to = o; }
+  const int bits = g.x.bits - 1;         // (the sums A + i B double the components: one bit less)
+  if constexpr (S::FIX) {
+#pragma unroll 1
+    for (int q = threadIdx.x; q < g.rows * nkx; q += blockDim.x) {
+      const int row = g.dkx(q), k = q - row * nkx;
+      const C<R> a = from[2 * row * nkx + k], b = from[(2 * row + 1) * nkx + k];
+      atomicMax(&rowkey[row], fix64::fit_key(fix64::abs_hi(a.x) | fix64::abs_hi(a.y) | fix64::abs_hi(b.x) | fix64::abs_hi(b.y),
+                                             colex[k]));
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < g.rows; i += blockDim.x)
+      exout[(size_t)plane * g.rows + i] = S::scale(rowkey[i], bits) + g.x.down;
+  }
+  // Z(k) = A + i B and Z(n0 - k) = conj(A) + i conj(B)
+#pragma unroll 1
+  for (int q = threadIdx.x; q < g.rows * nkx; q += blockDim.x) {
+    const int row = g.dkx(q), k = q - row * nkx;
+    C<R> a = from[2 * row * nkx + k], b = from[(2 * row + 1) * nkx + k];
+    if constexpr (S::FIX) {
+      const int E = S::scale(rowkey[row], bits), e = colex[k];
+      a = mk(S::work(a.x, e, E, 0), S::work(a.y, e, E, 0));
+      b = mk(S::work(b.x, e, E, 0), S::work(b.y, e, E, 0));
+    }
+    to[row_elem(row, n0, k)] = mk(a.x - b.y, a.y + b.x);
+    if (k > 0 && 2 * k < n0) to[row_elem(row, n0, n0 - k)] = mk(a.x + b.y, b.x - a.y);
+  }
+  __syncthreads();
+  auto xslot = [&](int q, int& t, int& tj) { t = g.dTx(q); tj = q - t * g.x.T; };
+  typename S::real* dst = out + (size_t)plane * g.n1 * n0;
+  auto put = [&](int row, int pos, C<R> v) {
+    dst[2 * row * n0 + pos] = (typename S::real)v.x;
+    dst[(2 * row + 1) * n0 + pos] = (typename S::real)v.y;
+  };
+  { C<R>* o = from; from = to; to = o; }
+  plane_pass<+1, R, true>(g.x, 0, g.rows * g.x.T, twx, xslot, [&](int row, int pos) { return from[row_elem(row, n0, pos)]; },
+                          [&](int row, int pos, C<R> v) {
+                            if (g.x.npass == 1) put(row, pos, v);
+                            else to[row_elem(row, n0, pos)] = v;
+                          });
+  for (int p = 1; p < g.x.npass; ++p) {
+    __syncthreads();
+    C<R>* o = from; from = to; to = o;
+    plane_pass<+1, R, false>(g.x, p, g.rows * g.x.T, twx, xslot, [&](int row, int pos) { return from[row_elem(row, n0, pos)]; },
+                             [&](int row, int pos, C<R> v) {
+                               if (p + 1 == g.x.npass) put(row, pos, v);
+                               else to[row_elem(row, n0, pos)] = v;
+                             });
   }
 }
 
@@ -949,6 +1235,46 @@ void make_plan(int n, FFTPlan* p) {
   for (; b > 0; --b) add(3);
 }
 
+Plane plane_of(const rve_s* h) {
+  Plane g;
+  g.n0 = h->n0; g.n1 = h->n1; g.nkx = h->nkx; g.rows = h->n1 / 2;
+  g.cap = std::max(g.rows * (h->n0 + (h->n0 >> 3) + 1), h->n1 * h->nkx);
+  g.x = to_dev(h->plan[0]);
+  g.y = to_dev(h->plan[1]);
+  g.dkx = make_div(h->nkx);
+  g.dTx = make_div(g.x.T);
+  return g;
+}
+// Whole planes per block where two buffers fit 47 KB (with the static part the 48 KB a launch
+// gets unasked): 48 x 48 in FP64, 64 x 64 in FP32.  Faster on every grid below the
+// line that was measured, by what two launches cost: an FP64 projection of 8^3 40.3 -> 36.6 us,
+// 16^3 44.0 -> 39.9, 32^3 54.3 -> 50.5, 36 x 54 x 27 58.6 -> 56.8, 48^3 67.9 -> 65.9,
+// 16 x 16 x 256 62.3 -> 58.0; a mixed increment of 32^3 12.25 -> 11.88 ms, of 64^3 80.5 -> 79.6 ms.
+// Above it few blocks share an SM and the passes within a block wait for each other: FP64
+// at 64^3 (84 KB) 79.6 -> 81.8 us.
+constexpr size_t PLANE_SMEM = 47 * 1024;
+template <typename R>
+bool planes_fit(const rve_s* h) { return plane_bytes<R>(plane_of(h), true) <= PLANE_SMEM; }
+template <typename R>
+int plane_threads(const Plane& g) {
+  return std::min(512, round32(std::max(g.rows * g.x.T, g.nkx * g.y.T)));
+}
+
+template <typename R, class S>
+void launch_xy(const rve_s* h, const typename S::real* in, cudaStream_t s, const double* done, const Fold& fold) {
+  const Plane g = plane_of(h);
+  ProfScope ps_(h, RVE_K_FFT_X_R2C, s);
+  launch_chained(h, k_fft_xy<R, S>, 3 * h->n2 + (fold.mean_blocks ? FOLD_BLOCKS : 0), plane_threads<R>(g),
+                 plane_bytes<R>(g, false), s, in, h->ex.div, spect<S>(h), h->ex.y, g, twt<R>(h, 0), twt<R>(h, 1), done, fold);
+}
+template <typename R, class S>
+void launch_yx(const rve_s* h, typename S::real* out, cudaStream_t s, const double* done) {
+  const Plane g = plane_of(h);
+  ProfScope ps_(h, RVE_K_FFT_X_C2R, s);
+  launch_chained(h, k_fft_yx<R, S>, 3 * h->n2, plane_threads<R>(g), plane_bytes<R>(g, true), s, spect<S>(h), h->ex.z, out,
+                 h->ex.u, h->n2, g, twt<R>(h, 0), twt<R>(h, 1), done);
+}
+
 // the block sums waiting to be added up, taken by the caller's Y pass
 Fold take_fold(const rve_s* h) {
   Fold f{};
@@ -980,6 +1306,12 @@ cudaError_t launch_fft9(const rve_s* h, const double* in, double* out, const Spe
 // stencils of this grid work on doubles
 cudaError_t launch_laplace_solve(const rve_s* h, const double* d, double* u, bool fixed, cudaStream_t s,
                                  const double* done) {
+  if (fixed && planes_fit<double>(h)) {
+    launch_xy<double, Fixed>(h, reinterpret_cast<const i64*>(d), s, done, take_fold(h));
+    launch_lap<double, Fixed>(h, s, done);
+    launch_yx<double, Fixed>(h, reinterpret_cast<i64*>(u), s, done);
+    return cudaGetLastError();
+  }
   if (fixed) launch_r2c<double, Fixed, Fixed>(h, reinterpret_cast<const i64*>(d), s, done, 3);
   else launch_r2c<double, Plain<double>, Fixed>(h, d, s, done, 3);
   launch_y<-1, double, Fixed>(h, s, done, 3, take_fold(h));
@@ -991,6 +1323,12 @@ cudaError_t launch_laplace_solve(const rve_s* h, const double* d, double* u, boo
 }
 cudaError_t launch_laplace_solve32(const rve_s* h, const float* d, float* u, cudaStream_t s, const double* done) {
   typedef Plain<float> S;
+  if (planes_fit<float>(h)) {
+    launch_xy<float, S>(h, d, s, done, take_fold(h));
+    launch_lap<float, S>(h, s, done);
+    launch_yx<float, S>(h, u, s, done);
+    return cudaGetLastError();
+  }
   launch_r2c<float, S, S>(h, d, s, done, 3);
   launch_y<-1, float, S>(h, s, done, 3, take_fold(h));
   launch_lap<float, S>(h, s, done);

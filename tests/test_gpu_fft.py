@@ -162,3 +162,26 @@ def test_rows_that_share_a_block_with_another_tensor_row(pkg, shape):
         assert not torch.isfinite(Z[3:6]).any()
         assert torch.equal(Z[:3], Y[:3]) and torch.equal(Z[6:], Y[6:])
     r.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 16, 16), (3, 2, 432), (2, 512, 2), (6, 128, 8), (3, 32, 64), (4, 48, 48), (3, 54, 36),
+                                   (3, 54, 48), (2, 64, 64)])
+def test_planes_in_one_block_and_above_the_line(pkg, shape):
+    """The X and Y passes fused per plane, up to the largest planes that take
+    them, and the separate passes just above: as accurate as the axis-length
+    test asks (4e-15 n), powers of two exact, zeros stay zero, a NaN stays
+    in its tensor row."""
+    import torch
+    X = np.random.default_rng(sum(shape)).standard_normal(shape + (3, 3))
+    ref = device_field(sp.project(X, MASK, 1e-5 / shape[2])).cpu()
+    Xd = device_field(X)
+    r = handle(pkg, shape)
+    Y = r.project(MASK, Xd).clone()
+    assert float((Y.cpu() - ref).abs().max()) < 4e-15 * max(shape) * float(ref.abs().max())
+    assert torch.equal(r.project(MASK, Xd * 2.0 ** -40), Y * 2.0 ** -40)
+    assert float(r.project(MASK, torch.zeros_like(Xd)).abs().max()) == 0.0
+    Xd[4, 5] = float("nan")
+    Z = r.project(MASK, Xd)
+    assert not torch.isfinite(Z[3:6]).any()
+    assert torch.equal(Z[:3], Y[:3]) and torch.equal(Z[6:], Y[6:])
+    r.close()
