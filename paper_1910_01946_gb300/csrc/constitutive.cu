@@ -261,6 +261,36 @@ __device__ void lu6_solve(const double* LU, const int* piv, double* b) {
   }
 }
 
+// double to float and back by integer instructions (the conversions of the
+// FP64 pipe cost as much as an FMA there); truncated; below 2^-126: zero
+__device__ __forceinline__ float f32_of(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  const unsigned m = (__funnelshift_l((unsigned)lo, (unsigned)hi, 3) - (896u << 23)) & 0x7fffffffu;
+  const unsigned v = e <= 896 ? 0u : (e >= 1151 ? 0x7f7fffffu : m);
+  return __uint_as_float(v | ((unsigned)hi & 0x80000000u));
+}
+__device__ __forceinline__ double f64_of(float x) {
+  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
+  const unsigned hi = (m >> 3) + (896u << 20);
+  return m < 0x00800000u ? 0.0 : __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
+}
+
+// k / sqrt(s), rounded once: a third-order step from the FP32 reciprocal root, its residual
+// e = 1 - s y^2 and k y each with their rounding error.  Ten FP64 operations in place of a square
+// root and a division: k_hardening of 64^3 412 -> 379 us (it is bound by the FP64 pipe); 0.5 units in
+// the last place where those two left 1.35.
+__device__ __forceinline__ double over_sqrt(double k, double s) {
+  const int hi = __double2hiint(s);
+  if (hi < 0x39b00000 || hi >= 0x46300000) return k / sqrt(s);      // not in [2^-100, 2^100)
+  const double y = f64_of(rsqrtf(f32_of(s)));
+  const double t = s * y, tl = fma(s, y, -t);
+  const double e = fma(-tl, y, fma(-t, y, 1.0));
+  const double g = e * fma(0.375, e, 0.5);
+  const double r = k * y, rl = fma(k, y, -r);
+  return r + fma(r, g, rl);
+}
+
 __global__ void __launch_bounds__(128) k_hardening(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
     const double* __restrict__ qhat, const double* __restrict__ Apinv, const int32_t* __restrict__ screw_of,
@@ -309,7 +339,7 @@ __global__ void __launch_bounds__(128) k_hardening(
     const double t = fma(amb, sqrt(s), c.tau0);
     tauc[a * nvox + v] = t;
     tinv[a * nvox + v] = 1.0 / t;      // read by every evaluation of the increment
-    ell[a * nvox + v] = c.K / sqrt(sum - rho[a]);
+    ell[a * nvox + v] = over_sqrt(c.K, sum - rho[a]);
   }
   double Fpv[9], Fi[9];
 #pragma unroll
@@ -365,21 +395,6 @@ __device__ __forceinline__ unsigned long long mag_bits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull;
 }
 constexpr unsigned long long INF_BITS = 0x7ff0000000000000ull;
-
-// double to float and back by integer instructions (the conversions of the
-// FP64 pipe cost as much as an FMA there); truncated; below 2^-126: zero
-__device__ __forceinline__ float f32_of(double x) {
-  const int hi = __double2hiint(x), lo = __double2loint(x);
-  const int e = (hi >> 20) & 0x7ff;
-  const unsigned m = (__funnelshift_l((unsigned)lo, (unsigned)hi, 3) - (896u << 23)) & 0x7fffffffu;
-  const unsigned v = e <= 896 ? 0u : (e >= 1151 ? 0x7f7fffffu : m);
-  return __uint_as_float(v | ((unsigned)hi & 0x80000000u));
-}
-__device__ __forceinline__ double f64_of(float x) {
-  const unsigned b = __float_as_uint(x), m = b & 0x7fffffffu;
-  const unsigned hi = (m >> 3) + (896u << 20);
-  return m < 0x00800000u ? 0.0 : __hiloint2double((int)(hi | (b & 0x80000000u)), (int)(b << 29));
-}
 
 // sqrt 6 times the resolved shears of the twelve systems: every one is a
 // difference of two normal components and a sum or difference of two shears
