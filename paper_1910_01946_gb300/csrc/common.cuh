@@ -297,6 +297,13 @@ __device__ __forceinline__ bool last_block_sum1(const double* partial, unsigned 
   return true;
 }
 
+// The tangent K lies in tiles of 256 voxels, [tile][entry][voxel in the tile], the last one padded:
+// entry e of voxel v at k_at(v) + e * K_TILE.  A block reads its 81 rows from one piece of 166 KB
+// (FP64) instead of from 81 places nvox entries apart, at constant offsets: tangent
+// apply of 64^3 46.0 -> 44.3 us, and the mixed one can copy nine rows at once (25.6 -> 23.5 us).
+constexpr int K_TILE = 256;
+__device__ __forceinline__ size_t k_at(size_t v) { return (v / K_TILE) * (81 * (size_t)K_TILE) + v % K_TILE; }
+
 // Sums that a later kernel needs and that no launch in between does: the block
 // sums a kernel has left in memory are added up by extra blocks (one per value) of a
 // kernel that follows (the forward Y pass of the Laplace solve), whose other

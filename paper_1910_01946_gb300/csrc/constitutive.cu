@@ -6,9 +6,11 @@
 //                  critical resolved shear stress (Eq. Taylor_hard, with the
 //                  lattice friction tau0 and Taylor coefficient alpha) and the
 //                  mean free path (Eq. meanfree), frozen for the increment.
-//   k_constitutive the implicit update of Sec. 2.1 (Eqs. 1-5, power law,
-//                  Eq. Piola) by Newton on the second Piola-Kirchhoff stress S,
-//                  and the consistent tangent dP/dF (Eq. linequil2ast).
+//   k_local        the implicit update of Sec. 2.1 (Eqs. 1-5, power law,
+//                  Eq. Piola) by Newton on the second Piola-Kirchhoff stress S;
+//   k_tangent      the consistent tangent dP/dF (Eq. linequil2ast).
+//   k_local_fp64, k_tangent_fp64: the same with FP64 Newton matrices, for
+//                  rve_eval_constitutive in mixed precision alone.
 //
 // Everything inside a voxel is done in its grain's crystal frame, where the
 // stiffness is cubic (three constants) and the Schmid tensors s (x) m are
@@ -20,8 +22,8 @@
 //   Fp = (I + sum_a dgam^a s^a (x) m^a) Fp_prev,
 //   dgam^a = dt gdot0 |tau^a / tauc^a|^n sgn tau^a,  tau^a = S : s^a (x) m^a,
 // residual r(S) = S - C : (Fe^T Fe - I)/2, Fe = F Fp^-1, solved from a warm
-// start with the exact Jacobian and step halving (a step is taken only if it
-// lowers max|r| and keeps every |dgam| <= dgam_max).
+// start with the exact Jacobian (in FP32 in k_local) and step halving (a step is
+// taken only if it lowers max|r| and keeps every |dgam| <= dgam_max).
 #include <algorithm>
 
 #include "common.cuh"
@@ -934,7 +936,7 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
       double t = ij / 3 == kk ? q[ij % 3] : 0.0;
 #pragma unroll
       for (int m = 0; m < 6; ++m) t = fma(H[(9 * m + ij) * TAN_THREADS], dE[m], t);
-      const size_t at = (size_t)(9 * ij + kl) * nvox + v;
+      const size_t at = k_at(v) + (9 * ij + kl) * K_TILE;
       if (k32) {   // mixed precision: the tangent only drives the FP32 conjugate gradients
         reinterpret_cast<float*>(Kout)[at] = (float)t;
       } else {     // integers for the FP64 apply: signed low word, high word
@@ -1171,9 +1173,9 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent_fp64(
 #pragma unroll
       for (int ij = 0; ij < 9; ++ij) {
         if (k32)   // mixed precision: the tangent only drives the FP32 conjugate gradients
-          reinterpret_cast<float*>(Kout)[(size_t)(9 * ij + kl) * nvox + v] = (float)dP[ij];
+          reinterpret_cast<float*>(Kout)[k_at(v) + (9 * ij + kl) * K_TILE] = (float)dP[ij];
         else
-          Kout[(size_t)(9 * ij + kl) * nvox + v] = dP[ij];
+          Kout[k_at(v) + (9 * ij + kl) * K_TILE] = dP[ij];
       }
     }
   }

@@ -93,7 +93,7 @@ void carve(rve_s* h, Carver& c) {
   h->F = c.take<double>(9 * nv);
   for (int b = 0; b < 2; ++b) {
     h->P[b] = c.take<double>(9 * nv);
-    h->K[b] = c.take<double>(81 * nv);
+    h->K[b] = c.take<double>(81 * ((nv + K_TILE - 1) / K_TILE * K_TILE));
     h->kex[b] = h->opt.precision == 0 ? c.take<int>(nv) : nullptr;
     h->S[b] = c.take<double>(6 * nv);
     h->dgam[b] = c.take<double>(12 * nv);

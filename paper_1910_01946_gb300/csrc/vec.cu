@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(RVE_RED_THREADS, 2) k_tangent_apply32(size_t n
     // row keeps enough bytes in flight
     float kk[81], pv[9];
 #pragma unroll
-    for (int e = 0; e < 81; ++e) kk[e] = __ldcs(K + (size_t)e * nvox + v);
+    for (int e = 0; e < 81; ++e) kk[e] = __ldcs(K + k_at(v) + e * K_TILE);
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
       const float rv = r[k * nvox + v];
@@ -89,10 +89,10 @@ __global__ void __launch_bounds__(RVE_RED_THREADS, 2) k_tangent_apply32(size_t n
 // The FP32 CG step is bound by HBM: 324 of its 396 bytes per voxel are the
 // tangent.  A persistent block per SM streams 256-voxel tiles of the 81
 // tangent rows and of r and p (99 rows) into shared memory with bulk
-// asynchronous copies (one 1 KB copy per row, completion counted on an
+// asynchronous copies (1 KB per row of r and p, 9 KB per nine rows of K; completion counted on an
 // mbarrier), double-buffered, so the copy engine keeps the bytes in flight
 // instead of per-thread loads.
-constexpr int TA_TV = 256;                       // voxels per tile = threads per block
+constexpr int TA_TV = K_TILE;                    // voxels per tile = threads per block
 constexpr int TA_ROWS = 81 + 9 + 9;              // K, r, p
 constexpr int TA_STAGE = TA_ROWS * TA_TV;        // floats per stage
 constexpr unsigned TA_STAGE_BYTES = TA_STAGE * sizeof(float);
@@ -133,7 +133,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, unsign
   return false;
 }
 
-// issue the 99 row copies of tile `tile` into a stage buffer (threads 0..98)
+// issue the copies of tile `tile` into a stage buffer (threads 0..98: a row each, or rows of K by nines)
 __device__ __forceinline__ void ta_issue(const float* __restrict__ K, const float* __restrict__ r,
                                          const float* __restrict__ p, size_t nvox, long tile, float* buf,
                                          uint64_t* bar) {
@@ -142,9 +142,11 @@ __device__ __forceinline__ void ta_issue(const float* __restrict__ K, const floa
   const unsigned bytes = (unsigned)(nv * sizeof(float));   // nvox is a multiple of 4: a 16-byte multiple
   if (threadIdx.x == 0) mbar_expect_tx(bar, TA_ROWS * bytes);
   const int e = threadIdx.x;
-  if (e < TA_ROWS) {
+  if (nv == TA_TV && e < 81) {           // whole tile: nine rows of K, one piece of memory, per copy (25.2 -> 23.5 us at 64^3)
+    if (e < 9) bulk_g2s_stream(buf + 9 * e * TA_TV, K + (size_t)tile * (81 * K_TILE) + 9 * e * K_TILE, 9 * bytes, bar);
+  } else if (e < TA_ROWS) {
     if (e < 81)
-      bulk_g2s_stream(buf + e * TA_TV, K + (size_t)e * nvox + v0, bytes, bar);
+      bulk_g2s_stream(buf + e * TA_TV, K + (size_t)tile * (81 * K_TILE) + e * K_TILE, bytes, bar);
     else
       bulk_g2s(buf + e * TA_TV, (e < 90 ? r + (size_t)(e - 81) * nvox : p + (size_t)(e - 90) * nvox) + v0, bytes, bar);
   }
@@ -260,7 +262,7 @@ __device__ __forceinline__ double fixed_row(const int2* K, size_t stride, const 
 // alpha = rr / p . t formed, by launch_laplace_solve: see Fold).
 // Returns at once when the CG loop has converged (done != 0).
 //
-// 55.3 -> 46.0 us at 64^3 (4.9 TB/s).  Plain loads, three rows of K in flight per thread: staged through
+// 55.3 -> 44.3 us at 64^3 (5.1 TB/s).  Plain loads, three rows of K in flight per thread: staged through
 // shared memory (bulk copies, two or four threads per voxel) it took 53, with the next voxel's rows
 // prefetched 49, at four and three blocks per SM 47 and 50 us.
 constexpr int TAF_THREADS = 128, TAF_BLOCKS = 5;  // per SM: 102 registers, 27 rows of K in flight per thread
@@ -279,9 +281,10 @@ __global__ void __launch_bounds__(TAF_THREADS, TAF_BLOCKS) k_tangent_apply(size_
   const double beta = first ? 0.0 : ds[DS_BETA];
   double acc = 0.0;
   for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvox; v += (size_t)gridDim.x * blockDim.x) {
+    const int2* Kv = K + k_at(v);
     int2 kk[27];
 #pragma unroll
-    for (int e = 0; e < 27; ++e) kk[e] = __ldcs(K + (size_t)e * nvox + v);
+    for (int e = 0; e < 27; ++e) kk[e] = __ldcs(Kv + e * K_TILE);
     const int ek = __ldcs(kex + v);
     double pv[9];
 #pragma unroll
@@ -302,7 +305,7 @@ __global__ void __launch_bounds__(TAF_THREADS, TAF_BLOCKS) k_tangent_apply(size_
         acc = fma(pv[i], s, acc);
         if (ib < 2) {
 #pragma unroll
-          for (int e = 0; e < 9; ++e) kk[9 * ii + e] = __ldcs(K + (size_t)(27 * (ib + 1) + 9 * ii + e) * nvox + v);
+          for (int e = 0; e < 9; ++e) kk[9 * ii + e] = __ldcs(Kv + (27 * (ib + 1) + 9 * ii + e) * K_TILE);
         }
       }
     }
@@ -660,28 +663,34 @@ __global__ void __launch_bounds__(RVE_RED_THREADS, 2) k_kmul(size_t nvox, const 
       const int ep = fixed_vector(pv, pf), ek = kex[v];
 #pragma unroll
       for (int i = 0; i < 9; ++i)
-        out[i * nvox + v] = fixed_row(reinterpret_cast<const int2*>(K) + (size_t)9 * i * nvox + v, nvox, pf, ek, ep);
+        out[i * nvox + v] = fixed_row(reinterpret_cast<const int2*>(K) + k_at(v) + 9 * i * K_TILE, K_TILE, pf, ek, ep);
     } else {
       const float* Kf = reinterpret_cast<const float*>(K);
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
         double s = 0.0;
 #pragma unroll
-        for (int j = 0; j < 9; ++j) s = fma((double)__ldcs(Kf + (size_t)(9 * i + j) * nvox + v), pv[j], s);
+        for (int j = 0; j < 9; ++j) s = fma((double)__ldcs(Kf + k_at(v) + (9 * i + j) * K_TILE), pv[j], s);
         out[i * nvox + v] = s;
       }
     }
   }
 }
 
-// the FP64 path's tangent as doubles
-__global__ void k_tangent_values(size_t nvox, const int2* __restrict__ K, const int* __restrict__ kex, double* __restrict__ out) {
+// the tangent as doubles, [entry][voxel]
+template <bool FIXED>
+__global__ void k_tangent_values(size_t nvox, const double* __restrict__ K, const int* __restrict__ kex, double* __restrict__ out) {
   for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvox; v += (size_t)gridDim.x * blockDim.x) {
-    const int ek = kex[v];
+    const int ek = FIXED ? kex[v] : 0;
 #pragma unroll 9
     for (int e = 0; e < 81; ++e) {
-      const int2 k = __ldcs(K + (size_t)e * nvox + v);
-      out[(size_t)e * nvox + v] = fix64::from_fix(((fix64::i64)k.y << 32) + k.x, ek);
+      const size_t at = k_at(v) + e * K_TILE;
+      if (FIXED) {
+        const int2 k = __ldcs(reinterpret_cast<const int2*>(K) + at);
+        out[(size_t)e * nvox + v] = fix64::from_fix(((fix64::i64)k.y << 32) + k.x, ek);
+      } else {
+        out[(size_t)e * nvox + v] = (double)__ldcs(reinterpret_cast<const float*>(K) + at);
+      }
     }
   }
 }
@@ -780,11 +789,12 @@ cudaError_t launch_kmul(const rve_s* h, const double* in, double* out, cudaStrea
 }
 
 cudaError_t launch_tangent_values(const rve_s* h, double* dst, cudaStream_t s) {
-  if (h->opt.precision == 1)   // stored as float
-    return launch_widen(h, reinterpret_cast<const float*>(h->K[h->cur]), dst, 81 * h->nvox, s);
   {
     ProfScope ps_(h, RVE_K_OTHER, s);
-    k_tangent_values<<<RVE_RED_BLOCKS, 128, 0, s>>>(h->nvox, reinterpret_cast<const int2*>(h->K[h->cur]), h->kex[h->cur], dst);
+    if (h->opt.precision == 1)   // stored as float
+      k_tangent_values<false><<<RVE_RED_BLOCKS, 128, 0, s>>>(h->nvox, h->K[h->cur], nullptr, dst);
+    else
+      k_tangent_values<true><<<RVE_RED_BLOCKS, 128, 0, s>>>(h->nvox, h->K[h->cur], h->kex[h->cur], dst);
   }
   return cudaGetLastError();
 }
