@@ -264,13 +264,19 @@ __device__ __forceinline__ double fixed_row(const int2* K, size_t stride, const 
 //
 // 55.3 -> 44.3 us at 64^3 (5.1 TB/s).  Plain loads, three rows of K in flight per thread: staged through
 // shared memory (bulk copies, two or four threads per voxel) it took 53, with the next voxel's rows
-// prefetched 49, at four and three blocks per SM 47 and 50 us.
-constexpr int TAF_THREADS = 128, TAF_BLOCKS = 5;  // per SM: 102 registers, 27 rows of K in flight per thread
-__global__ void __launch_bounds__(TAF_THREADS, TAF_BLOCKS) k_tangent_apply(size_t nvox, const int2* __restrict__ K,
-                                                                           const int* __restrict__ kex,
-                                                                           const double* __restrict__ r, double* __restrict__ p,
-                                                                           double* __restrict__ t, double* __restrict__ ds,
-                                                                           double* __restrict__ partial) {
+// prefetched 49, with three blocks per SM 50.
+//
+// BLOCKS per SM, ROWS of K in flight per thread.  Grids of up to two blocks per SM (about 38900
+// voxels) leave registers for all nine rows: 16^3 11.1 -> 10.2 us, 32^3 12.8 -> 12.1;
+// above, 64^3 takes 44.2 us with five blocks per SM, 45.7 with four.
+constexpr int TAF_THREADS = 128;
+constexpr int TAF_SMALL = 2, TAF_LARGE = 5;
+template <int BLOCKS, int ROWS>
+__global__ void __launch_bounds__(TAF_THREADS, BLOCKS) k_tangent_apply(size_t nvox, const int2* __restrict__ K,
+                                                                       const int* __restrict__ kex,
+                                                                       const double* __restrict__ r, double* __restrict__ p,
+                                                                       double* __restrict__ t, double* __restrict__ ds,
+                                                                       double* __restrict__ partial) {
   __shared__ double sh[32];
   chain_wait();
   if (ds[DS_DONE] != 0.0) return;
@@ -282,9 +288,9 @@ __global__ void __launch_bounds__(TAF_THREADS, TAF_BLOCKS) k_tangent_apply(size_
   double acc = 0.0;
   for (size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x; v < nvox; v += (size_t)gridDim.x * blockDim.x) {
     const int2* Kv = K + k_at(v);
-    int2 kk[27];
+    int2 kk[9 * ROWS];
 #pragma unroll
-    for (int e = 0; e < 27; ++e) kk[e] = __ldcs(Kv + e * K_TILE);
+    for (int e = 0; e < 9 * ROWS; ++e) kk[e] = __ldcs(Kv + e * K_TILE);
     const int ek = __ldcs(kex + v);
     double pv[9];
 #pragma unroll
@@ -296,16 +302,16 @@ __global__ void __launch_bounds__(TAF_THREADS, TAF_BLOCKS) k_tangent_apply(size_
     fix64::Sp pf[9];
     const int ep = fixed_vector(pv, pf);
 #pragma unroll
-    for (int ib = 0; ib < 3; ++ib) {
+    for (int ib = 0; ib < 9 / ROWS; ++ib) {
 #pragma unroll
-      for (int ii = 0; ii < 3; ++ii) {
-        const int i = 3 * ib + ii;
+      for (int ii = 0; ii < ROWS; ++ii) {
+        const int i = ROWS * ib + ii;
         const double s = fixed_row(kk + 9 * ii, 1, pf, ek, ep);
         t[i * nvox + v] = s;
         acc = fma(pv[i], s, acc);
-        if (ib < 2) {
+        if (ib + 1 < 9 / ROWS) {
 #pragma unroll
-          for (int e = 0; e < 9; ++e) kk[9 * ii + e] = __ldcs(Kv + (27 * (ib + 1) + 9 * ii + e) * K_TILE);
+          for (int e = 0; e < 9; ++e) kk[9 * ii + e] = __ldcs(Kv + (9 * ROWS * (ib + 1) + 9 * ii + e) * K_TILE);
         }
       }
     }
@@ -524,11 +530,13 @@ unsigned grid_for(size_t n, int threads) {
 
 cudaError_t launch_tangent_apply(const rve_s* h, cudaStream_t s) {
   // one wave of resident blocks, no more than the voxels need
-  const int blocks = (int)std::min<size_t>((h->nvox + TAF_THREADS - 1) / TAF_THREADS, (size_t)TAF_BLOCKS * h->num_sms);
+  const size_t need = (h->nvox + TAF_THREADS - 1) / TAF_THREADS;
+  const bool small = need <= (size_t)TAF_SMALL * h->num_sms;
+  const int blocks = (int)std::min<size_t>(need, (size_t)TAF_LARGE * h->num_sms);
   {
     ProfScope ps_(h, RVE_K_TANGENT_APPLY, s);
-    launch_chained(h, k_tangent_apply, blocks, TAF_THREADS, 0, s, h->nvox, reinterpret_cast<const
-                   int2*>(h->K[h->cur]), h->kex[h->cur], h->r, h->p, h->t, h->dscal, h->partial_pkp());
+    launch_chained(h, small ? k_tangent_apply<TAF_SMALL, 9> : k_tangent_apply<TAF_LARGE, 3>, blocks, TAF_THREADS, 0, s, h->nvox,
+                   reinterpret_cast<const int2*>(h->K[h->cur]), h->kex[h->cur], h->r, h->p, h->t, h->dscal, h->partial_pkp());
     h->fold.pkp_blocks = blocks;
   }
   return cudaGetLastError();

@@ -88,3 +88,25 @@ def test_mixed_evaluation_is_the_fp64_one_with_a_rounded_tangent(pkg, case):
     K = b["TANGENT"]
     assert np.array_equal(K, K.astype(np.float32).astype(np.float64))
     assert np.all(np.abs(K - a["TANGENT"]) <= 2.0 ** -24 * np.abs(a["TANGENT"]) + 1e-10 * np.abs(a["TANGENT"]).max())
+
+
+@pytest.mark.parametrize("shape", [(1, 2, 2), (27, 36, 36), (27, 36, 48)])
+def test_tangent_apply_forms_reach_one_increment(pkg, shape):
+    """K in tiles of 256 voxels, the last one part full, on both sides of the
+    line between the two FP64 forms of the apply (38912 voxels): conjugate
+    gradients in FP64 and in mixed precision (staged and plain loads) reach the increment
+    that BiCGStab reaches with its own product K : p, to the 1e-9 of the other
+    comparisons of two converged increments."""
+    n2, n1, n0 = shape
+    wl = rvegen.WORKLOADS["cu16"]
+    gid, _ = rvegen.voronoi_grain_map(0, 4, 3, shape=(n0, n1, n2))
+    quat, mat = rvegen.random_quaternions(4, 5), rvegen.material("Cu")
+    out = []
+    for options in (dict(krylov=1), dict(), dict(precision=1), dict(precision=1, tma=0)):
+        g = pkg.RVE(gid, quat, mat, wl.edge, **options)
+        assert g.step(wl.dFbar(), rvegen.UNIAXIAL_X_MASK, np.zeros(9), wl.dt)["converged"]
+        out.append([g.field(k).reshape(gid.size, -1) for k in ("P", "F", "RHO_GND")])
+        g.close()
+    for other in out[1:]:
+        for a, b in zip(other, out[0]):
+            assert np.abs(a - b).max() <= 1e-9 * np.abs(b).max()
