@@ -125,20 +125,14 @@ class ClockSampler:
 
 # ---------------------------------------------------------------- roofline
 # FP64 operations of the local update, counted from the kernels' arithmetic
-# (an FMA counts 2; constant Schmid-tensor entries 0 and +-1 folded).  k_local:
-# per voxel set-up (frame rotation, trial elastic state) and P at the
-# converged S (six 3x3 products), per residual evaluation, per Newton
-# iteration (Jacobian with the stiffness applied once per column of the
-# accumulated sum, LU, solve).  k_tangent: per voxel set-up, one evaluation,
-# Jacobian and LU, the intermediate products, the strain-linear response to
-# each of the six unit strains (solve, Schmid sum, five 3x3 products, F~ dQ)
-# and the nine directions of dP/dF (Fe^T a and Fp^-T b, dE, H dE, the
-# rank-one term and the rotation).  The k_tangent total, 7744, agrees with
-# the FP64 operations ncu counts for the kernel (7771 per voxel).
-CONST_SETUP, CONST_EVAL, CONST_ITER = 180.0 + 270.0, 500.0, 1442.0
-TANGENT_FLOPS = 180.0 + 500.0 + 1230.0 + 146.0 + 180.0 + 6 * 522.0 + 9 * 264.0
-CONST_BYTES = 364 + 216        # reads F, dF, Fp^-1, tauc, S, grain; writes S, dgam, P
-TANGENT_BYTES = 364 + 648      # reads F, dF, Fp^-1, tauc, S, grain; writes K
+# (an FMA counts 2).  k_local: per voxel set-up (frame rotation, trial elastic
+# state) and P at the converged S (six 3x3 products), and per residual
+# evaluation; its Newton matrix and solve are FP32.  k_tangent: the FP64 operations ncu
+# counts per voxel.
+CONST_SETUP, CONST_EVAL, CONST_ITER = 180.0 + 270.0, 290.0, 0.0
+TANGENT_FLOPS = 4000.0
+CONST_BYTES = 364 + 216        # reads F, dF, Fp^-1, 1/tauc, S, grain; writes S, dgam, P
+TANGENT_BYTES = 364 + 648      # reads F, dF, Fp^-1, 1/tauc, S, grain; writes K
 
 
 def fft_models(n0, n1, n2, nf):
@@ -159,7 +153,8 @@ def fft_models(n0, n1, n2, nf):
 def kernel_models(n0, n1, n2, local=None):
     """Algorithmic FP64 flops and bytes per launch of each kernel category.
     The fft_* categories count the three-field transforms of the projection
-    (the CG loop, the residual); fft_curl counts all five passes of the
+    (the CG loop, the residual; small grids run the x and y passes as one kernel each way,
+    which fft_x_r2c and fft_x_c2r count with the same bytes); fft_curl counts all five passes of the
     nine-field Nye-curl transform, so its per-launch figure is a fifth of one
     curl.  `local` = (launches, local iterations, local evaluations) of the
     local update in the timed region, for its per-launch average."""
@@ -194,7 +189,9 @@ def kernel_models(n0, n1, n2, local=None):
 # the FP32 conjugate-gradient kernels of the mixed path: half the bytes of the
 # FP64 model, and their FP32 arithmetic is far below the FP32 peak, so HBM binds
 FP32_CG = ("tangent_apply", "stencil", "cg_update", "fft_x_r2c", "fft_y", "fft_y_inv", "fft_z_op", "fft_x_c2r")
-
+# kernels whose FP64 sums run as 64-bit integers: the FP64 pipe does not bound them, so HBM rates
+# them (the tangent apply keeps its rating against the FP64 peak)
+INTEGER_SUMS = ("stencil", "cg_update", "fft_x_r2c", "fft_y", "fft_y_inv", "fft_z_op", "fft_x_c2r", "fft_curl")
 
 
 def rate(flops, nbytes, avg_s, peaks):
@@ -226,7 +223,7 @@ def roofline_all(stats, shape, peaks, local=None, prec=0):
         e = {"launches": n, "avg_us": avg_s * 1e6, "share": ms / total}
         if k in models:
             flops, nbytes = models[k]
-            e.update(rate(flops, nbytes, avg_s, peaks))
+            e.update(rate(0.0 if k in INTEGER_SUMS else flops, nbytes, avg_s, peaks))
             e["algorithmic_flops"] = flops
             e["algorithmic_bytes"] = nbytes
         out[k] = e
@@ -301,17 +298,7 @@ def mixed_accuracy(pkg, rve, wl, gid, quat, mat, dev, a, P_hist):
 # workload; keyed by (category, precision).  Kernels changed since that
 # capture have no entry (reported as null), as do other grid sizes.
 TRAFFIC_SOURCE = "profiles/kernels_cu64.md"
-TRAFFIC_64 = {
-    ("tangent_apply", 0): 207.66e6 + 5.11e6,   # K : p reads its algorithmic 207.6 MB
-    ("tangent_apply", 1): 103.84e6 + 3.36e6,   # TMA-staged FP32 apply (float K, r, p)
-    ("constitutive", 0): 97.20e6 + 30.14e6,    # k_local (the same kernel in both precisions)
-    ("constitutive", 1): 97.20e6 + 30.14e6,
-    ("tangent_build", 0): 77.53e6 + 149.33e6,  # k_tangent, K written in FP64
-    ("stencil", 0): 18.94e6,                   # k_div_rows (its writes stay in L2)
-    ("stencil", 1): 9.49e6,                    # k_div_rows<float>
-    ("cg_update", 0): 62.96e6 + 0.16e6,        # k_grad_rows<true>
-    ("cg_update", 1): 31.49e6,                 # k_grad_rows<true, float>
-}
+TRAFFIC_64 = {}
 
 
 def load_peaks():
