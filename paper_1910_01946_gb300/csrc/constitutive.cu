@@ -792,9 +792,9 @@ __global__ void __launch_bounds__(LOCAL_THREADS, LOCAL_BLOCKS) k_local(
 // so the six unit strains are carried to the sample frame once (H = U B W^T, 9 x 6 in shared
 // memory) and each of the nine directions costs H dE.
 //
-// Bound by the FP64 pipe: 2.6 thousand instructions per voxel, against 4.9
+// Bound by the FP64 pipe (91 % of its cycles): 2.9 thousand instructions per voxel, against 4.9
 // thousand with the Schmid sums, the products of dQ and the rotation formed per
-// strain and per direction: 2.39 -> 1.43 ms at 64^3.
+// strain and per direction: 2.39 -> 1.40 ms at 64^3.
 constexpr int TAN_THREADS = 64;
 
 constexpr int TAN_BITS = 60;        // of an integer entry of K (high words below 2^28: see fixed_row in vec.cu)
