@@ -799,6 +799,50 @@ constexpr int TAN_THREADS = 64;
 
 constexpr int TAN_BITS = 60;        // of an integer entry of K (high words below 2^28: see fixed_row in vec.cu)
 
+// Exponent field of K's scale at one voxel: |K| < 2^(ek - 1022), the largest entry at least a quarter
+// of that; 0x7ff where K is not finite.  H, U, W and W S W^T bound an entry only to a factor of some 2^6, and
+// those bits would be missing from every entry, so the 81 entries are formed once in FP32
+// first: H, U and W as numbers below 2 of one scale each, the 486 FMAs on the FP32 pipe, idle here.
+// That sum errs by less than 2^-14 (six products below 8, each 5 parts of 2^-23 off, and
+// their additions): the 2^-13 on top of the largest.
+__device__ __forceinline__ float f32_scaled(double x, int up) {     // x 2^-up, truncated; below 2^-126: zero
+  const int hi = __double2hiint(x), lo = __double2loint(x), e = ((hi >> 20) & 0x7ff) - up;
+  const unsigned m = ((unsigned)(e - 896) << 23) | (unsigned)(hi & 0xfffff) << 3 | (unsigned)lo >> 29;
+  return __uint_as_float((e <= 896 ? 0u : m) | ((unsigned)hi & 0x80000000u));
+}
+__device__ __forceinline__ int tangent_exp(const double* H, const double* T, unsigned mH, unsigned mU, unsigned mW,
+                                           unsigned mQ) {
+  // (exponents of at least 128: zeros stay zeros in f32_scaled)
+  auto up = [](unsigned m) { return max((int)(m >> 20), 128) - 1023; };
+  const int uH = up(mH), uU = up(mU), uW = up(mW), hu = uH + uU + uW, c = max(hu, up(mQ));
+  const float sh = __int_as_float(max(hu - c + 127, 0) << 23);
+  float Hf[54], most = 0.0f;
+#pragma unroll
+  for (int k = 0; k < 54; ++k) Hf[k] = f32_scaled(H[k * TAN_THREADS], uH);
+#pragma unroll 1
+  for (int kl = 0; kl < 9; ++kl) {
+    const int kk = kl / 3, ll = kl % 3;
+    float u[3], w[3], q[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      u[i] = f32_scaled(T[(3 * kk + i) * TAN_THREADS], uU);
+      w[i] = f32_scaled(T[(9 + 3 * ll + i) * TAN_THREADS], uW);
+      q[i] = f32_scaled(T[(18 + 3 * ll + i) * TAN_THREADS], c);
+    }
+    const float dE[6] = {u[0] * w[0], u[1] * w[1], u[2] * w[2], 0.5f * fmaf(u[1], w[2], u[2] * w[1]),
+                         0.5f * fmaf(u[0], w[2], u[2] * w[0]), 0.5f * fmaf(u[0], w[1], u[1] * w[0])};
+#pragma unroll
+    for (int ij = 0; ij < 9; ++ij) {
+      float t = 0.0f;
+#pragma unroll
+      for (int m = 0; m < 6; ++m) t = fmaf(Hf[9 * m + ij], dE[m], t);
+      most = fmaxf(most, fabsf(fmaf(sh, t, ij / 3 == kk ? q[ij % 3] : 0.0f)));
+    }
+  }
+  const int ek = max(c + (__float_as_int(most + 0x1p-13f) >> 23) + 896, fix64::EXP_MIN);
+  return max(max(mU, mW), max(mQ, mH)) < 0x7ff00000u && ek < 0x7ff ? ek : 0x7ff;
+}
+
 __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
     const double* __restrict__ Fin, const double* __restrict__ xdir, double lambda,
@@ -879,8 +923,7 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
     }
     lu6(J, piv);
   }
-  // scale of the voxel's tangent: |K| <= |W S W^T| + 6 |H| |U| |W| in largest entries
-  unsigned mU = 0u, mW = 0u, mQ = 0u, mH = 0u;
+  unsigned mU = 0u, mW = 0u, mQ = 0u, mH = 0u;     // largest magnitudes, for the scale of K
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     mU = max(mU, fix64::mag(U[k]));
@@ -908,10 +951,6 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
       mH = max(mH, fix64::mag(P[ij]));
     }
   }
-  const bool finite = max(max(mU, mW), max(mQ, mH)) < 0x7ff00000u;
-  const int ek = min(max(max((int)(mH >> 20) + (int)(mU >> 20) + (int)(mW >> 20) - 2046 + 5, (int)(mQ >> 20)) + 1,
-                         fix64::EXP_MIN), 0x7fe);
-  if (!k32) kex[v] = finite ? fix64::out_base(ek, TAN_BITS) : fix64::EXP_BAD;
   // T is done with: its place takes U, W and W S W^T for the rolled loop over directions
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
@@ -919,6 +958,8 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
     T[(9 + k) * TAN_THREADS] = W[k];
     T[(18 + k) * TAN_THREADS] = Qs[k];
   }
+  const int ek = k32 ? 0 : tangent_exp(H, T, mH, mU, mW, mQ);
+  if (!k32) kex[v] = ek < 0x7ff ? fix64::out_base(ek, TAN_BITS) : fix64::EXP_BAD;
 #pragma unroll 1
   for (int kl = 0; kl < 9; ++kl) {
     const int kk = kl / 3, ll = kl % 3;

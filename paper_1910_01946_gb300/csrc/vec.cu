@@ -230,7 +230,7 @@ __global__ void __launch_bounds__(TA_TV, 1) k_tangent_apply32_tma(size_t nvox, c
 // k_tangent stores K as integers on one scale per voxel (kex), each split into a high word and a
 // signed low word, p becomes integers on the scale of its largest component, and three 32 x 32
 // multiply-adds per entry sum the high and the mixed products exactly (the low words' product, below
-// 2^-58 of the row's largest, is dropped).  K keeps 54 or more bits of the voxel's
+// 2^-58 of the row's largest, is dropped).  K keeps 58 or more bits of the voxel's
 // largest entry, p 56 of its largest component, against the 2^-53 of each FP64 FMA.  FP64 keeps p = r + beta p and p . t (18 FMAs).
 constexpr int TAF_P_BITS = 56, TAF_SHIFT = 7;
 

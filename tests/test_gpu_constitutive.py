@@ -77,6 +77,22 @@ def test_local_update_and_tangent_match_oracle(pkg, case):
     assert relerr(out["TANGENT"], K.reshape(-1, 81)) < 1e-10
 
 
+@pytest.mark.parametrize("case", ["one block", "past a block", "linear flow", "soft bulk"])
+def test_tangent_entries_resolve_the_largest_one_to_58_bits(pkg, case):
+    """K is kept as integers on one scale per voxel, the largest entry at 2^58
+    or more: half of the small entries (below 2^53 of those units, so exact as
+    doubles) have their lowest set bit in the last of them or the one above, 2^-58
+    or less of the power of two above the largest entry."""
+    K = evaluate(pkg, state(case))["TANGENT"]
+    top = np.frexp(np.abs(K).max(axis=1))[1][:, None]
+    m, e = np.frexp(K)
+    i = np.abs(m * 2.0 ** 53).astype(np.int64)
+    small = (i > 0) & (np.abs(K) <= np.ldexp(1.0, top - 8))
+    low = (e - 53 + np.log2(np.where(i > 0, i & -i, 1)) - top)[small]
+    assert low.size > 50
+    assert np.median(low) <= -58
+
+
 @pytest.mark.parametrize("case", ["one block", "past a block", "real exponent"])
 def test_mixed_evaluation_is_the_fp64_one_with_a_rounded_tangent(pkg, case):
     """FP32 rounding of the tangent: half a unit of the last place, 2^-24."""
