@@ -797,7 +797,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, LOCAL_BLOCKS) k_local(
 // strain and per direction: 2.39 -> 1.40 ms at 64^3.
 constexpr int TAN_THREADS = 64;
 
-constexpr int TAN_BITS = 60;        // of an integer entry of K (high words below 2^28: see fixed_row in vec.cu)
+constexpr int TAN_BITS = 60;        // of an integer entry of K (high words below 2^28: see fix64::row9)
 
 // Exponent field of K's scale at one voxel: |K| < 2^(ek - 1022), the largest entry at least a quarter
 // of that; 0x7ff where K is not finite.  H, U, W and W S W^T bound an entry only to a factor of some 2^6, and

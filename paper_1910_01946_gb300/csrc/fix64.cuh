@@ -120,4 +120,39 @@ __host__ __device__ inline void split_q62(F w, int* h, int* l) {
   *h = (int)((v - lo) >> 32);
 }
 
+// ---- rows of K : p ----
+// K: 60-bit integers on the voxel's scale (the largest entry at 2^58 or more), each as a signed low word
+// and a high word.  p: 56 bits on the scale of its largest component, as h 2^29 + l 2^-3, so that
+// three 32 x 32 multiply-adds per entry give the high and the mixed products exactly and the low
+// ones, which are dropped, are below 2^59: 2^-55 of max|K| max|p| at the usual 2^59 and 2^55.  (Split at
+// 32 bits they reached 2^62, and the row erred by more than nine FP64 FMAs; kept by a fourth
+// multiply-add the apply of 64^3 took 44.8 us for 43.4.)  Sums: 9 (2^28 2^31 + 2^31 2^27) < 2^63.
+constexpr int P_BITS = 56, ROW_SHIFT = 4;
+struct Vec9 { int h[9], l[9], e; };
+__device__ __forceinline__ void vec9(const double* p, Vec9& f) {
+  unsigned m = 0u;
+#pragma unroll
+  for (int c = 0; c < 9; ++c) m = max(m, mag(p[c]));
+  const int e = tile_exp(m);
+#pragma unroll
+  for (int c = 0; c < 9; ++c) {
+    const i64 v = to_fix(p[c], e + 63 - P_BITS);
+    f.l[c] = (int)((unsigned)v << 3);
+    f.h[c] = (int)(v >> 29) - (f.l[c] >> 31);
+  }
+  f.e = out_base(e, P_BITS);
+}
+// one row of K (entries `stride` apart, on the scale ek) times p
+__device__ __forceinline__ double row9(const int2* K, size_t stride, const Vec9& p, int ek) {
+  i64 hi = 0, mid = 0;
+#pragma unroll
+  for (int j = 0; j < 9; ++j) {
+    const int2 k = K[j * stride];                          // low (signed), high
+    hi += wide(k.y, p.h[j]);
+    mid += wide(k.y, p.l[j]) + wide(k.x, p.h[j]);
+  }
+  const int eb = max(ek, p.e) >= EXP_BAD / 2 ? EXP_BAD : ek + p.e - 1029;
+  return eb < 70 ? 0.0 : from_fix((hi << ROW_SHIFT) + (mid >> (32 - ROW_SHIFT)), eb);
+}
+
 }  // namespace fix64

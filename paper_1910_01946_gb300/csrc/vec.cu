@@ -226,38 +226,10 @@ __global__ void __launch_bounds__(TA_TV, 1) k_tangent_apply32_tma(size_t nvox, c
 
 // ---- FP64 tangent apply ----
 // The 81 FMAs of K : p per voxel take 41 us at 64^3 on the FP64 pipe (2 lanes per clock and SM), the
-// bytes (648 of K of 936 in all) 31, so the products are formed in fixed point on the integer pipes:
-// k_tangent stores K as integers on one scale per voxel (kex), each split into a high word and a
-// signed low word, p becomes integers on the scale of its largest component, and three 32 x 32
-// multiply-adds per entry sum the high and the mixed products exactly (the low words' product, below
-// 2^-58 of the row's largest, is dropped).  K keeps 58 or more bits of the voxel's
-// largest entry, p 56 of its largest component, against the 2^-53 of each FP64 FMA.  FP64 keeps p = r + beta p and p . t (18 FMAs).
-constexpr int TAF_P_BITS = 56, TAF_SHIFT = 7;
-
-// p of one voxel as split integers; returns their scale
-__device__ __forceinline__ int fixed_vector(const double* pv, fix64::Sp* pf) {
-  unsigned pm = 0u;
-#pragma unroll
-  for (int c = 0; c < 9; ++c) pm = max(pm, fix64::mag(pv[c]));
-  const int e = fix64::tile_exp(pm);
-#pragma unroll
-  for (int c = 0; c < 9; ++c) pf[c] = fix64::split(fix64::to_fix(pv[c], e + 63 - TAF_P_BITS));
-  return fix64::out_base(e, TAF_P_BITS);
-}
-// one row of K (entries `stride` apart, on the scale ek) times p (on the scale ep)
-__device__ __forceinline__ double fixed_row(const int2* K, size_t stride, const fix64::Sp* pf, int ek, int ep) {
-  using namespace fix64;
-  i64 hi = 0, mid = 0;
-#pragma unroll
-  for (int j = 0; j < 9; ++j) {
-    const int2 k = K[j * stride];                          // low (signed), high
-    hi += wide(k.y, pf[j].h);
-    mid += wide(k.y, pf[j].l) + wide(k.x, pf[j].h);
-  }
-  const int eb = max(ek, ep) >= EXP_BAD / 2 ? EXP_BAD : ek + ep - 1022 - TAF_SHIFT;
-  return eb < 70 ? 0.0 : from_fix((hi << TAF_SHIFT) + (mid >> (32 - TAF_SHIFT)), eb);
-}
-
+// bytes (648 of K of 936 in all) 31, so the products are formed in fixed point on the integer pipes
+// (fix64::row9): k_tangent stores K as integers on one scale per voxel (kex), p becomes integers on the
+// scale of its largest component.  FP64 keeps p = r + beta p and p . t (18 FMAs).
+//
 // p = r (first) or r + beta p; t = K : p; block sums of p . t (added up, and
 // alpha = rr / p . t formed, by launch_laplace_solve: see Fold).
 // Returns at once when the CG loop has converged (done != 0).
@@ -299,14 +271,14 @@ __global__ void __launch_bounds__(TAF_THREADS, BLOCKS) k_tangent_apply(size_t nv
       pv[k] = first ? rv : fma(beta, p[k * nvox + v], rv);
       p[k * nvox + v] = pv[k];
     }
-    fix64::Sp pf[9];
-    const int ep = fixed_vector(pv, pf);
+    fix64::Vec9 pf;
+    fix64::vec9(pv, pf);
 #pragma unroll
     for (int ib = 0; ib < 9 / ROWS; ++ib) {
 #pragma unroll
       for (int ii = 0; ii < ROWS; ++ii) {
         const int i = ROWS * ib + ii;
-        const double s = fixed_row(kk + 9 * ii, 1, pf, ek, ep);
+        const double s = fix64::row9(kk + 9 * ii, 1, pf, ek);
         t[i * nvox + v] = s;
         acc = fma(pv[i], s, acc);
         if (ib + 1 < 9 / ROWS) {
@@ -667,11 +639,12 @@ __global__ void __launch_bounds__(RVE_RED_THREADS, 2) k_kmul(size_t nvox, const 
 #pragma unroll
     for (int k = 0; k < 9; ++k) pv[k] = in[k * nvox + v];
     if (FIXED) {
-      fix64::Sp pf[9];
-      const int ep = fixed_vector(pv, pf), ek = kex[v];
+      fix64::Vec9 pf;
+      fix64::vec9(pv, pf);
+      const int ek = kex[v];
 #pragma unroll
       for (int i = 0; i < 9; ++i)
-        out[i * nvox + v] = fixed_row(reinterpret_cast<const int2*>(K) + k_at(v) + 9 * i * K_TILE, K_TILE, pf, ek, ep);
+        out[i * nvox + v] = fix64::row9(reinterpret_cast<const int2*>(K) + k_at(v) + 9 * i * K_TILE, K_TILE, pf, ek);
     } else {
       const float* Kf = reinterpret_cast<const float*>(K);
 #pragma unroll
