@@ -1233,13 +1233,9 @@ rve_status rve_get_fields(rve_t* h, uint32_t which, void* dst, size_t bytes, int
     case RVE_FIELD_DGAM: src = h->dgam[h->cur]; break;
     case RVE_FIELD_TANGENT:
       RVE_TRY(build_stale_tangent(h));
-      // stored as floats or as integers: as doubles into the caller's device memory, or by way of the
-      // other evaluation buffer
-      if (dst_is_device) {
-        RVE_CUDA(h, launch_tangent_values(h, static_cast<double*>(dst), h->stream));
-        RVE_CUDA(h, cudaStreamSynchronize(h->stream));
-        return RVE_OK;
-      }
+      // stored as floats or as integers: made doubles in the other evaluation buffer (rebuilt before it
+      // is next read) and copied from there, like every field: dst may have any alignment and may lie on
+      // another device
       RVE_CUDA(h, launch_tangent_values(h, h->K[1 - h->cur], h->stream));
       src = h->K[1 - h->cur];
       break;

@@ -126,3 +126,26 @@ def test_tangent_apply_forms_reach_one_increment(pkg, shape):
     for other in out[1:]:
         for a, b in zip(other, out[0]):
             assert np.abs(a - b).max() <= 1e-9 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("field", ["TANGENT", "P_EVAL", "DGAM"])
+def test_fields_go_to_device_memory_of_any_alignment(pkg, precision, field):
+    """Device destinations that start 8, 4 and 1 bytes past a 16-byte boundary get
+    the bytes that a host destination gets."""
+    import torch
+    gid, quat, mat, F, Fp = state("past a block")
+    g = pkg.RVE(gid, quat, mat, 2e-5, precision=precision)
+    g.set_field("F", F.reshape(gid.shape + (9,)))
+    g.set_field("FP", Fp.reshape(gid.shape + (9,)))
+    assert g.eval_constitutive(1.0)[1] == 0
+    which, nc = pkg.FIELDS[field]
+    n = nc * gid.size * 8
+    host = np.empty(n, dtype=np.uint8)
+    assert pkg.rve_get_fields(g.h, which, host.ctypes.data, n, 0) == pkg.RVE_OK
+    for shift in (0, 8, 4, 1):
+        dst = torch.zeros(n + 16, dtype=torch.uint8, device="cuda")
+        assert pkg.rve_get_fields(g.h, which, dst.data_ptr() + shift, n, 1) == pkg.RVE_OK
+        assert np.array_equal(dst[shift:shift + n].cpu().numpy(), host)
+        assert not dst[shift + n:].any() and not dst[:shift].any()
+    g.close()
