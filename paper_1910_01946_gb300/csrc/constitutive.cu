@@ -634,9 +634,111 @@ __device__ __forceinline__ void load_F(size_t nvox, size_t v, const double* __re
   if (Ft) mat3_tmul(R, FR, Ft);
 }
 
+// P = Fe S Fp^-T = F~ (Fp^-1 S Fp^-T) in the crystal frame, rotated to the
+// sample frame, with Fp^-1 = Fp_prev^-1 M^-1 (Eq. Piola)
+__device__ __forceinline__ void piola(const VoxelIn& in, const double* S, const double* Minv, double* P) {
+  double Fpinv[9], Sf[9], W[9], Q[9], Pt[9], U[9];
+  mat3_mul(in.Fpi0, Minv, Fpinv);
+  sym_full(S, Sf);
+  mat3_mult(Sf, Fpinv, W);
+  mat3_mul(Fpinv, W, Q);
+  mat3_mul(in.Ft, Q, Pt);
+  mat3_mult(Pt, in.R, U);
+  mat3_mul(in.R, U, P);
+}
+
+// Local Newton on S at one voxel with the exact Jacobian in FP64, factorised with pivoting
+__device__ __forceinline__ void local_voxel_fp64(size_t nvox, size_t v, const int32_t* __restrict__ grain,
+                                            const double* __restrict__ grainR, const double* __restrict__ Fin,
+                                            const double* __restrict__ xdir, double lambda,
+                                            const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
+                                            const double* __restrict__ Swarm, double* __restrict__ Sout,
+                                            double* __restrict__ dgout, double* __restrict__ Pout, double dt,
+                                            const Consts& c, int& iters, int& evals, int& failed) {
+  VoxelIn in;
+  load_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, in);
+  const double* A = in.A;
+  const double* tinv = in.tinv;      // 1 / tauc
+  double S[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) S[k] = Swarm[k * nvox + v];
+
+  Eval e;
+  evaluate(c, S, A, tinv, dt, e);
+  ++evals;
+  if (!(e.rn < INFINITY)) {             // warm start rejected: restart from the elastic-free state
+#pragma unroll
+    for (int k = 0; k < 6; ++k) S[k] = 0.0;
+    evaluate(c, S, A, tinv, dt, e);
+    ++evals;
+  }
+  double J[36], dgp[12];
+  int piv[6];
+  bool conv = e.rn <= c.local_tol_abs;
+  while (!conv && iters < c.max_local) {
+    jacobian(c, e, tinv, dt, J, dgp);
+    lu6(J, piv);
+    double d[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) d[k] = -e.r[k];
+    lu6_solve(J, piv, d);
+    double lam = 1.0;
+    bool acc = false;
+    for (int hv = 0; hv <= c.max_halvings; ++hv) {
+      double St[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) St[k] = fma(lam, d[k], S[k]);
+      Eval et;
+      evaluate(c, St, A, tinv, dt, et);
+      ++evals;
+      if (et.rn < e.rn) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) S[k] = St[k];
+        e = et;
+        acc = true;
+        break;
+      }
+      lam *= 0.5;
+    }
+    ++iters;
+    if (!acc) {                          // no decrease: round-off floor or failure
+      conv = e.rn <= c.floor_abs;
+      break;
+    }
+    conv = e.rn <= c.local_tol_abs;
+  }
+  failed = conv ? 0 : 1;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) Sout[k * nvox + v] = S[k];
+#pragma unroll
+  for (int a = 0; a < 12; ++a) dgout[a * nvox + v] = e.dg[a];
+  double P[9];
+  piola(in, S, e.Minv, P);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Pout[k * nvox + v] = P[k];
+}
+
+// The same for a voxel that local_voxel could not solve.  Where the compliance is close to singular or
+// the rank-one terms outweigh it by more than FP32 holds, its factorisation without pivoting breaks
+// down and no halved step is accepted: with C11 - C12 = 1e-7 C11 1247 of 4096 voxels failed that this solves.
+// A function of its own, so that the loop of the others keeps its registers.
+struct Again { int iters, evals, failed; };
+static __device__ __noinline__ Again local_voxel_again(size_t nvox, size_t v, const int32_t* __restrict__ grain,
+                                                     const double* __restrict__ grainR, const double* __restrict__ Fin,
+                                                     const double* __restrict__ xdir, double lambda,
+                                                     const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
+                                                     const double* __restrict__ Swarm, double* __restrict__ Sout,
+                                                     double* __restrict__ dgout, double* __restrict__ Pout, double dt,
+                                                     Consts c) {
+  Again a{0, 0, 0};
+  local_voxel_fp64(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c, a.iters,
+                   a.evals, a.failed);
+  return a;
+}
+
 // Local Newton on S at one voxel (data-dependent iteration counts): writes S,
-// dgam and P; returns the Newton iterations, residual evaluations and whether
-// it failed.  One residual call serves the warm start, the restart from the
+// dgam and P; returns the Newton iterations (`again`: those of a second try in FP64), residual
+// evaluations and whether it failed.  One residual call serves the warm start, the restart from the
 // elastic-free state, the trials and their halvings; the slips go to memory at every
 // evaluation, and F and R are read again for P, so that few registers live through the loop.
 __device__ __forceinline__ void local_voxel(size_t nvox, size_t v, const int32_t* __restrict__ grain,
@@ -645,7 +747,7 @@ __device__ __forceinline__ void local_voxel(size_t nvox, size_t v, const int32_t
                                             const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
                                             const double* __restrict__ Swarm, double* __restrict__ Sout,
                                             double* __restrict__ dgout, double* __restrict__ Pout, double dt,
-                                            const Consts& c, int& iters, int& evals, int& failed) {
+                                            const Consts& c, int& iters, int& again, int& evals, int& failed) {
   double A[6], tq[12], S[6], St[6];
   const double* Rg = grainR + 9 * grain[v];
   {
@@ -707,7 +809,13 @@ __device__ __forceinline__ void local_voxel(size_t nvox, size_t v, const int32_t
 #pragma unroll
     for (int k = 0; k < 6; ++k) St[k] = fma(lam, f64_of(d[k]), S[k]);
   }
-  failed = conv ? 0 : 1;
+  if (!conv) {
+    const Again a = local_voxel_again(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c);
+    again = a.iters;
+    evals += a.evals;
+    failed = a.failed;
+    return;
+  }
 #pragma unroll
   for (int k = 0; k < 6; ++k) Sout[k * nvox + v] = S[k];
   // P = F~ Q rotated to the sample frame = (F R) Q R^T, Q = Fp^-1 S Fp^-T,
@@ -754,13 +862,13 @@ __global__ void __launch_bounds__(LOCAL_THREADS, LOCAL_BLOCKS) k_local(
     chunk = __shfl_sync(full, chunk, 0);
     if (chunk >= nchunks) break;
     const size_t v = (size_t)chunk * 32 + lane;
-    int iters = 0, failed = 0, evals = 0;
+    int iters = 0, again = 0, failed = 0, evals = 0;
     if (v < nvox)
       local_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c,
-                  iters, evals, failed);
-    mx = max(mx, iters);
+                  iters, again, evals, failed);
+    mx = max(mx, max(iters, again));
     nf += failed;
-    si += (unsigned)iters;
+    si += (unsigned)(iters + again);
     se += (unsigned)evals;
   }
   // counters: warp-aggregated
@@ -993,90 +1101,6 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
 // rounded to FP32 (see curl_fp64.cu): the exact Jacobian's Newton path and the order of the products stay as they
 // are, so that the rounded values are the same bits.  3.05 and 2.43 ms at 64^3 within an increment, against
 // 1.07 and 1.44 ms above.
-
-// P = Fe S Fp^-T = F~ (Fp^-1 S Fp^-T) in the crystal frame, rotated to the
-// sample frame, with Fp^-1 = Fp_prev^-1 M^-1 (Eq. Piola)
-__device__ __forceinline__ void piola(const VoxelIn& in, const double* S, const double* Minv, double* P) {
-  double Fpinv[9], Sf[9], W[9], Q[9], Pt[9], U[9];
-  mat3_mul(in.Fpi0, Minv, Fpinv);
-  sym_full(S, Sf);
-  mat3_mult(Sf, Fpinv, W);
-  mat3_mul(Fpinv, W, Q);
-  mat3_mul(in.Ft, Q, Pt);
-  mat3_mult(Pt, in.R, U);
-  mat3_mul(in.R, U, P);
-}
-
-// Local Newton on S at one voxel, with the exact Jacobian
-__device__ __forceinline__ void local_voxel_fp64(size_t nvox, size_t v, const int32_t* __restrict__ grain,
-                                            const double* __restrict__ grainR, const double* __restrict__ Fin,
-                                            const double* __restrict__ xdir, double lambda,
-                                            const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
-                                            const double* __restrict__ Swarm, double* __restrict__ Sout,
-                                            double* __restrict__ dgout, double* __restrict__ Pout, double dt,
-                                            const Consts& c, int& iters, int& evals, int& failed) {
-  VoxelIn in;
-  load_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, in);
-  const double* A = in.A;
-  const double* tinv = in.tinv;      // 1 / tauc
-  double S[6];
-#pragma unroll
-  for (int k = 0; k < 6; ++k) S[k] = Swarm[k * nvox + v];
-
-  Eval e;
-  evaluate(c, S, A, tinv, dt, e);
-  ++evals;
-  if (!(e.rn < INFINITY)) {             // warm start rejected: restart from the elastic-free state
-#pragma unroll
-    for (int k = 0; k < 6; ++k) S[k] = 0.0;
-    evaluate(c, S, A, tinv, dt, e);
-    ++evals;
-  }
-  double J[36], dgp[12];
-  int piv[6];
-  bool conv = e.rn <= c.local_tol_abs;
-  while (!conv && iters < c.max_local) {
-    jacobian(c, e, tinv, dt, J, dgp);
-    lu6(J, piv);
-    double d[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) d[k] = -e.r[k];
-    lu6_solve(J, piv, d);
-    double lam = 1.0;
-    bool acc = false;
-    for (int hv = 0; hv <= c.max_halvings; ++hv) {
-      double St[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) St[k] = fma(lam, d[k], S[k]);
-      Eval et;
-      evaluate(c, St, A, tinv, dt, et);
-      ++evals;
-      if (et.rn < e.rn) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) S[k] = St[k];
-        e = et;
-        acc = true;
-        break;
-      }
-      lam *= 0.5;
-    }
-    ++iters;
-    if (!acc) {                          // no decrease: round-off floor or failure
-      conv = e.rn <= c.floor_abs;
-      break;
-    }
-    conv = e.rn <= c.local_tol_abs;
-  }
-  failed = conv ? 0 : 1;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) Sout[k * nvox + v] = S[k];
-#pragma unroll
-  for (int a = 0; a < 12; ++a) dgout[a * nvox + v] = e.dg[a];
-  double P[9];
-  piola(in, S, e.Minv, P);
-#pragma unroll
-  for (int k = 0; k < 9; ++k) Pout[k * nvox + v] = P[k];
-}
 
 __global__ void __launch_bounds__(128) k_local_fp64(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,

@@ -128,6 +128,21 @@ def test_tangent_apply_forms_reach_one_increment(pkg, shape):
             assert np.abs(a - b).max() <= 1e-9 * np.abs(b).max()
 
 
+@pytest.mark.parametrize("shear", [1e-7, 1e-9])
+def test_voxels_whose_fp32_direction_breaks_down_are_solved_in_fp64(pkg, shear):
+    """A lattice with almost no stiffness in one shear (C11 - C12 = 1e-7 and 1e-9
+    C11): the FP32 factorisation of the compliance plus the slip terms is no
+    descent direction, the FP64 one with pivoting solves every voxel.  Both
+    handles end at residuals of 10 local_tol mu = 4.5e-9 MPa or less, and an
+    error of S is no larger than its residual, within a factor 3 in P:
+    2.7e-8 MPa of 667."""
+    gid, quat, _, F, Fp = state("past a block")
+    args = gid, quat, rvegen.material("Cu", C11=120e3 * (1 + shear), C12=120e3, C44=75e3, mu=45e3), F, Fp
+    a, b = evaluate(pkg, args), evaluate(pkg, args, precision=1)
+    assert relerr(a["P_EVAL"], b["P_EVAL"]) < 5e-11
+    assert relerr(a["S_EVAL"], b["S_EVAL"]) < 5e-11
+
+
 @pytest.mark.parametrize("precision", [0, 1])
 @pytest.mark.parametrize("field", ["TANGENT", "P_EVAL", "DGAM"])
 def test_fields_go_to_device_memory_of_any_alignment(pkg, precision, field):
