@@ -1037,7 +1037,7 @@ __global__ void __launch_bounds__(128) k_fft_z_op(double2* __restrict__ spec, in
                                                   const int4* __restrict__ tw, OpTables T, SpecParams sp) {
   chain_wait();
   typedef double R;
-  __shared__ int red[4][MAX_WARPS * 32];
+  __shared__ int red[6][MAX_WARPS * 32];
   typedef Plain<double> S;
   C<R>* b0 = reinterpret_cast<C<R>*>(fft_smem);
   C<R>* b1 = b0 + cpb * pl.n;
@@ -1075,7 +1075,7 @@ __global__ void __launch_bounds__(128) k_fft_z_op(double2* __restrict__ spec, in
         u[f][m] = S::store(z, eb);
       }
   }
-  int key = 0;
+  int key[3] = {0, 0, 0};                         // (a scale per field: a component of a curl does not depend on all three)
   if (on) {
     const int ky = pc / nkx, kx = pc - ky * nkx;
 #pragma unroll
@@ -1084,13 +1084,14 @@ __global__ void __launch_bounds__(128) k_fft_z_op(double2* __restrict__ spec, in
         cplx X0 = cmk(u[0][m].x, u[0][m].y), X1 = cmk(u[1][m].x, u[1][m].y), X2 = cmk(u[2][m].x, u[2][m].y);
         apply_op(T, sp, row, kx, ky, tj + m * pl.T, X0, X1, X2);
         u[0][m] = st2(X0.x, X0.y); u[1][m] = st2(X1.x, X1.y); u[2][m] = st2(X2.x, X2.y);
-        key = max(key, max(S::key(u[0][m], 0), max(S::key(u[1][m], 0), S::key(u[2][m], 0))));
+#pragma unroll
+        for (int f = 0; f < 3; ++f) key[f] = max(key[f], S::key(u[f][m], 0));
       }
   }
-  const int E = S::scale(column_max<R>(key, cpb, red[3]), pl.bits), eb = E + pl.down;
 #pragma unroll
   for (int f = 0; f < 3; ++f) {
     __syncthreads();                              // the previous results are read
+    const int E = S::scale(column_max<R>(key[f], cpb, red[3 + f]), pl.bits), eb = E + pl.down;
     C<R> a[RMAX];
 #pragma unroll
     for (int m = 0; m < RMAX; ++m) a[m] = mk(S::work(u[f][m].x, 0, E, pl.bits), S::work(u[f][m].y, 0, E, pl.bits));

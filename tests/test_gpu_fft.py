@@ -185,3 +185,33 @@ def test_planes_in_one_block_and_above_the_line(pkg, shape):
     assert not torch.isfinite(Z[3:6]).any()
     assert torch.equal(Z[:3], Y[:3]) and torch.equal(Z[6:], Y[6:])
     r.close()
+
+
+@pytest.mark.parametrize("scheme", [0, 1])
+@pytest.mark.parametrize("shape", [(6, 12, 16), (27, 8, 64), (1, 6, 12)])
+def test_curl_components_see_only_the_fields_they_depend_on(pkg, scheme, shape):
+    """G_ij = -eps_jkl D_k Fp_il: component i0 does not depend on Fp_i0, which
+    may be 2^60 as large as the others or hold a NaN without a bit of G_i0
+    changing (each field's inverse transform has its own scale)."""
+    rng = np.random.default_rng(sum(shape))
+    Fp = np.eye(3) + 1e-3 * rng.standard_normal(shape + (3, 3))
+    r = handle(pkg, shape)
+
+    def nye(F):
+        r.set_field("FP", F.reshape(shape + (9,)))
+        assert pkg.load_library().rve_eval_nye(r.h, scheme) == pkg.RVE_OK
+        return r.field("NYE").reshape(-1, 3, 3)
+
+    G = nye(Fp)
+    for bad in (2.0 ** 60, np.nan):
+        for l in range(3):
+            F = Fp.copy()
+            F[..., 1, l] *= bad if bad == bad else 1.0
+            if bad != bad:
+                F[0, 1, 2, 1, l] = bad
+            H = nye(F)
+            assert np.array_equal(H[:, 1, l], G[:, 1, l]), (bad, l)
+            assert np.array_equal(H[:, [0, 2]], G[:, [0, 2]])
+            for j in (j for j in range(3) if j != l and shape != (1, 6, 12)):
+                assert not np.array_equal(H[:, 1, j], G[:, 1, j])
+    r.close()
