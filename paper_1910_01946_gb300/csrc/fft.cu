@@ -363,7 +363,7 @@ template <typename R> struct Plain {
   __device__ static int scale(int key, int B) { return sizeof(R) == 4 ? 0 : fix64::out_base(fix64::tile_exp((unsigned)key), B); }
   __device__ static i64 work(double x, int, int E, int B) {
     // (NaN tiles: any shift; their results are marked by E)
-    return fix64::to_fix(x, E >= fix64::EXP_BAD ? 0x7ff : E - 1);
+    return fix64::to_fix(x, E >= fix64::EXP_BAD ? 0x7ff : fix64::fix_shift(E));
   }
   __device__ static float work(float x, int, int, int) { return x; }
   // a result on the scale eb

@@ -10,9 +10,9 @@
 // replaces leaves in a sum of the tile's values), and integer additions are
 // exact.
 //
-// A tile that holds an infinity or a NaN gives NaN throughout; a tile whose
-// values lie below 2^-767 is taken as zero (a sum of it is below 2^-767
-// times the sum's terms, an absolute error no FP64 caller here can see).
+// A tile that holds an infinity or a NaN gives NaN throughout.  Scales go down to
+// that of values of 2^-959: smaller ones keep the bits above 2^-1016 (FP64 itself
+// keeps those above 2^-1074).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -21,8 +21,8 @@ namespace fix64 {
 
 typedef long long i64;
 
-constexpr int EXP_MIN = 256;          // smallest common exponent field used
-constexpr int EXP_SLOW = 2000;        // output exponent bases above this take the checked path
+constexpr int EXP_MIN = 64;           // smallest common exponent field used (zeros and denormals are shifted out)
+constexpr int EXP_SLOW = 1930;        // output exponent bases above this, or negative, take the checked path
 constexpr int EXP_BAD = 1 << 20;      // scale of values that an infinity or a NaN went into
 constexpr int EXP_ZERO = -(1 << 20);  // scale of exact zeros
 
@@ -51,28 +51,30 @@ __device__ __forceinline__ i64 to_fix(double x, int s0) {
 
 static __device__ __noinline__ double from_fix_checked(i64 v, int eb) {
   if (eb >= EXP_BAD / 2) return __hiloint2double(0x7ff80000, 0);    // an infinity or NaN went in
-  return scalbn((double)v, eb - 1086);                              // may overflow to infinity
+  return v ? scalbn((double)v, eb - 1016) : 0.0;                    // may overflow to infinity or underflow
 }
 
-// v on the scale given by eb (the exponent field of 2^63 on that scale) as
-// a double, rounded to nearest (ties away from zero)
+// v on the scale given by eb (70 less than the exponent field of 2^63 on that scale, so that
+// a result of a base of zero is still a normal number) as a double, rounded to nearest (ties away from zero)
 __device__ __forceinline__ double from_fix(i64 v, int eb) {
-  if (eb > EXP_SLOW) return from_fix_checked(v, eb);
+  if ((unsigned)eb > (unsigned)EXP_SLOW) return from_fix_checked(v, eb);
   const i64 s = v >> 63;
   const uint64_t a = (uint64_t)((v ^ s) - s);
   const int lz = __clzll((i64)a);
   const uint64_t n = a << (lz & 63);
   const uint64_t t = (n >> 11) + ((n >> 10) & 1u);                   // implicit bit at 2^52
-  int hi = (int)(t >> 32) + ((eb - 1 - lz) << 20);
+  int hi = (int)(t >> 32) + ((eb + 69 - lz) << 20);
   hi = a ? (hi | ((int)s & (int)0x80000000)) : 0;
   return __hiloint2double(hi, (int)t);
 }
 // exponent base of from_fix for integers on the scale to_fix(., e + 63 - B) gave, times 2^sh
 __device__ __forceinline__ int out_base(int e, int B, int sh = 0) {
-  return e == 0x7ff ? EXP_BAD : e + 64 - B + sh;
+  return e == 0x7ff ? EXP_BAD : e - 6 - B + sh;
 }
+// s0 of to_fix for the scale eb
+__device__ __forceinline__ int fix_shift(int eb) { return eb + 69; }
 
-// ---- integers already on a scale eb (v 2^(eb - 1086), |v| < 2^63) ----
+// ---- integers already on a scale eb (v 2^(eb - 1016), |v| < 2^63) ----
 // |v| < 2^(33 + top_bit(high(v)))
 __device__ __forceinline__ int abs_hi(i64 v) { const int h = (int)(v >> 32); return h ^ (h >> 31); }
 __device__ __forceinline__ int top_bit(int h) { return 31 - __clz(h); }
@@ -151,8 +153,8 @@ __device__ __forceinline__ double row9(const int2* K, size_t stride, const Vec9&
     hi += wide(k.y, p.h[j]);
     mid += wide(k.y, p.l[j]) + wide(k.x, p.h[j]);
   }
-  const int eb = max(ek, p.e) >= EXP_BAD / 2 ? EXP_BAD : ek + p.e - 1029;
-  return eb < 70 ? 0.0 : from_fix((hi << ROW_SHIFT) + (mid >> (32 - ROW_SHIFT)), eb);
+  const int eb = max(ek, p.e) >= EXP_BAD / 2 ? EXP_BAD : ek + p.e - 959;
+  return from_fix((hi << ROW_SHIFT) + (mid >> (32 - ROW_SHIFT)), eb);
 }
 
 }  // namespace fix64

@@ -158,7 +158,7 @@ struct rve_s {
   double *R, *x, *r, *p, *t, *q;
   double *bv, *bs;      // BiCGStab vectors v and s
   double2* spec;        // 9 * nspec
-  // scales of the integers of the three-field FP64 transforms (v 2^(ex - 1086), see fix64.cuh)
+  // scales of the integers of the three-field FP64 transforms (v 2^(ex - 1016), see fix64.cuh)
   struct {
     int* div;           // divergence: per tensor row and x line (i, z, y)
     int* x;             // spectra after the X pass: per field and line pair

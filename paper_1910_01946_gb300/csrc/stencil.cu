@@ -764,7 +764,7 @@ __global__ void __launch_bounds__(32 * RW) k_grad_fix(Grid3 g, int lanes, const 
     };
     auto zero_modes = [&]() {
 #pragma unroll
-      for (int j = 0; j < 3; ++j) offx[j] = fix64::to_fix(off[j], E - 1);
+      for (int j = 0; j < 3; ++j) offx[j] = fix64::to_fix(off[j], fix64::fix_shift(E));
     };
     // z pair and difference of the loaded row on the strip's scale, which moves up if need be
     auto take = [&](i64 (&s)[NPL], i64 (&m)[NPL]) {

@@ -48,7 +48,7 @@ def test_rows_of_the_tangent_product(lib, rows, spread):
     K = np.zeros((n, 9), dtype=object)
     words = np.zeros((n, 9, 2), dtype=np.int32)
     p = rng.uniform(-1.0, 1.0, (n, 9)) * 2.0 ** -rng.uniform(0, spread, (n, 9)) * 2.0 ** rng.integers(-80, 80, (n, 1))
-    ek = rng.integers(1000, 1100, n).astype(np.int32)
+    ek = rng.integers(930, 1030, n).astype(np.int32)
     for i in range(n):
         row = [int(x) for x in ROWS[rows](rng)]
         row[i % 9] = int(np.sign(row[i % 9]) or 1) * max(abs(row[i % 9]), 2 ** 58)   # the largest: 2^58 or more
@@ -58,7 +58,7 @@ def test_rows_of_the_tangent_product(lib, rows, spread):
     ptr = lambda a: a.ctypes.data_as(C.c_void_p)
     lib.rows9(n, ptr(words), ptr(ek), ptr(p), ptr(out))
     for i in range(n):
-        unit = Fraction(2) ** int(ek[i] - 1086)
+        unit = Fraction(2) ** int(ek[i] - 1016)
         exact = sum(K[i, j] * Fraction(float(p[i, j])) for j in range(9)) * unit
         big = max(abs(k) for k in K[i]) * unit * Fraction(float(np.abs(p[i]).max()))
         err = abs(Fraction(float(out[i])) - exact)
@@ -70,8 +70,30 @@ def test_non_finite_and_zero_rows(lib):
     p = np.ones((3, 9))
     p[0, 4] = np.nan
     p[1] = 0.0
-    ek = np.array([1040, 1040, 1 << 20], dtype=np.int32)
+    ek = np.array([970, 970, 1 << 20], dtype=np.int32)
     out = np.zeros(3)
     ptr = lambda a: a.ctypes.data_as(C.c_void_p)
     lib.rows9(3, ptr(words), ptr(ek), ptr(p), ptr(out))
     assert np.isnan(out[0]) and out[1] == 0.0 and np.isnan(out[2])
+
+
+def test_values_near_the_bottom_of_the_range(lib):
+    """A value of 2^-959 or more keeps 53 bits through 56-bit integers on its own
+    scale, a smaller one the bits above 2^-1016; results below the normal range
+    round to denormals.  K = 2^59 on the scale that makes it 1."""
+    rng = np.random.default_rng(5)
+    n = 2000
+    p = np.zeros((n, 9))
+    p[:, 4] = np.ldexp(rng.uniform(1.0, 2.0, n) * rng.choice([-1, 1], n), rng.integers(-1074, -700, n))
+    words = np.zeros((n, 9, 2), dtype=np.int32)
+    words[:, 4, 1] = 2 ** 27
+    ek = np.full(n, 1016 - 59, dtype=np.int32)
+    out = np.zeros(n)
+    ptr = lambda a: a.ctypes.data_as(C.c_void_p)
+    lib.rows9(n, ptr(words), ptr(ek), ptr(p), ptr(out))
+    x = p[:, 4]
+    assert np.all(np.abs(out - x) <= np.where(np.abs(x) >= 2.0 ** -959, 2.0 ** -53 * np.abs(x), 2.0 ** -1014))
+    words[:, 4, 1] = 2 ** 27 + 2 ** 26
+    ek[:] = 1016 - 59 - 200                                # 1.5 2^-200 times p
+    lib.rows9(n, ptr(words), ptr(ek), ptr(p), ptr(out))
+    assert np.all(np.abs(out - 1.5 * 2.0 ** -200 * x) <= 2.0 ** -52 * np.abs(out) + 2.0 ** -1074)

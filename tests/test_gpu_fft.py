@@ -215,3 +215,27 @@ def test_curl_components_see_only_the_fields_they_depend_on(pkg, scheme, shape):
             for j in (j for j in range(3) if j != l and shape != (1, 6, 12)):
                 assert not np.array_equal(H[:, 1, j], G[:, 1, j])
     r.close()
+
+
+@pytest.mark.parametrize("options", [dict(), dict(stencils=1)])
+@pytest.mark.parametrize("shape", [(6, 12, 16), (9, 18, 64), (3, 8, 144)])
+def test_small_fields_keep_their_digits(pkg, shape, options):
+    """The projections and the curl are linear down to the bottom of the FP64
+    range: fields of 2^-800 and 2^-920 give the scaled result (1e-13, the
+    tolerance at the top of the range)."""
+    import torch
+    X = np.random.default_rng(7).standard_normal(shape + (3, 3))
+    Xd = device_field(X)
+    r = pkg.RVE(np.zeros(shape, dtype=np.int32), np.array([[1.0, 0, 0, 0]]), rvegen.material("Cu"), 1e-5, **options)
+
+    def nye(x):
+        r.set_field("FP", x.reshape(9, -1).T.reshape(shape + (9,)).cpu().numpy())
+        r.eval_nye()
+        return torch.from_numpy(np.ascontiguousarray(r.field("NYE"))).cuda()
+
+    for run in (lambda x: r.project(MASK, x).clone(), lambda x: noalloc(pkg, shape, x), nye):
+        Y = run(Xd)
+        for k in (-800, -920):
+            Z = run(Xd * 2.0 ** k) * 2.0 ** -k
+            assert float((Z - Y).abs().max()) < 1e-13 * float(Y.abs().max()), k
+    r.close()
