@@ -28,6 +28,18 @@ def test_fp64_cg_kernels_are_alu_bound_and_fp32_ones_hbm_bound():
     assert abs(r32["achieved"] - r32["algorithmic_bytes"] / 27e-6 / 1e9) < 1e-6 * r32["achieved"]
 
 
+def test_printed_line_rates_the_integer_tangent_apply_by_its_bytes():
+    # 81 of its 99 products per voxel run on the integer pipes: at 43.6 us per launch of 64^3 it would be at
+    # 0.95 of the nominal FP64 peak and above the measured FMA rate, which it cannot be
+    b = bench()
+    assert set(b.INTEGER_SUMS) < set(b.ON_INTEGERS)
+    _, r = b.roofline({"tangent_apply": (100, 4.36)}, (64, 64, 64), {"hbm_gbs": 6783.8}, prec=0, integers=b.ON_INTEGERS)
+    assert r["bound"] == "hbm" and r["unit"] == "GB/s" and r["algorithmic_flops"] == 64 ** 3 * 198
+    assert abs(r["frac"] - 64 ** 3 * 117 * 8 / 43.6e-6 / 6783.8e9) < 1e-12
+    import inspect
+    assert inspect.getsource(b.main).count("integers=ON_INTEGERS") == 2
+
+
 def test_dominant_kernel_and_share():
     b = bench()
     stats = {"tangent_apply": (10, 0.8), "stencil": (10, 0.5), "constitutive": (0, 0.0)}
