@@ -128,6 +128,27 @@ def test_tangent_apply_forms_reach_one_increment(pkg, shape):
             assert np.abs(a - b).max() <= 1e-9 * np.abs(b).max()
 
 
+@pytest.mark.parametrize("precision", [0, 1])
+def test_tangent_of_a_step_is_the_oracles(pkg, precision):
+    """TANGENT after rve_step: the kernel the conjugate gradients of either precision read
+    from, at the increment's own state.  FP32 storage: half a unit of the last
+    place, 2^-24; the rest as in the other comparisons with the oracle (1e-10 of the largest)."""
+    wl = rvegen.Workload("cu8", 8, 5, "Cu", 0.004, 4, seed=31)
+    gid, quat, mat = wl.inputs()
+    g = pkg.RVE(gid, quat, mat, wl.edge, precision=precision)
+    o = solver.RVE(gid, quat, mat, wl.edge)
+    for _ in range(3):
+        o.Fp, o.rho_ssd = g.field("FP").reshape(-1, 3, 3).copy(), g.field("RHO_SSD").reshape(-1, 12).copy()
+        assert g.step(wl.dFbar(), rvegen.UNIAXIAL_X_MASK, np.zeros(9), wl.dt)["converged"]
+    tauc, _ = o.hardening()
+    K = o.constitutive(g.field("F").reshape(-1, 3, 3), tauc, np.zeros_like(o.S), wl.dt)[1].reshape(-1, 81)
+    out = g.field("TANGENT").reshape(-1, 81)
+    if precision:
+        assert np.array_equal(out, out.astype(np.float32).astype(np.float64))
+    assert np.all(np.abs(out - K) <= (2.0 ** -24 if precision else 0.0) * np.abs(K) + 1e-10 * np.abs(K).max())
+    g.close()
+
+
 @pytest.mark.parametrize("shear", [1e-7, 1e-9])
 def test_voxels_whose_fp32_direction_breaks_down_are_solved_in_fp64(pkg, shear):
     """A lattice with almost no stiffness in one shear (C11 - C12 = 1e-7 and 1e-9
