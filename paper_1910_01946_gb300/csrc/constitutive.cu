@@ -10,7 +10,8 @@
 //                  Eq. Piola) by Newton on the second Piola-Kirchhoff stress S;
 //   k_tangent      the consistent tangent dP/dF (Eq. linequil2ast).
 //   k_local_fp64, k_tangent_fp64: the same with FP64 Newton matrices, for
-//                  rve_eval_constitutive in mixed precision alone.
+//                  rve_eval_constitutive in mixed precision alone (its Newton iteration
+//                  is also the second try of a voxel that k_local cannot solve).
 //
 // Everything inside a voxel is done in its grain's crystal frame, where the
 // stiffness is cubic (three constants) and the Schmid tensors s (x) m are
@@ -1100,7 +1101,7 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
 // For rve_eval_constitutive on a mixed-precision handle, whose tangent is
 // rounded to FP32 (see curl_fp64.cu): the exact Jacobian's Newton path and the order of the products stay as they
 // are, so that the rounded values are the same bits.  3.05 and 2.43 ms at 64^3 within an increment, against
-// 1.07 and 1.44 ms above.
+// 0.98 and 1.40 ms above.
 
 __global__ void __launch_bounds__(128) k_local_fp64(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
@@ -1152,7 +1153,7 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent_fp64(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
     const double* __restrict__ Fin, const double* __restrict__ xdir, double lambda,
     const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g, const double* __restrict__ Sin,
-    double* __restrict__ Kout, double dt, Consts c, int k32) {
+    float* __restrict__ Kout, double dt, Consts c) {
   __shared__ double Hs[54 * TAN_THREADS];     // H[9 m + ij] of this thread at Hs[(9 m + ij) T + tid]
   double* H = Hs + threadIdx.x;
   const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1236,12 +1237,7 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent_fp64(
       mat3_mult(dPt, R, U);
       mat3_mul(R, U, dP);
 #pragma unroll
-      for (int ij = 0; ij < 9; ++ij) {
-        if (k32)   // mixed precision: the tangent only drives the FP32 conjugate gradients
-          reinterpret_cast<float*>(Kout)[k_at(v) + (9 * ij + kl) * K_TILE] = (float)dP[ij];
-        else
-          Kout[k_at(v) + (9 * ij + kl) * K_TILE] = dP[ij];
-      }
+      for (int ij = 0; ij < 9; ++ij) Kout[k_at(v) + (9 * ij + kl) * K_TILE] = (float)dP[ij];
     }
   }
 }
@@ -1547,7 +1543,7 @@ cudaError_t launch_constitutive(const rve_s* h, double dt, double lambda, int ou
     const unsigned blocks = (unsigned)((h->nvox + TAN_THREADS - 1) / TAN_THREADS);
     ProfScope ps_(h, RVE_K_TANGENT_BUILD, s);
     k_tangent_fp64<<<blocks, TAN_THREADS, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv, h->tinv,
-                                                  h->S[out_buf], h->K[out_buf], dt, h->cst, 1);
+                                                  h->S[out_buf], reinterpret_cast<float*>(h->K[out_buf]), dt, h->cst);
   }
   return cudaGetLastError();
 }

@@ -28,10 +28,11 @@
 // does 2 lanes per clock and SM and held every FP64 pass of a 64^3 grid to
 // 24-50 us, where the bytes need about 2.  A block takes the
 // largest magnitude of each transform's values, converts them to integers on that
-// scale with 57 or more bits (so that no sum of the transform can overflow),
+// scale with 56 or more bits (57 to 61 at every length but 288, 384 and 512; one less in the
+// inverse X pass; so that no sum of the transform can overflow),
 // and converts back on the way out.  Twiddles are Q62; a twiddled pass leaves the
 // values a factor 4 down (the high words of the products, no shift), which is about what its
-// sums grow by.  The rounding errors of a pass are 0.3 units of 2^-57 ...
+// sums grow by.  The rounding errors of a pass are 0.3 units of 2^-55 ...
 // 2^-53 of the transform's largest value, below the 2^-53 of each
 // intermediate value that every FP64 operation of a butterfly would leave.
 #include <algorithm>
@@ -873,7 +874,7 @@ struct OpTables {
 // value (see the X pass); the operators scale by SPEC_SCALE / nvox.
 constexpr double SPEC_SCALE = 0.5;
 
-// Inverse-Laplacian weight of OP_LAPINV at one frequency, with SPEC_SCALE:
+// Inverse-Laplacian weight at one frequency, with SPEC_SCALE:
 // SPEC_SCALE / (64 nvox sum_m s2_m prod_{j!=m} c2_j), 0 where it vanishes
 __device__ __forceinline__ double lapinv_weight(const OpTables& T, double inv_nvox, int kx, int ky, int kz) {
   const double sx = T.s20[kx], sy = T.s21[ky], sz = T.s22[kz];
@@ -937,7 +938,7 @@ __device__ __forceinline__ void apply_op(const OpTables& T, const SpecParams& sp
   X0 = Y0; X1 = Y1; X2 = Y2;
 }
 
-// the OP_LAPINV weight of every spectrum point (layout of one field's half
+// the inverse-Laplacian weight of every spectrum point (layout of one field's half
 // spectrum, [kz][ky][kx]), built once per handle; w32: its rounding to float
 // for the FP32 transforms (nullable)
 __global__ void k_lapinv_table(double* __restrict__ w, float* __restrict__ w32, OpTables T, int nkx, int n1, int n2,

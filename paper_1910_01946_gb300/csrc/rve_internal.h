@@ -28,7 +28,7 @@ struct FFTPlan {
 // (The inverse Laplacian of the stencil-factored projection, three fields each
 // multiplied by 1 / (64 nvox sum_m s2_m prod_{j!=m} c2_j), the inverse of D^H D
 // for the unscaled rotated-scheme stencils and 0 where it vanishes, is a pass of
-// its own: launch_fft_lapinv.)
+// its own, k_fft_z_lap: see launch_laplace_solve.)
 enum SpecOp { OP_PROJECT = 0, OP_CURL = 1, OP_CURL_STD = 2 };
 
 struct SpecParams {
@@ -285,7 +285,6 @@ cudaError_t launch_tangent_apply32(const rve_s* h, cudaStream_t s);
 cudaError_t vec_init();
 cudaError_t launch_cg_init32(const rve_s* h, double eta, cudaStream_t s);
 cudaError_t launch_widen_x(const rve_s* h, cudaStream_t s);
-cudaError_t launch_widen(const rve_s* h, const float* a, double* b, size_t n, cudaStream_t s);
 // the tangent K[cur] as doubles (81 * nvox)
 cudaError_t launch_tangent_values(const rve_s* h, double* dst, cudaStream_t s);
 // x_c -= mean(x_c) for the components whose bit is set (uses DS_XMEAN)

@@ -7,8 +7,8 @@
 //   (D_j f)(n)   = sum_{a in {0,1}^3} s_j(a) f(n + a),
 //   (D_j^T g)(n) = sum_{a in {0,1}^3} s_j(a) g(n - a),   s_j(a) = +1 if a_j = 1 else -1,
 // so the projection is a divergence stencil (9 fields -> 3), a scalar Laplace
-// solve in Fourier space (3 fields instead of 9: OP_LAPINV, which also
-// carries the two 1/(4h) factors), and a gradient stencil (3 -> 9), plus the
+// solve in Fourier space (3 fields instead of 9: launch_laplace_solve, whose weights also
+// carry the two 1/(4h) factors), and a gradient stencil (3 -> 9), plus the
 // zero mode of the mixed control (the stress-controlled components of the
 // mean are kept).  Identical to the Fourier-space projection up to round-off.
 #include "common.cuh"
@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(32 * RW) k_div_fix(Grid3 g, int lanes, const d
 // the scales exu of their line pairs.  SP = u(z) + u(z+1), SM = u(z+1) - u(z); YS = SP(y) + SP(y+1), YD = SP(y+1) -
 // SP(y), YM = SM(y) + SM(y+1); q_i0 = YS(x+1) - YS(x), q_i1 = YD(x) + YD(x+1),
 // q_i2 = YM(x) + YM(x+1).  CG as in k_grad_t.  Sums of eight values below
-// 2^GRAD_BITS and the zero mode.  vec: Y is 16-byte aligned.
+// 2^GRAD_BITS and the zero mode.
 constexpr int GRAD_BITS = 58;
 template <bool CG, int NPL>
 __global__ void __launch_bounds__(32 * RW) k_grad_fix(Grid3 g, int lanes, const i64* __restrict__ u,

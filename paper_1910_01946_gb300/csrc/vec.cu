@@ -619,14 +619,6 @@ cudaError_t launch_widen_x(const rve_s* h, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_widen(const rve_s* h, const float* a, double* b, size_t n, cudaStream_t s) {
-  {
-    ProfScope ps_(h, RVE_K_OTHER, s);
-    k_widen<<<RVE_RED_BLOCKS, RVE_RED_THREADS, 0, s>>>(n, a, b);
-  }
-  return cudaGetLastError();
-}
-
 // ---- BiCGStab support (FP64): w = K : v; fused dot products; linear combinations
 namespace {
 
