@@ -130,7 +130,7 @@ class ClockSampler:
 # evaluation; its Newton matrix and solve are FP32.  k_tangent: the FP64 operations ncu
 # counts per voxel.
 CONST_SETUP, CONST_EVAL, CONST_ITER = 180.0 + 270.0, 290.0, 0.0
-TANGENT_FLOPS = 302.0 + 2 * 1764.0 + 814.0
+TANGENT_FLOPS = 297.0 + 2 * 1764.0 + 814.0
 CONST_BYTES = 364 + 216        # reads F, dF, Fp^-1, 1/tauc, S, grain; writes S, dgam, P
 TANGENT_BYTES = 364 + 648      # reads F, dF, Fp^-1, 1/tauc, S, grain; writes K
 
@@ -301,12 +301,11 @@ def mixed_accuracy(pkg, rve, wl, gid, quat, mat, dev, a, P_hist):
 # capture have no entry (reported as null), as do other grid sizes.
 TRAFFIC_SOURCE = "profiles/kernels_cu64.md"
 TRAFFIC_64 = {
-    ("tangent_apply", 0): 208.71e6 + 4.95e6,   # k_tangent_apply
+    ("tangent_apply", 0): 208.70e6 + 5.12e6,   # k_tangent_apply
     ("tangent_apply", 1): 103.83e6 + 3.20e6,   # k_tangent_apply32_tma
-    ("constitutive", 0): 98.46e6 + 30.79e6,    # k_local (the same kernel in both precisions)
-    ("constitutive", 1): 97.38e6 + 31.30e6,
-    ("tangent_build", 0): 76.77e6 + 110.99e6,  # k_tangent (part of K is still in L2 at its end)
-    ("tangent_build", 1): 76.75e6 + 35.77e6,
+    ("constitutive", 0): 100.40e6 + 44.55e6,   # k_local (the same kernel in both precisions)
+    ("constitutive", 1): 100.40e6 + 44.55e6,
+    ("tangent_build", 0): 76.79e6 + 111.04e6,  # k_tangent (part of K is still in L2 at its end)
     ("stencil", 0): 18.91e6,                   # k_div_fix (its writes stay in L2)
     ("stencil", 1): 9.45e6,                    # k_div_rows<float>
     ("cg_update", 0): 62.98e6 + 1.71e6,        # k_grad_fix<true>

@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(TA_TV, 1) k_tangent_apply32_tma(size_t nvox, c
 // alpha = rr / p . t formed, by launch_laplace_solve: see Fold).
 // Returns at once when the CG loop has converged (done != 0).
 //
-// 55.3 -> 44.3 us at 64^3 (5.1 TB/s).  Plain loads, three rows of K in flight per thread: staged through
+// 55.3 -> 43.3 us at 64^3 (5.66 TB/s).  Plain loads, three rows of K in flight per thread: staged through
 // shared memory (bulk copies, two or four threads per voxel) it took 53, with the next voxel's rows
 // prefetched 49, with three blocks per SM 50.
 //
