@@ -152,7 +152,8 @@ typedef struct {
  * Last local evaluation (the converged one after rve_step, or the one made by
  * rve_eval_constitutive):
  *   P_EVAL: 9; S_EVAL: 6; DGAM: 12 (slip increments); TANGENT: 81
- *   (K_ijkl = dP_ij / dF_kl at component 27*i + 9*j + 3*k + l).  rve_step does
+ *   (K_ijkl = dP_ij / dF_kl at component 27*i + 9*j + 3*k + l; precision 0: to
+ *   2^-58 of the voxel's largest entry, precision 1: rounded to FP32).  rve_step does
  *   not build the tangent of the converged evaluation (no solve needs it); the
  *   first TANGENT request, or rve_eval_hardening, builds it from that state. */
 enum {
