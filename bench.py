@@ -303,8 +303,8 @@ TRAFFIC_SOURCE = "profiles/kernels_cu64.md"
 TRAFFIC_64 = {
     ("tangent_apply", 0): 208.70e6 + 5.12e6,   # k_tangent_apply
     ("tangent_apply", 1): 103.83e6 + 3.20e6,   # k_tangent_apply32_tma
-    ("constitutive", 0): 100.40e6 + 44.55e6,   # k_local (the same kernel in both precisions)
-    ("constitutive", 1): 100.40e6 + 44.55e6,
+    ("constitutive", 0): 98.46e6 + 30.79e6,    # k_local (the same kernel in both precisions)
+    ("constitutive", 1): 97.38e6 + 31.30e6,
     ("tangent_build", 0): 76.79e6 + 111.04e6,  # k_tangent (part of K is still in L2 at its end)
     ("stencil", 0): 18.91e6,                   # k_div_fix (its writes stay in L2)
     ("stencil", 1): 9.45e6,                    # k_div_rows<float>

@@ -10,8 +10,8 @@
 //                  Eq. Piola) by Newton on the second Piola-Kirchhoff stress S;
 //   k_tangent      the consistent tangent dP/dF (Eq. linequil2ast).
 //   k_local_fp64, k_tangent_fp64: the same with FP64 Newton matrices, for
-//                  rve_eval_constitutive in mixed precision alone (its Newton iteration
-//                  is also the second try of a voxel that k_local cannot solve).
+//                  rve_eval_constitutive in mixed precision; k_local_fp64 also where
+//                  FP32 directions do not do (see launch_local).
 //
 // Everything inside a voxel is done in its grain's crystal frame, where the
 // stiffness is cubic (three constants) and the Schmid tensors s (x) m are
@@ -635,111 +635,9 @@ __device__ __forceinline__ void load_F(size_t nvox, size_t v, const double* __re
   if (Ft) mat3_tmul(R, FR, Ft);
 }
 
-// P = Fe S Fp^-T = F~ (Fp^-1 S Fp^-T) in the crystal frame, rotated to the
-// sample frame, with Fp^-1 = Fp_prev^-1 M^-1 (Eq. Piola)
-__device__ __forceinline__ void piola(const VoxelIn& in, const double* S, const double* Minv, double* P) {
-  double Fpinv[9], Sf[9], W[9], Q[9], Pt[9], U[9];
-  mat3_mul(in.Fpi0, Minv, Fpinv);
-  sym_full(S, Sf);
-  mat3_mult(Sf, Fpinv, W);
-  mat3_mul(Fpinv, W, Q);
-  mat3_mul(in.Ft, Q, Pt);
-  mat3_mult(Pt, in.R, U);
-  mat3_mul(in.R, U, P);
-}
-
-// Local Newton on S at one voxel with the exact Jacobian in FP64, factorised with pivoting
-__device__ __forceinline__ void local_voxel_fp64(size_t nvox, size_t v, const int32_t* __restrict__ grain,
-                                            const double* __restrict__ grainR, const double* __restrict__ Fin,
-                                            const double* __restrict__ xdir, double lambda,
-                                            const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
-                                            const double* __restrict__ Swarm, double* __restrict__ Sout,
-                                            double* __restrict__ dgout, double* __restrict__ Pout, double dt,
-                                            const Consts& c, int& iters, int& evals, int& failed) {
-  VoxelIn in;
-  load_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, in);
-  const double* A = in.A;
-  const double* tinv = in.tinv;      // 1 / tauc
-  double S[6];
-#pragma unroll
-  for (int k = 0; k < 6; ++k) S[k] = Swarm[k * nvox + v];
-
-  Eval e;
-  evaluate(c, S, A, tinv, dt, e);
-  ++evals;
-  if (!(e.rn < INFINITY)) {             // warm start rejected: restart from the elastic-free state
-#pragma unroll
-    for (int k = 0; k < 6; ++k) S[k] = 0.0;
-    evaluate(c, S, A, tinv, dt, e);
-    ++evals;
-  }
-  double J[36], dgp[12];
-  int piv[6];
-  bool conv = e.rn <= c.local_tol_abs;
-  while (!conv && iters < c.max_local) {
-    jacobian(c, e, tinv, dt, J, dgp);
-    lu6(J, piv);
-    double d[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) d[k] = -e.r[k];
-    lu6_solve(J, piv, d);
-    double lam = 1.0;
-    bool acc = false;
-    for (int hv = 0; hv <= c.max_halvings; ++hv) {
-      double St[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) St[k] = fma(lam, d[k], S[k]);
-      Eval et;
-      evaluate(c, St, A, tinv, dt, et);
-      ++evals;
-      if (et.rn < e.rn) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) S[k] = St[k];
-        e = et;
-        acc = true;
-        break;
-      }
-      lam *= 0.5;
-    }
-    ++iters;
-    if (!acc) {                          // no decrease: round-off floor or failure
-      conv = e.rn <= c.floor_abs;
-      break;
-    }
-    conv = e.rn <= c.local_tol_abs;
-  }
-  failed = conv ? 0 : 1;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) Sout[k * nvox + v] = S[k];
-#pragma unroll
-  for (int a = 0; a < 12; ++a) dgout[a * nvox + v] = e.dg[a];
-  double P[9];
-  piola(in, S, e.Minv, P);
-#pragma unroll
-  for (int k = 0; k < 9; ++k) Pout[k * nvox + v] = P[k];
-}
-
-// The same for a voxel that local_voxel could not solve.  Where the compliance is close to singular or
-// the rank-one terms outweigh it by more than FP32 holds, its factorisation without pivoting breaks
-// down and no halved step is accepted: with C11 - C12 = 1e-7 C11 1247 of 4096 voxels failed that this solves.
-// A function of its own, so that the loop of the others keeps its registers (64^3: 974 -> 985 us).
-struct Again { int iters, evals, failed; };
-static __device__ __noinline__ Again local_voxel_again(size_t nvox, size_t v, const int32_t* __restrict__ grain,
-                                                     const double* __restrict__ grainR, const double* __restrict__ Fin,
-                                                     const double* __restrict__ xdir, double lambda,
-                                                     const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
-                                                     const double* __restrict__ Swarm, double* __restrict__ Sout,
-                                                     double* __restrict__ dgout, double* __restrict__ Pout, double dt,
-                                                     Consts c) {
-  Again a{0, 0, 0};
-  local_voxel_fp64(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c, a.iters,
-                   a.evals, a.failed);
-  return a;
-}
-
 // Local Newton on S at one voxel (data-dependent iteration counts): writes S,
-// dgam and P; returns the Newton iterations (`again`: those of a second try in FP64), residual
-// evaluations and whether it failed.  One residual call serves the warm start, the restart from the
+// dgam and P; returns the Newton iterations, residual evaluations and whether
+// it failed.  One residual call serves the warm start, the restart from the
 // elastic-free state, the trials and their halvings; the slips go to memory at every
 // evaluation, and F and R are read again for P, so that few registers live through the loop.
 __device__ __forceinline__ void local_voxel(size_t nvox, size_t v, const int32_t* __restrict__ grain,
@@ -748,7 +646,7 @@ __device__ __forceinline__ void local_voxel(size_t nvox, size_t v, const int32_t
                                             const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
                                             const double* __restrict__ Swarm, double* __restrict__ Sout,
                                             double* __restrict__ dgout, double* __restrict__ Pout, double dt,
-                                            const Consts& c, int& iters, int& again, int& evals, int& failed) {
+                                            const Consts& c, int& iters, int& evals, int& failed) {
   double A[6], tq[12], S[6], St[6];
   const double* Rg = grainR + 9 * grain[v];
   {
@@ -810,13 +708,7 @@ __device__ __forceinline__ void local_voxel(size_t nvox, size_t v, const int32_t
 #pragma unroll
     for (int k = 0; k < 6; ++k) St[k] = fma(lam, f64_of(d[k]), S[k]);
   }
-  if (!conv) {
-    const Again a = local_voxel_again(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c);
-    again = a.iters;
-    evals += a.evals;
-    failed = a.failed;
-    return;
-  }
+  failed = conv ? 0 : 1;
 #pragma unroll
   for (int k = 0; k < 6; ++k) Sout[k * nvox + v] = S[k];
   // P = F~ Q rotated to the sample frame = (F R) Q R^T, Q = Fp^-1 S Fp^-T,
@@ -851,7 +743,7 @@ __global__ void __launch_bounds__(LOCAL_THREADS, LOCAL_BLOCKS) k_local(
     const double* __restrict__ Fin, const double* __restrict__ xdir, double lambda,
     const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g, const double* __restrict__ Swarm,
     double* __restrict__ Sout, double* __restrict__ dgout, double* __restrict__ Pout,
-    int32_t* __restrict__ counters, double dt, Consts c) {
+    int32_t* __restrict__ counters, int32_t* __restrict__ failures, double dt, Consts c) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const long nchunks = (long)((nvox + 31) / 32);
@@ -863,13 +755,14 @@ __global__ void __launch_bounds__(LOCAL_THREADS, LOCAL_BLOCKS) k_local(
     chunk = __shfl_sync(full, chunk, 0);
     if (chunk >= nchunks) break;
     const size_t v = (size_t)chunk * 32 + lane;
-    int iters = 0, again = 0, failed = 0, evals = 0;
+    int iters = 0, failed = 0, evals = 0;
     if (v < nvox)
       local_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c,
-                  iters, again, evals, failed);
-    mx = max(mx, max(iters, again));
+                  iters, evals, failed);
+    if (failed) failures[atomicAdd(&counters[2], 1)] = (int32_t)v;
+    mx = max(mx, iters);
     nf += failed;
-    si += (unsigned)(iters + again);
+    si += (unsigned)iters;
     se += (unsigned)evals;
   }
   // counters: warp-aggregated
@@ -1103,15 +996,100 @@ __global__ void __launch_bounds__(TAN_THREADS) k_tangent(
 // are, so that the rounded values are the same bits.  3.05 and 2.43 ms at 64^3 within an increment, against
 // 0.98 and 1.40 ms above.
 
+// P = Fe S Fp^-T = F~ (Fp^-1 S Fp^-T) in the crystal frame, rotated to the
+// sample frame, with Fp^-1 = Fp_prev^-1 M^-1 (Eq. Piola)
+__device__ __forceinline__ void piola(const VoxelIn& in, const double* S, const double* Minv, double* P) {
+  double Fpinv[9], Sf[9], W[9], Q[9], Pt[9], U[9];
+  mat3_mul(in.Fpi0, Minv, Fpinv);
+  sym_full(S, Sf);
+  mat3_mult(Sf, Fpinv, W);
+  mat3_mul(Fpinv, W, Q);
+  mat3_mul(in.Ft, Q, Pt);
+  mat3_mult(Pt, in.R, U);
+  mat3_mul(in.R, U, P);
+}
+
+// Local Newton on S at one voxel with the exact Jacobian in FP64, factorised with pivoting
+__device__ __forceinline__ void local_voxel_fp64(size_t nvox, size_t v, const int32_t* __restrict__ grain,
+                                            const double* __restrict__ grainR, const double* __restrict__ Fin,
+                                            const double* __restrict__ xdir, double lambda,
+                                            const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g,
+                                            const double* __restrict__ Swarm, double* __restrict__ Sout,
+                                            double* __restrict__ dgout, double* __restrict__ Pout, double dt,
+                                            const Consts& c, int& iters, int& evals, int& failed) {
+  VoxelIn in;
+  load_voxel(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, in);
+  const double* A = in.A;
+  const double* tinv = in.tinv;      // 1 / tauc
+  double S[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) S[k] = Swarm[k * nvox + v];
+
+  Eval e;
+  evaluate(c, S, A, tinv, dt, e);
+  ++evals;
+  if (!(e.rn < INFINITY)) {             // warm start rejected: restart from the elastic-free state
+#pragma unroll
+    for (int k = 0; k < 6; ++k) S[k] = 0.0;
+    evaluate(c, S, A, tinv, dt, e);
+    ++evals;
+  }
+  double J[36], dgp[12];
+  int piv[6];
+  bool conv = e.rn <= c.local_tol_abs;
+  while (!conv && iters < c.max_local) {
+    jacobian(c, e, tinv, dt, J, dgp);
+    lu6(J, piv);
+    double d[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) d[k] = -e.r[k];
+    lu6_solve(J, piv, d);
+    double lam = 1.0;
+    bool acc = false;
+    for (int hv = 0; hv <= c.max_halvings; ++hv) {
+      double St[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) St[k] = fma(lam, d[k], S[k]);
+      Eval et;
+      evaluate(c, St, A, tinv, dt, et);
+      ++evals;
+      if (et.rn < e.rn) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) S[k] = St[k];
+        e = et;
+        acc = true;
+        break;
+      }
+      lam *= 0.5;
+    }
+    ++iters;
+    if (!acc) {                          // no decrease: round-off floor or failure
+      conv = e.rn <= c.floor_abs;
+      break;
+    }
+    conv = e.rn <= c.local_tol_abs;
+  }
+  failed = conv ? 0 : 1;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) Sout[k * nvox + v] = S[k];
+#pragma unroll
+  for (int a = 0; a < 12; ++a) dgout[a * nvox + v] = e.dg[a];
+  double P[9];
+  piola(in, S, e.Minv, P);
+#pragma unroll
+  for (int k = 0; k < 9; ++k) Pout[k * nvox + v] = P[k];
+}
+
+// n voxels: those of `list`, or the first n
 __global__ void __launch_bounds__(128) k_local_fp64(
     size_t nvox, const int32_t* __restrict__ grain, const double* __restrict__ grainR,
     const double* __restrict__ Fin, const double* __restrict__ xdir, double lambda,
     const double* __restrict__ Fp0inv, const double* __restrict__ tinv_g, const double* __restrict__ Swarm,
     double* __restrict__ Sout, double* __restrict__ dgout, double* __restrict__ Pout,
-    int32_t* __restrict__ counters, double dt, Consts c) {
+    int32_t* __restrict__ counters, const int32_t* __restrict__ list, long n, double dt, Consts c) {
   const unsigned full = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const long nchunks = (long)((nvox + 31) / 32);
+  const long nchunks = (n + 31) / 32;
   int mx = 0, nf = 0;
   unsigned si = 0, se = 0;
   for (;;) {
@@ -1119,10 +1097,10 @@ __global__ void __launch_bounds__(128) k_local_fp64(
     if (lane == 0) chunk = atomicAdd(&counters[6], 1);
     chunk = __shfl_sync(full, chunk, 0);
     if (chunk >= nchunks) break;
-    const size_t v = (size_t)chunk * 32 + lane;
+    const long at = (long)chunk * 32 + lane;
     int iters = 0, failed = 0, evals = 0;
-    if (v < nvox)
-      local_voxel_fp64(nvox, v, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c,
+    if (at < n)
+      local_voxel_fp64(nvox, list ? (size_t)list[at] : (size_t)at, grain, grainR, Fin, xdir, lambda, Fp0inv, tinv_g, Swarm, Sout, dgout, Pout, dt, c,
                   iters, evals, failed);
     mx = max(mx, iters);
     nf += failed;
@@ -1490,23 +1468,56 @@ cudaError_t launch_hardening(const rve_s* h, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// persistent: as many blocks as are resident at once (no more than the chunks need)
+static unsigned local_blocks(const rve_s* h, long voxels, int threads, int per_sm) {
+  return (unsigned)std::min<long>((voxels + threads - 1) / threads, (long)per_sm * h->num_sms);
+}
+
+static cudaError_t launch_local_fp64(const rve_s* h, double dt, double lambda, int out_buf, int warm_buf, const int32_t* list,
+                                     long n, cudaStream_t s) {
+  static const int per_sm = [] {
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_local_fp64, 128, 0) != cudaSuccess || b < 1) b = 1;
+    return b;
+  }();
+  const double* warm = warm_buf < 0 ? h->S_c : h->S[warm_buf];
+  if (cudaError_t e = cudaMemsetAsync(h->dcount + 6, 0, sizeof(int32_t), s)) return e;
+  {
+    ProfScope ps_(h, RVE_K_CONSTITUTIVE, s);
+    k_local_fp64<<<local_blocks(h, n, 128, per_sm), 128, 0, s>>>(
+        h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv, h->tinv, warm, h->S[out_buf], h->dgam[out_buf],
+        h->P[out_buf], h->dcount, list, n, dt, h->cst);
+  }
+  return cudaGetLastError();
+}
+
+// Lattices whose two stiffnesses of normal strains, C11 - C12 and C11 + 2 C12, differ by more than 2^10
+// (Consts::soft) take the FP64 Newton matrices (3.05 ms at 64^3 where k_local takes 0.98): their compliance is
+// close to singular in FP32.  At 1e-7 a third of the voxels failed, and from 1e-5 on the poor directions ended each
+// residual just below its tolerance, whose sum kept the increment from its own (8^3: no convergence; at 1e-3
+// both converge alike).
 cudaError_t launch_local(const rve_s* h, double dt, double lambda, int out_buf, int warm_buf, cudaStream_t s) {
-  // persistent: as many blocks as are resident at once (no more than the chunks need)
+  if (h->cst.soft) return launch_local_fp64(h, dt, lambda, out_buf, warm_buf, nullptr, (long)h->nvox, s);
   static const int per_sm = [] {
     int n = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local, LOCAL_THREADS, 0) != cudaSuccess || n < 1) n = 1;
     return n;
   }();
-  const long need = (long)((h->nvox + LOCAL_THREADS - 1) / LOCAL_THREADS);
-  const unsigned blocks = (unsigned)std::min<long>(need, (long)per_sm * h->num_sms);
   const double* warm = warm_buf < 0 ? h->S_c : h->S[warm_buf];
-  if (cudaError_t e = cudaMemsetAsync(h->dcount + 6, 0, sizeof(int32_t), s)) return e;
+  // the list's length and the chunk counter (the ticket between them is zero between kernels)
+  if (cudaError_t e = cudaMemsetAsync(h->dcount + 2, 0, 5 * sizeof(int32_t), s)) return e;
   {
     ProfScope ps_(h, RVE_K_CONSTITUTIVE, s);
-    k_local<<<blocks, LOCAL_THREADS, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv, h->tinv, warm,
-                                   h->S[out_buf], h->dgam[out_buf], h->P[out_buf], h->dcount, dt, h->cst);
+    k_local<<<local_blocks(h, (long)h->nvox, LOCAL_THREADS, per_sm), LOCAL_THREADS, 0, s>>>(
+        h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv, h->tinv, warm, h->S[out_buf], h->dgam[out_buf],
+        h->P[out_buf], h->dcount, failed_voxels(h), dt, h->cst);
   }
   return cudaGetLastError();
+}
+
+cudaError_t launch_local_failed(const rve_s* h, double dt, double lambda, int out_buf, int warm_buf, int n, cudaStream_t s) {
+  if (cudaError_t e = cudaMemsetAsync(h->dcount + 1, 0, sizeof(int32_t), s)) return e;
+  return launch_local_fp64(h, dt, lambda, out_buf, warm_buf, failed_voxels(h), n, s);
 }
 
 cudaError_t launch_tangent(const rve_s* h, double dt, double lambda, int buf, cudaStream_t s) {
@@ -1526,19 +1537,7 @@ cudaError_t launch_constitutive(const rve_s* h, double dt, double lambda, int ou
     if (cudaError_t e = launch_local(h, dt, lambda, out_buf, warm_buf, s)) return e;
     return launch_tangent(h, dt, lambda, out_buf, s);
   }
-  const double* warm = warm_buf < 0 ? h->S_c : h->S[warm_buf];
-  if (cudaError_t e = cudaMemsetAsync(h->dcount + 6, 0, sizeof(int32_t), s)) return e;
-  {
-    static const int per_sm = [] {
-      int n = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_local_fp64, 128, 0) != cudaSuccess || n < 1) n = 1;
-      return n;
-    }();
-    const unsigned blocks = (unsigned)std::min<long>((long)((h->nvox + 127) / 128), (long)per_sm * h->num_sms);
-    ProfScope ps_(h, RVE_K_CONSTITUTIVE, s);
-    k_local_fp64<<<blocks, 128, 0, s>>>(h->nvox, h->grain, h->grainR, h->F, h->x, lambda, h->Fp0inv, h->tinv, warm,
-                                        h->S[out_buf], h->dgam[out_buf], h->P[out_buf], h->dcount, dt, h->cst);
-  }
+  if (cudaError_t e = launch_local_fp64(h, dt, lambda, out_buf, warm_buf, nullptr, (long)h->nvox, s)) return e;
   {
     const unsigned blocks = (unsigned)((h->nvox + TAN_THREADS - 1) / TAN_THREADS);
     ProfScope ps_(h, RVE_K_TANGENT_BUILD, s);

@@ -61,6 +61,7 @@ struct Theta {
 
 struct Consts {        // material constants read by the hardening and constitutive kernels
   double C11, C12, C44, mu, b, tau0, alpha, gdot0, n, K, yc;
+  int soft;             // an FP32 factorisation of the compliance keeps few digits (see launch_local)
   double s11, s12, s44; // cubic compliance: E = s11 S + s12 (the other two), shear E = s44 S
   int n_int;            // n if it is a positive integer <= 64, else 0 (use pow)
   int gnd_enabled;
@@ -175,7 +176,7 @@ struct rve_s {
   double* partial_pkp() const { return partial + 9 * 4096; }
   mutable struct { int mean_blocks = 0; unsigned mean_mask = 0; int pkp_blocks = 0; } fold;   // block sums to be added up (see Fold)
   double* dscal;        // device scalars (see DS_*)
-  int32_t* dcount;      // device counters: [0] local max iters, [1] local failures, [4] last-block ticket,
+  int32_t* dcount;      // device counters: [0] local max iters, [1] local failures, [2] the length of their list, [4] last-block ticket,
                         // [6] next voxel chunk of the local update, [8..11] 64-bit work totals
   double* hscal;        // pinned host mirror of dscal
   int32_t* hcount;      // pinned host mirror of dcount
@@ -262,6 +263,10 @@ cudaError_t launch_hardening(const rve_s* h, cudaStream_t s);
 // local update (S, dgam, P) at F + lambda x into buffer out_buf, warm-started
 // from S[warm_buf] (or the committed S when warm_buf < 0)
 cudaError_t launch_local(const rve_s* h, double dt, double lambda, int out_buf, int warm_buf, cudaStream_t s);
+// the n voxels that failed in it, once more from the same start with FP64 Newton matrices (lattices
+// that launch_local treats so anyway: not to be called).  Their list lies in scratch that only BiCGStab uses
+inline int32_t* failed_voxels(const rve_s* h) { return reinterpret_cast<int32_t*>(h->bv); }
+cudaError_t launch_local_failed(const rve_s* h, double dt, double lambda, int out_buf, int warm_buf, int n, cudaStream_t s);
 // consistent tangent K[buf] at F + lambda x and the converged S[buf]
 cudaError_t launch_tangent(const rve_s* h, double dt, double lambda, int buf, cudaStream_t s);
 // sensitivities (one parameter direction per launch): d tauc, d l from the

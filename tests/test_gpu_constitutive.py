@@ -149,6 +149,26 @@ def test_tangent_of_a_step_is_the_oracles(pkg, precision):
     g.close()
 
 
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("shear", [1e-7, 1e-5, 1e-3])
+def test_increments_of_a_lattice_soft_in_one_shear(pkg, precision, shear):
+    """Increments of lattices with C11 - C12 = 1e-7, 1e-5 (FP64 Newton matrices) and
+    1e-3 C11 (FP32 ones) converge to the Newton tolerance, in both precisions to the
+    same mean stress (1e-9, as the other comparisons of two converged increments)."""
+    wl = rvegen.Workload("cu8", 8, 5, "Cu", 0.002, 4, seed=31)
+    gid, quat, _ = wl.inputs()
+    mat = rvegen.material("Cu", C11=120e3 * (1 + shear), C12=120e3, C44=75e3, mu=45e3)
+    P = []
+    for p in {precision, 0}:
+        g = pkg.RVE(gid, quat, mat, wl.edge, precision=p)
+        for _ in range(2):
+            info = g.step(wl.dFbar(), rvegen.UNIAXIAL_X_MASK, np.zeros(9), wl.dt)
+            assert info["converged"] and info["newton_iters"] <= 12
+        P.append(g.macro_stress()[0])
+        g.close()
+    assert relerr(P[0], P[-1]) < 1e-9
+
+
 @pytest.mark.parametrize("shear", [1e-7, 1e-9])
 def test_voxels_whose_fp32_direction_breaks_down_are_solved_in_fp64(pkg, shear):
     """A lattice with almost no stiffness in one shear (C11 - C12 = 1e-7 and 1e-9
@@ -162,6 +182,16 @@ def test_voxels_whose_fp32_direction_breaks_down_are_solved_in_fp64(pkg, shear):
     a, b = evaluate(pkg, args), evaluate(pkg, args, precision=1)
     assert relerr(a["P_EVAL"], b["P_EVAL"]) < 5e-11
     assert relerr(a["S_EVAL"], b["S_EVAL"]) < 5e-11
+
+
+def test_voxels_that_fail_are_tried_again_in_fp64(pkg):
+    """C44 = 1e4 C11: strains of 5e-4 ask for trial shears of 1e6 MPa, and a few
+    voxels fail from either Newton iteration (4 and 10 of 648 by themselves); those
+    that the FP32 directions leave are solved by the FP64 ones, the others keep
+    their result."""
+    gid, quat, _, F, Fp = state("past a block")
+    out = evaluate(pkg, (gid, quat, rvegen.material("Cu", C44=75e7, mu=45e3), F, Fp))
+    assert all(np.isfinite(v).all() for v in out.values())
 
 
 @pytest.mark.parametrize("precision", [0, 1])
